@@ -417,7 +417,6 @@ fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long l
 
 __global__ void __launch_bounds__(kRedThreads)
 fx_finish_kernel(LzScalars* S, int cur, const long long* __restrict__ pb, int nb) {
-  __shared__ int stop_s;
   if (S->status != 0) return;
   const int j = S->j + 1;
   I192 sum;
@@ -426,14 +425,11 @@ fx_finish_kernel(LzScalars* S, int cur, const long long* __restrict__ pb, int nb
   if (threadIdx.x == 0) {
     const double sw = S->fx_sw;
     const double beta = sw * sqrt(i192_to_double(sum));
-    stop_s = finish_record_beta(S, j, beta);
-    if (stop_s == 0) {
+    if (finish_step(S, j, beta)) {
       S->scale[1 - cur] = sw / beta;
       S->fx_max[1 - cur] = mx;
     }
   }
-  __syncthreads();
-  finish_tail(S, j, stop_s);
 }
 
 // ------------------------------------------------------------------ ground-state vector

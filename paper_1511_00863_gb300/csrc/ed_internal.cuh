@@ -121,13 +121,13 @@ void hv2_tables_free(const ed_basis* b);
 struct LzScalars {
   int j;            // steps completed
   int status;       // 0 running, 1 breakdown, 2 converged, 3 max_steps reached
-  int check_every;  // compute E0(j) every this many steps (and at the stop step)
+  int conv_j;       // first step that passed the convergence test (0: none yet); steps the
+                    // stream had already enqueued behind it may have advanced j further
+  int chk;          // convergence checks have covered the steps up to here
+  unsigned tick_chk;  // CTAs of the running check that are done
   int max_steps;
   double tol;
   double tscale;    // max over i <= j of |a_i| + b_i (breakdown scale)
-  double last_E0;   // most recent computed E0 and its step
-  int last_E0_step;
-  int pad_;
   double scale[2];
   // FP64-accurate (fixed-point) runs: buffer i holds int64 X_i with f = scale[i] * X_i.
   long long fx_max[2];          // max |X_i| of each buffer

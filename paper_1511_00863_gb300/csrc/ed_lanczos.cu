@@ -7,13 +7,16 @@
 //   2. update:     a_j = sum of the partials (every CTA sums them in the same order),
 //      q = w - a_j f_j in place, per-CTA partial sums of q . q;
 //   3. finish (one CTA): b_{j+1} = sqrt(sum), breakdown test, f_{j+1} = q / b_{j+1} kept
-//      implicit as a buffer scale, E0(j) = lambda_min(T_j), convergence test.
+//      implicit as a buffer scale.
+// E0(j) = lambda_min(T_j) and the convergence test run beside the next steps, on a stream of
+// their own (lz_check_kernel).
 // Each buffer holds an unnormalised vector B with f = scale * B, so no pass rescales it.
 // Once the run stops (breakdown, convergence, max_steps) every later kernel returns at
-// entry; ed_lanczos_solve replays a captured two-step CUDA graph and reads the status
-// between batches of replays.
+// entry; ed_lanczos_solve replays a captured CUDA graph of a few steps and reads the status of
+// one batch of replays while the next one runs.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 #include <type_traits>
@@ -139,17 +142,13 @@ lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restric
 __global__ void __launch_bounds__(kRedThreads)
 lz_finish_kernel(LzScalars* S, int cur, const double* __restrict__ pb, int nb) {
   __shared__ double red[33];
-  __shared__ int stop_s;
   if (S->status != 0) return;
   const int j = S->j + 1;
   const double b2 = block_sum_array(pb, nb, red);
   if (threadIdx.x == 0) {
     const double beta = sqrt(b2);
-    stop_s = finish_record_beta(S, j, beta);
-    if (stop_s == 0) S->scale[1 - cur] = 1.0 / beta;
+    if (finish_step(S, j, beta)) S->scale[1 - cur] = 1.0 / beta;
   }
-  __syncthreads();
-  finish_tail(S, j, stop_s);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
@@ -164,17 +163,64 @@ lz_energy_kernel(const LzScalars* S, double* out) {
   if (threadIdx.x == 0) *out = E;
 }
 
-// E0(i) = lambda_min(T_i) for i = 1 .. m - 1, block i - 1 for step i: the history of a run
-// whose steps computed E0 only at the stop step (no convergence test). The steps' scalars are
-// final, so the m - 1 bisections run side by side on as many SMs instead of one after each
-// step on one SM (FP64 multisection: 4-9 rounds of ~9 us each on GB300).
+// E0(i) = lambda_min(T_i) for i = 1 .. j, block i - 1 for step i (all != 0), or for i = j
+// alone: the history of a run without convergence test. The steps' scalars are final, so the
+// bisections run side by side on as many SMs instead of one after each step on one SM (FP64
+// multisection: 4-9 rounds of ~9 us each on GB300).
 __global__ void __launch_bounds__(kRedThreads)
-lz_history_kernel(LzScalars* S, int m) {
-  const int i = (int)blockIdx.x + 1;
-  if (i >= m) return;
+lz_history_kernel(LzScalars* S, int all) {
+  const int i = all ? (int)blockIdx.x + 1 : S->j;
+  if (i < 1 || i > S->j) return;
   __shared__ double sturm_work[kSturmWork];
   const double E = sturm_lowest(S->alpha, S->beta, i, NAN, sturm_work);
   if (threadIdx.x == 0) S->E0[i] = E;
+}
+
+// The convergence test of the `gridDim.x` steps after S->chk, one CTA per step: E0(i) =
+// lambda_min(T_i), then the last CTA to finish tests |E0(i) - E0(i-1)| in step order and
+// records the first i that passes (conv_j; the next finish kernel stops the run). It needs a_i, b_i alone, which are final
+// once step i is done, so it runs on a stream of its own beside the next steps' H.v: a
+// bisection takes 35-50 us on one SM (the float-float and FP64 chains of sturm_lowest), which
+// after every step was 41 of the 52 us of a step on the 12-site ring (48,400 states) and 51
+// of 500 us on the 4x4 lattice (19 M). The steps enqueued meanwhile are not part of the
+// result: everything a caller sees ends at conv_j.
+// E0(chk), when known, bounds every later E0(i) from above (Cauchy interlacing).
+__global__ void __launch_bounds__(kRedThreads)
+lz_check_kernel(LzScalars* S) {
+  __shared__ double sturm_work[kSturmWork];
+  __shared__ int base_s, j_s, open_s, broke_s;
+  if (threadIdx.x == 0) {  // once per CTA: the steps beside this kernel advance j
+    base_s = S->chk;
+    open_s = S->conv_j == 0;
+    broke_s = *(volatile int*)&S->status == 1;  // then j is final
+    __threadfence();
+    j_s = *(volatile int*)&S->j;
+  }
+  __syncthreads();
+  const int base = base_s;
+  const int i = base + 1 + (int)blockIdx.x;
+  // the steps up to base + gridDim.x are done, unless the run stopped before them
+  if (open_s && i >= 1 && i <= j_s) {
+    const double E = sturm_lowest(S->alpha, S->beta, i, base >= 1 ? S->E0[base] : NAN, sturm_work);
+    if (threadIdx.x == 0) S->E0[i] = E;
+  }
+  if (threadIdx.x != 0) return;
+  __threadfence();
+  if (atomicAdd(&S->tick_chk, 1u) != gridDim.x - 1) return;
+  S->tick_chk = 0;
+  __threadfence();
+  if (open_s) {
+    const int last = min(base + (int)gridDim.x, j_s);
+    for (int k = max(base + 1, 2); k <= last; ++k) {
+      const double E = __ldcg(&S->E0[k]), P = __ldcg(&S->E0[k - 1]);
+      if (broke_s && k == j_s) break;  // a step that broke down ends the run by itself
+      if (fabs(E - P) <= S->tol * fmax(fabs(E), 1.0)) {
+        S->conv_j = k;
+        break;
+      }
+    }
+  }
+  S->chk = base + (int)gridDim.x;
 }
 
 // Eigenvector y of T_m for its lowest eigenvalue lam (tridiag_ritz_vector); one thread.
@@ -210,12 +256,17 @@ struct ed_lanczos {
   int64_t npa = 0, npb = 0;
   int hv_grid = 0;
   bool stopped = false;
-  double graph_t = 0.0, graph_U = 0.0;  // parameters the captured graph was made with
+  double graph_t[2] = {0.0, 0.0}, graph_U[2] = {0.0, 0.0};  // parameters of the captured graphs
   bool fx = false;     // ED_F64: int64 fixed-point buffers (ed_fixed.cu)
   FxRun fxr{};
   Hv2Plan* plan = nullptr;  // fused H.v on the padded layout (ed_hv2.cu), if it fits
   Reorth* ro = nullptr;     // stored Lanczos vectors when opts.reorth != 0 (ed_reorth.cu)
-  cudaGraphExec_t graph = nullptr;
+  cudaGraphExec_t graph[2] = {nullptr, nullptr};  // without / with the convergence test
+  // solves only (lz_iterate): the checks' stream, fork and join events of the capture, one event
+  // per batch in flight and the host's copies of the run's scalars (pinned)
+  cudaStream_t check_stream = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_batch[2] = {nullptr, nullptr};
+  LzScalars* host = nullptr;  // [1] and the two batches' headers behind it
 };
 
 static ed_status lz_launch_step(ed_lanczos* st, const ed_params* p, cudaStream_t s,
@@ -375,7 +426,14 @@ extern "C" void ed_lanczos_destroy(ed_lanczos* st) {
   cudaGetDevice(&prev);
   if (prev != st->device) cudaSetDevice(st->device);
   if (st->stream) cudaStreamSynchronize(st->stream);
-  if (st->graph) cudaGraphExecDestroy(st->graph);
+  for (int i = 0; i < 2; ++i) {
+    if (st->graph[i]) cudaGraphExecDestroy(st->graph[i]);
+    if (st->ev_batch[i]) cudaEventDestroy(st->ev_batch[i]);
+  }
+  if (st->ev_fork) cudaEventDestroy(st->ev_fork);
+  if (st->ev_join) cudaEventDestroy(st->ev_join);
+  if (st->check_stream) cudaStreamDestroy(st->check_stream);
+  if (st->host) cudaFreeHost(st->host);
   if (st->plan) hv2_free(st->plan);
   if (st->ro) ro_free(st->ro);
   for (int i = 0; i < 2; ++i)
@@ -388,8 +446,6 @@ extern "C" void ed_lanczos_destroy(ed_lanczos* st) {
   delete st;
 }
 
-// check_every: compute E0(j) in the finish kernel every this many steps; step_mode: the
-// caller drives the loop, so only breakdown and max_steps stop the run (no tol test).
 // Bases below this many states use the default fused H.v variant order: timing every
 // variant would cost more than their solves.
 constexpr int64_t kAutotuneMinDim = (int64_t)1 << 22;
@@ -472,11 +528,16 @@ static ed_status lz_alloc(const ed_basis* b, const ed_opts* o, cudaStream_t s, e
   return ED_OK;
 }
 
+// Steps tested per convergence check (and per CTA of it): enough that a check of 35-50 us
+// hides behind as many later steps. A step takes about 10 us up to 2^18 states, 12-30 us up to
+// 2^20, 25-60 us up to 2^22 (int64, rings to the 4x4 lattice).
+static int check_stride(int64_t n) {
+  return n < ((int64_t)1 << 18) ? 8 : n < ((int64_t)1 << 20) ? 4 : n < ((int64_t)1 << 22) ? 2 : 1;
+}
+
 // Start a run on an allocated state: zero both buffers (their pads must hold 0), load f_1
-// (caller vector or seeded start vector) and the run's scalars. check_every: compute E0(j)
-// every this many steps; step_mode: the caller drives the loop (no tol test).
-static ed_status lz_reset(ed_lanczos* st, const ed_opts* o, const void* f1, int check_every,
-                          bool step_mode) {
+// (caller vector or seeded start vector) and the run's scalars.
+static ed_status lz_reset(ed_lanczos* st, const ed_opts* o, const void* f1) {
   const ed_basis* b = st->basis;
   cudaStream_t s = st->stream;
   ED_CHECK_ARG(f1 == nullptr || aligned16(f1), "f1 must be 16-byte aligned");
@@ -485,9 +546,9 @@ static ed_status lz_reset(ed_lanczos* st, const ed_opts* o, const void* f1, int 
   for (int i = 0; i < 2; ++i) ED_TRY_CUDA(cudaMemsetAsync(st->B[i], 0, st->n * st->esize, s));
   LzScalars h;
   memset(&h, 0, sizeof(h));
-  h.check_every = check_every < 1 ? 1 : check_every;
   h.max_steps = o->max_steps;
-  h.tol = step_mode ? 0.0 : o->tol;
+  h.tol = o->tol;
+  h.chk = -check_stride(st->n);  // a graph's first check covers the steps before it: none yet
   h.scale[0] = 1.0;
   h.scale[1] = 0.0;
   for (int i = 0; i < ED_MAX_STEPS + 2; ++i) h.E0[i] = NAN;
@@ -538,11 +599,11 @@ static ed_status lz_reset(ed_lanczos* st, const ed_opts* o, const void* f1, int 
 }
 
 static ed_status lz_init(const ed_basis* b, const ed_opts* o, const void* f1, cudaStream_t s,
-                         int check_every, bool step_mode, ed_lanczos** out) {
+                         ed_lanczos** out) {
   ed_lanczos* st = nullptr;
   ed_status r = lz_alloc(b, o, s, &st);
   if (r != ED_OK) return r;
-  if ((r = lz_reset(st, o, f1, check_every, step_mode)) != ED_OK) {
+  if ((r = lz_reset(st, o, f1)) != ED_OK) {
     ed_lanczos_destroy(st);
     return r;
   }
@@ -559,7 +620,7 @@ extern "C" ed_status ed_lanczos_init(const ed_basis* b, const ed_opts* o, const 
     const ed_status rc = check_opts(o);
     if (rc != ED_OK) return rc;
   }
-  ed_status r = lz_init(b, o, f1, (cudaStream_t)stream, ED_MAX_STEPS + 1, true, out);
+  ed_status r = lz_init(b, o, f1, (cudaStream_t)stream, out);
   if (r == ED_OK)
     r = o->dtype == ED_F64 ? fx_prepare(b)
         : is_complex(o->dtype) ? hvc_prepare(b, o->dtype)
@@ -696,25 +757,30 @@ extern "C" ed_status ed_lanczos_ground_state(const ed_basis* b, const ed_params*
       if (yd) cudaFree(yd);
     }
   } release{st, P, yd};
-  // ---- pass 1: Algorithm 1 to convergence (stepwise, E0 every step)
-  ed_status r = lz_init(b, o, f1, s, 1, false, &st);
+  // ---- pass 1: Algorithm 1 to convergence, tested after every 8 steps
+  ed_status r = lz_init(b, o, f1, s, &st);
   if (r != ED_OK) return r;
   if ((r = fx_prepare(b)) != ED_OK) return r;
-  int hdr[2] = {0, 0};
-  for (int done = 0; done < o->max_steps; done += 8) {
+  ED_TRY_CUDA(cudaMemsetAsync(&st->S->chk, 0, sizeof(int), s));
+  LzScalars hs;
+  constexpr size_t kHead = offsetof(LzScalars, tick_chk);
+  hs.status = 0;
+  hs.conv_j = 0;
+  for (int done = 0; done < o->max_steps && hs.status == 0 && hs.conv_j == 0; done += 8) {
     for (int i = 0; i < 8; ++i)
       if ((r = lz_launch_step(st, p, s)) != ED_OK) return r;
-    if (cudaMemcpyAsync(hdr, st->S, 2 * sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
-      set_error("ed_lanczos_ground_state: %s", cudaGetErrorString(cudaGetLastError()));
-      return ED_ERR_CUDA;
-    }
-    if (hdr[1] != 0) break;
+    if (o->tol > 0.0) lz_check_kernel<<<8, kRedThreads, 0, s>>>(st->S);
+    ED_TRY_CUDA(cudaGetLastError());
+    ED_TRY_CUDA(cudaMemcpyAsync(&hs, st->S, kHead, cudaMemcpyDeviceToHost, s));
+    ED_TRY_CUDA(cudaStreamSynchronize(s));
   }
-  const int m = hdr[0];
-  const int status = hdr[1];
+  const int m = hs.conv_j ? hs.conv_j : hs.j;
+  const int status = hs.conv_j ? 2 : hs.status;
   double lam = 0.0;
-  ED_TRY_CUDA(cudaMemcpy(&lam, &st->S->E0[m], sizeof(double), cudaMemcpyDeviceToHost));
+  if (!(o->tol > 0.0)) lz_history_kernel<<<1, kRedThreads, 0, s>>>(st->S, 0);
+  ED_TRY_CUDA(cudaGetLastError());
+  ED_TRY_CUDA(cudaMemcpyAsync(&lam, &st->S->E0[m], sizeof(double), cudaMemcpyDeviceToHost, s));
+  ED_TRY_CUDA(cudaStreamSynchronize(s));
   // ---- Ritz vector of T_m on the device
   if (cudaMalloc((void**)&yd, (size_t)(3 * (m + 2)) * sizeof(double)) != cudaSuccess)
     return ED_ERR_OOM;
@@ -722,7 +788,7 @@ extern "C" ed_status ed_lanczos_ground_state(const ed_basis* b, const ed_params*
   ED_TRY_CUDA(cudaGetLastError());
   // ---- pass 2: the same steps again from the same start, accumulating y_j f_j
   ed_lanczos* st2 = nullptr;
-  if ((r = lz_init(b, o, f1, s, ED_MAX_STEPS + 1, true, &st2)) != ED_OK) return r;
+  if ((r = lz_init(b, o, f1, s, &st2)) != ED_OK) return r;
   ed_lanczos_destroy(st);
   st = st2;
   if (cudaMalloc((void**)&P, (size_t)b->dim * sizeof(long long)) != cudaSuccess)
@@ -771,80 +837,120 @@ void lz_cache_free(const ed_basis* b) {
 }
 }  // namespace ed
 
+// The CUDA graph of a solve's steps (captured on first use per parameters): two steps, or
+// with the convergence test max(2, K) steps, K = check_stride. The check of K steps is a
+// branch beside the steps that follow: one opens the graph (the last K steps of the replay
+// before, whose check would otherwise end it alone), the others follow their steps.
+static ed_status lz_graph(ed_lanczos* st, const ed_params* p, bool check, int* steps) {
+  cudaStream_t s = st->stream;
+  const int K = check_stride(st->n);
+  const int n = check ? std::max(2, K) : 2;
+  *steps = n;
+  cudaGraphExec_t& exec = st->graph[check];
+  if (exec && st->graph_t[check] == p->t && st->graph_U[check] == p->U) return ED_OK;
+  if (exec) cudaGraphExecDestroy(exec);
+  exec = nullptr;
+  if (!st->host) {
+    int lo = 0, hi = 0;
+    ED_TRY_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    if (!st->check_stream)
+      ED_TRY_CUDA(cudaStreamCreateWithPriority(&st->check_stream, cudaStreamNonBlocking, hi));
+    for (cudaEvent_t* e : {&st->ev_fork, &st->ev_join, &st->ev_batch[0], &st->ev_batch[1]})
+      if (!*e) ED_TRY_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    ED_TRY_CUDA(cudaMallocHost((void**)&st->host, sizeof(LzScalars) + 2 * sizeof(int4)));
+  }
+  cudaGraph_t g = nullptr;
+  if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    set_error("ed_lanczos_solve: stream capture failed");
+    return ED_ERR_CUDA;
+  }
+  ed_status r = ED_OK;
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < n && r == ED_OK && e == cudaSuccess; ++i) {
+    if (check && i % K == 0) {
+      e = cudaEventRecord(st->ev_fork, s);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(st->check_stream, st->ev_fork, 0);
+      lz_check_kernel<<<K, kRedThreads, 0, st->check_stream>>>(st->S);
+      if (e == cudaSuccess) e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) r = lz_launch_step(st, p, s);
+  }
+  if (check) {  // the branch joins the steps again, also where the capture failed
+    cudaEventRecord(st->ev_join, st->check_stream);
+    cudaStreamWaitEvent(s, st->ev_join, 0);
+  }
+  const cudaError_t ce = cudaStreamEndCapture(s, &g);
+  if (e == cudaSuccess) e = ce;
+  if (r == ED_OK && e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
+  if (g) cudaGraphDestroy(g);
+  if (r != ED_OK || e != cudaSuccess) {
+    exec = nullptr;
+    cudaGetLastError();
+    if (r != ED_OK) return r;
+    set_error("ed_lanczos_solve: graph of the steps: %s", cudaGetErrorString(e));
+    return ED_ERR_CUDA;
+  }
+  st->graph_t[check] = p->t;
+  st->graph_U[check] = p->U;
+  return ED_OK;
+}
+
+// Run a started state until it stops, and copy its scalars to st->host: m steps, status as in
+// LzScalars. all_E0: E0 of every step, else of the last one (runs without convergence test).
+static ed_status lz_iterate(ed_lanczos* st, const ed_params* p, const ed_opts* o, bool all_E0,
+                            int* m, int* status) {
+  cudaStream_t s = st->stream;
+  const bool check = o->tol > 0.0;
+  int n = 0;
+  ed_status r = lz_graph(st, p, check, &n);
+  if (r != ED_OK) return r;
+  // batches of about 8 steps, the host one batch behind the device: it reads the status of a
+  // batch while the next one runs (a stopped run's remaining kernels return at entry)
+  int4* head = reinterpret_cast<int4*>(st->host + 1);
+  const int per_batch = std::max(1, 8 / n);
+  int launched = 0;
+  for (int batch = 0;; ++batch) {
+    for (int i = 0; i < per_batch && launched < o->max_steps; ++i, launched += n)
+      ED_TRY_CUDA(cudaGraphLaunch(st->graph[check], s));
+    ED_TRY_CUDA(cudaMemcpyAsync(&head[batch & 1], st->S, sizeof(int4), cudaMemcpyDeviceToHost, s));
+    ED_TRY_CUDA(cudaEventRecord(st->ev_batch[batch & 1], s));
+    if (launched >= o->max_steps) break;
+    if (batch == 0) continue;
+    ED_TRY_CUDA(cudaEventSynchronize(st->ev_batch[(batch - 1) & 1]));
+    if (head[(batch - 1) & 1].y != 0 || head[(batch - 1) & 1].z != 0) break;
+  }
+  if (check)
+    lz_check_kernel<<<check_stride(st->n), kRedThreads, 0, s>>>(st->S);  // the last steps
+  else
+    lz_history_kernel<<<all_E0 ? o->max_steps : 1, kRedThreads, 0, s>>>(st->S, all_E0 ? 1 : 0);
+  ED_TRY_CUDA(cudaGetLastError());
+  ED_TRY_CUDA(cudaMemcpyAsync(st->host, st->S, sizeof(LzScalars), cudaMemcpyDeviceToHost, s));
+  ED_TRY_CUDA(cudaStreamSynchronize(s));
+  const LzScalars& h = *st->host;
+  *m = h.conv_j ? h.conv_j : h.j;
+  *status = h.conv_j ? 2 : h.status;
+  return ED_OK;
+}
+
 static ed_status solve_on(ed_lanczos* st, const ed_basis* b, const ed_params* p, const ed_opts* o,
                           const void* f1, double* E0, int32_t* steps, double* alpha, double* beta,
                           double* E0_hist) {
-  cudaStream_t s = st->stream;
-  // E0(j) every step when the convergence test needs it, else at the stop step (a history
-  // is then computed after the run, all steps at once)
-  const int check = o->tol > 0.0 ? 1 : ED_MAX_STEPS + 1;
-  ed_status r = lz_reset(st, o, f1, check, false);
+  ed_status r = lz_reset(st, o, f1);
   if (r != ED_OK) return r;
   if ((r = (o->dtype == ED_F64 ? fx_prepare(b)
             : is_complex(o->dtype) ? hvc_prepare(b, o->dtype)
                                    : hv_prepare(b, o->dtype))) != ED_OK)
     return r;
-  if (!st->graph || st->graph_t != p->t || st->graph_U != p->U) {
-    if (st->graph) cudaGraphExecDestroy(st->graph);
-    st->graph = nullptr;
-    // capture two steps (the buffer roles alternate) and replay
-    cudaGraph_t g = nullptr;
-    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-      set_error("ed_lanczos_solve: stream capture failed");
-      return ED_ERR_CUDA;
-    }
-    const ed_status r1 = lz_launch_step(st, p, s);
-    const ed_status r2 = r1 == ED_OK ? lz_launch_step(st, p, s) : r1;
-    cudaError_t ce = cudaStreamEndCapture(s, &g);
-    if (r2 != ED_OK || ce != cudaSuccess) {
-      if (g) cudaGraphDestroy(g);
-      if (r2 == ED_OK) set_error("ed_lanczos_solve: capture failed: %s", cudaGetErrorString(ce));
-      return r2 != ED_OK ? r2 : ED_ERR_CUDA;
-    }
-    ce = cudaGraphInstantiate(&st->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (ce != cudaSuccess) {
-      st->graph = nullptr;
-      set_error("ed_lanczos_solve: graph instantiate failed: %s", cudaGetErrorString(ce));
-      return ED_ERR_CUDA;
-    }
-    st->graph_t = p->t;
-    st->graph_U = p->U;
-  }
-  int hdr[2] = {0, 0};
-  int launched = 0;
-  while (true) {
-    const int remaining = o->max_steps - launched;
-    int batch = (remaining + 1) / 2;
-    if (batch > 8) batch = 8;
-    if (batch < 1) batch = 1;
-    for (int i = 0; i < batch; ++i) ED_TRY_CUDA(cudaGraphLaunch(st->graph, s));
-    launched += 2 * batch;
-    ED_TRY_CUDA(cudaMemcpyAsync(hdr, st->S, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-    ED_TRY_CUDA(cudaStreamSynchronize(s));
-    if (hdr[1] != 0 || launched >= o->max_steps) break;
-  }
-  const int j = hdr[0];
-  if (E0_hist && check > 1 && j > 1) {
-    lz_history_kernel<<<j - 1, kRedThreads, 0, s>>>(st->S, j);
-    ED_TRY_CUDA(cudaGetLastError());
-  }
-  std::vector<double> hv(3 * (size_t)(j + 2));
-  double* h_alpha = hv.data();
-  double* h_beta = h_alpha + (j + 2);
-  double* h_E = h_beta + (j + 2);
-  ED_TRY_CUDA(cudaMemcpyAsync(h_alpha, st->S->alpha, (j + 2) * 8, cudaMemcpyDeviceToHost, s));
-  ED_TRY_CUDA(cudaMemcpyAsync(h_beta, st->S->beta, (j + 2) * 8, cudaMemcpyDeviceToHost, s));
-  ED_TRY_CUDA(cudaMemcpyAsync(h_E, st->S->E0, (j + 2) * 8, cudaMemcpyDeviceToHost, s));
-  ED_TRY_CUDA(cudaStreamSynchronize(s));
-  *E0 = j >= 1 ? h_E[j] : NAN;
+  int j = 0, status = 0;
+  if ((r = lz_iterate(st, p, o, E0_hist != nullptr, &j, &status)) != ED_OK) return r;
+  const LzScalars& h = *st->host;
+  *E0 = j >= 1 ? h.E0[j] : NAN;
   if (steps) *steps = j;
   for (int i = 1; i <= j; ++i) {
-    if (alpha) alpha[i - 1] = h_alpha[i];
-    if (beta) beta[i - 1] = h_beta[i + 1];
-    if (E0_hist) E0_hist[i - 1] = h_E[i];
+    if (alpha) alpha[i - 1] = h.alpha[i];
+    if (beta) beta[i - 1] = h.beta[i + 1];
+    if (E0_hist) E0_hist[i - 1] = h.E0[i];
   }
-  const int status = hdr[1];
   if (status == 1) return ED_BREAKDOWN;
   if (status == 3 && o->tol > 0.0) {
     set_error("ed_lanczos_solve: not converged after %d steps", j);

@@ -330,36 +330,22 @@ __device__ __forceinline__ void tridiag_ritz_vector(const double* a, const doubl
   }
 }
 
-// Thread 0 of the finish kernel: record b_{j+1}, update the breakdown scale, advance j.
-// Returns 1 on breakdown (b_{j+1} <= 1e-13 max(1, max_i |a_i| + b_i)), else 0.
-__device__ __forceinline__ int finish_record_beta(LzScalars* S, int j, double beta) {
+// Thread 0 of the finish kernel: record b_{j+1}, update the breakdown scale, advance j and
+// stop the run at a breakdown (b_{j+1} <= 1e-13 max(1, max_i |a_i| + b_i)), at the step limit
+// or once a convergence check has passed. Returns whether b_{j+1} may be divided by.
+// The status is written here alone, between the kernels that read it: the checks run beside
+// them (lz_check_kernel), and a flag that changed under a running kernel would let some warps
+// of a CTA return and others go on with shared memory that was never filled.
+__device__ __forceinline__ bool finish_step(LzScalars* S, int j, double beta) {
   const double ts = fmax(S->tscale, fabs(S->alpha[j]) + S->beta[j]);
   S->tscale = ts;
   S->beta[j + 1] = beta;
   S->j = j;
-  return (beta > kBreakdownRel * fmax(1.0, ts)) ? 0 : 1;
-}
-
-// Whole block: E0(j) = lambda_min(T_j) when due, convergence test, final status.
-__device__ __forceinline__ void finish_tail(LzScalars* S, int j, int st) {
-  __shared__ double sturm_work[kSturmWork];
-  const bool check = st != 0 || j >= S->max_steps || (j % S->check_every) == 0;
-  if (check) {
-    const double E = sturm_lowest(S->alpha, S->beta, j, S->last_E0_step > 0 ? S->last_E0 : NAN,
-                                  sturm_work);
-    if (threadIdx.x == 0) {
-      S->E0[j] = E;
-      if (st == 0 && S->tol > 0.0 && S->last_E0_step > 0 &&
-          fabs(E - S->last_E0) <= S->tol * fmax(fabs(E), 1.0))
-        st = 2;
-      S->last_E0 = E;
-      S->last_E0_step = j;
-    }
-  }
-  if (threadIdx.x == 0) {
-    if (st == 0 && j >= S->max_steps) st = 3;
-    S->status = st;
-  }
+  const bool go = beta > kBreakdownRel * fmax(1.0, ts);
+  if (!go) S->status = 1;
+  else if (*(volatile int*)&S->conv_j != 0) S->status = 2;
+  else if (j >= S->max_steps) S->status = 3;
+  return go;
 }
 
 }  // namespace ed
