@@ -4,7 +4,7 @@
 // vb = 62 - ceil(log2(hops + n_max + 2))), so that a hop sum of up to `hops` elements and
 // the diagonal product n X never overflow. One step j on buffers cur (f_j) and prev
 // (f_{j-1}):
-//   plan   (1 thread):  choose W's scale s_w = s_cur 2^r so that |W| <= 2^(vb-1), and the
+//   plan   (1 thread, at the end of the step before): choose W's scale s_w = s_cur 2^r so that |W| <= 2^(vb-1), and the
 //                       integer coefficients of  W = round((a S + b n X + c P) 2^k)  with
 //                       a 2^k = -t 2^-r, b 2^k = U 2^-r, c 2^k = -b_j (s_prev/s_cur) 2^-r;
 //   H.v    (fused):     S = exact int64 hop sum (Sec. 4 Eqs. 5-6), P = X_prev, W written
@@ -34,73 +34,6 @@ FxRun fx_make(const ed_basis* b) {
   while ((1 << hb) < need) ++hb;
   f.vb = 62 - hb;
   return f;
-}
-
-// ------------------------------------------------------------------ reductions
-// Block reduction of a 192-bit sum and a max; thread 0 writes out[0..3] =
-// (lo bits 0..63, lo bits 64..127, hi, max).
-__device__ __forceinline__ void fx_block_reduce(I192 v, long long mx, long long* out) {
-  __shared__ unsigned long long sm[32][4];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const I192 w = i192_shfl_down(v, o);
-    i192_add(v, w);
-    mx = max(mx, (long long)__shfl_down_sync(0xffffffffu, mx, o));
-  }
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) {
-    sm[wid][0] = (unsigned long long)v.lo;
-    sm[wid][1] = (unsigned long long)(v.lo >> 64);
-    sm[wid][2] = (unsigned long long)v.hi;
-    sm[wid][3] = (unsigned long long)mx;
-  }
-  __syncthreads();
-  if (wid == 0) {
-    const int nw = blockDim.x >> 5;
-    I192 a;
-    i192_zero(a);
-    long long m = 0;
-    if (lane < nw) {
-      a.lo = ((u128)sm[lane][1] << 64) | (u128)sm[lane][0];
-      a.hi = (long long)sm[lane][2];
-      m = (long long)sm[lane][3];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const I192 w = i192_shfl_down(a, o);
-      i192_add(a, w);
-      m = max(m, (long long)__shfl_down_sync(0xffffffffu, m, o));
-    }
-    if (lane == 0) {
-      out[0] = (long long)(unsigned long long)a.lo;
-      out[1] = (long long)(unsigned long long)(a.lo >> 64);
-      out[2] = a.hi;
-      out[3] = m;
-    }
-  }
-  __syncthreads();
-}
-
-// Sum (exact) and max of n partial records of 4 words; every thread gets the result.
-__device__ __forceinline__ void fx_sum_partials(const long long* __restrict__ p, int n, I192& sum,
-                                                long long& mx) {
-  __shared__ long long out[4];
-  I192 v;
-  i192_zero(v);
-  long long m = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    I192 w;
-    w.lo = ((u128)(unsigned long long)p[4 * i + 1] << 64) | (u128)(unsigned long long)p[4 * i];
-    w.hi = p[4 * i + 2];
-    i192_add(v, w);
-    m = max(m, p[4 * i + 3]);
-  }
-  fx_block_reduce(v, m, out);
-  sum.lo = ((u128)(unsigned long long)out[1] << 64) | (u128)(unsigned long long)out[0];
-  sum.hi = out[2];
-  mx = out[3];
-  __syncthreads();
 }
 
 __device__ __forceinline__ long long sgn_apply(long long v, uint32_t e) {
@@ -213,9 +146,15 @@ fx_init_kernel(LzScalars* S, const long long* __restrict__ part, int n) {
 }
 
 // ------------------------------------------------------------------ one step
-__global__ void fx_plan_kernel(LzScalars* S, int cur, double t, double U, int hops, int nmax,
-                               int vb) {
-  if (threadIdx.x != 0 || S->status != 0) return;
+struct FxPlanArgs {
+  double t, U;
+  int hops, nmax, vb;
+};
+
+// One thread: the integer coefficients of the H.v of step S->j + 1 on buffer cur.
+__device__ __forceinline__ void fx_plan_step(LzScalars* S, int cur, const FxPlanArgs& p) {
+  const double t = p.t, U = p.U;
+  const int hops = p.hops, nmax = p.nmax, vb = p.vb;
   const int j = S->j + 1;
   const double sc = S->scale[cur], sp = S->scale[1 - cur];
   const double mc = (double)S->fx_max[cur], mp = (double)S->fx_max[1 - cur];
@@ -239,6 +178,10 @@ __global__ void fx_plan_kernel(LzScalars* S, int cur, double t, double U, int ho
   S->fx_k = k;
   S->fx_r = r;
   S->fx_sw = ldexp(sc, r);
+}
+
+__global__ void fx_plan_kernel(LzScalars* S, int cur, FxPlanArgs p) {
+  if (threadIdx.x == 0 && S->status == 0) fx_plan_step(S, cur, p);
 }
 
 struct FxHvArgs {
@@ -284,7 +227,7 @@ __device__ __forceinline__ void fx_add_hops(long long& s, const int32_t* tab, in
 template <int R>
 __global__ void __launch_bounds__(kFxThreads)
 fx_hv_staged_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __restrict__ y,
-                    const LzScalars* __restrict__ S, long long* __restrict__ part) {
+                    LzScalars* S, int cur, long long* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (S->status != 0) return;
   const long long ca = S->fx_a, cb = S->fx_b, cc = S->fx_c;
@@ -340,12 +283,13 @@ fx_hv_staged_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __re
     }
   }
   fx_block_reduce(dot, 0, part + 4 * blockIdx.x);
+  fx_hv_finish(S, cur, part);
 }
 
 // Fallback when a row does not fit in shared memory.
 __global__ void __launch_bounds__(kFxThreads)
 fx_hv_global_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __restrict__ y,
-                    const LzScalars* __restrict__ S, long long* __restrict__ part) {
+                    LzScalars* S, int cur, long long* __restrict__ part) {
   if (S->status != 0) return;
   const long long ca = S->fx_a, cb = S->fx_b, cc = S->fx_c;
   const int k = S->fx_k;
@@ -368,25 +312,35 @@ fx_hv_global_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __re
     i192_add(dot, (i128)w * xc);
   }
   fx_block_reduce(dot, 0, part + 4 * blockIdx.x);
+  fx_hv_finish(S, cur, part);
 }
 
+// Whole CTA: b_{j+1} and f_{j+1}'s scale from the n partial records of ||Q||^2, then the
+// coefficients of the next H.v.
+__device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long long* pb, int nb,
+                                               const FxPlanArgs& p) {
+  I192 sum;
+  long long mx;
+  fx_sum_partials(pb, nb, sum, mx);
+  if (threadIdx.x != 0) return;
+  const int j = S->j + 1;
+  const double sw = S->fx_sw;
+  const double beta = sw * sqrt(i192_to_double(sum));
+  if (finish_step(S, j, beta)) {
+    S->scale[1 - cur] = sw / beta;
+    S->fx_max[1 - cur] = mx;
+    fx_plan_step(S, 1 - cur, p);
+  }
+}
+
+// finish: the last CTA ends the step (fx_finish_step); otherwise fx_finish_kernel does, after
+// the reorthogonalisation.
 __global__ void __launch_bounds__(kFxThreads)
 fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long long* __restrict__ xp,
-                 int64_t n, const long long* __restrict__ pa, int na, long long* __restrict__ pb) {
+                 int64_t n, long long* __restrict__ pb, int finish, FxPlanArgs plan) {
   if (S->status != 0) return;
-  I192 sum;
-  long long unused;
-  fx_sum_partials(pa, na, sum, unused);
-  const double sc = S->scale[cur], sw = S->fx_sw;
-  const double alpha = sw * sc * i192_to_double(sum);
-  if (blockIdx.x == 0 && threadIdx.x == 0) S->alpha[S->j + 1] = alpha;
-  const double D = -alpha * (sc / sw);
-  long long d = 0;
-  int k2 = -1;
-  if (D != 0.0 && isfinite(D)) {
-    k2 = ilogb(D) - 61;
-    d = llrint(ldexp(D, -k2));
-  }
+  const long long d = S->fx_d;
+  const int k2 = S->fx_k2;
   A192 q2;
   long long mx = 0;
   // n is even (rows are padded to 32 elements): pairs of elements, two pairs in flight
@@ -413,23 +367,12 @@ fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long l
     if (two) p2[i + stride] = make_longlong2(upd(w1.x, c1.x), upd(w1.y, c1.y));
   }
   fx_block_reduce(a192_get(q2), mx, pb + 4 * blockIdx.x);
+  if (finish && last_cta(&S->tick_upd)) fx_finish_step(S, cur, pb, gridDim.x, plan);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
-fx_finish_kernel(LzScalars* S, int cur, const long long* __restrict__ pb, int nb) {
-  if (S->status != 0) return;
-  const int j = S->j + 1;
-  I192 sum;
-  long long mx;
-  fx_sum_partials(pb, nb, sum, mx);
-  if (threadIdx.x == 0) {
-    const double sw = S->fx_sw;
-    const double beta = sw * sqrt(i192_to_double(sum));
-    if (finish_step(S, j, beta)) {
-      S->scale[1 - cur] = sw / beta;
-      S->fx_max[1 - cur] = mx;
-    }
-  }
+fx_finish_kernel(LzScalars* S, int cur, const long long* __restrict__ pb, int nb, FxPlanArgs plan) {
+  if (S->status == 0) fx_finish_step(S, cur, pb, nb, plan);
 }
 
 // ------------------------------------------------------------------ ground-state vector
@@ -625,39 +568,44 @@ ed_status fx_copy_in(const ed_basis* b, const FxRun& fx, const double* f1, long 
   return ED_OK;
 }
 
+ed_status fx_plan(const FxRun& fx, double t, double U, int cur, LzScalars* S, cudaStream_t s) {
+  fx_plan_kernel<<<1, 32, 0, s>>>(S, cur, FxPlanArgs{t, U, fx.hops, fx.nmax, fx.vb});
+  ED_TRY_CUDA(cudaGetLastError());
+  return ED_OK;
+}
+
 ed_status fx_step(const ed_basis* b, const FxRun& fx, double t, double U, long long* const B[2],
                   int cur, int64_t ld, LzScalars* S, long long* pa, long long* pb,
                   cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, const Hv2Plan* plan,
                   const Reorth* ro) {
-  fx_plan_kernel<<<1, 32, 0, s>>>(S, cur, t, U, fx.hops, fx.nmax, fx.vb);
   if (ev0) ED_TRY_CUDA(cudaEventRecord(ev0, s));
   const FxHvArgs a = fx_args(b, ld);
   const int R = plan ? -1 : fx_rows(b);
-  int grid;
   if (plan) {
-    grid = hv2_grid(plan);
     ed_status r = hv2_launch(plan, b, t, U, B[cur], B[1 - cur], S, cur, pa, s);
     if (r != ED_OK) return r;
   } else if (R == 2) {
-    grid = (int)((b->up.dim + 1) / 2);
-    fx_hv_staged_kernel<2><<<grid, kFxThreads, fx_smem<2>(b), s>>>(a, B[cur], B[1 - cur], S, pa);
+    const int grid = (int)((b->up.dim + 1) / 2);
+    fx_hv_staged_kernel<2><<<grid, kFxThreads, fx_smem<2>(b), s>>>(a, B[cur], B[1 - cur], S, cur, pa);
   } else if (R == 1) {
-    grid = (int)b->up.dim;
-    fx_hv_staged_kernel<1><<<grid, kFxThreads, fx_smem<1>(b), s>>>(a, B[cur], B[1 - cur], S, pa);
+    const int grid = (int)b->up.dim;
+    fx_hv_staged_kernel<1><<<grid, kFxThreads, fx_smem<1>(b), s>>>(a, B[cur], B[1 - cur], S, cur, pa);
   } else {
-    grid = fx_red_grid(b->dim) * 2;
-    fx_hv_global_kernel<<<grid, kFxThreads, 0, s>>>(a, B[cur], B[1 - cur], S, pa);
+    const int grid = fx_red_grid(b->dim) * 2;
+    fx_hv_global_kernel<<<grid, kFxThreads, 0, s>>>(a, B[cur], B[1 - cur], S, cur, pa);
   }
   ED_TRY_CUDA(cudaGetLastError());
   if (ev1) ED_TRY_CUDA(cudaEventRecord(ev1, s));
   const int64_t n = b->up.dim * ld;
   const int ug = fx_red_grid(n);
-  fx_update_kernel<<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pa, grid, pb);
-  if (ro) {
+  const FxPlanArgs next = {t, U, fx.hops, fx.nmax, fx.vb};
+  const bool between = ro && ro_between(ro);  // passes between the update and the finish
+  fx_update_kernel<<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next);
+  if (between) {
     const ed_status r = ro_apply(ro, S, B[1 - cur], pb, ug, s);
     if (r != ED_OK) return r;
+    fx_finish_kernel<<<1, kRedThreads, 0, s>>>(S, cur, pb, ug, next);
   }
-  fx_finish_kernel<<<1, kRedThreads, 0, s>>>(S, cur, pb, ug);
   ED_TRY_CUDA(cudaGetLastError());
   if (ro) return ro_store(ro, S, 1 - cur, B[1 - cur], s);
   return ED_OK;

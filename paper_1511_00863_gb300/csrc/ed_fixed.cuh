@@ -10,6 +10,8 @@
 
 #include <stdint.h>
 
+#include "ed_internal.cuh"
+
 namespace ed {
 
 typedef __int128 i128;
@@ -171,5 +173,106 @@ struct FxCoef {
   long long m;
   int e;
 };
+
+// ------------------------------------------------------------------ reductions
+// Block reduction of a 192-bit sum and a max; thread 0 writes out[0..3] =
+// (lo bits 0..63, lo bits 64..127, hi, max).
+__device__ __forceinline__ void fx_block_reduce(I192 v, long long mx, long long* out) {
+  __shared__ unsigned long long sm[32][4];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const I192 w = i192_shfl_down(v, o);
+    i192_add(v, w);
+    mx = max(mx, (long long)__shfl_down_sync(0xffffffffu, mx, o));
+  }
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();
+  if (lane == 0) {
+    sm[wid][0] = (unsigned long long)v.lo;
+    sm[wid][1] = (unsigned long long)(v.lo >> 64);
+    sm[wid][2] = (unsigned long long)v.hi;
+    sm[wid][3] = (unsigned long long)mx;
+  }
+  __syncthreads();
+  if (wid == 0) {
+    const int nw = blockDim.x >> 5;
+    I192 a;
+    i192_zero(a);
+    long long m = 0;
+    if (lane < nw) {
+      a.lo = ((u128)sm[lane][1] << 64) | (u128)sm[lane][0];
+      a.hi = (long long)sm[lane][2];
+      m = (long long)sm[lane][3];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const I192 w = i192_shfl_down(a, o);
+      i192_add(a, w);
+      m = max(m, (long long)__shfl_down_sync(0xffffffffu, m, o));
+    }
+    if (lane == 0) {
+      out[0] = (long long)(unsigned long long)a.lo;
+      out[1] = (long long)(unsigned long long)(a.lo >> 64);
+      out[2] = a.hi;
+      out[3] = m;
+    }
+  }
+  __syncthreads();
+}
+
+// Sum (exact) and max of n partial records of 4 words; every thread gets the result. They may
+// come from other CTAs of the running launch: read from L2.
+__device__ __forceinline__ void fx_sum_partials(const long long* __restrict__ p, int n, I192& sum,
+                                                long long& mx) {
+  __shared__ long long out[4];
+  I192 v;
+  i192_zero(v);
+  long long m = 0;
+  for (int i = threadIdx.x; i < n; i += 4 * blockDim.x) {  // four records in flight
+    longlong2 r[4][2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int q = i + k * (int)blockDim.x;
+      const longlong2* w = reinterpret_cast<const longlong2*>(p + 4 * (int64_t)q);
+      r[k][0] = q < n ? __ldcg(w) : make_longlong2(0, 0);
+      r[k][1] = q < n ? __ldcg(w + 1) : make_longlong2(0, 0);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      I192 w;
+      w.lo = ((u128)(unsigned long long)r[k][0].y << 64) | (u128)(unsigned long long)r[k][0].x;
+      w.hi = r[k][1].x;
+      i192_add(v, w);
+      m = max(m, r[k][1].y);
+    }
+  }
+  fx_block_reduce(v, m, out);
+  sum.lo = ((u128)(unsigned long long)out[1] << 64) | (u128)(unsigned long long)out[0];
+  sum.hi = out[2];
+  mx = out[3];
+  __syncthreads();
+}
+
+// End of a fixed-point H.v: the last CTA records a_j and the update's integer coefficient
+// (Q = W + round(d X 2^k2), d 2^k2 = -a_j s_cur / s_w).
+__device__ __forceinline__ void fx_hv_finish(LzScalars* S, int cur, const long long* part) {
+  if (!last_cta(&S->tick_hv)) return;
+  I192 sum;
+  long long unused;
+  fx_sum_partials(part, gridDim.x, sum, unused);
+  if (threadIdx.x != 0) return;
+  const double sc = S->scale[cur], sw = S->fx_sw;
+  const double alpha = sw * sc * i192_to_double(sum);
+  S->alpha[S->j + 1] = alpha;
+  const double D = -alpha * (sc / sw);
+  long long d = 0;
+  int k2 = -1;
+  if (D != 0.0 && isfinite(D)) {
+    k2 = ilogb(D) - 61;
+    d = llrint(ldexp(D, -k2));
+  }
+  S->fx_d = d;
+  S->fx_k2 = k2;
+}
 
 }  // namespace ed

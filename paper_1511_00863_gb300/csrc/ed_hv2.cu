@@ -83,7 +83,7 @@ static bool kind_info(int kind, const ed_basis* b, int ld, KindInfo* ki) {
 #define HV2_INFO(K, E, R_, V_, T, MB)                                                     \
     case K:                                                                               \
       ki->smem = ((size_t)(ld + hv2_group<E, R_>()) * sizeof(E) * R_ + 15) / 16 * 16 +      \
-                 (size_t)R_ * MH * 12;                                                    \
+                 (size_t)R_ * MH * 8;                                                     \
       ki->R = R_;                                                                         \
       ki->V = V_;                                                                         \
       ki->G = hv2_group<E, R_>();                                                         \
@@ -217,7 +217,7 @@ static int split_slots(const SplitTables& t) {
 
 static size_t split_smem(const SplitTables& t, const ed_basis* b, size_t esize) {
   const int MH = b->up.maxhops > 0 ? b->up.maxhops : 1;
-  return ((size_t)split_slots(t) * esize + 15) / 16 * 16 + (size_t)MH * 12;
+  return ((size_t)split_slots(t) * esize + 15) / 16 * 16 + (size_t)MH * 8;
 }
 
 // The split tables of this basis for V = 2, G = 16 (int64 kernel) or V = 4, G = 32 (FP32
@@ -276,6 +276,17 @@ void hv2_split_free(const ed_basis* b) {
   b->hv2_split = nullptr;
 }
 
+// Opt in to the shared memory and cut the plan's grid (one CTA per row group) to the CTAs that
+// are resident at once: each then takes every grid-th row group.
+template <typename K>
+static cudaError_t one_wave(K kernel, int threads, Hv2Plan* p) {
+  cudaError_t e = allow_max_smem(kernel);
+  int per_sm = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, p->smem);
+  if (e == cudaSuccess && per_sm >= 1) p->grid = std::min(p->grid, per_sm * sm_count());
+  return e;
+}
+
 static ed_status hv2_build_split(const ed_basis* b, int mode, int ld, cudaStream_t s, Hv2Plan** out) {
   const int V = mode == kHv2Fx ? 2 : 4;
   const SplitTables* t = split_tables(b, V, s);
@@ -307,7 +318,7 @@ static ed_status hv2_build_split(const ed_basis* b, int mode, int ld, cudaStream
   if (e == cudaSuccess) e = cudaMemcpyAsync(p->colpos, t->pos.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
 #define HV2S_ATTR(K, E, V_, T, MB) \
-  if (e == cudaSuccess && p->kind == K) e = allow_max_smem(hv2s_kernel<E, V_, T, MB>);
+  if (e == cudaSuccess && p->kind == K) e = one_wave(hv2s_kernel<E, V_, T, MB>, T, p);
   HV2S_KINDS(HV2S_ATTR)
 #undef HV2S_ATTR
   if (e != cudaSuccess) {
@@ -361,12 +372,12 @@ ed_status hv2_build(const ed_basis* b, int mode, int ld, int schedule, cudaStrea
   cudaError_t e = cudaSuccess;
 #define HV2_ATTR(K, E, R_, V, T, MB)                                                     \
   if (kind == K)                                                                          \
-    e = allow_max_smem(hv2_kernel<E, R_, V, T, MB>);
+    e = one_wave(hv2_kernel<E, R_, V, T, MB>, T, p);
   HV2_KINDS(HV2_ATTR)
 #undef HV2_ATTR
 #define HV2C_ATTR(K, R_, V, T, MB)                                                         \
   if (kind == K)                                                                          \
-    e = allow_max_smem(hv2c_kernel<R_, V, T, MB>);
+    e = one_wave(hv2c_kernel<R_, V, T, MB>, T, p);
   HV2C_KINDS(HV2C_ATTR)
 #undef HV2C_ATTR
   if (e != cudaSuccess) {
@@ -383,7 +394,7 @@ const int32_t* hv2_colpos(const Hv2Plan* p) { return p ? p->colpos : nullptr; }
 int hv2_grid(const Hv2Plan* p) { return p ? p->grid : 0; }
 
 ed_status hv2_autotune(const ed_basis* b, int mode, int ld, void* x, void* y,
-                       const LzScalars* S, void* partial, cudaStream_t s, int* kind) {
+                       LzScalars* S, void* partial, cudaStream_t s, int* kind) {
   *kind = 0;
   if (b->up.dim < kMinRowsStaged) return ED_OK;  // few rows: the general kernels
   static const int cand_f32[] = {1, 2, 3, 4, 5, 6, 7, 14}, cand_fx[] = {8, 9, 10, 11, 12, 13},
@@ -432,7 +443,7 @@ ed_status hv2_autotune(const ed_basis* b, int mode, int ld, void* x, void* y,
 int hv2_kind(const Hv2Plan* p) { return p ? p->kind : 0; }
 
 ed_status hv2_launch(const Hv2Plan* p, const ed_basis* b, double t, double U, const void* x,
-                     void* y, const LzScalars* S, int cur, void* partial, cudaStream_t s) {
+                     void* y, LzScalars* S, int cur, void* partial, cudaStream_t s) {
   Hv2Args a;
   a.up_bits = b->up.bits;
   a.dn_bits = p->dn_pad;

@@ -96,9 +96,41 @@ struct Hv2Args {
   float t, U;  // FP32 variant
 };
 
+// The up-hop list of up row u by one warp: element offsets of the neighbour rows, those with
+// sign +1 first, each group in table order.
+__device__ __forceinline__ void hv2_up_list(const int32_t* __restrict__ hop_up, int maxhops, int64_t dim_up,
+                                            int64_t u, int64_t ld, int64_t* upoff, int* npos, int* nneg) {
+  const int lane = threadIdx.x & 31;
+  int total = 0;  // hops with sign +1
+  for (int k0 = 0; k0 < maxhops; k0 += 32) {
+    const int k = k0 + lane;
+    const uint32_t e = k < maxhops ? (uint32_t)hop_up[(int64_t)k * dim_up + u] : (uint32_t)dim_up;
+    total += __popc(__ballot_sync(0xffffffffu, (int64_t)(e & kTargetMask) < dim_up && !(e & kSignBit)));
+  }
+  int np = 0, nn = 0;
+  for (int k0 = 0; k0 < maxhops; k0 += 32) {
+    const int k = k0 + lane;
+    const uint32_t e = k < maxhops ? (uint32_t)hop_up[(int64_t)k * dim_up + u] : (uint32_t)dim_up;
+    const int64_t tg = (int64_t)(e & kTargetMask);
+    const bool hop = tg < dim_up, neg = (e & kSignBit) != 0;
+    const unsigned mp = __ballot_sync(0xffffffffu, hop && !neg), mn = __ballot_sync(0xffffffffu, hop && neg);
+    const unsigned below = (1u << lane) - 1u;
+    if (hop) upoff[neg ? total + nn + __popc(mn & below) : np + __popc(mp & below)] = tg * ld;
+    np += __popc(mp);
+    nn += __popc(mn);
+  }
+  if (lane == 0) {
+    *npos = np;
+    *nneg = nn;
+  }
+}
+
+// The grid is one resident wave (hv2_build): a CTA takes the row groups blockIdx.x,
+// blockIdx.x + gridDim.x, ..., so that its reduction and its ticket (each 1-2 us of waiting in a
+// CTA's 50) come once per launch and not once per row.
 template <typename E, int R, int V, int T, int MB>
 __global__ void __launch_bounds__(T, MB)
-hv2_kernel(Hv2Args a, const E* __restrict__ x, E* __restrict__ y, const LzScalars* __restrict__ S,
+hv2_kernel(Hv2Args a, const E* __restrict__ x, E* __restrict__ y, LzScalars* S,
            int cur, void* __restrict__ partial) {
   constexpr int G = hv2_group<E, R>();
   extern __shared__ __align__(16) unsigned char smem[];
@@ -110,64 +142,6 @@ hv2_kernel(Hv2Args a, const E* __restrict__ x, E* __restrict__ y, const LzScalar
   Pack<E, R>* xs = reinterpret_cast<Pack<E, R>*>(smem);
   int64_t* upoff = reinterpret_cast<int64_t*>(
       smem + ((size_t)(ld + G) * sizeof(Pack<E, R>) + 15) / 16 * 16);
-  uint32_t* upraw = reinterpret_cast<uint32_t*>(upoff + R * MH);
-  const int64_t g0 = (int64_t)blockIdx.x * R;
-  int64_t urow[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int64_t g = g0 + r;
-    urow[r] = g < a.dim_up ? (a.order ? (int64_t)a.order[g] : g) : a.dim_up;  // dim_up = none
-  }
-
-  // ---- stage the R rows (one d per thread: R coalesced loads, one vector store); slots
-  // ld .. ld + G - 1 are zero, one in each bank group
-  for (int d = threadIdx.x; d < ld + G; d += T) {
-    Pack<E, R> p;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int64_t u = urow[r];
-      p.v[r] = (d < ld && u < a.dim_up) ? x[u * ld + d] : E(0);
-    }
-    xs[d < ld ? (d & ~(G - 1)) | a.slot_lo[d] : d] = p;
-  }
-  // ---- up-hop lists: raw entries, then per row positives first, negatives after
-  for (int i = threadIdx.x; i < R * a.maxhops_up; i += T) {
-    const int r = i / a.maxhops_up, k = i - r * a.maxhops_up;
-    int64_t u = a.dim_up;
-#pragma unroll
-    for (int rr = 0; rr < R; ++rr)
-      if (rr == r) u = urow[rr];
-    upraw[i] = (u < a.dim_up) ? (uint32_t)a.hop_up[(int64_t)k * a.dim_up + u] : (uint32_t)a.dim_up;
-  }
-  __syncthreads();
-  if (threadIdx.x < R) {
-    const int r = threadIdx.x;
-    int np = 0, nn = 0;
-    for (int k = 0; k < a.maxhops_up; ++k) {
-      const uint32_t e = upraw[r * a.maxhops_up + k];
-      const int64_t tg = (int64_t)(e & kTargetMask);
-      if (tg >= a.dim_up) break;
-      if (!(e & kSignBit)) upoff[r * MH + np++] = tg * ld;
-    }
-    for (int k = 0; k < a.maxhops_up; ++k) {
-      const uint32_t e = upraw[r * a.maxhops_up + k];
-      const int64_t tg = (int64_t)(e & kTargetMask);
-      if (tg >= a.dim_up) break;
-      if (e & kSignBit) upoff[r * MH + np + nn++] = tg * ld;
-    }
-    npos_s[r] = np;
-    nneg_s[r] = nn;
-  }
-  __syncthreads();
-
-  uint32_t ub[R];
-  int npos[R], nneg[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    ub[r] = (urow[r] < a.dim_up) ? a.up_bits[urow[r]] : 0u;
-    npos[r] = npos_s[r];
-    nneg[r] = nneg_s[r];
-  }
   // per-run scalars
   float sc = 1.f, bsp = 0.f;
   long long ca = 0, cb = 0, cc = 0;
@@ -184,6 +158,49 @@ hv2_kernel(Hv2Args a, const E* __restrict__ x, E* __restrict__ y, const LzScalar
   }
   DotAcc<float> dotf;
   A192 dota;
+  const int ngroups = (int)((a.dim_up + R - 1) / R);
+  for (int g = blockIdx.x; g < ngroups; g += gridDim.x) {
+  int64_t urow[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int64_t q = (int64_t)g * R + r;
+    urow[r] = q < a.dim_up ? (a.order ? (int64_t)a.order[q] : q) : a.dim_up;  // dim_up = none
+  }
+  if (g != (int)blockIdx.x) __syncthreads();  // the gathers of the rows before are done
+
+  // ---- stage the R rows (one d per thread: R coalesced loads, one vector store); slots
+  // ld .. ld + G - 1 are zero, one in each bank group
+  for (int d = threadIdx.x; d < ld + G; d += T) {
+    Pack<E, R> p;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int64_t u = urow[r];
+      p.v[r] = (d < ld && u < a.dim_up) ? x[u * ld + d] : E(0);
+    }
+    xs[d < ld ? (d & ~(G - 1)) | a.slot_lo[d] : d] = p;
+  }
+  if (threadIdx.x < 32 * R) {
+    const int r = threadIdx.x >> 5;
+    int64_t u = a.dim_up;
+#pragma unroll
+    for (int rr = 0; rr < R; ++rr)
+      if (rr == r) u = urow[rr];
+    if (u < a.dim_up) {
+      hv2_up_list(a.hop_up, a.maxhops_up, a.dim_up, u, ld, upoff + r * MH, &npos_s[r], &nneg_s[r]);
+    } else if ((threadIdx.x & 31) == 0) {
+      npos_s[r] = nneg_s[r] = 0;
+    }
+  }
+  __syncthreads();
+
+  uint32_t ub[R];
+  int npos[R], nneg[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    ub[r] = (urow[r] < a.dim_up) ? a.up_bits[urow[r]] : 0u;
+    npos[r] = npos_s[r];
+    nneg[r] = nneg_s[r];
+  }
 
   for (int d0 = threadIdx.x * V; d0 < ld; d0 += T * V) {
     E acc[R][V];
@@ -283,45 +300,15 @@ hv2_kernel(Hv2Args a, const E* __restrict__ x, E* __restrict__ y, const LzScalar
       stcs_pack(reinterpret_cast<Pack<E, V>*>(yp), W);
     }
   }
+  }
   if constexpr (sizeof(E) == 4) {
     const double v = block_sum(dotf.get(), red);
     if (threadIdx.x == 0) reinterpret_cast<double*>(partial)[blockIdx.x] = v;
+    hv_finish(S, reinterpret_cast<const double*>(partial), red);
   } else {
-    // same record layout as the fixed-point reductions: (lo, lo >> 64, hi, max)
-    __shared__ unsigned long long sm[32][3];
-    I192 doti = a192_get(dota);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const I192 w = i192_shfl_down(doti, o);
-      i192_add(doti, w);
-    }
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-      sm[wid][0] = (unsigned long long)doti.lo;
-      sm[wid][1] = (unsigned long long)(doti.lo >> 64);
-      sm[wid][2] = (unsigned long long)doti.hi;
-    }
-    __syncthreads();
-    if (wid == 0) {
-      I192 s;
-      i192_zero(s);
-      if (lane < T / 32) {
-        s.lo = ((u128)sm[lane][1] << 64) | (u128)sm[lane][0];
-        s.hi = (long long)sm[lane][2];
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const I192 w = i192_shfl_down(s, o);
-        i192_add(s, w);
-      }
-      if (lane == 0) {
-        long long* out = reinterpret_cast<long long*>(partial) + 4 * blockIdx.x;
-        out[0] = (long long)(unsigned long long)s.lo;
-        out[1] = (long long)(unsigned long long)(s.lo >> 64);
-        out[2] = s.hi;
-        out[3] = 0;
-      }
-    }
+    long long* part = reinterpret_cast<long long*>(partial);
+    fx_block_reduce(a192_get(dota), 0, part + 4 * blockIdx.x);
+    fx_hv_finish(S, cur, part);
   }
 }
 

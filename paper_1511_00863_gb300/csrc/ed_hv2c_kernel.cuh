@@ -56,7 +56,7 @@ __device__ __forceinline__ void cmacf(float2& a, const float2& b, const float2& 
 template <int R, int V, int T, int MB>
 __global__ void __launch_bounds__(T, MB)
 hv2c_kernel(Hv2cArgs a, const float2* __restrict__ x, float2* __restrict__ y,
-            const LzScalars* __restrict__ S, int cur, double* __restrict__ partial) {
+            LzScalars* S, int cur, double* __restrict__ partial) {
   constexpr int G = hv2_group<float2, R>();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[33];
@@ -68,15 +68,22 @@ hv2c_kernel(Hv2cArgs a, const float2* __restrict__ x, float2* __restrict__ y,
   int64_t* upoff = reinterpret_cast<int64_t*>(amp + ((a.namp + 1) & ~1));
   int32_t* upamp = reinterpret_cast<int32_t*>(upoff + R * MH);
   __shared__ int nup_s[R];
-  const int64_t g0 = (int64_t)blockIdx.x * R;
+  for (int i = threadIdx.x; i < a.namp; i += T) amp[i] = hv2c_amp(a, i);
+  const int j = S->j + 1;
+  const float sc = (float)S->scale[cur];
+  const float bsp = (float)(S->beta[j] * S->scale[1 - cur]);
+  DotAcc<float> dot;
+  // one resident wave of CTAs, each takes the row groups blockIdx.x, blockIdx.x + gridDim.x, ...
+  const int ngroups = (int)((a.dim_up + R - 1) / R);
+  for (int g = blockIdx.x; g < ngroups; g += gridDim.x) {
+  if (g != (int)blockIdx.x) __syncthreads();
   int64_t urow[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const int64_t g = g0 + r;
-    urow[r] = g < a.dim_up ? (a.order ? (int64_t)a.order[g] : g) : a.dim_up;
+    const int64_t q = (int64_t)g * R + r;
+    urow[r] = q < a.dim_up ? (a.order ? (int64_t)a.order[q] : q) : a.dim_up;
   }
-  // ---- stage the R rows into their slots (zero slots ld .. ld + G - 1), the amplitude
-  // table, the up-hop lists
+  // ---- stage the R rows into their slots (zero slots ld .. ld + G - 1), the up-hop lists
   for (int d = threadIdx.x; d < ld + G; d += T) {
     Pack<float2, R> p;
 #pragma unroll
@@ -86,7 +93,6 @@ hv2c_kernel(Hv2cArgs a, const float2* __restrict__ x, float2* __restrict__ y,
     }
     xs[d < ld ? (d & ~(G - 1)) | a.slot_lo[d] : d] = p;
   }
-  for (int i = threadIdx.x; i < a.namp; i += T) amp[i] = hv2c_amp(a, i);
   for (int i = threadIdx.x; i < R * a.maxhops_up; i += T) {
     const int r = i / a.maxhops_up, k = i - r * a.maxhops_up;
     int64_t u = a.dim_up;
@@ -121,10 +127,6 @@ hv2c_kernel(Hv2cArgs a, const float2* __restrict__ x, float2* __restrict__ y,
     ub[r] = (urow[r] < a.dim_up) ? a.up_bits[urow[r]] : 0u;
     nup[r] = nup_s[r];
   }
-  const int j = S->j + 1;
-  const float sc = (float)S->scale[cur];
-  const float bsp = (float)(S->beta[j] * S->scale[1 - cur]);
-  DotAcc<float> dot;
 
   for (int d0 = threadIdx.x * V; d0 < ld; d0 += T * V) {
     float2 acc[R][V];
@@ -183,8 +185,10 @@ hv2c_kernel(Hv2cArgs a, const float2* __restrict__ x, float2* __restrict__ y,
       *reinterpret_cast<Pack<float2, V>*>(yp) = W;
     }
   }
+  }
   const double v = block_sum(dot.get(), red);
   if (threadIdx.x == 0) partial[blockIdx.x] = v;
+  hv_finish(S, partial, red);
 }
 
 }  // namespace ed

@@ -36,7 +36,7 @@ struct Hv2sArgs {
 template <typename E, int V, int T, int MB>
 __global__ void __launch_bounds__(T, MB)
 hv2s_kernel(Hv2sArgs a, const E* __restrict__ x, E* __restrict__ y,
-            const LzScalars* __restrict__ S, int cur, void* __restrict__ partial) {
+            LzScalars* S, int cur, void* __restrict__ partial) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int npos_s, nneg_s;
   __shared__ double red[33];
@@ -46,33 +46,6 @@ hv2s_kernel(Hv2sArgs a, const E* __restrict__ x, E* __restrict__ y,
   constexpr int G = hv2_group<E, 1>();
   E* xs = reinterpret_cast<E*>(smem);
   int64_t* upoff = reinterpret_cast<int64_t*>(smem + ((size_t)a.nslots * sizeof(E) + 15) / 16 * 16);
-  uint32_t* upraw = reinterpret_cast<uint32_t*>(upoff + MH);
-  const int64_t g = blockIdx.x;
-  const int64_t u = a.order ? (int64_t)a.order[g] : g;
-  // ---- up-hop list of the row: positives first, negatives after
-  for (int k = threadIdx.x; k < a.maxhops_up; k += T)
-    upraw[k] = (uint32_t)a.hop_up[(int64_t)k * a.dim_up + u];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int np = 0, nn = 0;
-    for (int k = 0; k < a.maxhops_up; ++k) {
-      const uint32_t e = upraw[k];
-      const int64_t tg = (int64_t)(e & kTargetMask);
-      if (tg >= a.dim_up) break;
-      if (!(e & kSignBit)) upoff[np++] = tg * ld;
-    }
-    for (int k = 0; k < a.maxhops_up; ++k) {
-      const uint32_t e = upraw[k];
-      const int64_t tg = (int64_t)(e & kTargetMask);
-      if (tg >= a.dim_up) break;
-      if (e & kSignBit) upoff[np + nn++] = tg * ld;
-    }
-    npos_s = np;
-    nneg_s = nn;
-  }
-  __syncthreads();
-  const int npos = npos_s, nneg = nneg_s;
-  const uint32_t ub = a.up_bits[u];
   float sc = 1.f, bsp = 0.f;
   long long ca = 0, cb = 0, cc = 0;
   int ck = 0;
@@ -88,6 +61,15 @@ hv2s_kernel(Hv2sArgs a, const E* __restrict__ x, E* __restrict__ y,
   }
   DotAcc<float> dotf;
   A192 dota;
+  // one resident wave of CTAs, each takes rows blockIdx.x, blockIdx.x + gridDim.x, ...
+  for (int g = blockIdx.x; g < (int)a.dim_up; g += gridDim.x) {
+  const int64_t u = a.order ? (int64_t)a.order[g] : g;
+  __syncthreads();
+  if (threadIdx.x < 32)
+    hv2_up_list(a.hop_up, a.maxhops_up, a.dim_up, u, ld, upoff, &npos_s, &nneg_s);
+  __syncthreads();
+  const int npos = npos_s, nneg = nneg_s;
+  const uint32_t ub = a.up_bits[u];
   const E* xrow = x + u * ld;
   for (int s = 0; s < 2; ++s) {
     const int c0 = s ? a.cstart1 : a.cstart0, c1 = s ? a.cstart2 : a.cstart1;
@@ -170,46 +152,15 @@ hv2s_kernel(Hv2sArgs a, const E* __restrict__ x, E* __restrict__ y,
       stcs_pack(reinterpret_cast<Pack<E, V>*>(yp), W);
     }
   }
+  }
   if constexpr (sizeof(E) == 4) {
     const double v = block_sum(dotf.get(), red);
     if (threadIdx.x == 0) reinterpret_cast<double*>(partial)[blockIdx.x] = v;
+    hv_finish(S, reinterpret_cast<const double*>(partial), red);
   } else {
-    // same record layout as the fixed-point reductions: (lo, lo >> 64, hi, max)
-    __shared__ unsigned long long sm[32][3];
-    I192 doti = a192_get(dota);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const I192 w = i192_shfl_down(doti, o);
-      i192_add(doti, w);
-    }
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) {
-      sm[wid][0] = (unsigned long long)doti.lo;
-      sm[wid][1] = (unsigned long long)(doti.lo >> 64);
-      sm[wid][2] = (unsigned long long)doti.hi;
-    }
-    __syncthreads();
-    if (wid == 0) {
-      I192 tot;
-      i192_zero(tot);
-      if (lane < T / 32) {
-        tot.lo = ((u128)sm[lane][1] << 64) | (u128)sm[lane][0];
-        tot.hi = (long long)sm[lane][2];
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const I192 w = i192_shfl_down(tot, o);
-        i192_add(tot, w);
-      }
-      if (lane == 0) {
-        long long* out = reinterpret_cast<long long*>(partial) + 4 * blockIdx.x;
-        out[0] = (long long)(unsigned long long)tot.lo;
-        out[1] = (long long)(unsigned long long)(tot.lo >> 64);
-        out[2] = tot.hi;
-        out[3] = 0;
-      }
-    }
+    long long* part = reinterpret_cast<long long*>(partial);
+    fx_block_reduce(a192_get(dota), 0, part + 4 * blockIdx.x);
+    fx_hv_finish(S, cur, part);
   }
 }
 

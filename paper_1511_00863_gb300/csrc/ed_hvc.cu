@@ -208,6 +208,7 @@ hvc_staged_kernel(HvcArgs a, const typename CVec<T>::type* __restrict__ x,
   if (kLz) {
     const double v = block_sum(dot.get(), red);
     if (threadIdx.x == 0) lz.partial[blockIdx.x] = v;
+    hv_finish(lz.S, lz.partial, red);
   }
 }
 
@@ -266,6 +267,7 @@ hvc_global_kernel(HvcArgs a, const typename CVec<T>::type* __restrict__ x,
   if (kLz) {
     const double v = block_sum(dot.get(), red);
     if (threadIdx.x == 0) lz.partial[blockIdx.x] = v;
+    hv_finish(lz.S, lz.partial, red);
   }
 }
 

@@ -125,6 +125,7 @@ struct LzScalars {
                     // stream had already enqueued behind it may have advanced j further
   int chk;          // convergence checks have covered the steps up to here
   unsigned tick_chk;  // CTAs of the running check that are done
+  unsigned tick_hv, tick_upd;  // CTAs of the running H.v / update pass that are done
   int max_steps;
   double tol;
   double tscale;    // max over i <= j of |a_i| + b_i (breakdown scale)
@@ -134,6 +135,8 @@ struct LzScalars {
   long long fx_a, fx_b, fx_c;   // H.v epilogue W = round((a S + b n X + c P) 2^fx_k)
   int fx_k, fx_r;               // ... and W's scale s_w = scale[cur] * 2^fx_r
   double fx_sw;
+  long long fx_d;               // update Q = W + round(d X 2^fx_k2)
+  int fx_k2, pad_;
   double alpha[ED_MAX_STEPS + 2];
   double beta[ED_MAX_STEPS + 2];
   double E0[ED_MAX_STEPS + 2];
@@ -142,8 +145,9 @@ struct LzScalars {
 // Extra arguments of the Lanczos-fused H.v pass:
 //   w = scale[cur] * H B_cur - b_j * scale[prev] * B_prev   (written over B_prev)
 //   partial[block] = sum over the block's elements of w * (scale[cur] * B_cur)
+// The last CTA sums the partials into alpha[j + 1].
 struct LzHvArgs {
-  const LzScalars* S;
+  LzScalars* S;
   int cur;
   double* partial;
 };
@@ -186,10 +190,13 @@ ed_status fx_copy_in(const ed_basis* b, const FxRun& fx, const double* f1, long 
                      int64_t ld, const int32_t* colpos, LzScalars* S, long long* part,
                      cudaStream_t s);
 // One step of Algorithm 1 on the fixed-point buffers (cur holds f_j, the other f_{j-1}).
+// Needs the step's integer coefficients: fx_plan before the first step of a call, afterwards
+// each step leaves the next one's (same t, U).
 ed_status fx_step(const ed_basis* b, const FxRun& fx, double t, double U, long long* const B[2],
                   int cur, int64_t ld, LzScalars* S, long long* pa, long long* pb,
                   cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, const struct Hv2Plan* plan,
                   const Reorth* ro = nullptr);
+ed_status fx_plan(const FxRun& fx, double t, double U, int cur, LzScalars* S, cudaStream_t s);
 ed_status fx_prepare(const ed_basis* b);
 // Ground-state vector (ed_lanczos_ground_state): P += round(y_j scale[cur] 2^60 X_cur),
 // and the final normalised, sign-gauged FP64 vector. part: >= 6 * 4 * sm_count longs.
@@ -208,6 +215,8 @@ ed_status ro_prepare(const Reorth* r);
 ed_status ro_reset(const Reorth* r, const LzScalars* S, const void* buf0, cudaStream_t s);
 // After the finish pass: store f_{j+1} (buffer buf, scale S->scale[buf]) in slot S->j.
 ed_status ro_store(const Reorth* r, const LzScalars* S, int buf, const void* src, cudaStream_t s);
+// Whether a run has passes between the update and the finish (modes 1 and 2).
+bool ro_between(const Reorth* r);
 // Between the update pass (residual Q, its partial norm records pb[nb]) and the finish pass.
 ed_status ro_apply(const Reorth* r, const LzScalars* S, void* Q, void* pb, int nb, cudaStream_t s);
 // Number of steps reorthogonalised so far in the current run (synchronises s).
@@ -238,9 +247,9 @@ int hv2_kind(const Hv2Plan* p);
 // Time every fused H.v variant that fits on x (f_j) and y (f_{j-1} / w) with scalars S
 // (zeroed: a neutral step) and return the fastest variant id (0 if none fits).
 ed_status hv2_autotune(const ed_basis* b, int mode, int ld, void* x, void* y,
-                       const LzScalars* S, void* partial, cudaStream_t s, int* kind);
+                       LzScalars* S, void* partial, cudaStream_t s, int* kind);
 ed_status hv2_launch(const Hv2Plan* p, const ed_basis* b, double t, double U, const void* x,
-                     void* y, const LzScalars* S, int cur, void* partial, cudaStream_t s);
+                     void* y, LzScalars* S, int cur, void* partial, cudaStream_t s);
 
 // Upper bound on the number of CTAs of any H.v launch of a Lanczos step (launch_hv,
 // launch_hvc, the fixed-point kernels, the fused plans): the size of the partial-sum buffer.
@@ -288,16 +297,52 @@ __device__ __forceinline__ double block_sum(double v, double* sm) {
   return v;
 }
 
-// Sum of n partials in a fixed order by one block (every thread gets the result).
+// True in the CTA that is the last of its launch to get here (for all its threads); it sees
+// what thread 0 of every other CTA wrote before. The reductions of a pass end in that CTA
+// instead of a launch of their own, or of every CTA of the next pass: summing the H.v's 4,368
+// records in each of the update pass's 608 CTAs took 4-5 us of its 91 on the 4x4 lattice.
+__device__ __forceinline__ bool last_cta(unsigned* ticket) {
+  __shared__ int last_s;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last_s = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last_s) return false;
+  if (threadIdx.x == 0) *ticket = 0;
+  __threadfence();
+  return true;
+}
+
+// Sum of n partials in a fixed order by one block (every thread gets the result). They may
+// come from other CTAs of the running launch: read from L2.
 __device__ __forceinline__ double block_sum_array(const double* p, int64_t n, double* sm) {
   double v = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) v += p[i];
+  // eight loads in flight, added in the order of a plain loop
+  for (int64_t i = threadIdx.x; i < n; i += 8 * (int64_t)blockDim.x) {
+    double w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int64_t q = i + k * (int64_t)blockDim.x;
+      w[k] = q < n ? __ldcg(p + q) : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (i + k * (int64_t)blockDim.x < n) v += w[k];
+  }
   v = block_sum(v, sm);
   if (threadIdx.x == 0) sm[32] = v;
   __syncthreads();
   v = sm[32];
   __syncthreads();
   return v;
+}
+
+// End of a Lanczos-fused H.v: the last CTA records a_{j+1} = the sum of the CTAs' partials.
+__device__ __forceinline__ void hv_finish(LzScalars* S, const double* partial, double* red) {
+  if (!last_cta(&S->tick_hv)) return;
+  const double a = block_sum_array(partial, gridDim.x, red);
+  if (threadIdx.x == 0) S->alpha[S->j + 1] = a;
 }
 
 }  // namespace ed

@@ -1,13 +1,13 @@
 // Lanczos iteration (Sec. 2.2, Algorithm 1) on the device, the random start vector, and
 // the lowest eigenvalue of the tridiagonal T by Sturm-sequence bisection in FP64.
 //
-// One step j is three launches on the run's stream:
+// One step j is two launches on the run's stream:
 //   1. fused H.v:  w = H f_j - b_j f_{j-1}, written over the f_{j-1} buffer, with per-CTA
-//      partial sums of w . f_j  (ed_hv.cu, LzHvArgs);
-//   2. update:     a_j = sum of the partials (every CTA sums them in the same order),
-//      q = w - a_j f_j in place, per-CTA partial sums of q . q;
-//   3. finish (one CTA): b_{j+1} = sqrt(sum), breakdown test, f_{j+1} = q / b_{j+1} kept
-//      implicit as a buffer scale.
+//      partial sums of w . f_j  (ed_hv.cu, LzHvArgs); the last CTA sums them to a_j;
+//   2. update:     q = w - a_j f_j in place, per-CTA partial sums of q . q; the last CTA sums
+//      them (finish): b_{j+1} = sqrt(sum), breakdown test, f_{j+1} = q / b_{j+1} kept implicit
+//      as a buffer scale.
+// (Reorthogonalisation runs between the update and a finish launch of its own.)
 // E0(j) = lambda_min(T_j) and the convergence test run beside the next steps, on a stream of
 // their own (lz_check_kernel).
 // Each buffer holds an unnormalised vector B with f = scale * B, so no pass rescales it.
@@ -104,16 +104,24 @@ __global__ void init_scalars_kernel(LzScalars* S, const double* __restrict__ par
 }
 
 // ------------------------------------------------------------------ update
+// Whole CTA: b_{j+1} and f_{j+1}'s scale from the nb partial sums of q . q.
+__device__ __forceinline__ void lz_finish_step(LzScalars* S, int cur, const double* pb, int nb,
+                                               double* red) {
+  const double b2 = block_sum_array(pb, nb, red);
+  if (threadIdx.x != 0) return;
+  const double beta = sqrt(b2);
+  if (finish_step(S, S->j + 1, beta)) S->scale[1 - cur] = 1.0 / beta;
+}
+
+// finish: the last CTA ends the step (lz_finish_step); otherwise lz_finish_kernel does, after
+// the reorthogonalisation.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
 lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restrict__ bprev,
-                 int64_t n, const double* __restrict__ pa, int na, double* __restrict__ pb) {
+                 int64_t n, double* __restrict__ pb, int finish) {
   __shared__ double red[33];
   if (S->status != 0) return;
-  const double a = block_sum_array(pa, na, red);
-  const int j = S->j + 1;
-  if (blockIdx.x == 0 && threadIdx.x == 0) S->alpha[j] = a;
-  const T coef = (T)(a * S->scale[cur]);
+  const T coef = (T)(S->alpha[S->j + 1] * S->scale[cur]);
   DotAcc<T> acc;
   // n is a multiple of 32 (padded rows): 16-byte vectors of 16 / sizeof(T) elements
   constexpr int VE = 16 / sizeof(T);
@@ -137,18 +145,13 @@ lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restric
   }
   const double v = block_sum(acc.get(), red);
   if (threadIdx.x == 0) pb[blockIdx.x] = v;
+  if (finish && last_cta(&S->tick_upd)) lz_finish_step(S, cur, pb, gridDim.x, red);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
 lz_finish_kernel(LzScalars* S, int cur, const double* __restrict__ pb, int nb) {
   __shared__ double red[33];
-  if (S->status != 0) return;
-  const int j = S->j + 1;
-  const double b2 = block_sum_array(pb, nb, red);
-  if (threadIdx.x == 0) {
-    const double beta = sqrt(b2);
-    if (finish_step(S, j, beta)) S->scale[1 - cur] = 1.0 / beta;
-  }
+  if (S->status == 0) lz_finish_step(S, cur, pb, nb, red);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
@@ -269,6 +272,11 @@ struct ed_lanczos {
   LzScalars* host = nullptr;  // [1] and the two batches' headers behind it
 };
 
+// Before the first step of a call: the fixed-point coefficients for these parameters.
+static ed_status lz_plan(const ed_lanczos* st, const ed_params* p) {
+  return st->fx ? fx_plan(st->fxr, p->t, p->U, st->cur, st->S, st->stream) : ED_OK;
+}
+
 static ed_status lz_launch_step(ed_lanczos* st, const ed_params* p, cudaStream_t s,
                                 cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr) {
   const ed_basis* b = st->basis;
@@ -281,38 +289,39 @@ static ed_status lz_launch_step(ed_lanczos* st, const ed_params* p, cudaStream_t
     return r;
   }
   LzHvArgs lz{st->S, c, st->pa};
-  int grid = 0;
   ed_status r;
   if (ev0) ED_TRY_CUDA(cudaEventRecord(ev0, s));
   const ed_dtype dt = st->opts.dtype;
   if (st->plan) {
-    grid = hv2_grid(st->plan);
     r = hv2_launch(st->plan, b, p->t, p->U, st->B[c], st->B[1 - c], st->S, c, st->pa, s);
   } else if (dt == ED_C32) {
-    r = launch_hvc<float>(b, p->t, p->U, st->B[c], st->B[1 - c], st->ld, s, &lz, &grid);
+    r = launch_hvc<float>(b, p->t, p->U, st->B[c], st->B[1 - c], st->ld, s, &lz);
   } else if (dt == ED_C64) {
-    r = launch_hvc<double>(b, p->t, p->U, st->B[c], st->B[1 - c], st->ld, s, &lz, &grid);
+    r = launch_hvc<double>(b, p->t, p->U, st->B[c], st->B[1 - c], st->ld, s, &lz);
   } else if (dt == ED_F64_NATIVE)
     r = launch_hv<double>(b, p->t, p->U, (const double*)st->B[c], (double*)st->B[1 - c], st->ld,
-                          s, &lz, &grid);
+                          s, &lz);
   else
     r = launch_hv<float>(b, p->t, p->U, (const float*)st->B[c], (float*)st->B[1 - c], st->ld,
-                         s, &lz, &grid);
+                         s, &lz);
   if (r != ED_OK) return r;
   if (ev1) ED_TRY_CUDA(cudaEventRecord(ev1, s));
   // the update works on scalars: a complex vector is 2 n of them (a_j, b_j are real)
   const int64_t ns = is_complex(dt) ? 2 * st->n : st->n;
   const int ug = red_grid(ns);
+  const bool between = st->ro && ro_between(st->ro);  // passes between the update and the finish
   if (dt == ED_F64_NATIVE || dt == ED_C64)
     lz_update_kernel<double><<<ug, kRedThreads, 0, s>>>(
-        st->S, c, (const double*)st->B[c], (double*)st->B[1 - c], ns, st->pa, grid, st->pb);
+        st->S, c, (const double*)st->B[c], (double*)st->B[1 - c], ns, st->pb, !between);
   else
     lz_update_kernel<float><<<ug, kRedThreads, 0, s>>>(
-        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pa, grid, st->pb);
+        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pb, !between);
   ED_TRY_CUDA(cudaGetLastError());
-  if (st->ro && (r = ro_apply(st->ro, st->S, st->B[1 - c], st->pb, ug, s)) != ED_OK) return r;
-  lz_finish_kernel<<<1, kRedThreads, 0, s>>>(st->S, c, st->pb, ug);
-  ED_TRY_CUDA(cudaGetLastError());
+  if (between) {
+    if ((r = ro_apply(st->ro, st->S, st->B[1 - c], st->pb, ug, s)) != ED_OK) return r;
+    lz_finish_kernel<<<1, kRedThreads, 0, s>>>(st->S, c, st->pb, ug);
+    ED_TRY_CUDA(cudaGetLastError());
+  }
   if (st->ro && (r = ro_store(st->ro, st->S, 1 - c, st->B[1 - c], s)) != ED_OK) return r;
   st->cur = 1 - c;
   return ED_OK;
@@ -637,7 +646,8 @@ extern "C" ed_status ed_lanczos_step(ed_lanczos* st, const ed_params* p, double*
   clear_error();
   ED_CHECK_ARG(st != nullptr && p != nullptr, "ed_lanczos_step: state or params is NULL");
   ED_CHECK_ARG(!st->stopped, "ed_lanczos_step: the run has stopped (breakdown or max_steps)");
-  ed_status r = lz_launch_step(st, p, st->stream);
+  ed_status r = lz_plan(st, p);
+  if (r == ED_OK) r = lz_launch_step(st, p, st->stream);
   if (r != ED_OK) return r;
   int hdr[2];
   ED_TRY_CUDA(cudaMemcpyAsync(hdr, st->S, 2 * sizeof(int), cudaMemcpyDeviceToHost, st->stream));
@@ -657,6 +667,10 @@ extern "C" ed_status ed_lanczos_run(ed_lanczos* st, const ed_params* p, int32_t 
   clear_error();
   ED_CHECK_ARG(st != nullptr && p != nullptr, "ed_lanczos_run: state or params is NULL");
   ED_CHECK_ARG(nsteps >= 0 && nsteps <= ED_MAX_STEPS, "ed_lanczos_run: nsteps out of range");
+  {
+    const ed_status r = lz_plan(st, p);
+    if (r != ED_OK) return r;
+  }
   if (!hv_ms) {
     for (int i = 0; i < nsteps; ++i) {
       ed_status r = lz_launch_step(st, p, st->stream);
@@ -760,7 +774,7 @@ extern "C" ed_status ed_lanczos_ground_state(const ed_basis* b, const ed_params*
   // ---- pass 1: Algorithm 1 to convergence, tested after every 8 steps
   ed_status r = lz_init(b, o, f1, s, &st);
   if (r != ED_OK) return r;
-  if ((r = fx_prepare(b)) != ED_OK) return r;
+  if ((r = fx_prepare(b)) != ED_OK || (r = lz_plan(st, p)) != ED_OK) return r;
   ED_TRY_CUDA(cudaMemsetAsync(&st->S->chk, 0, sizeof(int), s));
   LzScalars hs;
   constexpr size_t kHead = offsetof(LzScalars, tick_chk);
@@ -794,6 +808,7 @@ extern "C" ed_status ed_lanczos_ground_state(const ed_basis* b, const ed_params*
   if (cudaMalloc((void**)&P, (size_t)b->dim * sizeof(long long)) != cudaSuccess)
     return ED_ERR_OOM;
   ED_TRY_CUDA(cudaMemsetAsync(P, 0, (size_t)b->dim * sizeof(long long), s));
+  if ((r = lz_plan(st, p)) != ED_OK) return r;
   for (int j = 1; j <= m; ++j) {
     if ((r = fx_psi_accum(b, st->S, st->cur, yd, j, (const long long*)st->B[st->cur], st->ld,
                           hv2_colpos(st->plan), P, s)) != ED_OK)
@@ -903,6 +918,7 @@ static ed_status lz_iterate(ed_lanczos* st, const ed_params* p, const ed_opts* o
   const bool check = o->tol > 0.0;
   int n = 0;
   ed_status r = lz_graph(st, p, check, &n);
+  if (r == ED_OK) r = lz_plan(st, p);
   if (r != ED_OK) return r;
   // batches of about 8 steps, the host one batch behind the device: it reads the status of a
   // batch while the next one runs (a stopped run's remaining kernels return at entry)

@@ -488,9 +488,11 @@ ed_status ro_prepare(const Reorth* r) {
   return ED_OK;
 }
 
+// Mode 3 stores the vectors and never reorthogonalises.
+bool ro_between(const Reorth* r) { return r->mode != 3; }
+
 // Between the update pass (q and its partial norms in pb, nb records) and the finish pass.
 ed_status ro_apply(const Reorth* r, const LzScalars* S, void* Q, void* pb, int nb, cudaStream_t s) {
-  if (r->mode == 3) return ED_OK;  // vectors are stored, never reorthogonalised
   ro_decide_kernel<<<1, kRoThreads, 0, s>>>(S, r->F, r->omega, r->mode, r->kind, pb, nb, r->slots,
                                             r->eps, r->psi);
   if (r->kind == 0)
