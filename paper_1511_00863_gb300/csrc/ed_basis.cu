@@ -260,6 +260,7 @@ extern "C" ed_status ed_build_basis(const ed_lattice* L, int32_t n_up, int32_t n
       ED_CHECK_ARG(std::isfinite(L->t_bond[b]), "ed_build_basis: t_bond[%d] is not finite", b);
   cudaStream_t s = (cudaStream_t)stream;
   ed_basis* B = new ed_basis();
+  psi_pool_basis(+1);
   cudaGetDevice(&B->device);
   B->n_sites = L->n_sites;
   B->n_up = n_up;
@@ -373,6 +374,7 @@ extern "C" void ed_basis_destroy(ed_basis* B) {
   if (B->up_order) cudaFree(B->up_order);
   if (B->tau) cudaFree(B->tau);
   if (prev != B->device) cudaSetDevice(prev);
+  psi_pool_basis(-1);
   delete B;
 }
 

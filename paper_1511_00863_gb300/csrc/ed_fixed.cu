@@ -318,7 +318,7 @@ fx_hv_global_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __re
 // Whole CTA: b_{j+1} and f_{j+1}'s scale from the n partial records of ||Q||^2, then the
 // coefficients of the next H.v.
 __device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long long* pb, int nb,
-                                               const FxPlanArgs& p) {
+                                               const FxPlanArgs& p, double* vscale) {
   I192 sum;
   long long mx;
   fx_sum_partials(pb, nb, sum, mx);
@@ -329,6 +329,7 @@ __device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long
   if (finish_step(S, j, beta)) {
     S->scale[1 - cur] = sw / beta;
     S->fx_max[1 - cur] = mx;
+    if (vscale) vscale[j] = sw / beta;
     fx_plan_step(S, 1 - cur, p);
   }
 }
@@ -337,8 +338,9 @@ __device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long
 // the reorthogonalisation.
 __global__ void __launch_bounds__(kFxThreads)
 fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long long* __restrict__ xp,
-                 int64_t n, long long* __restrict__ pb, int finish, FxPlanArgs plan) {
+                 int64_t n, long long* __restrict__ pb, int finish, FxPlanArgs plan, LzStore store) {
   if (S->status != 0) return;
+  longlong2* const keep = store.slots ? (longlong2*)store.slots[S->j + 1] : nullptr;
   const long long d = S->fx_d;
   const int k2 = S->fx_k2;
   A192 q2;
@@ -363,16 +365,22 @@ fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long l
       w1 = p2[i + stride];
       c1 = c2[i + stride];
     }
-    p2[i] = make_longlong2(upd(w0.x, c0.x), upd(w0.y, c0.y));
-    if (two) p2[i + stride] = make_longlong2(upd(w1.x, c1.x), upd(w1.y, c1.y));
+    const longlong2 r0 = make_longlong2(upd(w0.x, c0.x), upd(w0.y, c0.y));
+    p2[i] = r0;
+    if (keep) __stcs(keep + i, r0);
+    if (two) {
+      const longlong2 r1 = make_longlong2(upd(w1.x, c1.x), upd(w1.y, c1.y));
+      p2[i + stride] = r1;
+      if (keep) __stcs(keep + i + stride, r1);
+    }
   }
   fx_block_reduce(a192_get(q2), mx, pb + 4 * blockIdx.x);
-  if (finish && last_cta(&S->tick_upd)) fx_finish_step(S, cur, pb, gridDim.x, plan);
+  if (finish && last_cta(&S->tick_upd)) fx_finish_step(S, cur, pb, gridDim.x, plan, store.vscale);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
 fx_finish_kernel(LzScalars* S, int cur, const long long* __restrict__ pb, int nb, FxPlanArgs plan) {
-  if (S->status == 0) fx_finish_step(S, cur, pb, nb, plan);
+  if (S->status == 0) fx_finish_step(S, cur, pb, nb, plan, nullptr);
 }
 
 // ------------------------------------------------------------------ ground-state vector
@@ -398,19 +406,123 @@ fx_psi_accum_kernel(const LzScalars* __restrict__ S, int cur, const double* __re
   }
 }
 
-// Largest |P_i| and its lowest index: partial records (value, index) per CTA.
+// Partial records of max |P| with its lowest index and of ||P||^2 (exact).
+__device__ __forceinline__ void fx_psi_records(long long bv, long long bi, const I192& nrm,
+                                               long long* amax, long long* part) {
+  __shared__ long long sv[32], si[32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long v2 = __shfl_down_sync(0xffffffffu, bv, o), i2 = __shfl_down_sync(0xffffffffu, bi, o);
+    if (v2 > bv || (v2 == bv && i2 < bi)) bv = v2, bi = i2;
+  }
+  if ((threadIdx.x & 31) == 0) sv[threadIdx.x >> 5] = bv, si[threadIdx.x >> 5] = bi;
+  fx_block_reduce(nrm, 0, part + 4 * blockIdx.x);  // (a barrier in it covers sv, si)
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+      if (sv[w] > bv || (sv[w] == bv && si[w] < bi)) bv = sv[w], bi = si[w];
+    amax[2 * blockIdx.x] = bv;
+    amax[2 * blockIdx.x + 1] = bi;
+  }
+}
+
+// rank[p] = the down rank at column p of the stored rows, -1 for a pad.
+__global__ void fx_rank_kernel(const int32_t* __restrict__ colpos, int64_t cols, int64_t ld,
+                               int32_t* __restrict__ rank, int pads) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (pads ? ld : cols);
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (pads) rank[i] = -1;
+    else rank[colpos ? colpos[i] : i] = (int32_t)i;
+  }
+}
+
+// P = sum_k round(y_{k+1} s_k 2^60 X_k) over the m stored vectors, two columns per thread, and
+// the records of P. HBM bound: every vector is read once, coalesced, four of them in flight;
+// the element goes to its rank (scattered within its row) once. Against regenerating the
+// vectors (a second run of the m H.v and update passes and a read-modify-write of P per step)
+// the half-filled 14-site ring's 78 vectors of 94 MB take about 1.4 ms instead of 26.
 __global__ void __launch_bounds__(kFxThreads)
-fx_psi_argmax_kernel(const long long* __restrict__ P, int64_t n, long long* __restrict__ part) {
-  __shared__ long long sv[kFxThreads];
-  __shared__ long long si[kFxThreads];
+fx_psi_sum_kernel(const double* __restrict__ y, int m, LzStore store, int64_t rows, int64_t cols,
+                  int64_t ld, const int32_t* __restrict__ rank, long long* __restrict__ P,
+                  long long* __restrict__ amax, long long* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char psi_smem[];
+  long long* mant = reinterpret_cast<long long*>(psi_smem);
+  const longlong2** vec = reinterpret_cast<const longlong2**>(mant + m);
+  int* expo = reinterpret_cast<int*>(vec + m);
+  for (int k = threadIdx.x; k < m; k += blockDim.x) {
+    const double c = y[k + 1] * store.vscale[k] * 0x1.0p60;
+    long long q = 0;
+    int e = -1;
+    if (c != 0.0 && isfinite(c)) {
+      e = ilogb(c) - 61;
+      q = llrint(ldexp(c, -e));
+    }
+    mant[k] = q;
+    expo[k] = e;
+    vec[k] = reinterpret_cast<const longlong2*>(store.slots[k]);
+  }
+  __syncthreads();
+  const int64_t pairs = rows * (ld / 2);
   long long bv = -1, bi = 0;
+  A192 nrm;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < pairs;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    long long s0 = 0, s1 = 0;
+    int k = 0;
+    for (; k + 4 <= m; k += 4) {
+      longlong2 x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[q] = __ldcs(vec[k + q] + i);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        s0 += round_shift128(smul128(mant[k + q], x[q].x), expo[k + q]);
+        s1 += round_shift128(smul128(mant[k + q], x[q].y), expo[k + q]);
+      }
+    }
+    for (; k < m; ++k) {
+      const longlong2 x = __ldcs(vec[k] + i);
+      s0 += round_shift128(smul128(mant[k], x.x), expo[k]);
+      s1 += round_shift128(smul128(mant[k], x.y), expo[k]);
+    }
+    const int64_t r = i / (ld / 2), p = 2 * (i - r * (ld / 2));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int32_t d = rank[p + q];
+      if (d < 0) continue;
+      const long long v = q ? s1 : s0, e = r * cols + d;
+      P[e] = v;
+      const long long av = v < 0 ? -v : v;
+      a192_add_sq(nrm, (unsigned long long)av);
+      if (av > bv || (av == bv && e < bi)) bv = av, bi = e;
+    }
+  }
+  fx_psi_records(bv, bi, a192_get(nrm), amax, part);
+}
+
+// The same records for a P in memory.
+__global__ void __launch_bounds__(kFxThreads)
+fx_psi_records_kernel(const long long* __restrict__ P, int64_t n, long long* __restrict__ amax,
+                      long long* __restrict__ part) {
+  long long bv = -1, bi = 0;
+  A192 nrm;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const long long v = P[i] < 0 ? -P[i] : P[i];
-    if (v > bv) {
-      bv = v;
-      bi = i;
-    }
+    const long long v = P[i], av = v < 0 ? -v : v;
+    a192_add_sq(nrm, (unsigned long long)av);
+    if (av > bv) bv = av, bi = i;
+  }
+  fx_psi_records(bv, bi, a192_get(nrm), amax, part);
+}
+
+// psi (FP64) = gauge * P 2^-60 / ||P 2^-60||, gauge making the largest entry positive. The
+// factor g (one CTA): 2 x 608 records, a thread per record.
+__global__ void __launch_bounds__(kFxThreads)
+fx_psi_gauge_kernel(const long long* __restrict__ P, const long long* __restrict__ amax,
+                    const long long* __restrict__ part, int n, double* __restrict__ g) {
+  __shared__ long long sv[kFxThreads], si[kFxThreads];
+  long long bv = -1, bi = 0;
+  for (int b = threadIdx.x; b < n; b += blockDim.x) {
+    const long long v = amax[2 * b], i = amax[2 * b + 1];
+    if (v > bv || (v == bv && i < bi)) bv = v, bi = i;
   }
   sv[threadIdx.x] = bv;
   si[threadIdx.x] = bi;
@@ -425,47 +537,19 @@ fx_psi_argmax_kernel(const long long* __restrict__ P, int64_t n, long long* __re
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = sv[0];
-    part[2 * blockIdx.x + 1] = si[0];
-  }
-}
-
-// psi (FP64) = gauge * P 2^-60 / ||P 2^-60||, gauge making the largest entry positive.
-__global__ void __launch_bounds__(kFxThreads)
-fx_psi_out_kernel(const long long* __restrict__ P, int64_t n, const long long* __restrict__ amax,
-                  int namax, const long long* __restrict__ nrm_part, int nn, double* __restrict__ out) {
-  __shared__ long long best_i;
-  if (threadIdx.x == 0) {
-    long long bv = -1, bi = 0;
-    for (int b = 0; b < namax; ++b) {
-      const long long v = amax[2 * b], i = amax[2 * b + 1];
-      if (v > bv || (v == bv && i < bi)) {
-        bv = v;
-        bi = i;
-      }
-    }
-    best_i = bi;
-  }
   I192 sum;
   long long unused;
-  fx_sum_partials(nrm_part, nn, sum, unused);
-  const double nrm = sqrt(i192_to_double(sum));
-  const double g = (P[best_i] < 0 ? -1.0 : 1.0) / nrm;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (double)P[i] * g;
+  fx_sum_partials(part, n, sum, unused);
+  if (threadIdx.x == 0) *g = (P[si[0]] < 0 ? -1.0 : 1.0) / sqrt(i192_to_double(sum));
 }
 
-// Partial sums of P_i^2 (exact).
+// In place: the int64 P becomes the FP64 psi.
 __global__ void __launch_bounds__(kFxThreads)
-fx_psi_norm_kernel(const long long* __restrict__ P, int64_t n, long long* __restrict__ part) {
-  I192 acc;
-  i192_zero(acc);
+fx_psi_out_kernel(long long* __restrict__ P, int64_t n, const double* __restrict__ gauge) {
+  const double g = *gauge;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
-    i192_add(acc, (i128)P[i] * P[i]);
-  fx_block_reduce(acc, 0, part + 4 * blockIdx.x);
+    P[i] = __double_as_longlong((double)P[i] * g);
 }
 
 // ------------------------------------------------------------------ host side
@@ -518,12 +602,25 @@ ed_status fx_psi_accum(const ed_basis* b, const LzScalars* S, int cur, const dou
   return ED_OK;
 }
 
-ed_status fx_psi_finish(const ed_basis* b, const long long* P, long long* part, double* out,
+ed_status fx_psi_sum(const ed_basis* b, const double* y, int m, const LzStore& store, int64_t ld,
+                     const int32_t* colpos, int32_t* rank, long long* P, long long* part,
+                     cudaStream_t s) {
+  const int g = fx_red_grid(b->dim);
+  fx_rank_kernel<<<g, kFxThreads, 0, s>>>(colpos, b->dn.dim, ld, rank, 1);
+  fx_rank_kernel<<<g, kFxThreads, 0, s>>>(colpos, b->dn.dim, ld, rank, 0);
+  fx_psi_sum_kernel<<<g, kFxThreads, (size_t)m * 20, s>>>(y, m, store, b->up.dim, b->dn.dim, ld, rank,
+                                                          P, part, part + 2 * g);
+  ED_TRY_CUDA(cudaGetLastError());
+  return ED_OK;
+}
+
+ed_status fx_psi_finish(const ed_basis* b, long long* P, bool have_records, long long* part,
                         cudaStream_t s) {
   const int g = fx_red_grid(b->dim);
-  fx_psi_argmax_kernel<<<g, kFxThreads, 0, s>>>(P, b->dim, part);
-  fx_psi_norm_kernel<<<g, kFxThreads, 0, s>>>(P, b->dim, part + 2 * g);
-  fx_psi_out_kernel<<<g, kFxThreads, 0, s>>>(P, b->dim, part, g, part + 2 * g, g, out);
+  if (!have_records) fx_psi_records_kernel<<<g, kFxThreads, 0, s>>>(P, b->dim, part, part + 2 * g);
+  double* gauge = reinterpret_cast<double*>(part + 6 * g);
+  fx_psi_gauge_kernel<<<1, kFxThreads, 0, s>>>(P, part, part + 2 * g, g, gauge);
+  fx_psi_out_kernel<<<g, kFxThreads, 0, s>>>(P, b->dim, gauge);
   ED_TRY_CUDA(cudaGetLastError());
   return ED_OK;
 }
@@ -577,7 +674,7 @@ ed_status fx_plan(const FxRun& fx, double t, double U, int cur, LzScalars* S, cu
 ed_status fx_step(const ed_basis* b, const FxRun& fx, double t, double U, long long* const B[2],
                   int cur, int64_t ld, LzScalars* S, long long* pa, long long* pb,
                   cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, const Hv2Plan* plan,
-                  const Reorth* ro) {
+                  const LzStore& store, const Reorth* ro) {
   if (ev0) ED_TRY_CUDA(cudaEventRecord(ev0, s));
   const FxHvArgs a = fx_args(b, ld);
   const int R = plan ? -1 : fx_rows(b);
@@ -600,14 +697,14 @@ ed_status fx_step(const ed_basis* b, const FxRun& fx, double t, double U, long l
   const int ug = fx_red_grid(n);
   const FxPlanArgs next = {t, U, fx.hops, fx.nmax, fx.vb};
   const bool between = ro && ro_between(ro);  // passes between the update and the finish
-  fx_update_kernel<<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next);
+  fx_update_kernel<<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next, store);
   if (between) {
     const ed_status r = ro_apply(ro, S, B[1 - cur], pb, ug, s);
     if (r != ED_OK) return r;
     fx_finish_kernel<<<1, kRedThreads, 0, s>>>(S, cur, pb, ug, next);
   }
   ED_TRY_CUDA(cudaGetLastError());
-  if (ro) return ro_store(ro, S, 1 - cur, B[1 - cur], s);
+  if (between) return ro_store(ro, S, 1 - cur, B[1 - cur], s);
   return ED_OK;
 }
 

@@ -112,6 +112,9 @@ inline cudaError_t allow_max_smem(K kernel) {
 
 // Free the solve workspaces cached on a basis (called by ed_basis_destroy).
 void lz_cache_free(const ed_basis* b);
+// A basis was built (+1) or destroyed (-1): with the last one the ground-state pool (memory of
+// kept Lanczos vectors, ed_lanczos.cu) is given back.
+void psi_pool_basis(int delta);
 // Free the fused H.v down tables cached on a basis (called by ed_basis_destroy).
 void hv2_tables_free(const ed_basis* b);
 
@@ -171,6 +174,13 @@ ed_status launch_hvc(const ed_basis* b, double t, double U, const void* x, void*
 ed_status hvc_prepare(const ed_basis* b, ed_dtype dtype);
 inline bool is_complex(ed_dtype d) { return d == ED_C32 || d == ED_C64; }
 
+// Where a run keeps its Lanczos vectors (device tables; slots NULL: nowhere): slot k receives
+// the raw vector of f_{k+1} from the update pass, vscale[k] its scale. A NULL slot is skipped.
+struct LzStore {
+  void* const* slots;
+  double* vscale;
+};
+
 struct Reorth;  // stored Lanczos vectors for reorthogonalisation (ed_reorth.cu)
 
 // FP64-accurate Lanczos path (int64 fixed point, ed_fixed.cu).
@@ -195,21 +205,32 @@ ed_status fx_copy_in(const ed_basis* b, const FxRun& fx, const double* f1, long 
 ed_status fx_step(const ed_basis* b, const FxRun& fx, double t, double U, long long* const B[2],
                   int cur, int64_t ld, LzScalars* S, long long* pa, long long* pb,
                   cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, const struct Hv2Plan* plan,
-                  const Reorth* ro = nullptr);
+                  const LzStore& store, const Reorth* ro = nullptr);
 ed_status fx_plan(const FxRun& fx, double t, double U, int cur, LzScalars* S, cudaStream_t s);
 ed_status fx_prepare(const ed_basis* b);
-// Ground-state vector (ed_lanczos_ground_state): P += round(y_j scale[cur] 2^60 X_cur),
-// and the final normalised, sign-gauged FP64 vector. part: >= 6 * 4 * sm_count longs.
+// Ground-state vector (ed_lanczos_ground_state) in fixed point, P = psi 2^60 (rank order), from
+// the coefficients y (1-based) of f_1 .. f_m:
+//   fx_psi_sum    P = sum_j round(y_j s_j 2^60 X_j) over stored vectors, with the records of
+//                 max |P| and ||P||^2 (part: >= 6 * 4 * sm_count longs; rank: b->dn.dim
+//                 padded to ld ints of scratch);
+//   fx_psi_accum  one term of the same sum, from the running vector of step j;
+//   fx_psi_finish the records for a P summed by fx_psi_accum (have_records: already there),
+//                 then P normalised and sign-gauged in place as FP64.
+ed_status fx_psi_sum(const ed_basis* b, const double* y, int m, const LzStore& store, int64_t ld,
+                     const int32_t* colpos, int32_t* rank, long long* P, long long* part,
+                     cudaStream_t s);
 ed_status fx_psi_accum(const ed_basis* b, const LzScalars* S, int cur, const double* y, int j,
                        const long long* X, int64_t ld, const int32_t* colpos, long long* P,
                        cudaStream_t s);
-ed_status fx_psi_finish(const ed_basis* b, const long long* P, long long* part, double* out,
+ed_status fx_psi_finish(const ed_basis* b, long long* P, bool have_records, long long* part,
                         cudaStream_t s);
 
 // Reorthogonalisation of the Lanczos residual (ed_reorth.cu; ed_opts.reorth 1 = full,
 // 2 = partial): the run keeps every Lanczos vector on the device.
 ed_status ro_create(int mode, ed_dtype dtype, int64_t n, int max_steps, int64_t dim, Reorth** out);
 void ro_free(Reorth* r);
+// The slots and scales of the vectors (mode 3: the update pass writes them).
+LzStore ro_slots(const Reorth* r);
 ed_status ro_prepare(const Reorth* r);
 // Start of a run: clear the estimates, store f_1 (buffer 0).
 ed_status ro_reset(const Reorth* r, const LzScalars* S, const void* buf0, cudaStream_t s);

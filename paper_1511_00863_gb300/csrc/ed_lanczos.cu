@@ -106,11 +106,15 @@ __global__ void init_scalars_kernel(LzScalars* S, const double* __restrict__ par
 // ------------------------------------------------------------------ update
 // Whole CTA: b_{j+1} and f_{j+1}'s scale from the nb partial sums of q . q.
 __device__ __forceinline__ void lz_finish_step(LzScalars* S, int cur, const double* pb, int nb,
-                                               double* red) {
+                                               double* red, double* vscale) {
   const double b2 = block_sum_array(pb, nb, red);
   if (threadIdx.x != 0) return;
   const double beta = sqrt(b2);
-  if (finish_step(S, S->j + 1, beta)) S->scale[1 - cur] = 1.0 / beta;
+  const int j = S->j + 1;
+  if (finish_step(S, j, beta)) {
+    S->scale[1 - cur] = 1.0 / beta;
+    if (vscale) vscale[j] = 1.0 / beta;
+  }
 }
 
 // finish: the last CTA ends the step (lz_finish_step); otherwise lz_finish_kernel does, after
@@ -118,7 +122,7 @@ __device__ __forceinline__ void lz_finish_step(LzScalars* S, int cur, const doub
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
 lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restrict__ bprev,
-                 int64_t n, double* __restrict__ pb, int finish) {
+                 int64_t n, double* __restrict__ pb, int finish, LzStore store) {
   __shared__ double red[33];
   if (S->status != 0) return;
   const T coef = (T)(S->alpha[S->j + 1] * S->scale[cur]);
@@ -128,6 +132,7 @@ lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restric
   typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type Vec;
   const Vec* c4 = reinterpret_cast<const Vec*>(bcur);
   Vec* p4 = reinterpret_cast<Vec*>(bprev);
+  Vec* const keep = store.slots ? (Vec*)store.slots[S->j + 1] : nullptr;
   const int64_t nv = n / VE;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nv;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -142,16 +147,17 @@ lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restric
       acc.add(q, q);
     }
     p4[i] = w;
+    if (keep) __stcs(keep + i, w);
   }
   const double v = block_sum(acc.get(), red);
   if (threadIdx.x == 0) pb[blockIdx.x] = v;
-  if (finish && last_cta(&S->tick_upd)) lz_finish_step(S, cur, pb, gridDim.x, red);
+  if (finish && last_cta(&S->tick_upd)) lz_finish_step(S, cur, pb, gridDim.x, red, store.vscale);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
 lz_finish_kernel(LzScalars* S, int cur, const double* __restrict__ pb, int nb) {
   __shared__ double red[33];
-  if (S->status == 0) lz_finish_step(S, cur, pb, nb, red);
+  if (S->status == 0) lz_finish_step(S, cur, pb, nb, red, nullptr);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
@@ -259,12 +265,19 @@ struct ed_lanczos {
   int64_t npa = 0, npb = 0;
   int hv_grid = 0;
   bool stopped = false;
-  double graph_t[2] = {0.0, 0.0}, graph_U[2] = {0.0, 0.0};  // parameters of the captured graphs
+  double graph_t[4] = {}, graph_U[4] = {};  // parameters of the captured graphs
   bool fx = false;     // ED_F64: int64 fixed-point buffers (ed_fixed.cu)
   FxRun fxr{};
   Hv2Plan* plan = nullptr;  // fused H.v on the padded layout (ed_hv2.cu), if it fits
   Reorth* ro = nullptr;     // stored Lanczos vectors when opts.reorth != 0 (ed_reorth.cu)
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};  // without / with the convergence test
+  LzStore store{nullptr, nullptr};  // where the update pass keeps the vectors
+  cudaGraphExec_t graph[4] = {};  // without / with the convergence test, + 2: vectors kept in `slots`
+  // ground-state vectors only: slot table and scales of the kept vectors, y of T_m with the
+  // inverse iteration's work, ranks by column
+  void** slots = nullptr;
+  double* vscale = nullptr;
+  double* ywork = nullptr;
+  int32_t* rank = nullptr;
   // solves only (lz_iterate): the checks' stream, fork and join events of the capture, one event
   // per batch in flight and the host's copies of the run's scalars (pinned)
   cudaStream_t check_stream = nullptr;
@@ -284,7 +297,7 @@ static ed_status lz_launch_step(ed_lanczos* st, const ed_params* p, cudaStream_t
   if (st->fx) {
     long long* const B[2] = {(long long*)st->B[0], (long long*)st->B[1]};
     ed_status r = fx_step(b, st->fxr, p->t, p->U, B, c, st->ld, st->S, (long long*)st->pa,
-                          (long long*)st->pb, s, ev0, ev1, st->plan, st->ro);
+                          (long long*)st->pb, s, ev0, ev1, st->plan, st->store, st->ro);
     if (r == ED_OK) st->cur = 1 - c;
     return r;
   }
@@ -312,17 +325,17 @@ static ed_status lz_launch_step(ed_lanczos* st, const ed_params* p, cudaStream_t
   const bool between = st->ro && ro_between(st->ro);  // passes between the update and the finish
   if (dt == ED_F64_NATIVE || dt == ED_C64)
     lz_update_kernel<double><<<ug, kRedThreads, 0, s>>>(
-        st->S, c, (const double*)st->B[c], (double*)st->B[1 - c], ns, st->pb, !between);
+        st->S, c, (const double*)st->B[c], (double*)st->B[1 - c], ns, st->pb, !between, st->store);
   else
     lz_update_kernel<float><<<ug, kRedThreads, 0, s>>>(
-        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pb, !between);
+        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pb, !between, st->store);
   ED_TRY_CUDA(cudaGetLastError());
   if (between) {
     if ((r = ro_apply(st->ro, st->S, st->B[1 - c], st->pb, ug, s)) != ED_OK) return r;
     lz_finish_kernel<<<1, kRedThreads, 0, s>>>(st->S, c, st->pb, ug);
     ED_TRY_CUDA(cudaGetLastError());
   }
-  if (st->ro && (r = ro_store(st->ro, st->S, 1 - c, st->B[1 - c], s)) != ED_OK) return r;
+  if (between && (r = ro_store(st->ro, st->S, 1 - c, st->B[1 - c], s)) != ED_OK) return r;
   st->cur = 1 - c;
   return ED_OK;
 }
@@ -435,10 +448,12 @@ extern "C" void ed_lanczos_destroy(ed_lanczos* st) {
   cudaGetDevice(&prev);
   if (prev != st->device) cudaSetDevice(st->device);
   if (st->stream) cudaStreamSynchronize(st->stream);
-  for (int i = 0; i < 2; ++i) {
-    if (st->graph[i]) cudaGraphExecDestroy(st->graph[i]);
-    if (st->ev_batch[i]) cudaEventDestroy(st->ev_batch[i]);
-  }
+  for (cudaGraphExec_t g : st->graph)
+    if (g) cudaGraphExecDestroy(g);
+  for (cudaEvent_t e : st->ev_batch)
+    if (e) cudaEventDestroy(e);
+  for (void* q : {(void*)st->slots, (void*)st->vscale, (void*)st->ywork, (void*)st->rank})
+    if (q) cudaFree(q);
   if (st->ev_fork) cudaEventDestroy(st->ev_fork);
   if (st->ev_join) cudaEventDestroy(st->ev_join);
   if (st->check_stream) cudaStreamDestroy(st->check_stream);
@@ -489,7 +504,7 @@ static ed_status lz_alloc(const ed_basis* b, const ed_opts* o, cudaStream_t s, e
   st->n = b->up.dim * st->ld;
   // partial sums: one double per CTA, or four int64 words per CTA on the fixed-point path
   st->npa = hv_max_grid(b) * (st->fx ? 4 : 1);
-  st->npb = (int64_t)sm_count() * 4 * (st->fx ? 6 : 1);
+  st->npb = (int64_t)sm_count() * 4 * (st->fx ? 6 : 1) + 8;
   auto fail = [&](ed_status e) {
     ed_lanczos_destroy(st);
     return e;
@@ -504,6 +519,7 @@ static ed_status lz_alloc(const ed_basis* b, const ed_opts* o, cudaStream_t s, e
   if (o->reorth != 0) {
     const ed_status rr = ro_create(o->reorth, o->dtype, st->n, o->max_steps, b->dim, &st->ro);
     if (rr != ED_OK) return fail(rr);
+    if (!ro_between(st->ro)) st->store = ro_slots(st->ro);  // mode 3
   }
   if (cudaMalloc((void**)&st->S, sizeof(LzScalars)) != cudaSuccess ||
       cudaMalloc((void**)&st->pa, st->npa * sizeof(double)) != cudaSuccess ||
@@ -746,86 +762,6 @@ extern "C" ed_status ed_lanczos_energy(ed_lanczos* st, double* E0, int32_t* step
   return ED_OK;
 }
 
-extern "C" ed_status ed_lanczos_ground_state(const ed_basis* b, const ed_params* p,
-                                             const ed_opts* o, const void* f1, void* stream,
-                                             double* psi, double* E0, int32_t* steps) {
-  clear_error();
-  ED_CHECK_ARG(b && p && o && psi && E0, "ed_lanczos_ground_state: NULL argument");
-  ED_CHECK_ARG(o->dtype == ED_F64, "ed_lanczos_ground_state: dtype must be ED_F64");
-  {
-    const ed_status rc = check_opts(o);
-    if (rc != ED_OK) return rc;
-  }
-  ED_CHECK_ARG(aligned16(psi), "ed_lanczos_ground_state: psi must be 16-byte aligned");
-  cudaStream_t s = (cudaStream_t)stream;
-  ed_lanczos* st = nullptr;
-  long long* P = nullptr;
-  double* yd = nullptr;
-  struct ReleaseOnReturn {  // frees the state and scratch on every return path
-    ed_lanczos*& st;
-    long long*& P;
-    double*& yd;
-    ~ReleaseOnReturn() {
-      if (st) ed_lanczos_destroy(st);
-      if (P) cudaFree(P);
-      if (yd) cudaFree(yd);
-    }
-  } release{st, P, yd};
-  // ---- pass 1: Algorithm 1 to convergence, tested after every 8 steps
-  ed_status r = lz_init(b, o, f1, s, &st);
-  if (r != ED_OK) return r;
-  if ((r = fx_prepare(b)) != ED_OK || (r = lz_plan(st, p)) != ED_OK) return r;
-  ED_TRY_CUDA(cudaMemsetAsync(&st->S->chk, 0, sizeof(int), s));
-  LzScalars hs;
-  constexpr size_t kHead = offsetof(LzScalars, tick_chk);
-  hs.status = 0;
-  hs.conv_j = 0;
-  for (int done = 0; done < o->max_steps && hs.status == 0 && hs.conv_j == 0; done += 8) {
-    for (int i = 0; i < 8; ++i)
-      if ((r = lz_launch_step(st, p, s)) != ED_OK) return r;
-    if (o->tol > 0.0) lz_check_kernel<<<8, kRedThreads, 0, s>>>(st->S);
-    ED_TRY_CUDA(cudaGetLastError());
-    ED_TRY_CUDA(cudaMemcpyAsync(&hs, st->S, kHead, cudaMemcpyDeviceToHost, s));
-    ED_TRY_CUDA(cudaStreamSynchronize(s));
-  }
-  const int m = hs.conv_j ? hs.conv_j : hs.j;
-  const int status = hs.conv_j ? 2 : hs.status;
-  double lam = 0.0;
-  if (!(o->tol > 0.0)) lz_history_kernel<<<1, kRedThreads, 0, s>>>(st->S, 0);
-  ED_TRY_CUDA(cudaGetLastError());
-  ED_TRY_CUDA(cudaMemcpyAsync(&lam, &st->S->E0[m], sizeof(double), cudaMemcpyDeviceToHost, s));
-  ED_TRY_CUDA(cudaStreamSynchronize(s));
-  // ---- Ritz vector of T_m on the device
-  if (cudaMalloc((void**)&yd, (size_t)(3 * (m + 2)) * sizeof(double)) != cudaSuccess)
-    return ED_ERR_OOM;
-  lz_ritz_kernel<<<1, 32, 0, s>>>(st->S, m, lam, yd, yd + (m + 2));
-  ED_TRY_CUDA(cudaGetLastError());
-  // ---- pass 2: the same steps again from the same start, accumulating y_j f_j
-  ed_lanczos* st2 = nullptr;
-  if ((r = lz_init(b, o, f1, s, &st2)) != ED_OK) return r;
-  ed_lanczos_destroy(st);
-  st = st2;
-  if (cudaMalloc((void**)&P, (size_t)b->dim * sizeof(long long)) != cudaSuccess)
-    return ED_ERR_OOM;
-  ED_TRY_CUDA(cudaMemsetAsync(P, 0, (size_t)b->dim * sizeof(long long), s));
-  if ((r = lz_plan(st, p)) != ED_OK) return r;
-  for (int j = 1; j <= m; ++j) {
-    if ((r = fx_psi_accum(b, st->S, st->cur, yd, j, (const long long*)st->B[st->cur], st->ld,
-                          hv2_colpos(st->plan), P, s)) != ED_OK)
-      return r;
-    if (j < m && (r = lz_launch_step(st, p, s)) != ED_OK) return r;
-  }
-  if ((r = fx_psi_finish(b, P, (long long*)st->pb, (double*)psi, s)) != ED_OK) return r;
-  ED_TRY_CUDA(cudaStreamSynchronize(s));
-  *E0 = lam;
-  if (steps) *steps = m;
-  if (status == 3 && o->tol > 0.0) {
-    set_error("ed_lanczos_ground_state: not converged after %d steps", m);
-    return ED_ERR_NOT_CONVERGED;
-  }
-  return ED_OK;
-}
-
 // ------------------------------------------------------------------ solve
 // ed_lanczos_solve keeps, per basis, one allocated state per (dtype, schedule) and its
 // instantiated two-step graph, so repeated solves skip allocation and capture; a solve that
@@ -856,13 +792,18 @@ void lz_cache_free(const ed_basis* b) {
 // with the convergence test max(2, K) steps, K = check_stride. The check of K steps is a
 // branch beside the steps that follow: one opens the graph (the last K steps of the replay
 // before, whose check would otherwise end it alone), the others follow their steps.
+static int lz_graph_index(const ed_lanczos* st, bool check) {
+  return (check ? 1 : 0) + (st->slots && st->store.slots == st->slots ? 2 : 0);
+}
+
 static ed_status lz_graph(ed_lanczos* st, const ed_params* p, bool check, int* steps) {
   cudaStream_t s = st->stream;
   const int K = check_stride(st->n);
   const int n = check ? std::max(2, K) : 2;
   *steps = n;
-  cudaGraphExec_t& exec = st->graph[check];
-  if (exec && st->graph_t[check] == p->t && st->graph_U[check] == p->U) return ED_OK;
+  const int gi = lz_graph_index(st, check);
+  cudaGraphExec_t& exec = st->graph[gi];
+  if (exec && st->graph_t[gi] == p->t && st->graph_U[gi] == p->U) return ED_OK;
   if (exec) cudaGraphExecDestroy(exec);
   exec = nullptr;
   if (!st->host) {
@@ -905,15 +846,17 @@ static ed_status lz_graph(ed_lanczos* st, const ed_params* p, bool check, int* s
     set_error("ed_lanczos_solve: graph of the steps: %s", cudaGetErrorString(e));
     return ED_ERR_CUDA;
   }
-  st->graph_t[check] = p->t;
-  st->graph_U[check] = p->U;
+  st->graph_t[gi] = p->t;
+  st->graph_U[gi] = p->U;
   return ED_OK;
 }
 
 // Run a started state until it stops, and copy its scalars to st->host: m steps, status as in
 // LzScalars. all_E0: E0 of every step, else of the last one (runs without convergence test).
+// before(n): called before the steps up to n are enqueued.
+template <typename Before>
 static ed_status lz_iterate(ed_lanczos* st, const ed_params* p, const ed_opts* o, bool all_E0,
-                            int* m, int* status) {
+                            int* m, int* status, Before before) {
   cudaStream_t s = st->stream;
   const bool check = o->tol > 0.0;
   int n = 0;
@@ -925,9 +868,11 @@ static ed_status lz_iterate(ed_lanczos* st, const ed_params* p, const ed_opts* o
   int4* head = reinterpret_cast<int4*>(st->host + 1);
   const int per_batch = std::max(1, 8 / n);
   int launched = 0;
+  const int gi = lz_graph_index(st, check);
   for (int batch = 0;; ++batch) {
+    if ((r = before(std::min(launched + per_batch * n, o->max_steps))) != ED_OK) return r;
     for (int i = 0; i < per_batch && launched < o->max_steps; ++i, launched += n)
-      ED_TRY_CUDA(cudaGraphLaunch(st->graph[check], s));
+      ED_TRY_CUDA(cudaGraphLaunch(st->graph[gi], s));
     ED_TRY_CUDA(cudaMemcpyAsync(&head[batch & 1], st->S, sizeof(int4), cudaMemcpyDeviceToHost, s));
     ED_TRY_CUDA(cudaEventRecord(st->ev_batch[batch & 1], s));
     if (launched >= o->max_steps) break;
@@ -958,7 +903,8 @@ static ed_status solve_on(ed_lanczos* st, const ed_basis* b, const ed_params* p,
                                    : hv_prepare(b, o->dtype))) != ED_OK)
     return r;
   int j = 0, status = 0;
-  if ((r = lz_iterate(st, p, o, E0_hist != nullptr, &j, &status)) != ED_OK) return r;
+  if ((r = lz_iterate(st, p, o, E0_hist != nullptr, &j, &status, [](int) { return ED_OK; })) != ED_OK)
+    return r;
   const LzScalars& h = *st->host;
   *E0 = j >= 1 ? h.E0[j] : NAN;
   if (steps) *steps = j;
@@ -1037,6 +983,193 @@ extern "C" ed_status ed_lanczos_solve(const ed_basis* b, const ed_params* p, con
   if (r != ED_OK) return r;
   return with_state(b, o, (cudaStream_t)stream, [&](ed_lanczos* st) {
     return solve_on(st, b, p, o, f1, E0, steps, alpha, beta, E0_hist);
+  });
+}
+
+// ------------------------------------------------------------------ ground-state vector
+namespace ed {
+// Memory of the vectors a ground-state call keeps: a pool per device, so that the next call
+// does not map the same gigabytes again (0.75 ms per GB). It holds at most kPsiKeep bytes while
+// idle and gives them back when the last basis is destroyed.
+constexpr uint64_t kPsiKeep = 16ull << 30;
+static std::mutex g_psi_mu;
+static cudaMemPool_t g_psi_pool[64] = {};
+static int64_t g_psi_bases = 0;
+
+static cudaMemPool_t psi_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> lk(g_psi_mu);
+  if (g_psi_pool[dev]) return g_psi_pool[dev];
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  uint64_t keep = kPsiKeep;
+  cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  return g_psi_pool[dev] = pool;
+}
+
+void psi_pool_basis(int delta) {
+  std::lock_guard<std::mutex> lk(g_psi_mu);
+  g_psi_bases += delta;
+  if (g_psi_bases > 0) return;
+  for (cudaMemPool_t p : g_psi_pool)
+    if (p) cudaMemPoolTrimTo(p, 0);
+}
+}  // namespace ed
+
+namespace {
+
+// The Lanczos vectors of a ground-state call: blocks of up to 512 MB from the pool, taken as
+// the run goes on (a run is far shorter than its step limit), at most half the free device
+// memory and 96 GB in all. Returned to the pool on destruction, after the stream's work.
+struct KeptVectors {
+  ed_lanczos* st;
+  size_t vbytes;
+  int per_block, ready = 0;  // slots with memory
+  double left;               // bytes still allowed
+  bool complete = true;      // every slot asked for has memory
+  cudaMemPool_t pool;
+  std::vector<void*> blocks;
+
+  explicit KeptVectors(ed_lanczos* state) : st(state), pool(ed::psi_pool()) {
+    vbytes = (size_t)st->n * st->esize;
+    per_block = (int)std::min<size_t>(std::max<size_t>((512ull << 20) / vbytes, 1), 64);
+    size_t free_b = 0, total_b = 0;
+    uint64_t reserved = 0, used = 0;
+    if (!pool || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+      cudaGetLastError();
+      complete = false;
+    }
+    left = std::min(0.5 * ((double)free_b + (double)(reserved - used)), 96e9);
+  }
+  ~KeptVectors() {
+    for (void* q : blocks) cudaFreeAsync(q, st->stream);
+  }
+  // Slots 0 .. n - 1; what does not fit leaves the run without kept vectors (complete false).
+  ed_status grow(int n) {
+    while (complete && ready < n) {
+      const size_t bytes = (size_t)per_block * vbytes;
+      void* q = nullptr;
+      if ((double)bytes > left || cudaMallocFromPoolAsync(&q, bytes, pool, st->stream) != cudaSuccess) {
+        cudaGetLastError();
+        complete = false;
+        break;
+      }
+      left -= (double)bytes;
+      blocks.push_back(q);
+      std::vector<void*> slot(std::min(per_block, ED_MAX_STEPS + 2 - ready));
+      for (size_t k = 0; k < slot.size(); ++k) slot[k] = (char*)q + k * vbytes;
+      ED_TRY_CUDA(cudaMemcpyAsync(st->slots + ready, slot.data(), slot.size() * sizeof(void*),
+                                  cudaMemcpyHostToDevice, st->stream));
+      ready += (int)slot.size();
+    }
+    return ED_OK;
+  }
+};
+
+}  // namespace
+
+// psi on a started state: Algorithm 1 with its vectors kept where memory allows (then one pass
+// over them sums psi; the run itself is most of the time), else a second run of the same steps
+// that adds y_j f_j step by step. Both sums are the same integers.
+static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p, const ed_opts* o,
+                           const void* f1, long long* P, double* E0, int32_t* steps) {
+  cudaStream_t s = st->stream;
+  if (!st->ywork) {
+    if (cudaMalloc((void**)&st->slots, (ED_MAX_STEPS + 2) * sizeof(void*)) != cudaSuccess ||
+        cudaMalloc((void**)&st->vscale, (ED_MAX_STEPS + 2) * sizeof(double)) != cudaSuccess ||
+        cudaMalloc((void**)&st->rank, (size_t)st->ld * sizeof(int32_t)) != cudaSuccess ||
+        cudaMalloc((void**)&st->ywork, 3 * (ED_MAX_STEPS + 4) * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      for (void* q : {(void*)st->slots, (void*)st->vscale, (void*)st->rank})
+        if (q) cudaFree(q);
+      st->slots = nullptr, st->vscale = nullptr, st->rank = nullptr;
+      set_error("ed_lanczos_ground_state: out of device memory");
+      return ED_ERR_OOM;
+    }
+  }
+  ed_status r = lz_reset(st, o, f1);
+  if (r != ED_OK) return r;
+  if ((r = fx_prepare(b)) != ED_OK) return r;
+  int m = 0, status = 0;
+  double* y = st->ywork;
+  bool summed = false;
+  {
+    struct Unset {  // later solves on the state keep no vectors
+      ed_lanczos* st;
+      ~Unset() { st->store = LzStore{nullptr, nullptr}; }
+    } unset{st};
+    KeptVectors kept(st);
+    const bool own = !st->ro;  // a reorthogonalising run keeps its vectors by itself
+    if (own) {
+      ED_TRY_CUDA(cudaMemsetAsync(st->slots, 0, (ED_MAX_STEPS + 2) * sizeof(void*), s));
+      if ((r = kept.grow(1)) != ED_OK) return r;
+      if (kept.complete) {
+        ED_TRY_CUDA(cudaMemcpyAsync(kept.blocks[0], st->B[0], kept.vbytes, cudaMemcpyDeviceToDevice, s));
+        ED_TRY_CUDA(cudaMemcpyAsync(st->vscale, &st->S->scale[0], sizeof(double), cudaMemcpyDeviceToDevice, s));
+        st->store = LzStore{st->slots, st->vscale};
+      }
+    }
+    r = lz_iterate(st, p, o, false, &m, &status,
+                   [&](int n) { return own ? kept.grow(n + 1) : ED_OK; });
+    if (r != ED_OK) return r;
+    if (m < 1) {
+      set_error("ed_lanczos_ground_state: the run took no step");
+      return ED_ERR_ARG;
+    }
+    lz_ritz_kernel<<<1, 32, 0, s>>>(st->S, m, st->host->E0[m], y, y + (m + 2));
+    ED_TRY_CUDA(cudaGetLastError());
+    summed = !own || kept.complete;
+    if (summed &&
+        (r = fx_psi_sum(b, y, m, own ? st->store : ro_slots(st->ro), st->ld, hv2_colpos(st->plan),
+                        st->rank, P, (long long*)st->pb, s)) != ED_OK)
+      return r;
+  }
+  const double lam = st->host->E0[m];
+  if (!summed) {
+    if ((r = lz_reset(st, o, f1)) != ED_OK) return r;
+    ED_TRY_CUDA(cudaMemsetAsync(P, 0, (size_t)b->dim * sizeof(long long), s));
+    if ((r = lz_plan(st, p)) != ED_OK) return r;
+    for (int j = 1; j <= m; ++j) {
+      if ((r = fx_psi_accum(b, st->S, st->cur, y, j, (const long long*)st->B[st->cur], st->ld,
+                            hv2_colpos(st->plan), P, s)) != ED_OK)
+        return r;
+      if (j < m && (r = lz_launch_step(st, p, s)) != ED_OK) return r;
+    }
+  }
+  if ((r = fx_psi_finish(b, P, summed, (long long*)st->pb, s)) != ED_OK) return r;
+  ED_TRY_CUDA(cudaStreamSynchronize(s));
+  *E0 = lam;
+  if (steps) *steps = m;
+  if (status == 3 && o->tol > 0.0) {
+    set_error("ed_lanczos_ground_state: not converged after %d steps", m);
+    return ED_ERR_NOT_CONVERGED;
+  }
+  return ED_OK;
+}
+
+extern "C" ed_status ed_lanczos_ground_state(const ed_basis* b, const ed_params* p,
+                                             const ed_opts* o, const void* f1, void* stream,
+                                             double* psi, double* E0, int32_t* steps) {
+  clear_error();
+  ED_CHECK_ARG(b && p && o && psi && E0, "ed_lanczos_ground_state: NULL argument");
+  ED_CHECK_ARG(o->dtype == ED_F64, "ed_lanczos_ground_state: dtype must be ED_F64");
+  {
+    const ed_status rc = check_opts(o);
+    if (rc != ED_OK) return rc;
+  }
+  ED_CHECK_ARG(aligned16(psi), "ed_lanczos_ground_state: psi must be 16-byte aligned");
+  return with_state(b, o, (cudaStream_t)stream, [&](ed_lanczos* st) {
+    return ground_on(st, b, p, o, f1, (long long*)psi, E0, steps);
   });
 }
 

@@ -26,6 +26,7 @@
 // passes, when the step does not reorthogonalise.
 #include <cmath>
 #include <type_traits>
+#include <vector>
 
 #include "ed_fixed.cuh"
 #include "ed_internal.cuh"
@@ -51,6 +52,7 @@ struct Reorth {
   int G = 0;           // CTAs of the dot-product kernel
   void* V = nullptr;   // [slots][n]
   double* vscale = nullptr;  // [slots]
+  void** slot = nullptr;     // [slots] the vectors of V
   double* coef = nullptr;    // [slots]
   void* part = nullptr;      // [slots][G] doubles, or [slots][G][3] words (fixed point)
   double* omega = nullptr;   // [3][slots + 2]
@@ -388,6 +390,7 @@ void ro_free(Reorth* r) {
   if (!r) return;
   if (r->V) cudaFree(r->V);
   if (r->vscale) cudaFree(r->vscale);
+  if (r->slot) cudaFree(r->slot);
   if (r->coef) cudaFree(r->coef);
   if (r->part) cudaFree(r->part);
   if (r->omega) cudaFree(r->omega);
@@ -427,9 +430,22 @@ ed_status ro_create(int mode, ed_dtype dtype, int64_t n, int max_steps, int64_t 
     set_error("reorthogonalisation: out of device memory");
     return ED_ERR_OOM;
   }
+  {
+    std::vector<void*> slot(r->slots);
+    for (int k = 0; k < r->slots; ++k) slot[k] = (char*)r->V + (size_t)k * n * ro_esize(r->kind);
+    if (cudaMalloc((void**)&r->slot, slot.size() * sizeof(void*)) != cudaSuccess ||
+        cudaMemcpy(r->slot, slot.data(), slot.size() * sizeof(void*), cudaMemcpyHostToDevice) != cudaSuccess) {
+      cudaGetLastError();
+      ro_free(r);
+      set_error("stored Lanczos vectors: out of device memory");
+      return ED_ERR_OOM;
+    }
+  }
   *out = r;
   return ED_OK;
 }
+
+LzStore ro_slots(const Reorth* r) { return LzStore{r->slot, r->vscale}; }
 
 template <typename T>
 static void ro_store_t(const Reorth* r, const LzScalars* S, int buf, const void* src, cudaStream_t s) {
