@@ -335,12 +335,15 @@ __device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long
 }
 
 // finish: the last CTA ends the step (fx_finish_step); otherwise fx_finish_kernel does, after
-// the reorthogonalisation.
-__global__ void __launch_bounds__(kFxThreads)
+// the reorthogonalisation. kKeep: Q goes to the step's slot of `store` too. The grid is 4 CTAs
+// per SM: with more registers than that leaves (it takes 70 unbounded) a third of it ran as a
+// second wave, 102 instead of 81 us on the 4x4 lattice.
+template <bool kKeep>
+__global__ void __launch_bounds__(kFxThreads, 4)
 fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long long* __restrict__ xp,
                  int64_t n, long long* __restrict__ pb, int finish, FxPlanArgs plan, LzStore store) {
   if (S->status != 0) return;
-  longlong2* const keep = store.slots ? (longlong2*)store.slots[S->j + 1] : nullptr;
+  longlong2* const keep = kKeep ? (longlong2*)store.slots[S->j + 1] : nullptr;
   const long long d = S->fx_d;
   const int k2 = S->fx_k2;
   A192 q2;
@@ -367,15 +370,15 @@ fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long l
     }
     const longlong2 r0 = make_longlong2(upd(w0.x, c0.x), upd(w0.y, c0.y));
     p2[i] = r0;
-    if (keep) __stcs(keep + i, r0);
+    if (kKeep && keep) __stcs(keep + i, r0);
     if (two) {
       const longlong2 r1 = make_longlong2(upd(w1.x, c1.x), upd(w1.y, c1.y));
       p2[i + stride] = r1;
-      if (keep) __stcs(keep + i + stride, r1);
+      if (kKeep && keep) __stcs(keep + i + stride, r1);
     }
   }
   fx_block_reduce(a192_get(q2), mx, pb + 4 * blockIdx.x);
-  if (finish && last_cta(&S->tick_upd)) fx_finish_step(S, cur, pb, gridDim.x, plan, store.vscale);
+  if (finish && last_cta(&S->tick_upd)) fx_finish_step(S, cur, pb, gridDim.x, plan, kKeep ? store.vscale : nullptr);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
@@ -697,7 +700,10 @@ ed_status fx_step(const ed_basis* b, const FxRun& fx, double t, double U, long l
   const int ug = fx_red_grid(n);
   const FxPlanArgs next = {t, U, fx.hops, fx.nmax, fx.vb};
   const bool between = ro && ro_between(ro);  // passes between the update and the finish
-  fx_update_kernel<<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next, store);
+  if (store.slots)
+    fx_update_kernel<true><<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next, store);
+  else
+    fx_update_kernel<false><<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next, store);
   if (between) {
     const ed_status r = ro_apply(ro, S, B[1 - cur], pb, ug, s);
     if (r != ED_OK) return r;

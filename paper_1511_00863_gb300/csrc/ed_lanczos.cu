@@ -118,8 +118,8 @@ __device__ __forceinline__ void lz_finish_step(LzScalars* S, int cur, const doub
 }
 
 // finish: the last CTA ends the step (lz_finish_step); otherwise lz_finish_kernel does, after
-// the reorthogonalisation.
-template <typename T>
+// the reorthogonalisation. kKeep: q goes to the step's slot of `store` too.
+template <typename T, bool kKeep>
 __global__ void __launch_bounds__(kRedThreads)
 lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restrict__ bprev,
                  int64_t n, double* __restrict__ pb, int finish, LzStore store) {
@@ -132,7 +132,7 @@ lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restric
   typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type Vec;
   const Vec* c4 = reinterpret_cast<const Vec*>(bcur);
   Vec* p4 = reinterpret_cast<Vec*>(bprev);
-  Vec* const keep = store.slots ? (Vec*)store.slots[S->j + 1] : nullptr;
+  Vec* const keep = kKeep ? (Vec*)store.slots[S->j + 1] : nullptr;
   const int64_t nv = n / VE;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nv;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -147,11 +147,11 @@ lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restric
       acc.add(q, q);
     }
     p4[i] = w;
-    if (keep) __stcs(keep + i, w);
+    if (kKeep && keep) __stcs(keep + i, w);
   }
   const double v = block_sum(acc.get(), red);
   if (threadIdx.x == 0) pb[blockIdx.x] = v;
-  if (finish && last_cta(&S->tick_upd)) lz_finish_step(S, cur, pb, gridDim.x, red, store.vscale);
+  if (finish && last_cta(&S->tick_upd)) lz_finish_step(S, cur, pb, gridDim.x, red, kKeep ? store.vscale : nullptr);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
@@ -323,11 +323,15 @@ static ed_status lz_launch_step(ed_lanczos* st, const ed_params* p, cudaStream_t
   const int64_t ns = is_complex(dt) ? 2 * st->n : st->n;
   const int ug = red_grid(ns);
   const bool between = st->ro && ro_between(st->ro);  // passes between the update and the finish
-  if (dt == ED_F64_NATIVE || dt == ED_C64)
-    lz_update_kernel<double><<<ug, kRedThreads, 0, s>>>(
+  const bool keep = st->store.slots != nullptr;
+  if (dt == ED_F64_NATIVE || dt == ED_C64)  // (only FP32 and fixed-point runs keep their vectors here)
+    lz_update_kernel<double, false><<<ug, kRedThreads, 0, s>>>(
         st->S, c, (const double*)st->B[c], (double*)st->B[1 - c], ns, st->pb, !between, st->store);
+  else if (keep)
+    lz_update_kernel<float, true><<<ug, kRedThreads, 0, s>>>(
+        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pb, !between, st->store);
   else
-    lz_update_kernel<float><<<ug, kRedThreads, 0, s>>>(
+    lz_update_kernel<float, false><<<ug, kRedThreads, 0, s>>>(
         st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pb, !between, st->store);
   ED_TRY_CUDA(cudaGetLastError());
   if (between) {
