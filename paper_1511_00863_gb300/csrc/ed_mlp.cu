@@ -61,12 +61,6 @@ __device__ __forceinline__ float tanh_sfu(float x) {
   return y;
 }
 
-// Rounded weights into shared memory (sw has P floats).
-__device__ __forceinline__ void load_weights(const float* __restrict__ params, int P, float* sw) {
-  for (int i = threadIdx.x; i < P; i += blockDim.x) sw[i] = bf16r(params[i]);
-  __syncthreads();
-}
-
 // ------------------------------------------------------------------ inference
 // 5th-generation tensor cores: a CTA of 4 warps evaluates tiles of 128 basis states, one
 // state per thread (TMEM lane). The features of the tile (bits as 0/1, bf16(U/8), zero
@@ -254,84 +248,174 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
 }
 
 // ------------------------------------------------------------------ loss and gradient
-// Each CTA walks tiles of kTile samples; thread t owns fixed gradient entries and sums them
-// over its CTA's tiles in order; partial[cta][P] and lpart[cta] are then reduced in order.
-__global__ void __launch_bounds__(kMThreads)
+// A CTA takes tiles of kTile samples. Every product of a tile (X W1, bf16(h1) W2, G2 W2^T and the
+// two weight gradients) is a 64-wide matrix product out of shared memory in FP32; each of the 256
+// threads holds a 4 x 4 block of the result in registers, so that two or four 16-byte loads feed
+// 16 or 64 multiply-adds (with one output per thread and two 4-byte loads per multiply-add the
+// kernel took 176 us for 16,384 samples of 29 features; 300 M multiply-adds are 8 us at the FP32
+// rate). Rows are kLdT floats apart: eight consecutive rows start in eight different bank groups.
+// A thread keeps its blocks of the weight gradients over all tiles of its CTA; partial[cta][P] and
+// lpart[cta] are then reduced in CTA order.
+constexpr int kLdT = 68;  // row stride of the tiles: 64 features (65 of X) and the bank offset
+
+struct GradLayout {
+  int W1, W2, small, X, H1, H1B, H2, DO, total;  // in floats
+};
+__host__ __device__ inline GradLayout grad_layout(int nin) {
+  GradLayout g;
+  const int n4 = (nin + 3) / 4 * 4;
+  g.W1 = 0;                       // [n4][64]
+  g.W2 = g.W1 + n4 * kH;          // [64][kLdT]
+  g.small = g.W2 + kH * kLdT;     // b1 | b2 | W3 (o, c) | b3
+  g.X = g.small + 4 * kH + 4;     // [kTile][kLdT]
+  g.H1 = g.X + kTile * kLdT;      // h1, then G1
+  g.H1B = g.H1 + kTile * kLdT;    // bf16(h1)
+  g.H2 = g.H1B + kTile * kLdT;    // h2, then G2
+  g.DO = g.H2 + kTile * kLdT;     // [kTile][2]
+  g.total = g.DO + 2 * kTile;
+  return g;
+}
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float get4(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+
+// acc[q][r] += sum_{k < K} A[(ty + 16 q)][k] B[k][4 tx + r] (K a multiple of 4; rows of A kLdT
+// apart, rows of B ldb).
+__device__ __forceinline__ void mm_forward(float (&acc)[4][4], const float* A, const float* B, int ldb, int K,
+                                           int ty, int tx) {
+  for (int k = 0; k < K; k += 4) {
+    float4 a[4], b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = ld4(A + (ty + 16 * q) * kLdT + k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) b[i] = ld4(B + (k + i) * ldb + 4 * tx);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[q][r] = fmaf(get4(a[q], i), get4(b[i], r), acc[q][r]);
+  }
+}
+
+// acc[q][r] += sum_s A[s][4 ty + q] B[s][4 tx + r] over the tile's samples in order.
+__device__ __forceinline__ void mm_outer(float (&acc)[4][4], const float* A, const float* B, int ty, int tx) {
+#pragma unroll 4
+  for (int t = 0; t < kTile; ++t) {
+    const float4 a = ld4(A + t * kLdT + 4 * ty), b = ld4(B + t * kLdT + 4 * tx);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc[q][r] = fmaf(get4(a, q), get4(b, r), acc[q][r]);
+  }
+}
+
+__global__ void __launch_bounds__(kMThreads, 2)
 mlp_grad_kernel(const float* __restrict__ params, int L, float U, const uint32_t* __restrict__ upb,
                 const uint32_t* __restrict__ dnb, int64_t dim_dn, const int64_t* __restrict__ idx,
                 const double* __restrict__ target, int64_t n, double wscale,
                 float* __restrict__ partial, double* __restrict__ lpart) {
-  extern __shared__ float smem[];
+  extern __shared__ __align__(16) float gsm[];
+  __shared__ uint32_t ubits[kTile], dbits[kTile];
+  __shared__ double lred[kTile];
   const MlpDims d = mlp_dims(L);
-  float* sw = smem;                     // P
-  float* X = sw + ((d.P + 3) / 4) * 4;  // [kTile][nin]
-  float* H1 = X + kTile * kMaxIn;       // [kTile][kH]
-  float* H2 = H1 + kTile * kH;          // [kTile][kH]
-  float* G2 = H2 + kTile * kH;          // [kTile][kH]
-  float* G1 = G2 + kTile * kH;          // [kTile][kH]
-  float* DO = G1 + kTile * kH;          // [kTile][2]
-  float* H1B = DO + 2 * kTile;          // [kTile][kH] bf16-rounded h1 (input of layer 2)
-  __shared__ double lred[kMThreads];
-  load_weights(params, d.P, sw);
+  const GradLayout g = grad_layout(d.nin);
+  const int n4 = (d.nin + 3) / 4 * 4;
+  float* W1 = gsm + g.W1;
+  float* W2 = gsm + g.W2;
+  float* sb1 = gsm + g.small;
+  float* sb2 = sb1 + kH;
+  float* W3 = sb2 + kH;
+  float* sb3 = W3 + 2 * kH;
+  float* X = gsm + g.X;
+  float* H1 = gsm + g.H1;
+  float* H1B = gsm + g.H1B;
+  float* H2 = gsm + g.H2;
+  float* DO = gsm + g.DO;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  // ---- rounded weights
+  for (int i = tid; i < n4 * kH; i += kMThreads) W1[i] = i < d.nin * kH ? bf16r(params[d.oW1 + i]) : 0.f;
+  for (int i = tid; i < kH * kH; i += kMThreads) W2[(i / kH) * kLdT + i % kH] = bf16r(params[d.oW2 + i]);
+  for (int i = tid; i < kH; i += kMThreads) {
+    sb1[i] = bf16r(params[d.ob1 + i]);
+    sb2[i] = bf16r(params[d.ob2 + i]);
+  }
+  for (int i = tid; i < 2 * kH; i += kMThreads) W3[i] = bf16r(params[d.oW3 + i]);
+  if (tid < 2) sb3[tid] = bf16r(params[d.ob3 + tid]);
   const float u8b = bf16r(U * 0.125f);
-  // owned gradient entries: W2 (kH*kH), W1 (nin*kH), W3 (2*kH), b1, b2 (kH each), b3 (2)
-  constexpr int kOwnW2 = kH * kH / kMThreads;  // 16
-  float gW2[kOwnW2];
-  constexpr int kOwnW1 = (kMaxIn * kH + kMThreads - 1) / kMThreads;  // 17
-  float gW1[kOwnW1];
+  float gW2[4][4] = {}, gW1[4][4] = {};
+  float gW1last = 0.f;  // W1's row 64 (32 sites: the U feature), entry tid < 64
   float gX = 0.f;   // thread t: W3 entry t (t < 128), b1 (t < 192), b2 (t < 256)
   float gB3 = 0.f;  // threads 0 and 1: b3
-  const int nW1 = d.nin * kH;
-  const int nW1own = (nW1 + kMThreads - 1) / kMThreads;
-#pragma unroll
-  for (int q = 0; q < kOwnW2; ++q) gW2[q] = 0.f;
-#pragma unroll
-  for (int q = 0; q < kOwnW1; ++q) gW1[q] = 0.f;
   double lsum = 0.0;
   const int64_t ntiles = (n + kTile - 1) / kTile;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t s0 = tile * kTile;
-    // ---- forward: one thread per (sample, half of the hidden units) for layer 1 and 2
-    for (int i = threadIdx.x; i < kTile * d.nin; i += blockDim.x) {
-      const int sidx = i / d.nin, f = i - sidx * d.nin;
-      const int64_t k = s0 + sidx;
-      float v = 0.f;
-      if (k < n) {
-        const int64_t g = idx[k];
-        const int64_t u = g / dim_dn, dd = g - u * dim_dn;
-        if (f < L) v = (float)((upb[u] >> f) & 1u);
-        else if (f < 2 * L) v = (float)((dnb[dd] >> (f - L)) & 1u);
-        else v = u8b;
+    __syncthreads();
+    if (tid < kTile) {
+      uint32_t ub = 0, db = 0;
+      if (s0 + tid < n) {
+        const int64_t e = idx[s0 + tid];
+        const int64_t u = e / dim_dn;
+        ub = upb[u];
+        db = dnb[e - u * dim_dn];
       }
-      X[sidx * kMaxIn + f] = v;
+      ubits[tid] = ub;
+      dbits[tid] = db;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kTile * kH; i += blockDim.x) {
-      const int sidx = i / kH, o = i - sidx * kH;
-      float s = sw[d.ob1 + o];
-      for (int f = 0; f < d.nin; ++f) s = fmaf(X[sidx * kMaxIn + f], sw[d.oW1 + f * kH + o], s);
-      const float h = tanhf(s);
-      H1[sidx * kH + o] = h;
-      H1B[sidx * kH + o] = bf16r(h);
+    for (int i = tid; i < kTile * n4; i += kMThreads) {
+      const int t = i / n4, f = i - t * n4;
+      float v = 0.f;
+      if (s0 + t < n) {
+        if (f < L) v = (float)((ubits[t] >> f) & 1u);
+        else if (f < 2 * L) v = (float)((dbits[t] >> (f - L)) & 1u);
+        else if (f == 2 * L) v = u8b;
+      }
+      X[t * kLdT + f] = v;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kTile * kH; i += blockDim.x) {
-      const int sidx = i / kH, o = i - sidx * kH;
-      float s = sw[d.ob2 + o];
-      for (int f = 0; f < kH; ++f) s = fmaf(H1B[sidx * kH + f], sw[d.oW2 + f * kH + o], s);
-      H2[sidx * kH + o] = tanhf(s);
+    // ---- forward
+    {
+      float acc[4][4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[q][r] = sb1[4 * tx + r];
+      mm_forward(acc, X, W1, kH, n4, ty, tx);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float4 h, hb;
+        h = make_float4(tanhf(acc[q][0]), tanhf(acc[q][1]), tanhf(acc[q][2]), tanhf(acc[q][3]));
+        hb = make_float4(bf16r(h.x), bf16r(h.y), bf16r(h.z), bf16r(h.w));
+        *reinterpret_cast<float4*>(H1 + (ty + 16 * q) * kLdT + 4 * tx) = h;
+        *reinterpret_cast<float4*>(H1B + (ty + 16 * q) * kLdT + 4 * tx) = hb;
+      }
+    }
+    __syncthreads();
+    {
+      float acc[4][4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[q][r] = sb2[4 * tx + r];
+      mm_forward(acc, H1B, W2, kLdT, kH, ty, tx);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<float4*>(H2 + (ty + 16 * q) * kLdT + 4 * tx) =
+            make_float4(tanhf(acc[q][0]), tanhf(acc[q][1]), tanhf(acc[q][2]), tanhf(acc[q][3]));
     }
     __syncthreads();
     // ---- outputs, loss and d(loss)/d(a, z) per sample
-    if (threadIdx.x < kTile) {
-      const int sidx = threadIdx.x;
-      const int64_t k = s0 + sidx;
+    if (tid < kTile) {
+      const int64_t k = s0 + tid;
       float da = 0.f, dz = 0.f;
       if (k < n) {
-        float a = sw[d.ob3], z = sw[d.ob3 + 1];
+        float a = sb3[0], z = sb3[1];
+        const float* h = H2 + tid * kLdT;
         for (int o = 0; o < kH; ++o) {
-          a = fmaf(H2[sidx * kH + o], sw[d.oW3 + 2 * o], a);
-          z = fmaf(H2[sidx * kH + o], sw[d.oW3 + 2 * o + 1], z);
+          a = fmaf(h[o], W3[2 * o], a);
+          z = fmaf(h[o], W3[2 * o + 1], z);
         }
         const double psi = target[k];
         if (psi != 0.0) {
@@ -340,101 +424,123 @@ mlp_grad_kernel(const float* __restrict__ params, int L, float U, const uint32_t
           const double sg = psi >= 0.0 ? 1.0 : -1.0;
           const double diff = (double)a - l;
           const double mz = -sg * (double)z;
-          const double sp = mz > 0.0 ? mz + log1p(exp(-mz)) : log1p(exp(mz));
-          lsum += w * (diff * diff + sp);
+          const double E = exp(-fabs(mz));  // softplus and its slope from one exponential
+          lsum += w * (diff * diff + (mz > 0.0 ? mz : 0.0) + log1p(E));
           da = (float)(w * 2.0 * diff / (double)n);
-          dz = (float)(w * (-sg) / (1.0 + exp(sg * (double)z)) / (double)n);
+          dz = (float)(w * (-sg) * (mz >= 0.0 ? 1.0 : E) / (1.0 + E) / (double)n);
         }
       }
-      DO[2 * sidx] = da;
-      DO[2 * sidx + 1] = dz;
+      DO[2 * tid] = da;
+      DO[2 * tid + 1] = dz;
     }
     __syncthreads();
-    // ---- backward through layer 2 and 1
-    for (int i = threadIdx.x; i < kTile * kH; i += blockDim.x) {
-      const int sidx = i / kH, o = i - sidx * kH;
-      const float h = H2[sidx * kH + o];
-      const float g = fmaf(DO[2 * sidx], sw[d.oW3 + 2 * o], DO[2 * sidx + 1] * sw[d.oW3 + 2 * o + 1]);
-      G2[sidx * kH + o] = g * (1.f - h * h);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kTile * kH; i += blockDim.x) {
-      const int sidx = i / kH, o = i - sidx * kH;
-      float g = 0.f;
-      for (int f = 0; f < kH; ++f) g = fmaf(G2[sidx * kH + f], sw[d.oW2 + o * kH + f], g);
-      const float h = H1[sidx * kH + o];
-      G1[sidx * kH + o] = g * (1.f - h * h);
-    }
-    __syncthreads();
-    // ---- weight gradients owned by this thread (sum over the tile's samples in order)
-#pragma unroll
-    for (int q = 0; q < kOwnW2; ++q) {
-      const int e = threadIdx.x + q * kMThreads;  // W2 entry (i, o)
-      const int i = e / kH, o = e - i * kH;
+    // ---- output layer's gradient (reads h2), then G2 over h2
+    if (tid < 2 * kH) {  // W3 (o, c)
+      const int o = tid >> 1, c = tid & 1;
       float acc = 0.f;
-      for (int sidx = 0; sidx < kTile; ++sidx) acc = fmaf(H1B[sidx * kH + i], G2[sidx * kH + o], acc);
-      gW2[q] += acc;
-    }
-#pragma unroll
-    for (int q = 0; q < kOwnW1; ++q) {
-      const int e = threadIdx.x + q * kMThreads;
-      if (q < nW1own && e < nW1) {
-        const int f = e / kH, o = e - f * kH;
-        float acc = 0.f;
-        for (int sidx = 0; sidx < kTile; ++sidx) acc = fmaf(X[sidx * kMaxIn + f], G1[sidx * kH + o], acc);
-        gW1[q] += acc;
-      }
-    }
-    if (threadIdx.x < 2) {
-      float acc = 0.f;
-      for (int sidx = 0; sidx < kTile; ++sidx) acc += DO[2 * sidx + threadIdx.x];
-      gB3 += acc;
-    }
-    {
-      const int t = threadIdx.x;
-      float acc = 0.f;
-      if (t < 2 * kH) {  // W3 (o, c)
-        const int o = t >> 1, c = t & 1;
-        for (int sidx = 0; sidx < kTile; ++sidx) acc = fmaf(H2[sidx * kH + o], DO[2 * sidx + c], acc);
-      } else if (t < 3 * kH) {  // b1
-        for (int sidx = 0; sidx < kTile; ++sidx) acc += G1[sidx * kH + (t - 2 * kH)];
-      } else if (t < 4 * kH) {  // b2
-        for (int sidx = 0; sidx < kTile; ++sidx) acc += G2[sidx * kH + (t - 3 * kH)];
-      }
+      for (int t = 0; t < kTile; ++t) acc = fmaf(H2[t * kLdT + o], DO[2 * t + c], acc);
       gX += acc;
     }
+    if (tid < 2) {
+      float acc = 0.f;
+      for (int t = 0; t < kTile; ++t) acc += DO[2 * t + tid];
+      gB3 += acc;
+    }
     __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int t = ty + 16 * q;
+      const float da = DO[2 * t], dz = DO[2 * t + 1];
+      float4* p = reinterpret_cast<float4*>(H2 + t * kLdT + 4 * tx);
+      const float4 h = *p, wa = ld4(W3 + 8 * tx), wb = ld4(W3 + 8 * tx + 4);
+      *p = make_float4(fmaf(da, wa.x, dz * wa.y) * (1.f - h.x * h.x), fmaf(da, wa.z, dz * wa.w) * (1.f - h.y * h.y),
+                       fmaf(da, wb.x, dz * wb.y) * (1.f - h.z * h.z), fmaf(da, wb.z, dz * wb.w) * (1.f - h.w * h.w));
+    }
+    __syncthreads();
+    // ---- G1 = (G2 W2^T) (1 - h1^2), over h1: rows ty + 16 q, hidden units tx + 16 r
+    {
+      float acc[4][4] = {};
+      for (int o = 0; o < kH; o += 4) {
+        float4 a[4], b[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = ld4(H2 + (ty + 16 * q) * kLdT + o);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) b[r] = ld4(W2 + (tx + 16 * r) * kLdT + o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[q][r] = fmaf(get4(a[q], i), get4(b[r], i), acc[q][r]);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          float* p = H1 + (ty + 16 * q) * kLdT + tx + 16 * r;
+          const float h = *p;
+          *p = acc[q][r] * (1.f - h * h);
+        }
+    }
+    __syncthreads();
+    // ---- weight gradients
+    mm_outer(gW2, H1B, H2, ty, tx);
+    if (4 * ty < n4) mm_outer(gW1, X, H1, ty, tx);
+    if (d.nin > kH && tid < kH)
+      for (int t = 0; t < kTile; ++t) gW1last = fmaf(X[t * kLdT + kH], H1[t * kLdT + tid], gW1last);
+    if (tid >= 2 * kH) {  // b1, b2
+      const float* G = tid < 3 * kH ? H1 + (tid - 2 * kH) : H2 + (tid - 3 * kH);
+      float acc = 0.f;
+      for (int t = 0; t < kTile; ++t) acc += G[t * kLdT];
+      gX += acc;
+    }
   }
   float* out = partial + (size_t)blockIdx.x * d.P;
 #pragma unroll
-  for (int q = 0; q < kOwnW2; ++q) out[d.oW2 + threadIdx.x + q * kMThreads] = gW2[q];
+  for (int q = 0; q < 4; ++q)
 #pragma unroll
-  for (int q = 0; q < kOwnW1; ++q) {
-    const int e = threadIdx.x + q * kMThreads;
-    if (q < nW1own && e < nW1) out[d.oW1 + e] = gW1[q];
-  }
-  if (threadIdx.x < 2) out[d.ob3 + threadIdx.x] = gB3;
-  if (threadIdx.x < 2 * kH) out[d.oW3 + threadIdx.x] = gX;
-  else if (threadIdx.x < 3 * kH) out[d.ob1 + threadIdx.x - 2 * kH] = gX;
-  else if (threadIdx.x < 4 * kH) out[d.ob2 + threadIdx.x - 3 * kH] = gX;
-  lred[threadIdx.x] = lsum;
+    for (int r = 0; r < 4; ++r) out[d.oW2 + (4 * ty + q) * kH + 4 * tx + r] = gW2[q][r];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (4 * ty + q < d.nin)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) out[d.oW1 + (4 * ty + q) * kH + 4 * tx + r] = gW1[q][r];
+  if (d.nin > kH && tid < kH) out[d.oW1 + kH * kH + tid] = gW1last;
+  if (tid < 2) out[d.ob3 + tid] = gB3;
+  if (tid < 2 * kH) out[d.oW3 + tid] = gX;
+  else if (tid < 3 * kH) out[d.ob1 + tid - 2 * kH] = gX;
+  else out[d.ob2 + tid - 3 * kH] = gX;
+  if (tid < kTile) lred[tid] = lsum;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < kMThreads; ++i) s += lred[i];
-    lpart[blockIdx.x] = s / (double)n;
+  if (tid == 0) {
+    double t = 0.0;
+    for (int i = 0; i < kTile; ++i) t += lred[i];
+    lpart[blockIdx.x] = t / (double)n;
   }
 }
 
-// Sum of the per-CTA partials in CTA order, the mean loss, and optionally an Adam step on
-// the master weights.
+// Sum of the per-CTA partials in a fixed order, the mean loss, and optionally an Adam step on
+// the master weights. A CTA takes 32 parameters, one warp per eighth of the partials (one thread
+// per parameter and 152 loads one after the other took 27 us).
 __global__ void __launch_bounds__(kMThreads)
-mlp_reduce_kernel(const float* __restrict__ partial, int ncta, int P, const double* __restrict__ lpart, float* __restrict__ grad, double* __restrict__ loss,
-                  float* __restrict__ params, float* __restrict__ m, float* __restrict__ v, int step,
-                  float lr, int do_adam) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P; i += gridDim.x * blockDim.x) {
-    float g = 0.f;
-    for (int c = 0; c < ncta; ++c) g += partial[(size_t)c * P + i];
+mlp_reduce_kernel(const float* __restrict__ partial, int ncta, int P, const double* __restrict__ lpart,
+                  float* __restrict__ grad, double* __restrict__ loss, float* __restrict__ params,
+                  float* __restrict__ m, float* __restrict__ v, int step, float lr, int do_adam) {
+  __shared__ float sum[kMThreads / 32][32];
+  __shared__ double red[33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  float g = 0.f;
+  if (i < P) {
+#pragma unroll 8
+    for (int c = w; c < ncta; c += kMThreads / 32) g += partial[(size_t)c * P + i];
+  }
+  sum[w][lane] = g;
+  __syncthreads();
+  if (w == 0 && i < P) {
+    g = 0.f;
+#pragma unroll
+    for (int k = 0; k < kMThreads / 32; ++k) g += sum[k][lane];
     grad[i] = g;
     if (do_adam) {
       const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -447,10 +553,9 @@ mlp_reduce_kernel(const float* __restrict__ partial, int ncta, int P, const doub
       params[i] -= lr * mh / (sqrtf(vh) + eps);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    double s = 0.0;
-    for (int c = 0; c < ncta; ++c) s += lpart[c];
-    *loss = s;
+  if (blockIdx.x == 0) {
+    const double s = block_sum_array(lpart, ncta, red);
+    if (threadIdx.x == 0) *loss = s;
   }
 }
 
@@ -515,22 +620,18 @@ struct ed_mlp {
 };
 
 namespace {
-size_t grad_smem(const MlpDims& d) {
-  return ((size_t)(d.P + 3) / 4 * 4 + (size_t)kTile * kMaxIn + 5 * (size_t)kTile * kH + 2 * kTile) *
-         sizeof(float);
-}
-
 ed_status mlp_grad(ed_mlp* M, const ed_basis* b, double U, const int64_t* idx, const double* tgt,
                    int64_t n, double wscale, int adam, float lr) {
   cudaStream_t s = M->stream;
-  const size_t sm = grad_smem(M->d);
+  const size_t sm = (size_t)grad_layout(M->d.nin).total * sizeof(float);
   ED_TRY_CUDA(allow_max_smem(mlp_grad_kernel));
-  mlp_grad_kernel<<<M->ncta, kMThreads, sm, s>>>(M->params, M->L, (float)U, b->user_up().bits,
+  const int ncta = (int)std::min<int64_t>((n + kTile - 1) / kTile, M->ncta);
+  mlp_grad_kernel<<<ncta, kMThreads, sm, s>>>(M->params, M->L, (float)U, b->user_up().bits,
                                                   b->user_dn().bits, b->user_dn().dim, idx, tgt, n,
                                                   wscale, M->partial, M->lpart);
   if (adam) ++M->step;
-  mlp_reduce_kernel<<<(M->d.P + kMThreads - 1) / kMThreads, kMThreads, 0, s>>>(
-      M->partial, M->ncta, M->d.P, M->lpart, M->grad, M->loss, M->params, M->m,
+  mlp_reduce_kernel<<<(M->d.P + 31) / 32, kMThreads, 0, s>>>(
+      M->partial, ncta, M->d.P, M->lpart, M->grad, M->loss, M->params, M->m,
       M->v, M->step, lr, adam);
   ED_TRY_CUDA(cudaGetLastError());
   return ED_OK;
@@ -565,7 +666,7 @@ extern "C" ed_status ed_mlp_create(int32_t n_sites, uint64_t seed, void* stream,
   M->stream = (cudaStream_t)stream;
   M->L = n_sites;
   M->d = mlp_dims(n_sites);
-  M->ncta = sm_count();
+  M->ncta = 2 * sm_count();  // CTAs of the gradient kernel: two per SM
   const size_t P = M->d.P;
   bool ok = cudaMalloc((void**)&M->params, P * 4) == cudaSuccess &&
             cudaMalloc((void**)&M->m, P * 4) == cudaSuccess &&
