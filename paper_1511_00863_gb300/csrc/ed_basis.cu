@@ -316,6 +316,7 @@ extern "C" ed_status ed_build_basis(const ed_lattice* L, int32_t n_up, int32_t n
       return fail(ED_ERR_CUDA);
     }
   }
+  if ((st = rows_build(B, L->t_bond, s)) != ED_OK) return fail(st);
   if (cudaStreamSynchronize(s) != cudaSuccess) {
     set_error("ed_build_basis: %s", cudaGetErrorString(cudaGetLastError()));
     return fail(ED_ERR_CUDA);
@@ -368,6 +369,7 @@ extern "C" void ed_basis_destroy(ed_basis* B) {
   if (prev != B->device) cudaSetDevice(B->device);
   lz_cache_free(B);
   hv2_tables_free(B);
+  rows_free(B);
   free_species(B->up);
   free_species(B->dn);
   if (B->binom) cudaFree(B->binom);

@@ -49,6 +49,22 @@ struct SpeciesTables {
   int32_t* hopa = nullptr;
 };
 
+// Tables of the row-ordered H.v (ed_rows.cu), built with the basis where its rows are short
+// enough; C = 0: none.
+constexpr int kMaxClasses = 16;
+struct HvRows {
+  int C = 0;                 // hop classes: distinct amplitudes up to sign
+  int nchunks = 0;           // groups of 32 down columns
+  void* mem = nullptr;       // one allocation, the arrays below point into it
+  double2* amp = nullptr;    // [C] relative amplitude of a class
+  int32_t* perm = nullptr;   // [32 nchunks] down rank of a column (-1 pad), by hop counts
+  int32_t* base = nullptr;   // [nchunks] start of a chunk in tab
+  uint8_t* kc = nullptr;     // [nchunks][C] table rows
+  uint16_t* tab = nullptr;   // 32 entries per row: target | sign << 15
+  int32_t* up = nullptr;     // [maxhops_up][dim_up] up hops class by class
+  uint8_t* ucnt = nullptr;   // [dim_up][C] up hops per class (NULL: one class)
+};
+
 }  // namespace ed
 
 struct ed_basis {
@@ -61,6 +77,7 @@ struct ed_basis {
   // up-species hop graph), so that rows sharing up-neighbours are processed close in
   // time and the neighbours stay resident in L2. NULL = rank order.
   int32_t* up_order = nullptr;
+  ed::HvRows rows;  // tables of the row-ordered H.v
   // Workspaces of ed_lanczos_solve kept between calls (ed_lanczos.cu); freed with the basis.
   mutable void* solve_cache = nullptr;
   // Fused H.v variant chosen by timing for this basis, per dtype (0 = not tuned yet).
@@ -180,6 +197,17 @@ struct LzStore {
   void* const* slots;
   double* vscale;
 };
+
+// Row-ordered H.v (ed_rows.cu): tables built with the basis (t_bond: host amplitudes or NULL);
+// E = float, double, float2 or double2 (complex). Preferred to launch_hv / launch_hvc where
+// rows_usable.
+ed_status rows_build(ed_basis* b, const double* t_bond, cudaStream_t s);
+void rows_free(ed_basis* b);
+template <typename E>
+bool rows_usable(const ed_basis* b);
+template <typename E>
+ed_status launch_hv_rows(const ed_basis* b, double t, double U, const E* x, E* y, int64_t ld,
+                         cudaStream_t s, const LzHvArgs* lz, int* grid_out);
 
 struct Reorth;  // stored Lanczos vectors for reorthogonalisation (ed_reorth.cu)
 
