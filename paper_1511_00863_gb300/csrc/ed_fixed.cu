@@ -9,7 +9,7 @@
 //                       a 2^k = -t 2^-r, b 2^k = U 2^-r, c 2^k = -b_j (s_prev/s_cur) 2^-r;
 //   H.v    (fused):     S = exact int64 hop sum (Sec. 4 Eqs. 5-6), P = X_prev, W written
 //                       over P; partial sums of W X_cur exact in 192 bits;
-//   update:             a_j = s_w s_cur sum(W X_cur) (one FP64 rounding),
+//   update:             a_j = s_w s_cur sum(W X_cur) (one FP64 rounding, one thread per CTA),
 //                       Q = W + round(d X_cur 2^k2) with d 2^k2 = -a_j s_cur / s_w,
 //                       exact partial sums of Q^2 and max |Q|;
 //   finish (1 CTA):     b_{j+1} = s_w sqrt(sum Q^2), f_{j+1} = (s_w / b_{j+1}) Q.
@@ -161,23 +161,23 @@ __device__ __forceinline__ void fx_plan_step(LzScalars* S, int cur, const FxPlan
   const double cp = sc != 0.0 ? S->beta[j] * sp / sc : 0.0;
   const double bound = (fabs(t) * hops + fabs(U) * nmax) * mc + fabs(cp) * mp;
   int r = 0;
-  if (bound > 0.0 && isfinite(bound)) r = ilogb(bound) + 1 - (vb - 1);
-  const double A = ldexp(-t, -r), B = ldexp(U, -r), C = ldexp(-cp, -r);
+  if (bound > 0.0 && isfinite(bound)) r = exponent2(bound) + 1 - (vb - 1);
+  const double A = scale2(-t, -r), B = scale2(U, -r), C = scale2(-cp, -r);
   const double M = fmax(fabs(A), fmax(fabs(B), fabs(C)));
   int k = 0;
   long long a = 0, b = 0, c = 0;
   if (M > 0.0 && isfinite(M)) {
-    k = ilogb(M) - 61;
-    a = llrint(ldexp(A, -k));
-    b = llrint(ldexp(B, -k));
-    c = llrint(ldexp(C, -k));
+    k = exponent2(M) - 61;
+    a = llrint(scale2(A, -k));
+    b = llrint(scale2(B, -k));
+    c = llrint(scale2(C, -k));
   }
   S->fx_a = a;
   S->fx_b = b;
   S->fx_c = c;
   S->fx_k = k;
   S->fx_r = r;
-  S->fx_sw = ldexp(sc, r);
+  S->fx_sw = scale2(sc, r);
 }
 
 __global__ void fx_plan_kernel(LzScalars* S, int cur, FxPlanArgs p) {
@@ -227,7 +227,7 @@ __device__ __forceinline__ void fx_add_hops(long long& s, const int32_t* tab, in
 template <int R>
 __global__ void __launch_bounds__(kFxThreads)
 fx_hv_staged_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __restrict__ y,
-                    LzScalars* S, int cur, long long* __restrict__ part) {
+                    LzScalars* S) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (S->status != 0) return;
   const long long ca = S->fx_a, cb = S->fx_b, cc = S->fx_c;
@@ -282,14 +282,13 @@ fx_hv_staged_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __re
       }
     }
   }
-  fx_block_reduce(dot, 0, part + 4 * blockIdx.x);
-  fx_hv_finish(S, cur, part);
+  fx_hv_add(S, dot);
 }
 
 // Fallback when a row does not fit in shared memory.
 __global__ void __launch_bounds__(kFxThreads)
 fx_hv_global_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __restrict__ y,
-                    LzScalars* S, int cur, long long* __restrict__ part) {
+                    LzScalars* S) {
   if (S->status != 0) return;
   const long long ca = S->fx_a, cb = S->fx_b, cc = S->fx_c;
   const int k = S->fx_k;
@@ -311,8 +310,7 @@ fx_hv_global_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __re
     *yp = w;
     i192_add(dot, (i128)w * xc);
   }
-  fx_block_reduce(dot, 0, part + 4 * blockIdx.x);
-  fx_hv_finish(S, cur, part);
+  fx_hv_add(S, dot);
 }
 
 // Whole CTA: b_{j+1} and f_{j+1}'s scale from the n partial records of ||Q||^2, then the
@@ -322,6 +320,7 @@ __device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long
   I192 sum;
   long long mx;
   fx_sum_partials(pb, nb, sum, mx);
+  if (threadIdx.x < 6) S->fx_dot[threadIdx.x] = 0;
   if (threadIdx.x != 0) return;
   const int j = S->j + 1;
   const double sw = S->fx_sw;
@@ -334,18 +333,33 @@ __device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long
   }
 }
 
+// kReady: the H.v left a_j finished (hv2_ticket), else its sum in S->fx_dot.
 // finish: the last CTA ends the step (fx_finish_step); otherwise fx_finish_kernel does, after
 // the reorthogonalisation. kKeep: Q goes to the step's slot of `store` too. The grid is 4 CTAs
 // per SM: with more registers than that leaves (it takes 70 unbounded) a third of it ran as a
 // second wave, 102 instead of 81 us on the 4x4 lattice.
-template <bool kKeep>
+template <bool kKeep, bool kReady>
 __global__ void __launch_bounds__(kFxThreads, 4)
 fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long long* __restrict__ xp,
                  int64_t n, long long* __restrict__ pb, int finish, FxPlanArgs plan, LzStore store) {
   if (S->status != 0) return;
+  long long d;
+  int k2;
+  if constexpr (kReady) {
+    d = S->fx_d;
+    k2 = S->fx_k2;
+  } else {
+    __shared__ long long d_s;
+    __shared__ int k2_s;
+    if (threadIdx.x == 0) {
+      const double alpha = fx_alpha(S, cur, fx_hv_dot(S), d_s, k2_s);
+      if (blockIdx.x == 0) S->alpha[S->j + 1] = alpha;
+    }
+    __syncthreads();
+    d = d_s;
+    k2 = k2_s;
+  }
   longlong2* const keep = kKeep ? (longlong2*)store.slots[S->j + 1] : nullptr;
-  const long long d = S->fx_d;
-  const int k2 = S->fx_k2;
   A192 q2;
   long long mx = 0;
   // n is even (rows are padded to 32 elements): pairs of elements, two pairs in flight
@@ -686,13 +700,13 @@ ed_status fx_step(const ed_basis* b, const FxRun& fx, double t, double U, long l
     if (r != ED_OK) return r;
   } else if (R == 2) {
     const int grid = (int)((b->up.dim + 1) / 2);
-    fx_hv_staged_kernel<2><<<grid, kFxThreads, fx_smem<2>(b), s>>>(a, B[cur], B[1 - cur], S, cur, pa);
+    fx_hv_staged_kernel<2><<<grid, kFxThreads, fx_smem<2>(b), s>>>(a, B[cur], B[1 - cur], S);
   } else if (R == 1) {
     const int grid = (int)b->up.dim;
-    fx_hv_staged_kernel<1><<<grid, kFxThreads, fx_smem<1>(b), s>>>(a, B[cur], B[1 - cur], S, cur, pa);
+    fx_hv_staged_kernel<1><<<grid, kFxThreads, fx_smem<1>(b), s>>>(a, B[cur], B[1 - cur], S);
   } else {
     const int grid = fx_red_grid(b->dim) * 2;
-    fx_hv_global_kernel<<<grid, kFxThreads, 0, s>>>(a, B[cur], B[1 - cur], S, cur, pa);
+    fx_hv_global_kernel<<<grid, kFxThreads, 0, s>>>(a, B[cur], B[1 - cur], S);
   }
   ED_TRY_CUDA(cudaGetLastError());
   if (ev1) ED_TRY_CUDA(cudaEventRecord(ev1, s));
@@ -700,10 +714,10 @@ ed_status fx_step(const ed_basis* b, const FxRun& fx, double t, double U, long l
   const int ug = fx_red_grid(n);
   const FxPlanArgs next = {t, U, fx.hops, fx.nmax, fx.vb};
   const bool between = ro && ro_between(ro);  // passes between the update and the finish
-  if (store.slots)
-    fx_update_kernel<true><<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next, store);
-  else
-    fx_update_kernel<false><<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next, store);
+  const bool ready = plan && hv2_ticket(plan);
+  const auto update = store.slots ? (ready ? fx_update_kernel<true, true> : fx_update_kernel<true, false>)
+                                  : (ready ? fx_update_kernel<false, true> : fx_update_kernel<false, false>);
+  update<<<ug, kFxThreads, 0, s>>>(S, cur, B[cur], B[1 - cur], n, pb, !between, next, store);
   if (between) {
     const ed_status r = ro_apply(ro, S, B[1 - cur], pb, ug, s);
     if (r != ED_OK) return r;

@@ -51,6 +51,21 @@ __device__ __forceinline__ I192 i192_shfl_down(const I192& a, int off) {
   return r;
 }
 
+// x 2^e, exactly ldexp: an addition to the exponent field while x and the result are normal (one
+// thread waits 270 cycles for an ldexp on GB300, and the scalars of a step are one thread's work).
+__device__ __forceinline__ double scale2(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7FF), r = ex + e;
+  if (ex == 0 || ex == 0x7FF || r < 1 || r > 0x7FE) return ldexp(x, e);
+  return __longlong_as_double(b + ((long long)e << 52));
+}
+
+// ilogb of a finite nonzero x.
+__device__ __forceinline__ int exponent2(double x) {
+  const int ex = (int)((__double_as_longlong(x) >> 52) & 0x7FF);
+  return ex ? ex - 1023 : ilogb(x);
+}
+
 // Correctly rounded (nearest) conversion of the 192-bit integer to double.
 __device__ __forceinline__ double i192_to_double(const I192& a) {
   const bool neg = a.hi < 0;
@@ -81,7 +96,7 @@ __device__ __forceinline__ double i192_to_double(const I192& a) {
   }
   // fold the sticky bit into bit 0: the 11 discarded bits of `top` then round correctly
   const double m = __ull2double_rn(top | (sticky ? 1ull : 0ull));
-  const double v = ldexp(m, shift);
+  const double v = scale2(m, shift);
   return neg ? -v : v;
 }
 
@@ -253,26 +268,70 @@ __device__ __forceinline__ void fx_sum_partials(const long long* __restrict__ p,
   __syncthreads();
 }
 
-// End of a fixed-point H.v: the last CTA records a_j and the update's integer coefficient
-// (Q = W + round(d X 2^k2), d 2^k2 = -a_j s_cur / s_w).
-__device__ __forceinline__ void fx_hv_finish(LzScalars* S, int cur, const long long* part) {
+// End of a fixed-point H.v without a ticket: a CTA's sum of W X goes to the run's (no fence, no
+// wait).
+__device__ __forceinline__ void fx_hv_add(LzScalars* S, const I192& v) {
+  __shared__ long long tot[4];
+  fx_block_reduce(v, 0, tot);
+  if (threadIdx.x < 6)
+    atomicAdd(&S->fx_dot[threadIdx.x], (unsigned long long)reinterpret_cast<const uint32_t*>(tot)[threadIdx.x]);
+}
+
+// One thread: a_j from the sum of W X, and the update's integer coefficient (Q = W +
+// round(d X 2^k2), d 2^k2 = -a_j s_cur / s_w, s_cur / s_w = 2^-r).
+__device__ __forceinline__ double fx_alpha(const LzScalars* S, int cur, const I192& sum, long long& d, int& k2) {
+  const double alpha = S->fx_sw * S->scale[cur] * i192_to_double(sum);
+  const double D = scale2(-alpha, -S->fx_r);
+  d = 0;
+  k2 = -1;
+  if (D != 0.0 && isfinite(D)) {
+    k2 = exponent2(D) - 61;
+    d = llrint(scale2(D, -k2));
+  }
+  return alpha;
+}
+
+// ... with a ticket: the last CTA records a_j and the coefficient.
+__device__ __forceinline__ void fx_hv_finish(LzScalars* S, int cur, const I192& v, long long* part) {
+  fx_block_reduce(v, 0, part + 4 * blockIdx.x);
   if (!last_cta(&S->tick_hv)) return;
   I192 sum;
   long long unused;
   fx_sum_partials(part, gridDim.x, sum, unused);
   if (threadIdx.x != 0) return;
-  const double sc = S->scale[cur], sw = S->fx_sw;
-  const double alpha = sw * sc * i192_to_double(sum);
-  S->alpha[S->j + 1] = alpha;
-  const double D = -alpha * (sc / sw);
-  long long d = 0;
-  int k2 = -1;
-  if (D != 0.0 && isfinite(D)) {
-    k2 = ilogb(D) - 61;
-    d = llrint(ldexp(D, -k2));
-  }
+  long long d;
+  int k2;
+  S->alpha[S->j + 1] = fx_alpha(S, cur, sum, d, k2);
+  S->row_next = 0;
   S->fx_d = d;
   S->fx_k2 = k2;
+}
+
+// Either end, out of line: inlined, its registers cost the H.v's loops spills.
+static __device__ __noinline__ void fx_hv_end(LzScalars* S, int cur, unsigned long long w0, unsigned long long w1,
+                                              unsigned long long w2, long long* part, int ticket) {
+  A192 a;
+  a.w0 = w0;
+  a.w1 = w1;
+  a.w2 = w2;
+  if (ticket) fx_hv_finish(S, cur, a192_get(a), part);
+  else fx_hv_add(S, a192_get(a));
+}
+
+// The sum the H.v's CTAs added up.
+__device__ __forceinline__ I192 fx_hv_dot(const LzScalars* S) {
+  uint32_t w[6];
+  unsigned long long c = 0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    c += S->fx_dot[i];
+    w[i] = (uint32_t)c;
+    c >>= 32;
+  }
+  I192 r;
+  r.lo = ((u128)w[3] << 96) | ((u128)w[2] << 64) | ((u128)w[1] << 32) | (u128)w[0];
+  r.hi = (long long)(((unsigned long long)w[5] << 32) | w[4]);
+  return r;
 }
 
 }  // namespace ed

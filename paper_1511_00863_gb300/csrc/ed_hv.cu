@@ -126,7 +126,6 @@ hv_staged_kernel(HvArgs a, const T* __restrict__ x, T* __restrict__ y, LzHvArgs 
   if (kLz) {
     const double v = block_sum(dot.get(), red);
     if (threadIdx.x == 0) lz.partial[blockIdx.x] = v;
-    hv_finish(lz.S, lz.partial, red);
   }
 }
 
@@ -166,7 +165,6 @@ hv_global_kernel(HvArgs a, const T* __restrict__ x, T* __restrict__ y, LzHvArgs 
   if (kLz) {
     const double v = block_sum(dot.get(), red);
     if (threadIdx.x == 0) lz.partial[blockIdx.x] = v;
-    hv_finish(lz.S, lz.partial, red);
   }
 }
 

@@ -20,6 +20,8 @@ struct Hv2Plan {
   size_t smem = 0;
   int grid = 0;
   int ld = 0;
+  bool ticket = false;        // the H.v's last CTA finishes a_j
+  int nstatic = 0;            // row groups dealt out by index (plain plans)
   void* dtab = nullptr;       // [rows][ld] 16-bit slots
   uchar2* kpn = nullptr;      // per chunk of 32 V columns: positive, negative table rows
   uint8_t* slot_lo = nullptr;  // per column: slot within its group of G
@@ -296,6 +298,7 @@ static ed_status hv2_build_split(const ed_basis* b, int mode, int ld, cudaStream
   p->smem = split_smem(*t, b, mode == kHv2Fx ? 8 : 4);
   p->ld = ld;
   p->grid = (int)b->up.dim;
+  p->ticket = b->up.dim * (int64_t)ld >= kTicketMin;
   p->nslots = split_slots(*t);
   for (int i = 0; i < 3; ++i) p->cst[i] = t->cstart[i];
   const int64_t n = b->dn.dim;
@@ -362,6 +365,7 @@ ed_status hv2_build(const ed_basis* b, int mode, int ld, int schedule, cudaStrea
   p->smem = ki.smem;
   p->ld = ld;
   p->grid = (int)((b->up.dim + ki.R - 1) / ki.R);
+  p->ticket = b->up.dim * (int64_t)ld >= kTicketMin;
   const DownTables* t = nullptr;
   ed_status r = down_tables(b, ld, ki, s, &t);
   if (r == ED_OK) r = upload_down_tables(*t, b->dn.dim, s, p);
@@ -385,6 +389,11 @@ ed_status hv2_build(const ed_basis* b, int mode, int ld, int schedule, cudaStrea
     set_error("H.v tables: %s", cudaGetErrorString(e));
     return ED_ERR_CUDA;
   }
+  // groups handed out by the counter: all beyond the first round for exact sums, the last
+  // quarter or so for FP32 ones (a reduction per group); none without a ticket to reset it
+  const int groups = (int)((b->up.dim + ki.R - 1) / ki.R), rounds = groups / p->grid;
+  p->nstatic = groups;
+  if (p->ticket && rounds >= 2) p->nstatic = mode == kHv2Fx ? p->grid : p->grid * std::max(1, rounds * 3 / 4);
   *out = p;
   return ED_OK;
 }
@@ -392,6 +401,7 @@ ed_status hv2_build(const ed_basis* b, int mode, int ld, int schedule, cudaStrea
 const int32_t* hv2_colpos(const Hv2Plan* p) { return p ? p->colpos : nullptr; }
 
 int hv2_grid(const Hv2Plan* p) { return p ? p->grid : 0; }
+bool hv2_ticket(const Hv2Plan* p) { return p && p->ticket; }
 
 ed_status hv2_autotune(const ed_basis* b, int mode, int ld, void* x, void* y,
                        LzScalars* S, void* partial, cudaStream_t s, int* kind) {
@@ -455,6 +465,8 @@ ed_status hv2_launch(const Hv2Plan* p, const ed_basis* b, double t, double U, co
   a.dim_up = b->up.dim;
   a.ld = p->ld;
   a.maxhops_up = b->up.maxhops;
+  a.ticket = p->ticket;
+  a.nstatic = p->nstatic;
   a.t = (float)t;
   a.U = (float)U;
 #define HV2_LAUNCH(K, E, R_, V, T, MB)                                                     \
@@ -476,6 +488,7 @@ ed_status hv2_launch(const Hv2Plan* p, const ed_basis* b, double t, double U, co
     c.dim_up = b->up.dim;
     c.ld = p->ld;
     c.maxhops_up = b->up.maxhops;
+    c.ticket = p->ticket;
     c.nslots = p->nslots;
     c.cstart0 = p->cst[0];
     c.cstart1 = p->cst[1];
@@ -502,6 +515,7 @@ ed_status hv2_launch(const Hv2Plan* p, const ed_basis* b, double t, double U, co
     c.dim_up = b->up.dim;
     c.ld = p->ld;
     c.maxhops_up = b->up.maxhops;
+    c.ticket = p->ticket;
     c.namp = hv2c_namp(b);
     c.t = (float)t;
     c.U = (float)U;

@@ -92,7 +92,8 @@ struct Hv2Args {
   const int32_t* __restrict__ hop_up;    // basis table [maxhops_up][dim_up]
   const int32_t* __restrict__ order;     // up-row visit order (NULL = rank order)
   int64_t dim_up;
-  int ld, maxhops_up;
+  int ld, maxhops_up, ticket;
+  int nstatic;  // row groups dealt out by index; the others by S->row_next
   float t, U;  // FP32 variant
 };
 
@@ -126,8 +127,12 @@ __device__ __forceinline__ void hv2_up_list(const int32_t* __restrict__ hop_up, 
 }
 
 // The grid is one resident wave (hv2_build): a CTA takes the row groups blockIdx.x,
-// blockIdx.x + gridDim.x, ..., so that its reduction and its ticket (each 1-2 us of waiting in a
-// CTA's 50) come once per launch and not once per row.
+// blockIdx.x + gridDim.x, ..., so that its reduction (1-2 us of a CTA's 50) comes once per launch and
+// not once per row, and the next pass has a few hundred records to add, not thousands. The SMs do
+// not run at one speed (with all rows dealt out they were busy 91% of the launch on average), so
+// groups from nstatic on are handed out by a counter, asked for one group ahead. Integer sums do
+// not mind which CTA took which row; FP32 runs write one partial sum per handed-out group, and
+// start handing out late (hv2_build), so that their sums too are the same in every run.
 template <typename E, int R, int V, int T, int MB>
 __global__ void __launch_bounds__(T, MB)
 hv2_kernel(Hv2Args a, const E* __restrict__ x, E* __restrict__ y, LzScalars* S,
@@ -159,15 +164,24 @@ hv2_kernel(Hv2Args a, const E* __restrict__ x, E* __restrict__ y, LzScalars* S,
   DotAcc<float> dotf;
   A192 dota;
   const int ngroups = (int)((a.dim_up + R - 1) / R);
-  for (int g = blockIdx.x; g < ngroups; g += gridDim.x) {
+  __shared__ int next_s;
+  bool flushed = false;  // FP32: the sum over the fixed groups is written
+  for (int g = blockIdx.x; g < ngroups;) {
+  const bool ask = g + (int)gridDim.x >= a.nstatic && a.nstatic < ngroups;
+  int asked = 0;
+  if (ask && threadIdx.x == 0) asked = atomicAdd(&S->row_next, 1);
+  if (sizeof(E) == 4 && g >= a.nstatic && !flushed) {
+    const double v = block_sum(dotf.get(), red);
+    if (threadIdx.x == 0) reinterpret_cast<double*>(partial)[blockIdx.x] = v;
+    dotf = DotAcc<float>();
+    flushed = true;
+  }
   int64_t urow[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int64_t q = (int64_t)g * R + r;
     urow[r] = q < a.dim_up ? (a.order ? (int64_t)a.order[q] : q) : a.dim_up;  // dim_up = none
   }
-  if (g != (int)blockIdx.x) __syncthreads();  // the gathers of the rows before are done
-
   // ---- stage the R rows (one d per thread: R coalesced loads, one vector store); slots
   // ld .. ld + G - 1 are zero, one in each bank group
   for (int d = threadIdx.x; d < ld + G; d += T) {
@@ -300,15 +314,24 @@ hv2_kernel(Hv2Args a, const E* __restrict__ x, E* __restrict__ y, LzScalars* S,
       stcs_pack(reinterpret_cast<Pack<E, V>*>(yp), W);
     }
   }
+  if (sizeof(E) == 4 && flushed) {
+    const double v = block_sum(dotf.get(), red);
+    if (threadIdx.x == 0) reinterpret_cast<double*>(partial)[gridDim.x + g - a.nstatic] = v;
+    dotf = DotAcc<float>();
+  }
+  if (ask && threadIdx.x == 0) next_s = a.nstatic + asked;
+  __syncthreads();  // the gathers of these rows are done
+  g = ask ? next_s : g + (int)gridDim.x;
   }
   if constexpr (sizeof(E) == 4) {
-    const double v = block_sum(dotf.get(), red);
-    if (threadIdx.x == 0) reinterpret_cast<double*>(partial)[blockIdx.x] = v;
-    hv_finish(S, reinterpret_cast<const double*>(partial), red);
+    if (!flushed) {
+      const double v = block_sum(dotf.get(), red);
+      if (threadIdx.x == 0) reinterpret_cast<double*>(partial)[blockIdx.x] = v;
+    }
+    if (a.ticket)
+      hv_finish(S, reinterpret_cast<const double*>(partial), (int)gridDim.x + ngroups - a.nstatic, red);
   } else {
-    long long* part = reinterpret_cast<long long*>(partial);
-    fx_block_reduce(a192_get(dota), 0, part + 4 * blockIdx.x);
-    fx_hv_finish(S, cur, part);
+    fx_hv_end(S, cur, dota.w0, dota.w1, dota.w2, reinterpret_cast<long long*>(partial), a.ticket);
   }
 }
 

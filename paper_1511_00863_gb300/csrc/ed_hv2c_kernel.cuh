@@ -29,7 +29,7 @@ struct Hv2cArgs {
   const int32_t* __restrict__ order;     // up-row visit order (NULL = rank order)
   const double2* __restrict__ tau;       // per-bond relative amplitudes (NULL: all 1)
   int64_t dim_up;
-  int ld, maxhops_up, namp;  // namp = 4 n_bonds with tau, else 2
+  int ld, maxhops_up, namp, ticket;  // namp = 4 n_bonds with tau, else 2
   float t, U;
 };
 
@@ -188,7 +188,7 @@ hv2c_kernel(Hv2cArgs a, const float2* __restrict__ x, float2* __restrict__ y,
   }
   const double v = block_sum(dot.get(), red);
   if (threadIdx.x == 0) partial[blockIdx.x] = v;
-  hv_finish(S, partial, red);
+  if (a.ticket) hv_finish(S, partial, gridDim.x, red);
 }
 
 }  // namespace ed

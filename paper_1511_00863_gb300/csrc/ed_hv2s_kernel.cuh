@@ -28,7 +28,7 @@ struct Hv2sArgs {
   const int32_t* __restrict__ hop_up;    // basis table [maxhops_up][dim_up]
   const int32_t* __restrict__ order;     // up-row visit order (NULL = rank order)
   int64_t dim_up;
-  int ld, maxhops_up, nslots;            // nslots: longest slice + G
+  int ld, maxhops_up, nslots, ticket;    // nslots: longest slice + G
   int cstart0, cstart1, cstart2;         // slices [cstart0, cstart1), [cstart1, cstart2)
   float t, U;                            // FP32 variant
 };
@@ -156,11 +156,9 @@ hv2s_kernel(Hv2sArgs a, const E* __restrict__ x, E* __restrict__ y,
   if constexpr (sizeof(E) == 4) {
     const double v = block_sum(dotf.get(), red);
     if (threadIdx.x == 0) reinterpret_cast<double*>(partial)[blockIdx.x] = v;
-    hv_finish(S, reinterpret_cast<const double*>(partial), red);
+    if (a.ticket) hv_finish(S, reinterpret_cast<const double*>(partial), gridDim.x, red);
   } else {
-    long long* part = reinterpret_cast<long long*>(partial);
-    fx_block_reduce(a192_get(dota), 0, part + 4 * blockIdx.x);
-    fx_hv_finish(S, cur, part);
+    fx_hv_end(S, cur, dota.w0, dota.w1, dota.w2, reinterpret_cast<long long*>(partial), a.ticket);
   }
 }
 

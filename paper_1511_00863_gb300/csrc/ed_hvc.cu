@@ -208,7 +208,6 @@ hvc_staged_kernel(HvcArgs a, const typename CVec<T>::type* __restrict__ x,
   if (kLz) {
     const double v = block_sum(dot.get(), red);
     if (threadIdx.x == 0) lz.partial[blockIdx.x] = v;
-    hv_finish(lz.S, lz.partial, red);
   }
 }
 
@@ -267,7 +266,6 @@ hvc_global_kernel(HvcArgs a, const typename CVec<T>::type* __restrict__ x,
   if (kLz) {
     const double v = block_sum(dot.get(), red);
     if (threadIdx.x == 0) lz.partial[blockIdx.x] = v;
-    hv_finish(lz.S, lz.partial, red);
   }
 }
 

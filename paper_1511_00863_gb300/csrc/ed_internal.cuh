@@ -146,6 +146,7 @@ struct LzScalars {
   int chk;          // convergence checks have covered the steps up to here
   unsigned tick_chk;  // CTAs of the running check that are done
   unsigned tick_hv, tick_upd;  // CTAs of the running H.v / update pass that are done
+  int row_next;     // row groups of the running H.v handed out beyond the fixed ones
   int max_steps;
   double tol;
   double tscale;    // max over i <= j of |a_i| + b_i (breakdown scale)
@@ -155,6 +156,9 @@ struct LzScalars {
   long long fx_a, fx_b, fx_c;   // H.v epilogue W = round((a S + b n X + c P) 2^fx_k)
   int fx_k, fx_r;               // ... and W's scale s_w = scale[cur] * 2^fx_r
   double fx_sw;
+  // sum of W X over the H.v's CTAs, 32 bits of the 192-bit value per word (the words' sums keep
+  // their carries): integer additions, so the order does not matter; zeroed by the step's finish
+  unsigned long long fx_dot[6];
   long long fx_d;               // update Q = W + round(d X 2^fx_k2)
   int fx_k2, pad_;
   double alpha[ED_MAX_STEPS + 2];
@@ -165,9 +169,8 @@ struct LzScalars {
 // Extra arguments of the Lanczos-fused H.v pass:
 //   w = scale[cur] * H B_cur - b_j * scale[prev] * B_prev   (written over B_prev)
 //   partial[block] = sum over the block's elements of w * (scale[cur] * B_cur)
-// The last CTA sums the partials into alpha[j + 1].
 struct LzHvArgs {
-  LzScalars* S;
+  const LzScalars* S;
   int cur;
   double* partial;
 };
@@ -275,6 +278,13 @@ ed_status ro_count(const Reorth* r, cudaStream_t s, int* count);
 ed_status ro_ritz_vector(const Reorth* r, const double* y, int m, int64_t dim, int64_t cols,
                          int64_t ld, const int32_t* colpos, double* psi, cudaStream_t s);
 
+// Vectors from this length on let the fused H.v's last CTA finish a_j (a fence and a ticket per
+// CTA and the last one's sum, 6-8 us in all); below, every CTA of the update pass sums the H.v's
+// records first (2-9 us, growing with the waiting memory traffic): H.v + update 440 against 453
+// us on the 4x4 lattice (19 M), 18.5 against 19.5 us on the 12-site ring (48,400). Kernels with
+// many short-lived CTAs (the general ones) never take tickets: 28 -> 39 us at 0.9 M elements.
+constexpr int64_t kTicketMin = (int64_t)1 << 20;
+
 // Lanczos-fused H.v on the library's padded vectors (ed_hv2.cu). hv2_build leaves *out
 // NULL when no variant fits in shared memory (the general kernels are used then).
 struct Hv2Plan;
@@ -285,6 +295,8 @@ ed_status hv2_build(const ed_basis* b, int mode, int ld, int schedule, cudaStrea
                     Hv2Plan** out);
 void hv2_free(Hv2Plan* p);
 int hv2_grid(const Hv2Plan* p);
+// Whether the plan's H.v leaves a_j finished (else its records, hv2_grid of them).
+bool hv2_ticket(const Hv2Plan* p);
 // Row stride the fused H.v needs for this basis and precision when its rows only fit in
 // shared memory as two slices (the split-row kernel), else 0 (the stride is then dim_dn
 // rounded up to 32). Builds and caches the split tables on the basis.
@@ -347,9 +359,9 @@ __device__ __forceinline__ double block_sum(double v, double* sm) {
 }
 
 // True in the CTA that is the last of its launch to get here (for all its threads); it sees
-// what thread 0 of every other CTA wrote before. The reductions of a pass end in that CTA
-// instead of a launch of their own, or of every CTA of the next pass: summing the H.v's 4,368
-// records in each of the update pass's 608 CTAs took 4-5 us of its 91 on the 4x4 lattice.
+// what thread 0 of every other CTA wrote before. The update pass ends in that CTA instead of a
+// launch of its own (the fence and the ticket take 2-4 us, so passes whose CTAs are many or
+// short-lived, the H.v, leave their records to the next pass).
 __device__ __forceinline__ bool last_cta(unsigned* ticket) {
   __shared__ int last_s;
   if (threadIdx.x == 0) {
@@ -387,11 +399,33 @@ __device__ __forceinline__ double block_sum_array(const double* p, int64_t n, do
   return v;
 }
 
-// End of a Lanczos-fused H.v: the last CTA records a_{j+1} = the sum of the CTAs' partials.
-__device__ __forceinline__ void hv_finish(LzScalars* S, const double* partial, double* red) {
+// End of a Lanczos-fused H.v with a ticket: the last CTA records a_{j+1} = the sum of the n
+// partials.
+__device__ __forceinline__ void hv_finish(LzScalars* S, const double* partial, int n, double* red) {
   if (!last_cta(&S->tick_hv)) return;
-  const double a = block_sum_array(partial, gridDim.x, red);
-  if (threadIdx.x == 0) S->alpha[S->j + 1] = a;
+  const double a = block_sum_array(partial, n, red);
+  if (threadIdx.x != 0) return;
+  S->alpha[S->j + 1] = a;
+  S->row_next = 0;
+}
+
+// Sum of n partials in a fixed order by one warp (every lane gets it): a CTA of the update pass
+// adds the H.v's few hundred records this way while its other warps wait, 20-40 FP64 additions
+// per lane of one warp instead of as many in each of eight.
+__device__ __forceinline__ double warp_sum_array(const double* p, int n) {
+  const int lane = threadIdx.x & 31;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int i = lane; i < n; i += 128) {
+    double w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = i + 32 * k < n ? p[i + 32 * k] : 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] += w[k];
+  }
+  double t = (v[0] + v[1]) + (v[2] + v[3]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
 }
 
 }  // namespace ed

@@ -3,9 +3,10 @@
 //
 // One step j is two launches on the run's stream:
 //   1. fused H.v:  w = H f_j - b_j f_{j-1}, written over the f_{j-1} buffer, with per-CTA
-//      partial sums of w . f_j  (ed_hv.cu, LzHvArgs); the last CTA sums them to a_j;
-//   2. update:     q = w - a_j f_j in place, per-CTA partial sums of q . q; the last CTA sums
-//      them (finish): b_{j+1} = sqrt(sum), breakdown test, f_{j+1} = q / b_{j+1} kept implicit
+//      partial sums of w . f_j  (ed_hv.cu, LzHvArgs);
+//   2. update:     a_j = the sum of the partials (one warp of every CTA, in the same order, or
+//      on long vectors the last CTA of the H.v: kTicketMin), q = w - a_j f_j in place, per-CTA partial sums of q . q; the last CTA sums them
+//      (finish): b_{j+1} = sqrt(sum), breakdown test, f_{j+1} = q / b_{j+1} kept implicit
 //      as a buffer scale.
 // (Reorthogonalisation runs between the update and a finish launch of its own.)
 // E0(j) = lambda_min(T_j) and the convergence test run beside the next steps, on a stream of
@@ -122,10 +123,25 @@ __device__ __forceinline__ void lz_finish_step(LzScalars* S, int cur, const doub
 template <typename T, bool kKeep>
 __global__ void __launch_bounds__(kRedThreads)
 lz_update_kernel(LzScalars* S, int cur, const T* __restrict__ bcur, T* __restrict__ bprev,
-                 int64_t n, double* __restrict__ pb, int finish, LzStore store) {
+                 int64_t n, const double* __restrict__ pa, int na, double* __restrict__ pb, int finish,
+                 LzStore store) {
   __shared__ double red[33];
+  __shared__ double alpha_s;
   if (S->status != 0) return;
-  const T coef = (T)(S->alpha[S->j + 1] * S->scale[cur]);
+  if (na == 0) {  // the H.v left a_j finished
+    if (threadIdx.x == 0) alpha_s = S->alpha[S->j + 1];
+  } else if (na <= 2048) {
+    if (threadIdx.x < 32) {
+      const double a = warp_sum_array(pa, na);
+      if (threadIdx.x == 0) alpha_s = a;
+    }
+  } else {
+    const double a = block_sum_array(pa, na, red);
+    if (threadIdx.x == 0) alpha_s = a;
+  }
+  __syncthreads();
+  if (na > 0 && blockIdx.x == 0 && threadIdx.x == 0) S->alpha[S->j + 1] = alpha_s;
+  const T coef = (T)(alpha_s * S->scale[cur]);
   DotAcc<T> acc;
   // n is a multiple of 32 (padded rows): 16-byte vectors of 16 / sizeof(T) elements
   constexpr int VE = 16 / sizeof(T);
@@ -302,21 +318,23 @@ static ed_status lz_launch_step(ed_lanczos* st, const ed_params* p, cudaStream_t
     return r;
   }
   LzHvArgs lz{st->S, c, st->pa};
+  int grid = 0;
   ed_status r;
   if (ev0) ED_TRY_CUDA(cudaEventRecord(ev0, s));
   const ed_dtype dt = st->opts.dtype;
   if (st->plan) {
+    grid = hv2_ticket(st->plan) ? 0 : hv2_grid(st->plan);  // (0: a_j is finished)
     r = hv2_launch(st->plan, b, p->t, p->U, st->B[c], st->B[1 - c], st->S, c, st->pa, s);
   } else if (dt == ED_C32) {
-    r = launch_hvc<float>(b, p->t, p->U, st->B[c], st->B[1 - c], st->ld, s, &lz);
+    r = launch_hvc<float>(b, p->t, p->U, st->B[c], st->B[1 - c], st->ld, s, &lz, &grid);
   } else if (dt == ED_C64) {
-    r = launch_hvc<double>(b, p->t, p->U, st->B[c], st->B[1 - c], st->ld, s, &lz);
+    r = launch_hvc<double>(b, p->t, p->U, st->B[c], st->B[1 - c], st->ld, s, &lz, &grid);
   } else if (dt == ED_F64_NATIVE)
     r = launch_hv<double>(b, p->t, p->U, (const double*)st->B[c], (double*)st->B[1 - c], st->ld,
-                          s, &lz);
+                          s, &lz, &grid);
   else
     r = launch_hv<float>(b, p->t, p->U, (const float*)st->B[c], (float*)st->B[1 - c], st->ld,
-                         s, &lz);
+                         s, &lz, &grid);
   if (r != ED_OK) return r;
   if (ev1) ED_TRY_CUDA(cudaEventRecord(ev1, s));
   // the update works on scalars: a complex vector is 2 n of them (a_j, b_j are real)
@@ -326,13 +344,13 @@ static ed_status lz_launch_step(ed_lanczos* st, const ed_params* p, cudaStream_t
   const bool keep = st->store.slots != nullptr;
   if (dt == ED_F64_NATIVE || dt == ED_C64)  // (only FP32 and fixed-point runs keep their vectors here)
     lz_update_kernel<double, false><<<ug, kRedThreads, 0, s>>>(
-        st->S, c, (const double*)st->B[c], (double*)st->B[1 - c], ns, st->pb, !between, st->store);
+        st->S, c, (const double*)st->B[c], (double*)st->B[1 - c], ns, st->pa, grid, st->pb, !between, st->store);
   else if (keep)
     lz_update_kernel<float, true><<<ug, kRedThreads, 0, s>>>(
-        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pb, !between, st->store);
+        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pa, grid, st->pb, !between, st->store);
   else
     lz_update_kernel<float, false><<<ug, kRedThreads, 0, s>>>(
-        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pb, !between, st->store);
+        st->S, c, (const float*)st->B[c], (float*)st->B[1 - c], ns, st->pa, grid, st->pb, !between, st->store);
   ED_TRY_CUDA(cudaGetLastError());
   if (between) {
     if ((r = ro_apply(st->ro, st->S, st->B[1 - c], st->pb, ug, s)) != ED_OK) return r;

@@ -337,7 +337,8 @@ __device__ __forceinline__ void tridiag_ritz_vector(const double* a, const doubl
 // them (lz_check_kernel), and a flag that changed under a running kernel would let some warps
 // of a CTA return and others go on with shared memory that was never filled.
 __device__ __forceinline__ bool finish_step(LzScalars* S, int j, double beta) {
-  const double ts = fmax(S->tscale, fabs(S->alpha[j]) + S->beta[j]);
+  // (a_j was written by another CTA of this launch)
+  const double ts = fmax(S->tscale, fabs(__ldcg(&S->alpha[j])) + S->beta[j]);
   S->tscale = ts;
   S->beta[j + 1] = beta;
   S->j = j;

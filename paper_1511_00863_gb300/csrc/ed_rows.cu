@@ -440,7 +440,6 @@ hv_rows_kernel(RowsArgs a, const E* __restrict__ x, E* __restrict__ y, LzHvArgs 
   if (kLz) {
     const double v = block_sum(dot.get(), red);
     if (threadIdx.x == 0) lz.partial[blockIdx.x] = v;
-    hv_finish(lz.S, lz.partial, red);
   }
 }
 
