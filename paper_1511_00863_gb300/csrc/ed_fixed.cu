@@ -41,36 +41,7 @@ __device__ __forceinline__ long long sgn_apply(long long v, uint32_t e) {
   return (v ^ m) - m;
 }
 
-// ------------------------------------------------------------------ start vectors
-__device__ __forceinline__ long long shift_signed(long long v, int sh) {
-  if (sh >= 0) return v << sh;
-  return round_shift((i128)v, sh);
-}
-
-// X_i = (2 u_i - 1) 2^53 exactly (u_i from SplitMix64 as in ed_start_vector), moved to the
-// 2^vb range.
-__global__ void __launch_bounds__(kFxThreads)
-fx_start_kernel(uint64_t seed, int64_t n, int64_t cols, int64_t ld, const int32_t* __restrict__ colpos,
-                int vb, long long* __restrict__ X, long long* __restrict__ part) {
-  I192 acc;
-  i192_zero(acc);
-  long long mx = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t z = seed + ((uint64_t)i + 1ull) * 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    z = z ^ (z >> 31);
-    long long v = (long long)(2ull * (z >> 11)) - (1LL << 53);
-    v = shift_signed(v, vb - 53);
-    const int64_t r = i / cols, c = i - r * cols;
-    X[r * ld + (colpos ? colpos[c] : c)] = v;
-    i192_add(acc, (i128)v * v);
-    mx = max(mx, v < 0 ? -v : v);
-  }
-  fx_block_reduce(acc, mx, part + 4 * blockIdx.x);
-}
-
+// ------------------------------------------------------------------ caller vectors
 // Largest |f_i| as its IEEE bit pattern (sign cleared); a non-finite entry gives the
 // pattern of infinity or NaN, which the host rejects.
 __global__ void __launch_bounds__(kFxThreads)
@@ -92,42 +63,19 @@ fx_absmax_kernel(const double* __restrict__ f, int64_t n, unsigned long long* __
   }
 }
 
-__global__ void fx_absmax_final(const unsigned long long* __restrict__ part, int n,
-                                unsigned long long* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    unsigned long long m = 0;
-    for (int i = 0; i < n; ++i) m = max(m, part[i]);
+__global__ void __launch_bounds__(kFxThreads)
+fx_absmax_final(const unsigned long long* __restrict__ part, int n, unsigned long long* __restrict__ out) {
+  __shared__ unsigned long long sm[32];
+  unsigned long long m = 0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) m = max(m, part[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max(m, sm[w]);
     *out = m;
   }
-}
-
-// X_i = f_i 2^(vb - E) with |f| < 2^E, by integer manipulation of the IEEE fields (round
-// half up where bits fall off).
-__global__ void __launch_bounds__(kFxThreads)
-fx_copy_in_kernel(const double* __restrict__ f, int64_t n, int64_t cols, int64_t ld,
-                  const int32_t* __restrict__ colpos, int vb, int E, long long* __restrict__ X,
-                  long long* __restrict__ part) {
-  I192 acc;
-  i192_zero(acc);
-  long long mx = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(f[i]);
-    const int ef = (int)((bits >> 52) & 0x7FF);
-    long long mant = (long long)(bits & 0xFFFFFFFFFFFFFull);
-    int e2 = -1074;
-    if (ef) {
-      mant |= 1LL << 52;
-      e2 = ef - 1075;
-    }
-    long long v = shift_signed(mant, e2 + vb - E);
-    if (bits >> 63) v = -v;
-    const int64_t r = i / cols, c = i - r * cols;
-    X[r * ld + (colpos ? colpos[c] : c)] = v;
-    i192_add(acc, (i128)v * v);
-    mx = max(mx, v < 0 ? -v : v);
-  }
-  fx_block_reduce(acc, mx, part + 4 * blockIdx.x);
 }
 
 // f_1 = X / ||X||: scale[0] = 1 / sqrt(sum X^2), fx_max[0] = max |X|.
@@ -442,16 +390,6 @@ __device__ __forceinline__ void fx_psi_records(long long bv, long long bi, const
   }
 }
 
-// rank[p] = the down rank at column p of the stored rows, -1 for a pad.
-__global__ void fx_rank_kernel(const int32_t* __restrict__ colpos, int64_t cols, int64_t ld,
-                               int32_t* __restrict__ rank, int pads) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (pads ? ld : cols);
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (pads) rank[i] = -1;
-    else rank[colpos ? colpos[i] : i] = (int32_t)i;
-  }
-}
-
 // P = sum_k round(y_{k+1} s_k 2^60 X_k) over the m stored vectors, two columns per thread, and
 // the records of P. HBM bound: every vector is read once, coalesced, four of them in flight;
 // the element goes to its rank (scattered within its row) once. Against regenerating the
@@ -620,11 +558,8 @@ ed_status fx_psi_accum(const ed_basis* b, const LzScalars* S, int cur, const dou
 }
 
 ed_status fx_psi_sum(const ed_basis* b, const double* y, int m, const LzStore& store, int64_t ld,
-                     const int32_t* colpos, int32_t* rank, long long* P, long long* part,
-                     cudaStream_t s) {
+                     const int32_t* rank, long long* P, long long* part, cudaStream_t s) {
   const int g = fx_red_grid(b->dim);
-  fx_rank_kernel<<<g, kFxThreads, 0, s>>>(colpos, b->dn.dim, ld, rank, 1);
-  fx_rank_kernel<<<g, kFxThreads, 0, s>>>(colpos, b->dn.dim, ld, rank, 0);
   fx_psi_sum_kernel<<<g, kFxThreads, (size_t)m * 20, s>>>(y, m, store, b->up.dim, b->dn.dim, ld, rank,
                                                           P, part, part + 2 * g);
   ED_TRY_CUDA(cudaGetLastError());
@@ -651,22 +586,17 @@ ed_status fx_prepare(const ed_basis* b) {
   return ED_OK;
 }
 
-ed_status fx_start(const ed_basis* b, const FxRun& fx, uint64_t seed, long long* X, int64_t ld,
-                   const int32_t* colpos, LzScalars* S, long long* part, cudaStream_t s) {
-  const int g = fx_red_grid(b->dim);
-  fx_start_kernel<<<g, kFxThreads, 0, s>>>(seed, b->dim, b->dn.dim, ld, colpos, fx.vb, X, part);
-  fx_init_kernel<<<1, kFxThreads, 0, s>>>(S, part, g);
+ed_status fx_init(LzScalars* S, const long long* part, int n, cudaStream_t s) {
+  fx_init_kernel<<<1, kFxThreads, 0, s>>>(S, part, n);
   ED_TRY_CUDA(cudaGetLastError());
   return ED_OK;
 }
 
-ed_status fx_copy_in(const ed_basis* b, const FxRun& fx, const double* f1, long long* X,
-                     int64_t ld, const int32_t* colpos, LzScalars* S, long long* part,
-                     cudaStream_t s) {
+ed_status fx_exponent(const ed_basis* b, const double* f1, long long* part, cudaStream_t s, int* E) {
   const int g = fx_red_grid(b->dim);
   unsigned long long* pm = reinterpret_cast<unsigned long long*>(part);
   fx_absmax_kernel<<<g, kFxThreads, 0, s>>>(f1, b->dim, pm);
-  fx_absmax_final<<<1, 32, 0, s>>>(pm, g, pm + g);
+  fx_absmax_final<<<1, kFxThreads, 0, s>>>(pm, g, pm + g);
   ED_TRY_CUDA(cudaGetLastError());
   unsigned long long mb = 0;
   ED_TRY_CUDA(cudaMemcpyAsync(&mb, pm + g, sizeof(mb), cudaMemcpyDeviceToHost, s));
@@ -674,11 +604,7 @@ ed_status fx_copy_in(const ed_basis* b, const FxRun& fx, const double* f1, long 
   const int ef = (int)(mb >> 52);
   ED_CHECK_ARG(ef != 0x7FF, "f1 holds a non-finite value");
   ED_CHECK_ARG(mb != 0, "f1 is the zero vector");
-  const int E = ef ? ef - 1022 : -1022;  // |f1| < 2^E
-  fx_copy_in_kernel<<<g, kFxThreads, 0, s>>>(f1, b->dim, b->dn.dim, ld, colpos, fx.vb, E, X,
-                                              part);
-  fx_init_kernel<<<1, kFxThreads, 0, s>>>(S, part, g);
-  ED_TRY_CUDA(cudaGetLastError());
+  *E = ef ? ef - 1022 : -1022;  // |f1| < 2^E
   return ED_OK;
 }
 

@@ -183,6 +183,21 @@ __device__ __forceinline__ I192 a192_get(const A192& a) {
   return r;
 }
 
+__device__ __forceinline__ long long shift_signed(long long v, int sh) {
+  if (sh >= 0) return v << sh;
+  return round_shift((i128)v, sh);
+}
+
+// Element i of the random start vector as an integer: the top 53 bits of the (i+1)-th output of
+// SplitMix64 (Steele, Lea & Flood 2014) seeded with `seed`, minus 2^52 (2 u - 1 = h 2^-52).
+__device__ __forceinline__ long long start_int(uint64_t seed, uint64_t i) {
+  uint64_t z = seed + (i + 1ull) * 0x9E3779B97F4A7C15ull;
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  z = z ^ (z >> 31);
+  return (long long)(z >> 11) - (1LL << 52);
+}
+
 // Coefficient c = m * 2^e with m an int64 mantissa, |m| < 2^62 for the largest of a set.
 struct FxCoef {
   long long m;

@@ -221,15 +221,11 @@ struct FxRun {
   int nmax;    // max doubly occupied sites = min(n_up, n_dn)
 };
 FxRun fx_make(const ed_basis* b);
-// Start vector of SplitMix64 `seed` (exact in fixed point) into X (layout rows x ld, down
-// rank d at column colpos[d], or d if colpos is NULL), and the run's initial scalars
-// (scale[0], fx_max[0]). part: >= 4 * 4 * sm_count longs.
-ed_status fx_start(const ed_basis* b, const FxRun& fx, uint64_t seed, long long* X, int64_t ld,
-                   const int32_t* colpos, LzScalars* S, long long* part, cudaStream_t s);
-// Caller FP64 vector f1 (dense, rank order) converted to fixed point (exponent from max |f1|).
-ed_status fx_copy_in(const ed_basis* b, const FxRun& fx, const double* f1, long long* X,
-                     int64_t ld, const int32_t* colpos, LzScalars* S, long long* part,
-                     cudaStream_t s);
+// Largest exponent of a caller's FP64 vector f1 (dim elements): |f1| < 2^E; ED_ERR_ARG for a zero or
+// non-finite one. part: >= 4 * 4 * sm_count longs. Synchronises s.
+ed_status fx_exponent(const ed_basis* b, const double* f1, long long* part, cudaStream_t s, int* E);
+// The run's initial scalars (scale[0], fx_max[0]) from the n records of sum X^2 and max |X|.
+ed_status fx_init(LzScalars* S, const long long* part, int n, cudaStream_t s);
 // One step of Algorithm 1 on the fixed-point buffers (cur holds f_j, the other f_{j-1}).
 // Needs the step's integer coefficients: fx_plan before the first step of a call, afterwards
 // each step leaves the next one's (same t, U).
@@ -242,14 +238,13 @@ ed_status fx_prepare(const ed_basis* b);
 // Ground-state vector (ed_lanczos_ground_state) in fixed point, P = psi 2^60 (rank order), from
 // the coefficients y (1-based) of f_1 .. f_m:
 //   fx_psi_sum    P = sum_j round(y_j s_j 2^60 X_j) over stored vectors, with the records of
-//                 max |P| and ||P||^2 (part: >= 6 * 4 * sm_count longs; rank: b->dn.dim
-//                 padded to ld ints of scratch);
+//                 max |P| and ||P||^2 (part: >= 6 * 4 * sm_count longs; rank: down rank by
+//                 column, -1 for pads);
 //   fx_psi_accum  one term of the same sum, from the running vector of step j;
 //   fx_psi_finish the records for a P summed by fx_psi_accum (have_records: already there),
 //                 then P normalised and sign-gauged in place as FP64.
 ed_status fx_psi_sum(const ed_basis* b, const double* y, int m, const LzStore& store, int64_t ld,
-                     const int32_t* colpos, int32_t* rank, long long* P, long long* part,
-                     cudaStream_t s);
+                     const int32_t* rank, long long* P, long long* part, cudaStream_t s);
 ed_status fx_psi_accum(const ed_basis* b, const LzScalars* S, int cur, const double* y, int j,
                        const long long* X, int64_t ld, const int32_t* colpos, long long* P,
                        cudaStream_t s);

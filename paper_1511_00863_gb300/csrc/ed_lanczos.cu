@@ -23,77 +23,177 @@
 #include <type_traits>
 #include <vector>
 
+#include "ed_fixed.cuh"
 #include "ed_internal.cuh"
 #include "ed_lanczos_dev.cuh"
 
 namespace ed {
 
-
 // ------------------------------------------------------------------ start vector
-// SplitMix64 (Steele, Lea & Flood 2014): the (i+1)-th output of the generator seeded with
-// `seed`; element i of the start vector is 2 * (top 53 bits * 2^-53) - 1.
-__device__ __forceinline__ double start_element(uint64_t seed, uint64_t i) {
-  uint64_t z = seed + (i + 1ull) * 0x9E3779B97F4A7C15ull;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  z = z ^ (z >> 31);
-  return 2.0 * ((double)(z >> 11) * 0x1.0p-53) - 1.0;
-}
+// Element i of the start vector is h_i 2^-52 / ||.||, h_i = (top 53 bits of the (i+1)-th
+// SplitMix64 output) - 2^52 (split_mix, ed_fixed.cuh). Everything per element is integer
+// arithmetic: GB300's FP64 rate made the conversion, the product and the rounding of an element
+// 15-17 ps and its share of the norm 7 ps (2.8 ms of a 166 M element FP32 start).
 
-// Partial sums of x_i^2 over the raw start vector.
+// Partial sums of x_i^2 = h_i^2 2^-104 over the raw start vector, exact per CTA.
 __global__ void __launch_bounds__(kRedThreads)
 start_norm_kernel(uint64_t seed, int64_t n, double* __restrict__ partial) {
-  __shared__ double red[33];
-  double v = 0.0;
+  __shared__ long long tot[4];
+  A192 acc;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const double e = start_element(seed, (uint64_t)i);
-    v = fma(e, e, v);
+    const long long h = start_int(seed, (uint64_t)i);
+    a192_add_sq(acc, (unsigned long long)(h < 0 ? -h : h));
   }
-  v = block_sum(v, red);
-  if (threadIdx.x == 0) partial[blockIdx.x] = v;
+  fx_block_reduce(a192_get(acc), 0, tot);
+  if (threadIdx.x == 0) {
+    I192 v;
+    v.lo = ((u128)(unsigned long long)tot[1] << 64) | (u128)(unsigned long long)tot[0];
+    v.hi = tot[2];
+    partial[blockIdx.x] = scale2(i192_to_double(v), -104);
+  }
 }
 
-// Scalar i of the vector (row r = i / cols, column c = i % cols) goes to out[r ld + p] with
-// p = cx colpos[c / cx] + c % cx (cx = 2 for the (re, im) scalars of a complex element) or
-// p = c when colpos is NULL.
-__device__ __forceinline__ int64_t col_of(const int32_t* colpos, int64_t c, int cx) {
-  if (!colpos) return c;
-  const int64_t e = c / cx;
-  return cx * (int64_t)colpos[e] + (c - e * cx);
+// RN(h 2^-52 inv) in FP64, then to T (both to nearest even): the product of the 52-bit h and
+// inv's mantissa M 2^-63 (top bit set; inv = M 2^(e_inv - 63)) in integers.
+template <typename T>
+__device__ __forceinline__ T start_scaled(long long h, unsigned long long M, int e_inv) {
+  if (h == 0) return T(0);
+  const unsigned long long a = (unsigned long long)(h < 0 ? -h : h);
+  const int lz = __clzll(a);
+  const unsigned long long an = a << lz;
+  unsigned long long hi = __umul64hi(an, M), lo = an * M;
+  int e = e_inv - lz + 12;  // exponent of the product with hi's top bit set
+  if (!(hi >> 63)) {
+    hi = (hi << 1) | (lo >> 63);
+    lo <<= 1;
+    --e;
+  }
+  // 64 significant bits and a sticky remainder: to 53 bits
+  unsigned long long m = hi >> 11, rem = (hi & 0x7FF) | (lo ? 1ull : 0ull);
+  m += rem > 0x400 || (rem == 0x400 && (m & 1));
+  if (m >> 53) {
+    m >>= 1;
+    ++e;
+  }
+  if constexpr (sizeof(T) == 8) {
+    return __longlong_as_double((long long)((m & ((1ull << 52) - 1)) | ((unsigned long long)(e + 1023) << 52) |
+                                            (h < 0 ? 1ull << 63 : 0ull)));
+  } else {
+    const unsigned r = (unsigned)(m & ((1u << 29) - 1));
+    unsigned f = (unsigned)(m >> 29);
+    f += r > (1u << 28) || (r == (1u << 28) && (f & 1u));
+    // (a carry out of the 24 bits moves into the exponent field by itself)
+    return __uint_as_float(f - (1u << 23) + ((unsigned)(e + 127) << 23) + (h < 0 ? 1u << 31 : 0u));
+  }
 }
 
-// out[row, col_of(c)] = raw_i / ||raw|| rounded to T.
+// A vector in the library's layout: row r, scalar p of a row (cx = 2 scalars (re, im) per complex
+// element) at out[r lds + p]; the element at column e = p / cx is the one of down rank
+// rank[e] (-1: a pad, holds 0; rank NULL: rank e for e < cols). CTAs take runs of kRun scalars of
+// a row and write them in column order, pads included.
+constexpr int kRun = 2048;
+struct RowRuns {
+  int64_t rows, cols, lds, runs;  // cols in elements, lds in scalars, runs per row
+  const int32_t* __restrict__ rank;
+  int cx;
+};
+
+// f(i, o) for every scalar: i its index in the dense vector (-1: a pad), o its place.
+template <typename F>
+__device__ __forceinline__ void for_rows(const RowRuns& L, F f) {
+  for (int64_t it = blockIdx.x; it < L.rows * L.runs; it += gridDim.x) {
+    const int64_t r = it / L.runs, c0 = (it - r * L.runs) * kRun;
+    const int64_t c1 = c0 + kRun < L.lds ? c0 + kRun : L.lds;
+    for (int64_t p = c0 + threadIdx.x; p < c1; p += blockDim.x) {
+      const int64_t e = L.cx == 2 ? p >> 1 : p;
+      const int64_t d = L.rank ? (int64_t)L.rank[e] : (e < L.cols ? e : -1);
+      f(d < 0 ? -1 : L.cx * (r * L.cols + d) + (L.cx == 2 ? p & 1 : 0), r * L.lds + p);
+    }
+  }
+}
+
+// raw_i / ||raw|| rounded to T, in the layout L.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-start_write_kernel(uint64_t seed, int64_t n, int64_t cols, int64_t ld, const int32_t* __restrict__ colpos,
-                   int cx, const double* __restrict__ partial, int nparts, T* __restrict__ out) {
+start_write_kernel(uint64_t seed, RowRuns L, const double* __restrict__ partial, int nparts, T* __restrict__ out) {
   __shared__ double red[33];
   const double inv = 1.0 / sqrt(block_sum_array(partial, nparts, red));
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / cols, c = i - r * cols;
-    out[r * ld + col_of(colpos, c, cx)] = (T)(start_element(seed, (uint64_t)i) * inv);
-  }
+  const unsigned long long b = (unsigned long long)__double_as_longlong(inv);
+  const unsigned long long M = (b << 11) | (1ull << 63);  // inv is positive and normal
+  const int e_inv = (int)(b >> 52) - 1023;
+  for_rows(L, [&](int64_t i, int64_t o) {
+    out[o] = i < 0 ? T(0) : start_scaled<T>(start_int(seed, (uint64_t)i), M, e_inv);
+  });
 }
 
-// Copy a dense caller vector into the padded layout and accumulate its squared norm.
+// Copy a dense caller vector into the layout L and accumulate its squared norm.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-copy_in_kernel(const T* __restrict__ src, int64_t n, int64_t cols, int64_t ld,
-               const int32_t* __restrict__ colpos, int cx, T* __restrict__ dst,
-               double* __restrict__ partial) {
+copy_in_kernel(const T* __restrict__ src, RowRuns L, T* __restrict__ dst, double* __restrict__ partial) {
   __shared__ double red[33];
   DotAcc<T> acc;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / cols, c = i - r * cols;
-    const T v = src[i];
-    dst[r * ld + col_of(colpos, c, cx)] = v;
+  for_rows(L, [&](int64_t i, int64_t o) {
+    const T v = i < 0 ? T(0) : src[i];
+    dst[o] = v;
     acc.add(v, v);
-  }
+  });
   const double v = block_sum(acc.get(), red);
   if (threadIdx.x == 0) partial[blockIdx.x] = v;
+}
+
+// The same copies in fixed point (ed_fixed.cu): X_i = 2 h_i moved to the 2^vb range, and a
+// caller's FP64 vector X_i = f_i 2^(vb - E), |f| < 2^E, by integer manipulation of the IEEE fields
+// (round half up where bits fall off); records of sum X^2 (exact) and max |X|.
+__global__ void __launch_bounds__(kRedThreads)
+fx_start_kernel(uint64_t seed, RowRuns L, int vb, long long* __restrict__ X, long long* __restrict__ part) {
+  A192 acc;
+  long long mx = 0;
+  for_rows(L, [&](int64_t i, int64_t o) {
+    const long long v = i < 0 ? 0 : shift_signed(2 * start_int(seed, (uint64_t)i), vb - 53);
+    X[o] = v;
+    const long long av = v < 0 ? -v : v;
+    a192_add_sq(acc, (unsigned long long)av);
+    mx = max(mx, av);
+  });
+  fx_block_reduce(a192_get(acc), mx, part + 4 * blockIdx.x);
+}
+
+__global__ void __launch_bounds__(kRedThreads)
+fx_copy_in_kernel(const double* __restrict__ f, RowRuns L, int vb, int E, long long* __restrict__ X,
+                  long long* __restrict__ part) {
+  A192 acc;
+  long long mx = 0;
+  for_rows(L, [&](int64_t i, int64_t o) {
+    long long v = 0;
+    if (i >= 0) {
+      const unsigned long long bits = (unsigned long long)__double_as_longlong(f[i]);
+      const int ef = (int)((bits >> 52) & 0x7FF);
+      long long mant = (long long)(bits & 0xFFFFFFFFFFFFFull);
+      int e2 = -1074;
+      if (ef) {
+        mant |= 1LL << 52;
+        e2 = ef - 1075;
+      }
+      v = shift_signed(mant, e2 + vb - E);
+      if (bits >> 63) v = -v;
+    }
+    X[o] = v;
+    const long long av = v < 0 ? -v : v;
+    a192_add_sq(acc, (unsigned long long)av);
+    mx = max(mx, av);
+  });
+  fx_block_reduce(a192_get(acc), mx, part + 4 * blockIdx.x);
+}
+
+// rank[p] = the down rank at column p, -1 for a pad.
+__global__ void rank_kernel(const int32_t* __restrict__ colpos, int64_t cols, int64_t ld,
+                            int32_t* __restrict__ rank, int pads) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (pads ? ld : cols);
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (pads) rank[i] = -1;
+    else rank[colpos ? colpos[i] : i] = (int32_t)i;
+  }
 }
 
 __global__ void init_scalars_kernel(LzScalars* S, const double* __restrict__ partial,
@@ -254,6 +354,10 @@ __global__ void lz_ritz_kernel(const LzScalars* S, int m, double lam, double* y,
   tridiag_ritz_vector(S->alpha, S->beta, m, lam, y, work);
 }
 
+static RowRuns row_runs(int64_t rows, int64_t cols, int64_t ld, int cx, const int32_t* rank) {
+  return RowRuns{rows, cols, cx * ld, (cx * ld + kRun - 1) / kRun, rank, cx};
+}
+
 static int red_grid(int64_t n) {
   const int64_t want = (n + kRedThreads - 1) / kRedThreads;
   const int64_t cap = (int64_t)sm_count() * 4;
@@ -390,13 +494,12 @@ extern "C" ed_status ed_start_vector(int64_t dim, uint64_t seed, ed_dtype dtype,
   const int g = red_grid(dim);
   double* part = nullptr;
   ED_TRY_CUDA(cudaMallocAsync((void**)&part, g * sizeof(double), s));
+  const RowRuns dense = row_runs(1, dim, dim, 1, nullptr);
   start_norm_kernel<<<g, kRedThreads, 0, s>>>(seed, dim, part);
   if (dtype != ED_F32)
-    start_write_kernel<double><<<g, kRedThreads, 0, s>>>(seed, dim, dim, dim, nullptr, 1, part, g,
-                                                         (double*)out);
+    start_write_kernel<double><<<g, kRedThreads, 0, s>>>(seed, dense, part, g, (double*)out);
   else
-    start_write_kernel<float><<<g, kRedThreads, 0, s>>>(seed, dim, dim, dim, nullptr, 1, part, g,
-                                                        (float*)out);
+    start_write_kernel<float><<<g, kRedThreads, 0, s>>>(seed, dense, part, g, (float*)out);
   cudaError_t e = cudaGetLastError();
   cudaFreeAsync(part, s);
   if (e != cudaSuccess) {
@@ -453,13 +556,12 @@ extern "C" ed_status ed_start_vector_noalloc(int64_t dim, uint64_t seed, ed_dtyp
   const ed_status r = noalloc_scratch(&part);
   if (r != ED_OK) return r;
   cudaStream_t s = (cudaStream_t)stream;
+  const RowRuns dense = row_runs(1, dim, dim, 1, nullptr);
   start_norm_kernel<<<g, kRedThreads, 0, s>>>(seed, dim, part);
   if (dtype != ED_F32)
-    start_write_kernel<double><<<g, kRedThreads, 0, s>>>(seed, dim, dim, dim, nullptr, 1, part, g,
-                                                         (double*)out);
+    start_write_kernel<double><<<g, kRedThreads, 0, s>>>(seed, dense, part, g, (double*)out);
   else
-    start_write_kernel<float><<<g, kRedThreads, 0, s>>>(seed, dim, dim, dim, nullptr, 1, part, g,
-                                                        (float*)out);
+    start_write_kernel<float><<<g, kRedThreads, 0, s>>>(seed, dense, part, g, (float*)out);
   ED_TRY_CUDA(cudaGetLastError());
   return ED_OK;
 }
@@ -495,6 +597,22 @@ extern "C" void ed_lanczos_destroy(ed_lanczos* st) {
 // Bases below this many states use the default fused H.v variant order: timing every
 // variant would cost more than their solves.
 constexpr int64_t kAutotuneMinDim = (int64_t)1 << 22;
+
+// The state's table of ranks by column (built on first use).
+static ed_status lz_rank(ed_lanczos* st) {
+  if (st->rank) return ED_OK;
+  if (cudaMalloc((void**)&st->rank, (size_t)st->ld * sizeof(int32_t)) != cudaSuccess) {
+    cudaGetLastError();
+    st->rank = nullptr;
+    set_error("Lanczos column ranks: out of device memory");
+    return ED_ERR_OOM;
+  }
+  const int g = red_grid(st->ld);
+  rank_kernel<<<g, kRedThreads, 0, st->stream>>>(hv2_colpos(st->plan), st->basis->dn.dim, st->ld, st->rank, 1);
+  rank_kernel<<<g, kRedThreads, 0, st->stream>>>(hv2_colpos(st->plan), st->basis->dn.dim, st->ld, st->rank, 0);
+  ED_TRY_CUDA(cudaGetLastError());
+  return ED_OK;
+}
 
 static ed_status lz_alloc(const ed_basis* b, const ed_opts* o, cudaStream_t s, ed_lanczos** out) {
   *out = nullptr;
@@ -571,6 +689,16 @@ static ed_status lz_alloc(const ed_basis* b, const ed_opts* o, cudaStream_t s, e
     ed_status pr = hv2_build(b, mode, (int)st->ld, sched, s, &st->plan);
     if (pr != ED_OK) return fail(pr);
   }
+  // pads hold 0 from here on: every pass writes 0 there or leaves them
+  for (int i = 0; i < 2; ++i)
+    if (cudaMemsetAsync(st->B[i], 0, st->n * st->esize, s) != cudaSuccess) {
+      set_error("Lanczos work vectors: clearing failed");
+      return fail(ED_ERR_CUDA);
+    }
+  if (st->plan) {
+    const ed_status rr = lz_rank(st);
+    if (rr != ED_OK) return fail(rr);
+  }
   *out = st;
   return ED_OK;
 }
@@ -582,15 +710,16 @@ static int check_stride(int64_t n) {
   return n < ((int64_t)1 << 18) ? 8 : n < ((int64_t)1 << 20) ? 4 : n < ((int64_t)1 << 22) ? 2 : 1;
 }
 
-// Start a run on an allocated state: zero both buffers (their pads must hold 0), load f_1
-// (caller vector or seeded start vector) and the run's scalars.
+// Start a run on an allocated state: load f_1 (caller vector or seeded start vector) with its pads
+// and the run's scalars. The other buffer enters the first step with factor 0; it is cleared only
+// in floating point, where what an earlier run left there may not be finite.
 static ed_status lz_reset(ed_lanczos* st, const ed_opts* o, const void* f1) {
   const ed_basis* b = st->basis;
   cudaStream_t s = st->stream;
   ED_CHECK_ARG(f1 == nullptr || aligned16(f1), "f1 must be 16-byte aligned");
   st->opts = *o;
   st->stopped = false;
-  for (int i = 0; i < 2; ++i) ED_TRY_CUDA(cudaMemsetAsync(st->B[i], 0, st->n * st->esize, s));
+  if (!st->fx) ED_TRY_CUDA(cudaMemsetAsync(st->B[1], 0, st->n * st->esize, s));
   LzScalars h;
   memset(&h, 0, sizeof(h));
   h.max_steps = o->max_steps;
@@ -600,40 +729,41 @@ static ed_status lz_reset(ed_lanczos* st, const ed_opts* o, const void* f1) {
   h.scale[1] = 0.0;
   for (int i = 0; i < ED_MAX_STEPS + 2; ++i) h.E0[i] = NAN;
   ED_TRY_CUDA(cudaMemcpyAsync(st->S, &h, sizeof(h), cudaMemcpyHostToDevice, s));
-  // a complex vector is seen as scalars: dim (re, im) pairs = 2 dim scalars, rows of 2 cols
-  // scalars with stride 2 ld, so the real kernels below write the interleaved layout
+  // a complex vector is seen as scalars: dim (re, im) pairs = 2 dim scalars (for_rows)
   const int cx = is_complex(o->dtype) ? 2 : 1;
-  const int64_t dim = cx * b->dim, cols = cx * b->dn.dim, lds = cx * st->ld;
+  const int64_t dim = cx * b->dim;
   const bool dbl = o->dtype == ED_F64_NATIVE || o->dtype == ED_C64;
   const int g = red_grid(dim);
   ED_CHECK_ARG((int64_t)g <= st->npb, "internal: partial buffer too small");
   st->cur = 0;
-  const int32_t* colpos = hv2_colpos(st->plan);  // NULL: rank order (general kernels)
+  // rank order (general kernels) without a plan
+  const RowRuns L = row_runs(b->up.dim, b->dn.dim, st->ld, cx, st->plan ? st->rank : nullptr);
   if (st->fx) {
-    const ed_status r = f1 == nullptr
-        ? fx_start(b, st->fxr, o->seed, (long long*)st->B[0], st->ld, colpos, st->S,
-                   (long long*)st->pb, s)
-        : fx_copy_in(b, st->fxr, (const double*)f1, (long long*)st->B[0], st->ld, colpos, st->S,
-                     (long long*)st->pb, s);
+    long long* part = (long long*)st->pb;
+    if (f1 == nullptr) {
+      fx_start_kernel<<<g, kRedThreads, 0, s>>>(o->seed, L, st->fxr.vb, (long long*)st->B[0], part);
+    } else {
+      int E = 0;
+      const ed_status r = fx_exponent(b, (const double*)f1, part, s, &E);
+      if (r != ED_OK) return r;
+      fx_copy_in_kernel<<<g, kRedThreads, 0, s>>>((const double*)f1, L, st->fxr.vb, E, (long long*)st->B[0], part);
+    }
+    const ed_status r = fx_init(st->S, part, g, s);
     if (r != ED_OK || !st->ro) return r;
     return ro_reset(st->ro, st->S, st->B[0], s);
   }
   if (f1 == nullptr) {
     start_norm_kernel<<<g, kRedThreads, 0, s>>>(o->seed, dim, st->pb);
     if (dbl)
-      start_write_kernel<double><<<g, kRedThreads, 0, s>>>(o->seed, dim, cols, lds, colpos, cx,
-                                                           st->pb, g, (double*)st->B[0]);
+      start_write_kernel<double><<<g, kRedThreads, 0, s>>>(o->seed, L, st->pb, g, (double*)st->B[0]);
     else
-      start_write_kernel<float><<<g, kRedThreads, 0, s>>>(o->seed, dim, cols, lds, colpos, cx,
-                                                          st->pb, g, (float*)st->B[0]);
+      start_write_kernel<float><<<g, kRedThreads, 0, s>>>(o->seed, L, st->pb, g, (float*)st->B[0]);
     init_scalars_kernel<<<1, 32, 0, s>>>(st->S, st->pb, g, 0);
   } else {
     if (dbl)
-      copy_in_kernel<double><<<g, kRedThreads, 0, s>>>((const double*)f1, dim, cols, lds,
-                                                       colpos, cx, (double*)st->B[0], st->pb);
+      copy_in_kernel<double><<<g, kRedThreads, 0, s>>>((const double*)f1, L, (double*)st->B[0], st->pb);
     else
-      copy_in_kernel<float><<<g, kRedThreads, 0, s>>>((const float*)f1, dim, cols, lds,
-                                                      colpos, cx, (float*)st->B[0], st->pb);
+      copy_in_kernel<float><<<g, kRedThreads, 0, s>>>((const float*)f1, L, (float*)st->B[0], st->pb);
     init_scalars_kernel<<<1, kRedThreads, 0, s>>>(st->S, st->pb, g, 1);
   }
   const cudaError_t e = cudaGetLastError();
@@ -1109,17 +1239,17 @@ static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p
   if (!st->ywork) {
     if (cudaMalloc((void**)&st->slots, (ED_MAX_STEPS + 2) * sizeof(void*)) != cudaSuccess ||
         cudaMalloc((void**)&st->vscale, (ED_MAX_STEPS + 2) * sizeof(double)) != cudaSuccess ||
-        cudaMalloc((void**)&st->rank, (size_t)st->ld * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc((void**)&st->ywork, 3 * (ED_MAX_STEPS + 4) * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
-      for (void* q : {(void*)st->slots, (void*)st->vscale, (void*)st->rank})
+      for (void* q : {(void*)st->slots, (void*)st->vscale})
         if (q) cudaFree(q);
-      st->slots = nullptr, st->vscale = nullptr, st->rank = nullptr;
+      st->slots = nullptr, st->vscale = nullptr;
       set_error("ed_lanczos_ground_state: out of device memory");
       return ED_ERR_OOM;
     }
   }
-  ed_status r = lz_reset(st, o, f1);
+  ed_status r = lz_rank(st);
+  if (r == ED_OK) r = lz_reset(st, o, f1);
   if (r != ED_OK) return r;
   if ((r = fx_prepare(b)) != ED_OK) return r;
   int m = 0, status = 0;
@@ -1152,8 +1282,7 @@ static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p
     ED_TRY_CUDA(cudaGetLastError());
     summed = !own || kept.complete;
     if (summed &&
-        (r = fx_psi_sum(b, y, m, own ? st->store : ro_slots(st->ro), st->ld, hv2_colpos(st->plan),
-                        st->rank, P, (long long*)st->pb, s)) != ED_OK)
+        (r = fx_psi_sum(b, y, m, own ? st->store : ro_slots(st->ro), st->ld, st->rank, P, (long long*)st->pb, s)) != ED_OK)
       return r;
   }
   const double lam = st->host->E0[m];
