@@ -13,7 +13,9 @@
 //   phase 3: b_{j+1}, scale of f_{j+1}, every `check` steps E0(j) = lambda_min(T_j) by
 //            Sturm bisection (leader CTA), convergence / breakdown / max_steps.
 // The H.v phase stages blocks of up rows in shared memory (down-hop gathers there) and reads
-// up-neighbour rows coalesced; vectors of the batch stay in L2.
+// up-neighbour rows coalesced; vectors of the batch stay in L2. Instances with tables of the
+// row-ordered H.v (ed_rows.cu) take 32 columns of equal hop counts per warp, one table entry for
+// two rows, and read neighbour rows in 16-byte loads; the others go element by element.
 // ed_lanczos_solve_batched_mixed carries the FP32 batch to FP64 accuracy: the FP32 run keeps
 // its vectors, a Ritz vector is assembled per instance and FP64 steps refine it
 // (batched_ritz_kernel and the `refine` form of the FP64 kernel, below).
@@ -40,6 +42,7 @@ constexpr int bctas_per_sm() { return sizeof(T) == 4 ? kBCtasPerSm : 4; }
 // Staging area of the H.v phase (a block of up rows, at most kBRowFloats * 4 bytes); the same
 // shared buffer holds the leader CTA's bisection workspace at another time.
 constexpr int kBRowFloats = 4096;
+constexpr int kBLists = 128;  // up-hop list entries in it (row-ordered H.v)
 // Dynamic shared memory of the batched kernels: the row-block staging area, or the bisection
 // workspace of T_m for m <= max_steps, whichever is larger (sized per run, so short runs keep
 // the L1 data cache that the hop tables are read through).
@@ -54,6 +57,12 @@ struct BInst {
   const int32_t* hu;
   const int32_t* hd;
   int dim_up, dim_dn, mhu, mhd;
+  int ld;  // row stride of the vectors: dim_dn, or rounded up to 4 where the tables below serve
+  // tables of the row-ordered H.v (ed_rows.cu: columns by hop count, one class), or tab NULL
+  const int32_t* perm;
+  const int32_t* base;
+  const uint8_t* kc;
+  const uint16_t* tab;
   void* B0;  // two work vectors of the instance (FP32 or FP64 elements)
   void* B1;
   double t, U;
@@ -213,6 +222,126 @@ __device__ bool group_barrier(unsigned* count, unsigned* gen, int g, long long m
 template <typename T>
 __device__ __forceinline__ T ld_shared_f(const T* p, bool multi) { return multi ? __ldcg(p) : *p; }
 
+// ---- H.v of a block of up rows through the row-ordered tables
+template <typename T> struct BWide;
+template <> struct BWide<float> { typedef float4 V; static constexpr int kRows = 2; };
+template <> struct BWide<double> { typedef double2 V; static constexpr int kRows = 1; };
+template <typename T, int N>
+struct alignas(sizeof(T) * N) BPack {
+  T v[N];
+};
+template <typename T>
+__device__ __forceinline__ T b_sign(T x, uint32_t s) {  // s: 0 or the sign bit in bit 31
+  if constexpr (sizeof(T) == 4) return __uint_as_float(__float_as_uint(x) ^ s);
+  else return __hiloint2double(__double2hiint(x) ^ (int)s, __double2loint(x));
+}
+// 16-byte load; from L2 when other CTAs of the group wrote the data
+template <typename V>
+__device__ __forceinline__ V b_ld16(const V* p, bool multi) { return multi ? __ldcg(p) : *p; }
+
+// Row packs (kRows rows each) per block of a CTA: what the staging area holds, but no more than
+// leaves every CTA of the group four blocks.
+template <typename T>
+__device__ __forceinline__ int b_packs(const BInst& I, int g) {
+  constexpr int R = BWide<T>::kRows;
+  const int fit = (kBRowFloats * 4 - 4 * kBLists) / ((2 * I.ld + 1) * R * (int)sizeof(T));
+  const int share = I.dim_up / (4 * R * g);
+  return max(1, min(min(fit, share), min(kBLists / max(1, R * I.mhu), 2048 / (R * I.ld))));
+}
+
+template <typename T>
+__device__ __forceinline__ void hv_block(const BInst& I, const T* xc, T* xp, float* vj, int u0, int packs,
+                                         bool multi, T sc, T bsp, DotAcc<T>& dot, unsigned char* bsm) {
+  constexpr int R = BWide<T>::kRows, W = 16 / (int)sizeof(T);
+  typedef typename BWide<T>::V V;
+  const int dn = I.dim_dn, ld = I.ld, MH = I.mhu;
+  BPack<T, R>* xs = reinterpret_cast<BPack<T, R>*>(bsm);               // [packs][ld + 1]
+  T* ys = reinterpret_cast<T*>(xs + packs * (ld + 1));                 // [packs * R][ld]
+  uint32_t* ue = reinterpret_cast<uint32_t*>(ys + (packs * R) * ld);   // [packs * R][MH]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const T tt = (T)I.t, UU = (T)I.U;
+  __syncthreads();
+  for (int b = 0; b < packs; ++b)
+    for (int d = threadIdx.x; d <= ld; d += blockDim.x) {
+      BPack<T, R> p;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int u = u0 + b * R + r;
+        p.v[r] = d < ld && u < I.dim_up ? ld_shared_f(xc + (int64_t)u * ld + d, multi) : T(0);
+      }
+      xs[b * (ld + 1) + d] = p;
+    }
+  for (int i = threadIdx.x; i < packs * R * MH; i += blockDim.x) {
+    const int r = i / MH, k = i - r * MH;
+    ue[i] = u0 + r < I.dim_up ? (uint32_t)I.hu[(int64_t)k * I.dim_up + u0 + r] : (uint32_t)I.dim_up;
+  }
+  __syncthreads();
+  // ---- down part: 32 columns of (nearly) equal hop counts per warp and pack
+  const int nch = (dn + 31) >> 5;
+  for (int task = warp; task < nch * packs; task += kBThreads / 32) {
+    const int b = task / nch, ch = task - b * nch;
+    const int p = I.perm[32 * ch + lane], n = I.kc[ch];
+    const uint16_t* tp = I.tab + I.base[ch] + lane;
+    const BPack<T, R>* xb = xs + b * (ld + 1);
+    T acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = T(0);
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+      const uint32_t e = tp[32 * k];  // target (dim_dn: a zero column) | sign << 15
+      const BPack<T, R> q = xb[e & 0x7FFFu];
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r] += b_sign(q.v[r], (e & 0x8000u) << 16);
+    }
+    if (p >= 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) ys[(b * R + r) * ld + p] = acc[r];
+    }
+  }
+  __syncthreads();
+  // ---- up part, diagonal and the Lanczos update: 16 bytes of a row per thread (pads hold 0)
+  const int per_row = ld / W;
+  for (int q = threadIdx.x; q < packs * R * per_row; q += blockDim.x) {
+    const int r = q / per_row, d0 = (q - r * per_row) * W, u = u0 + r;
+    if (u >= I.dim_up) break;
+    const uint32_t* ul = ue + r * MH;
+    T acc[W];
+#pragma unroll
+    for (int v = 0; v < W; ++v) acc[v] = d0 + v < dn ? ys[r * ld + d0 + v] : T(0);
+    const T* xd = xc + d0;
+#pragma unroll 2
+    for (int k = 0; k < MH; ++k) {
+      const uint32_t e = ul[k];
+      const int tg = (int)(e & kTargetMask);
+      if (tg >= I.dim_up) break;
+      const V x4 = b_ld16(reinterpret_cast<const V*>(xd + (int64_t)tg * ld), multi);
+      const T* xv = reinterpret_cast<const T*>(&x4);
+#pragma unroll
+      for (int v = 0; v < W; ++v) acc[v] += b_sign(xv[v], e & kSignBit);
+    }
+    const int64_t e0 = (int64_t)u * ld + d0;
+    const V P4 = b_ld16(reinterpret_cast<const V*>(xp + e0), multi);
+    const T* P = reinterpret_cast<const T*>(&P4);
+    const uint32_t ub = I.upb[u];
+    V w4, x4;
+    T* w = reinterpret_cast<T*>(&w4);
+    T* xo = reinterpret_cast<T*>(&x4);
+#pragma unroll
+    for (int v = 0; v < W; ++v) {
+      const T xv = xs[(r / R) * (ld + 1) + d0 + v].v[r % R];
+      const uint32_t db = d0 + v < dn ? I.dnb[d0 + v] : 0u;
+      const T hx = fma(-tt, acc[v], UU * (T)__popc(ub & db) * xv);
+      w[v] = fma(sc, hx, -bsp * P[v]);
+      xo[v] = xv;
+      dot.add(w[v], sc * xv);
+    }
+    *reinterpret_cast<V*>(xp + e0) = w4;
+    if constexpr (sizeof(T) == 4) {
+      if (vj) __stcs(reinterpret_cast<V*>(vj + e0), x4);
+    }
+  }
+}
+
 __device__ __forceinline__ double bstart_element(uint64_t seed, uint64_t i) {
   uint64_t z = seed + (i + 1ull) * 0x9E3779B97F4A7C15ull;
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -249,15 +378,21 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
   double* al = R.al;
   double* be = R.be;
   double* e0 = R.e0;
-  const int dim = I.dim_up * I.dim_dn;
+  const int dim = I.dim_up * I.ld;  // elements of a vector, pads included
   const int64_t gt = (int64_t)g * blockDim.x;
   const int64_t t0 = (int64_t)c * blockDim.x + threadIdx.x;
+  // element e of the seeded start vector (0 in a pad)
+  auto start = [&](int64_t e) {
+    if (I.ld == I.dim_dn) return bstart_element(a.seed, (uint64_t)e);
+    const int r = (int)e / I.ld, d = (int)e - r * I.ld;
+    return d < I.dim_dn ? bstart_element(a.seed, (uint64_t)((int64_t)r * I.dim_dn + d)) : 0.0;
+  };
   // ---- start vector: raw values (SplitMix64 or the given FP64 vector), FP64 norm,
   // normalised then rounded
   {
     double v = 0.0;
     for (int64_t e = t0; e < dim; e += gt) {
-      const double x = R.f1 ? ld_shared_f(R.f1 + e, multi) : bstart_element(a.seed, (uint64_t)e);
+      const double x = R.f1 ? ld_shared_f(R.f1 + e, multi) : start(e);
       v = fma(x, x, v);
     }
     v = block_sum(v, red);
@@ -265,7 +400,7 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
     if (!group_barrier(bc, bg, g, a.max_spin, a.error)) return false;
     const double inv = 1.0 / sqrt(group_sum(a.part_a, first_cta, g, red));
     for (int64_t e = t0; e < dim; e += gt) {
-      const double x = R.f1 ? ld_shared_f(R.f1 + e, multi) : bstart_element(a.seed, (uint64_t)e);
+      const double x = R.f1 ? ld_shared_f(R.f1 + e, multi) : start(e);
       ((T*)R.B0)[e] = (T)(x * inv);
       ((T*)R.B1)[e] = T(0);
     }
@@ -292,7 +427,11 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
     const T bsp = (T)(__ldcg(&be[j]) * __ldcg(&S->scale[1 - cur]));
     const T tt = (T)I.t, UU = (T)I.U;
     DotAcc<T> dot;
-    if (I.dim_dn <= kRowElems) {
+    if (I.tab) {
+      const int packs = b_packs<T>(I, g), rows = packs * BWide<T>::kRows;
+      for (int u0 = c * rows; u0 < I.dim_up; u0 += g * rows)
+        hv_block<T>(I, xc, xp, vj, u0, packs, multi, sc, bsp, dot, bsm);
+    } else if (I.dim_dn <= kRowElems) {
       // blocks of BR consecutive up rows staged in shared memory (coalesced loads; from L2
       // when other CTAs of the group wrote them): down-hop gathers read shared memory,
       // up-hop gathers read whole neighbour rows coalesced
@@ -368,10 +507,27 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
     const T coef = (T)(alpha * __ldcg(&S->scale[cur]));
     DotAcc<T> q2;
     // (phase 1 wrote w by row blocks: other CTAs' values are read from L2)
-    for (int64_t e = t0; e < dim; e += gt) {
-      const T q = ld_shared_f(xp + e, multi) - coef * ld_shared_f(xc + e, multi);
-      xp[e] = q;
-      q2.add(q, q);
+    if (I.tab) {  // (rows of a multiple of 16 bytes)
+      typedef typename BWide<T>::V V;
+      constexpr int W = 16 / (int)sizeof(T);
+      for (int64_t e = t0; e < dim / W; e += gt) {
+        V w4 = b_ld16(reinterpret_cast<const V*>(xp) + e, multi);
+        const V c4 = b_ld16(reinterpret_cast<const V*>(xc) + e, multi);
+        T* w = reinterpret_cast<T*>(&w4);
+        const T* x = reinterpret_cast<const T*>(&c4);
+#pragma unroll
+        for (int v = 0; v < W; ++v) {
+          w[v] = w[v] - coef * x[v];
+          q2.add(w[v], w[v]);
+        }
+        reinterpret_cast<V*>(xp)[e] = w4;
+      }
+    } else {
+      for (int64_t e = t0; e < dim; e += gt) {
+        const T q = ld_shared_f(xp + e, multi) - coef * ld_shared_f(xc + e, multi);
+        xp[e] = q;
+        q2.add(q, q);
+      }
     }
     {
       const double v = block_sum(q2.get(), red);
@@ -503,7 +659,7 @@ batched_ritz_kernel(BArgs a) {
     for (int j = 1 + threadIdx.x; j <= m; j += blockDim.x)
       coef[j] = (float)(__ldcg(&y[j]) * __ldcg(&rw[j]));
     __syncthreads();
-    const int dim = I.dim_up * I.dim_dn;
+    const int dim = I.dim_up * I.ld;
     for (int64_t e = (int64_t)c * blockDim.x + threadIdx.x; e < dim; e += (int64_t)g * blockDim.x) {
       float p = 0.f;
       for (int j = 1; j <= m; ++j) p = fmaf(coef[j], ld_shared_f(I.V + (size_t)(j - 1) * I.dpad + e, multi), p);
@@ -659,6 +815,17 @@ cudaMemPool_t vstore_pool() {
   pools[dev] = pool;
   return pool;
 }
+
+// Layout of an instance's vectors: the row-ordered H.v where the basis has its tables (one hop
+// class) and a block of rows and its up-hop lists fit the staging area, with rows padded to 4
+// elements; else dense rows. Rows shorter than 96 columns leave most warps of the down part idle.
+bool blayout_rows(const ed_basis* b) {
+  const int64_t ld = (b->dn.dim + 3) / 4 * 4;
+  return b->rows.C == 1 && b->rows.ucnt == nullptr && b->dn.dim >= 96 && b->up.maxhops * 2 <= kBLists &&
+         (2 * ld + 1) * 8 + 4 * kBLists <= kBRowFloats * 4;
+}
+int blayout_ld(const ed_basis* b) { return blayout_rows(b) ? (int)((b->dn.dim + 3) / 4 * 4) : (int)b->dn.dim; }
+size_t blayout_elems(const ed_basis* b) { return ((size_t)b->up.dim * blayout_ld(b) + 3) / 4 * 4; }
 
 struct BatchRun {
   int n = 0;
@@ -920,7 +1087,8 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
     ED_CHECK_ARG(b->dim < (1LL << 31), "%s: instance %d too large", fn, i);
     R.dims[i] = (int)b->dim;
     R.work[i] = (long long)b->dim * (b->up.maxhops + b->dn.maxhops + 4);
-    total += (size_t)((b->dim + 3) / 4 * 4);
+    ED_CHECK_ARG(b->up.dim * (int64_t)blayout_ld(b) < (1LL << 31), "%s: instance %d too large", fn, i);
+    total += blayout_elems(b);
   }
   const size_t esize = o->dtype == ED_F64_NATIVE ? 8 : 4;
   const size_t stride = (size_t)o->max_steps + 2;
@@ -961,7 +1129,13 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
     I.dim_dn = (int)b->dn.dim;
     I.mhu = b->up.maxhops;
     I.mhd = b->dn.maxhops;
-    const size_t dpad = (size_t)(b->dim + 3) / 4 * 4;
+    const bool rows = blayout_rows(b);
+    I.ld = blayout_ld(b);
+    I.perm = b->rows.perm;
+    I.base = b->rows.base;
+    I.kc = b->rows.kc;
+    I.tab = rows ? b->rows.tab : nullptr;
+    const size_t dpad = blayout_elems(b);
     I.dpad = (int)dpad;
     // the two work vectors of an instance side by side (per instance: B0, B1; D0, D1)
     I.B0 = (char*)R.vec + 2 * off * esize;
