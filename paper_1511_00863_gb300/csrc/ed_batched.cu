@@ -51,6 +51,9 @@ static size_t bsmem_bytes(int max_steps) {
   return sturm > (size_t)kBRowFloats * 4 ? sturm : (size_t)kBRowFloats * 4;
 }
 
+// ... of batched_ritz_kernel: a, b, y and the two arrays of the inverse iteration.
+static size_t ritz_bytes(int max_steps) { return 5 * (size_t)(max_steps + 2) * sizeof(double); }
+
 struct BInst {
   const uint32_t* upb;
   const uint32_t* dnb;
@@ -79,7 +82,7 @@ struct BState {
   int j, status;
   double scale[2];
   double tscale;
-  double last_E0;
+  double last_E0, last_lo;  // bracket of E0(last_E0_step), the last tested step's
   int last_E0_step;
   int pad_;
 };
@@ -362,6 +365,56 @@ __device__ __forceinline__ double group_sum(const double* part, int first, int g
   return v;
 }
 
+// sturm_lowest out of line: inlined three times it cost the kernel's loops 700 bytes of spills.
+__device__ __noinline__ double group_sturm(const double* al, const double* be, int m, double hint, double* work,
+                                           int cap, double* rough_lo) {
+  return sturm_lowest(al, be, m, hint, work, cap, rough_lo);
+}
+
+// The stop test of step j (whole leader CTA; st: 1 after a breakdown): the new status. It compares
+// E0(j) with the last tested step's, but away from convergence a rough bracket of each decides it
+// for a quarter of the time (two float-float rounds instead of those and the FP64 ones): while the
+// brackets lie further apart than tol, the test fails whatever the exact values are. Otherwise, and
+// at the last step, both are computed exactly.
+__device__ __noinline__ int group_stop_test(BState* S, const RunSpec& R, const double* al, const double* be, double* e0, int j,
+                               int st, double* work) {
+  const int cap = R.max_steps + 2;
+  const bool last = st != 0 || j >= R.max_steps;
+  const int prev = S->last_E0_step;
+  const double plo = S->last_lo, phi = S->last_E0;  // [plo, phi] holds E0(prev); plo == phi: exact
+  __syncthreads();
+  double E, lo;
+  if (prev > 0 && !last) {
+    E = group_sturm(al, be, j, phi, work, cap, &lo);
+    const double mag = fmax(fmax(fabs(lo), fabs(E)), 1.0);
+    if (plo - E > 1.001 * R.tol * mag) {
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        S->last_lo = lo;
+        S->last_E0 = E;
+        S->last_E0_step = j;
+      }
+      return 0;
+    }
+    __syncthreads();
+  }
+  double P = phi;
+  if (prev > 0 && st == 0 && R.tol > 0.0 && plo != phi) {
+    P = group_sturm(al, be, prev, phi, work, cap, nullptr);
+    __syncthreads();
+  }
+  E = group_sturm(al, be, j, prev > 0 ? P : NAN, work, cap, nullptr);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    e0[j] = E;
+    S->last_lo = E;
+    S->last_E0 = E;
+    S->last_E0_step = j;
+  }
+  if (st == 0 && R.tol > 0.0 && prev > 0 && fabs(E - P) <= R.tol * fmax(fabs(E), 1.0)) return 2;
+  return st == 0 && j >= R.max_steps ? 3 : st;
+}
+
 // T = float (ED_F32) or double (ED_F64_NATIVE): vector elements and H.v arithmetic; the
 // scalars are FP64 either way.
 // Algorithm 1 for instance I on its group (CTA c of g, leader = c == 0), FP32 or FP64
@@ -411,20 +464,29 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
       S->scale[1] = 0.0;
       S->tscale = 0.0;
       S->last_E0_step = 0;
-      S->last_E0 = 0.0;
+      S->last_E0 = S->last_lo = 0.0;
       be[1] = 0.0;
     }
     if (!group_barrier(bc, bg, g, a.max_spin, a.error)) return false;
   }
+  // the scalars of the running step, one copy per CTA (all CTAs compute the same)
+  __shared__ struct {
+    double scale, scale_prev, beta, tscale;  // of f_j and f_{j-1}; b_j
+  } run_s;
+  if (threadIdx.x == 0) {
+    run_s.scale = 1.0;
+    run_s.scale_prev = run_s.beta = run_s.tscale = 0.0;
+  }
+  __syncthreads();
   int cur = 0;
   for (int j = 1; j <= R.max_steps; ++j) {
     T* xc = (T*)(cur ? R.B1 : R.B0);
     T* xp = (T*)(cur ? R.B0 : R.B1);
     float* vj = R.V ? R.V + (size_t)(j - 1) * R.dpad : nullptr;
-    if (vj && leader && threadIdx.x == 0) R.vscale[j] = __ldcg(&S->scale[cur]);
+    if (vj && leader && threadIdx.x == 0) R.vscale[j] = run_s.scale;
     // ---- phase 1: fused H.v
-    const T sc = (T)__ldcg(&S->scale[cur]);
-    const T bsp = (T)(__ldcg(&be[j]) * __ldcg(&S->scale[1 - cur]));
+    const T sc = (T)run_s.scale;
+    const T bsp = (T)(run_s.beta * run_s.scale_prev);
     const T tt = (T)I.t, UU = (T)I.U;
     DotAcc<T> dot;
     if (I.tab) {
@@ -504,7 +566,7 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
     // ---- phase 2: a_j, update
     const double alpha = group_sum(a.part_a, first_cta, g, red);
     if (leader && threadIdx.x == 0) al[j] = alpha;
-    const T coef = (T)(alpha * __ldcg(&S->scale[cur]));
+    const T coef = (T)(alpha * run_s.scale);
     DotAcc<T> q2;
     // (phase 1 wrote w by row blocks: other CTAs' values are read from L2)
     if (I.tab) {  // (rows of a multiple of 16 bytes)
@@ -534,41 +596,37 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
       if (threadIdx.x == 0) a.part_b[blockIdx.x] = v;
     }
     if (!group_barrier(bc, bg, g, a.max_spin, a.error)) return false;
-    // ---- phase 3: b_{j+1}, E0(j), stop test (leader), then everyone reads the status
+    // ---- phase 3: b_{j+1} (every CTA, from the same partials); the stop test when due: E0(j) by
+    // the leader, then everyone reads the status
     const double b2 = group_sum(a.part_b, first_cta, g, red);
-    if (leader) {
-      if (threadIdx.x == 0) {
-        const double beta = sqrt(b2);
-        const double ts = fmax(S->tscale, fabs(alpha) + be[j]);
-        S->tscale = ts;
+    if (threadIdx.x == 0) {
+      const double beta = sqrt(b2);
+      const double ts = fmax(run_s.tscale, fabs(alpha) + run_s.beta);
+      const int st = (beta > kBreakdownRel * fmax(1.0, ts)) ? 0 : 1;
+      run_s.tscale = ts;
+      run_s.beta = beta;
+      run_s.scale_prev = run_s.scale;
+      run_s.scale = st == 0 ? 1.0 / beta : 0.0;
+      if (leader) {
         be[j + 1] = beta;
         S->j = j;
-        int st = (beta > kBreakdownRel * fmax(1.0, ts)) ? 0 : 1;
-        if (st == 0) S->scale[1 - cur] = 1.0 / beta;
-        *stop_s = st;
+        if (st == 0) S->scale[1 - cur] = run_s.scale;
       }
-      __syncthreads();
-      int st = *stop_s;
-      if (st != 0 || j >= R.max_steps || (j % R.check) == 0) {
-        const double E = sturm_lowest(al, be, j, S->last_E0_step > 0 ? S->last_E0 : NAN,
-                                      reinterpret_cast<double*>(bsm), R.max_steps + 2);
+      *stop_s = st;
+    }
+    __syncthreads();
+    int st = *stop_s;
+    if (st != 0 || j >= R.max_steps || (R.tol > 0.0 && j % R.check == 0)) {
+      if (leader) {
+        st = group_stop_test(S, R, al, be, e0, j, st, reinterpret_cast<double*>(bsm));
         if (threadIdx.x == 0) {
-          e0[j] = E;
-          if (st == 0 && R.tol > 0.0 && S->last_E0_step > 0 &&
-              fabs(E - S->last_E0) <= R.tol * fmax(fabs(E), 1.0))
-            st = 2;
-          S->last_E0 = E;
-          S->last_E0_step = j;
+          S->status = st;
+          __threadfence();
         }
       }
-      if (threadIdx.x == 0) {
-        if (st == 0 && j >= R.max_steps) st = 3;
-        S->status = st;
-        __threadfence();
-      }
+      if (!group_barrier(bc, bg, g, a.max_spin, a.error)) return false;
+      if (__ldcg(&S->status) != 0) break;
     }
-    if (!group_barrier(bc, bg, g, a.max_spin, a.error)) return false;
-    if (__ldcg(&S->status) != 0) break;
     cur = 1 - cur;
   }
   return true;
@@ -633,6 +691,7 @@ batched_lanczos_kernel(BArgs a) {
 __global__ void __launch_bounds__(kBThreads, kBCtasPerSm)
 batched_ritz_kernel(BArgs a) {
   __shared__ __align__(16) float coef[ED_MAX_STEPS + 2];  // y_j times the stored vector's scale
+  extern __shared__ __align__(16) unsigned char bsm[];    // the leader's T_m, y and work
   const int gi = a.group_of_cta[blockIdx.x];
   const BGroup G = a.groups[gi];
   const int c = blockIdx.x - G.first_cta, g = G.ncta;
@@ -648,8 +707,14 @@ batched_ritz_kernel(BArgs a) {
     const double* be = a.beta + (size_t)id * stride;
     const int m = __ldcg(&a.st[id].j);
     double* y = rw + stride;
-    if (c == 0 && threadIdx.x == 0) {
-      if (m >= 1) tridiag_ritz_vector(al, be, m, __ldcg(&a.E0[(size_t)id * stride + m]), y, rw + 2 * stride);
+    if (c == 0) {  // in shared memory: one thread's chain of dependent operations
+      double *as = reinterpret_cast<double*>(bsm), *bs = as + stride, *ys = bs + stride, *work = ys + stride;
+      for (int i = threadIdx.x; i < m + 2 && m >= 1; i += blockDim.x) as[i] = al[i], bs[i] = be[i];
+      __syncthreads();
+      if (threadIdx.x == 0 && m >= 1)
+        tridiag_ritz_vector(as, bs, m, __ldcg(&a.E0[(size_t)id * stride + m]), ys, work);
+      __syncthreads();
+      for (int i = threadIdx.x; i < m + 2 && m >= 1; i += blockDim.x) y[i] = ys[i];
       __threadfence();
     }
     if (!group_barrier(bc, bg, g, a.max_spin, a.error)) return;
@@ -956,7 +1021,8 @@ ed_status run_plan(BatchRun& R, const Plan& p, const Plan* p2, const ed_opts* o,
   const size_t dsm = bsmem_bytes(o->max_steps), dsm2 = bsmem_bytes(R.refine_steps);
   cudaError_t le = cudaLaunchCooperativeKernel(kernel, p.grid, kBThreads, args, dsm, s);
   if (le == cudaSuccess && R.mixed)
-    le = cudaLaunchCooperativeKernel((const void*)batched_ritz_kernel, p2->grid, kBThreads, argsr, 0, s);
+    le = cudaLaunchCooperativeKernel((const void*)batched_ritz_kernel, p2->grid, kBThreads, argsr,
+                                     ritz_bytes(o->max_steps), s);
   if (le == cudaSuccess && R.mixed)
     le = cudaLaunchCooperativeKernel((const void*)batched_lanczos_kernel<double>, p2->grid, kBThreads,
                                      args2, dsm2, s);
@@ -1164,7 +1230,8 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
                                                               kBThreads, bsmem_bytes(o->max_steps)));
   if (mixed) {  // the Ritz and refinement launches share a plan
     int pm = 0, pd = 0;
-    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pm, batched_ritz_kernel, kBThreads, 0));
+    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pm, batched_ritz_kernel, kBThreads,
+                                                              ritz_bytes(o->max_steps)));
     ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pd, batched_lanczos_kernel<double>,
                                                               kBThreads, bsmem_bytes(refine_steps)));
     per_sm2 = std::min(pm, pd);

@@ -166,9 +166,15 @@ constexpr int kSturmWork = sturm_work_doubles(kSturmCap);
 // FP64, so the result has the precision of an all-FP64 multisection at about half its FP64
 // work. With a hint (a previous lambda_min of a leading block of T_m, an upper bound by
 // Cauchy interlacing; NaN = none), a first round probes geometrically spaced points below
-// it, so a bracket of the size of the last change is found in one round.
+// it, so a bracket of the size of the last change is found in one round. With rough_lo the search
+// ends after the probe and one more float-float round (about a quarter of the time): it returns
+// the upper and *rough_lo the lower end of a bracket that holds lambda_min, about 1/1000 as wide as
+// the distance to the hint. (One FP64 division, logarithm or power of the few scalars of a round
+// costs as much as ten rows of a count, so they are multiplications and FP32 functions: the points
+// need not be exact, only the same wherever they are formed.)
 __device__ __forceinline__ double sturm_lowest(const double* a, const double* b, int m,
-                                               double hint, double* work, int cap = kSturmCap) {
+                                               double hint, double* work, int cap = kSturmCap,
+                                               double* rough_lo = nullptr) {
   constexpr int P = 128;
   double* aa = work;
   double* bb = work + cap;
@@ -223,10 +229,10 @@ __device__ __forceinline__ double sturm_lowest(const double* a, const double* b,
     const double tiny = delta;
     if (D > 2.0 * tiny) {
       // x_i = hi - D r^i, i = 0..P-2 (x_0 = lo), r^(P-2) = tiny / D; lane P-1 checks x = hi
-      const double lr = log2(tiny / D) / (double)(P - 2);
+      const float lr = log2f((float)tiny / (float)D) * (1.0f / (float)(P - 2));
       if (threadIdx.x < P) {
         const int i = threadIdx.x;
-        const double x = (i == P - 1) ? hi : hi - D * exp2(lr * (double)i);
+        const double x = (i == P - 1) ? hi : hi - D * (double)exp2f(lr * (float)i);
         const int c = (x > lo && x <= hi) ? sturm_count_ff(af, bf, m, ff_of(x)) : (x <= lo ? 0 : 1);
         if (i == P - 1) {
           top_s = c;
@@ -238,8 +244,8 @@ __device__ __forceinline__ double sturm_lowest(const double* a, const double* b,
       if (threadIdx.x == 0 && top_s >= 1) {
         const int k = last0_s;  // largest probe index still below lambda_min
         if (k >= 0) {
-          const double nlo = hi - D * exp2(lr * (double)k);
-          const double nhi = (k + 1 <= P - 2) ? hi - D * exp2(lr * (double)(k + 1)) : hi;
+          const double nlo = hi - D * (double)exp2f(lr * (float)k);
+          const double nhi = (k + 1 <= P - 2) ? hi - D * (double)exp2f(lr * (float)(k + 1)) : hi;
           lo_s = fmax(nlo, lo);
           hi_s = fmin(nhi, hi);
         } else {
@@ -254,6 +260,10 @@ __device__ __forceinline__ double sturm_lowest(const double* a, const double* b,
   // within 4 units in the last place of its ends or stops shrinking
   bool fp64 = false;
   for (int round = 0; round < 160; ++round) {
+    if (rough_lo && (round > 0 || !(hi_s - lo_s > 4.0 * delta))) {
+      *rough_lo = lo_s - delta;
+      return hi_s + delta;
+    }
     if (!fp64 && !(hi_s - lo_s > 4.0 * delta)) {
       fp64 = true;
       __syncthreads();
@@ -265,7 +275,7 @@ __device__ __forceinline__ double sturm_lowest(const double* a, const double* b,
     }
     const int np = fp64 ? P : 2 * P;
     const double lo = lo_s, hi = hi_s;
-    const double w = (hi - lo) / (double)(np + 1);
+    const double w = (hi - lo) * (fp64 ? 1.0 / (double)(P + 1) : 1.0 / (double)(2 * P + 1));
     if (threadIdx.x == 0) first_s = np;
     __syncthreads();
     if (threadIdx.x < P) {
@@ -295,7 +305,9 @@ __device__ __forceinline__ double sturm_lowest(const double* a, const double* b,
       const double mid = 0.5 * (lo_s + hi_s);
       if (!(mid > lo_s && mid < hi_s)) break;
       const double mag = fmax(fabs(lo_s), fabs(hi_s));
-      if (hi_s - lo_s <= 4.0 * (mag > 0.0 ? ldexp(1.0, ilogb(mag) - 52) : 0.0)) break;
+      // 4 units in the last place: 2^(exponent - 50) from the exponent field
+      const long long ulp4 = (__double_as_longlong(mag) >> 52) - 50;
+      if (hi_s - lo_s <= (ulp4 > 0 ? __longlong_as_double(ulp4 << 52) : 0.0)) break;
     }
   }
   return hi_s;
