@@ -1,5 +1,5 @@
 // Batched Lanczos (Sec. 2.2, Algorithm 1) over many independent (lattice, filling, U)
-// instances in ONE persistent cooperative kernel launch, captured in a CUDA graph.
+// instances in ONE persistent cooperative kernel launch.
 //
 // Instances are packed onto groups of co-resident CTAs by a schedule (kScheds): an instance
 // whose dimension reaches a threshold gets a group of several CTAs, smaller instances run
@@ -20,9 +20,11 @@
 // its vectors, a Ritz vector is assembled per instance and FP64 steps refine it
 // (batched_ritz_kernel and the `refine` form of the FP64 kernel, below).
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <map>
 #include <mutex>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -81,7 +83,6 @@ struct BInst {
 struct BState {
   int j, status;
   double scale[2];
-  double tscale;
   double last_E0, last_lo;  // bracket of E0(last_E0_step), the last tested step's
   int last_E0_step;
   int pad_;
@@ -440,6 +441,15 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
     const int r = (int)e / I.ld, d = (int)e - r * I.ld;
     return d < I.dim_dn ? bstart_element(a.seed, (uint64_t)((int64_t)r * I.dim_dn + d)) : 0.0;
   };
+  // the scalars of the running step, one copy per CTA (all CTAs compute the same)
+  __shared__ struct {
+    double scale, scale_prev, beta, tscale;  // of f_j and f_{j-1}; b_j
+  } run_s;
+  if (threadIdx.x == 0) {
+    run_s.scale = 1.0;
+    run_s.scale_prev = run_s.beta = run_s.tscale = 0.0;
+  }
+  __syncthreads();
   // ---- start vector: raw values (SplitMix64 or the given FP64 vector), FP64 norm,
   // normalised then rounded
   {
@@ -462,22 +472,12 @@ __device__ bool run_instance(const BArgs& a, const BInst& I, const RunSpec& R, i
       S->status = 0;
       S->scale[0] = 1.0;
       S->scale[1] = 0.0;
-      S->tscale = 0.0;
       S->last_E0_step = 0;
       S->last_E0 = S->last_lo = 0.0;
       be[1] = 0.0;
     }
     if (!group_barrier(bc, bg, g, a.max_spin, a.error)) return false;
   }
-  // the scalars of the running step, one copy per CTA (all CTAs compute the same)
-  __shared__ struct {
-    double scale, scale_prev, beta, tscale;  // of f_j and f_{j-1}; b_j
-  } run_s;
-  if (threadIdx.x == 0) {
-    run_s.scale = 1.0;
-    run_s.scale_prev = run_s.beta = run_s.tscale = 0.0;
-  }
-  __syncthreads();
   int cur = 0;
   for (int j = 1; j <= R.max_steps; ++j) {
     T* xc = (T*)(cur ? R.B1 : R.B0);
@@ -738,13 +738,12 @@ batched_ritz_kernel(BArgs a) {
 // A schedule maps instances to CTA groups: instances with dim >= big get `gbig` CTAs,
 // with dim >= mid get `gmid` CTAs, the rest are queued on single-CTA groups; queues are
 // balanced by estimated work (dim x hops x 1), longest first.
-// Schedules 5 and 6 instead size groups in proportion to a weight: with T = total weight /
-// CTAs, an instance of at least 4096 states and weight w >= 1.5 T gets about w / T CTAs, the
-// rest are queued. The weight is the work per step (5), or the work times log2 dim (6), an
-// estimate of the steps the instance will take growing with its dimension: a random start
-// overlaps the ground state by about dim^-1/2, and the batch's slowest-converging instances
-// are its large ones (on the 256-instance batch: FP32 54.8 ms against 56.0 ms with 5; a
-// stronger weight, work^1.25, took 71 ms).
+// Schedules 5 and 6 instead size groups in proportion to a weight, the work per step (5) or that
+// times log2 dim (6), an estimate of the steps growing with the dimension (a random start overlaps
+// the ground state by about dim^-1/2): with the smallest load t per CTA that fits, an instance of
+// at least 4096 states and weight w > t gets ceil(w / t) CTAs, the rest are queued, largest first,
+// on queues of load t. (With round(w / T) from w = 1.5 T on, T = total / CTAs, the instances just
+// below took twice the step time of the average and ended the batch: 27.4 ms, CTAs busy 44%.)
 struct Sched {
   int big, gbig, mid, gmid;
   int weight;  // proportional schedules: 0 work, 1 work x log2 dim
@@ -783,33 +782,41 @@ static Plan make_plan(const std::vector<long long>& work_in, const std::vector<i
   const bool prop = sc.gbig == 0;
   std::vector<int> gprop(n, 1);
   if (prop) {
-    // T = work per CTA if the batch were spread evenly over all but one CTA; instances of
-    // at least 4096 states and 1.5 T get round(w / T) CTAs; the largest groups give CTAs
-    // back until the groups fit
-    long long W = 0;
-    for (long long w : work) W += w;
-    const int cap = std::max(1, max_ctas - 1);
-    const double T = (double)W / (double)cap;
-    long long total = 0;
-    for (int i = 0; i < n; ++i) {
-      if (dims[i] >= 4096 && (double)work[i] >= 1.5 * T)
-        gprop[i] = (int)std::min((double)cap, std::floor((double)work[i] / T + 0.5));
-      if (gprop[i] > 1) total += gprop[i];
+    // the smallest t by bisection: groups for w > t, the others on queues of load <= t
+    auto fits = [&](double t) {
+      long long used = 0;
+      for (int i : idx)
+        if (dims[i] >= 4096 && (double)work[i] > t) used += (long long)std::ceil((double)work[i] / t);
+      const long long left = max_ctas - used;
+      std::priority_queue<double, std::vector<double>, std::greater<double>> load;
+      for (int i : idx) {
+        if (dims[i] >= 4096 && (double)work[i] > t) continue;
+        if (left < 1) return false;
+        double l = (double)work[i];
+        if ((long long)load.size() >= left) {
+          l += load.top();
+          load.pop();
+          if (l > t) return false;
+        }
+        load.push(l);
+      }
+      return used <= max_ctas;
+    };
+    double lo = 0.0, hi = 1.0;
+    for (int i = 0; i < n; ++i) hi += (double)work[i];
+    lo = hi / (2.0 * max_ctas);
+    for (int it = 0; it < 20 && hi > 1.01 * lo; ++it) {
+      const double t = std::sqrt(lo * hi);
+      if (fits(t)) hi = t;
+      else lo = t;
     }
-    while (total > cap) {
-      int big = 0;
-      for (int i = 1; i < n; ++i)
-        if (gprop[i] > gprop[big]) big = i;
-      if (gprop[big] <= 1) break;
-      --gprop[big];
-      --total;
-      if (gprop[big] == 1) --total;  // queued from now on
-    }
+    for (int i = 0; i < n; ++i)
+      if (dims[i] >= 4096 && (double)work[i] > hi) gprop[i] = (int)std::ceil((double)work[i] / hi);
   }
   for (int i : idx) {
     int gsz = dims[i] >= sc.big ? sc.gbig : (dims[i] >= sc.mid ? sc.gmid : 1);
     if (prop) gsz = gprop[i];
-    const int cap = prop ? max_ctas - 1 : max_ctas / 2;
+    const int cap = prop ? max_ctas : max_ctas / 2;
     if (gsz > 1 && ctas + gsz <= cap) {
       BGroup G{ctas, gsz, (int)p.order.size(), (int)p.order.size() + 1};
       p.order.push_back(i);
@@ -894,95 +901,82 @@ size_t blayout_elems(const ed_basis* b) { return ((size_t)b->up.dim * blayout_ld
 
 struct BatchRun {
   int n = 0;
-  cudaStream_t stream = nullptr;  // frees the pooled store
-  bool pooled = false;
+  cudaStream_t stream = nullptr;  // frees the pooled memory
   std::vector<BInst> hinst;
   std::vector<int> dims;
   std::vector<long long> work;
-  void* vec = nullptr;
+  std::vector<BState> hs, hs2;  // the instances' final states of the two phases
+  int max_ctas = 0, max_ctas2 = 0;
+  void* mem = nullptr;        // one block from the library's bounded pool for all but the store:
+  void* vec = nullptr;        //   work vectors
   BInst* d_inst = nullptr;
   BState* d_state = nullptr;
-  double* d_scal = nullptr;  // alpha | beta | E0
-  int* d_misc = nullptr;     // error flag
+  double* d_scal = nullptr;   //   alpha | beta | E0
+  int* d_misc = nullptr;      //   error flag
+  void* d_plan = nullptr;     //   the launches' plans
+  void* d_plan2 = nullptr;
   // mixed solves
   bool mixed = false;
   int refine_steps = 0;
   double refine_tol = 0.0;
   void* vstore = nullptr;     // FP32 Lanczos vectors of every instance
-  void* dvec = nullptr;       // FP64 refinement vectors
+  bool pooled = false;
+  void* dvec = nullptr;       //   FP64 refinement vectors
   double* d_rwork = nullptr;
   BState* d_state2 = nullptr;
-  double* d_scal2 = nullptr;  // alpha | beta | E0 of the refinement
+  double* d_scal2 = nullptr;  //   alpha | beta | E0 of the refinement
   ~BatchRun() {
-    if (vec) cudaFree(vec);
-    if (d_inst) cudaFree(d_inst);
-    if (d_state) cudaFree(d_state);
-    if (d_scal) cudaFree(d_scal);
-    if (d_misc) cudaFree(d_misc);
+    if (mem) cudaFreeAsync(mem, stream);
     if (vstore && pooled) cudaFreeAsync(vstore, stream);
     if (vstore && !pooled) cudaFree(vstore);
-    if (dvec) cudaFree(dvec);
-    if (d_rwork) cudaFree(d_rwork);
-    if (d_state2) cudaFree(d_state2);
-    if (d_scal2) cudaFree(d_scal2);
   }
 };
 
-struct PlanDev {
-  BGroup* groups = nullptr;
-  int* goc = nullptr;
-  int* order = nullptr;
-  double* part = nullptr;
-  unsigned* bar = nullptr;
-  ~PlanDev() {
-    if (groups) cudaFree(groups);
-    if (goc) cudaFree(goc);
-    if (order) cudaFree(order);
-    if (part) cudaFree(part);
-    if (bar) cudaFree(bar);
-  }
-};
+// Device copy of a plan on at most max_ctas CTAs, in one block.
+size_t plan_bytes(int max_ctas, int n) {
+  return (size_t)max_ctas * (sizeof(BGroup) + sizeof(int) + 2 * sizeof(double) + 2 * sizeof(unsigned)) +
+         (size_t)n * sizeof(int) + 64;
+}
 
-ed_status upload_plan(const Plan& p, PlanDev& d, cudaStream_t s) {
-  ED_TRY_CUDA(cudaMalloc((void**)&d.groups, p.groups.size() * sizeof(BGroup)));
-  ED_TRY_CUDA(cudaMalloc((void**)&d.goc, p.group_of_cta.size() * sizeof(int)));
-  ED_TRY_CUDA(cudaMalloc((void**)&d.order, p.order.size() * sizeof(int)));
-  ED_TRY_CUDA(cudaMalloc((void**)&d.part, 2 * (size_t)p.grid * sizeof(double)));
-  ED_TRY_CUDA(cudaMalloc((void**)&d.bar, 2 * p.groups.size() * sizeof(unsigned)));
-  ED_TRY_CUDA(cudaMemcpyAsync(d.groups, p.groups.data(), p.groups.size() * sizeof(BGroup), cudaMemcpyHostToDevice, s));
-  ED_TRY_CUDA(cudaMemcpyAsync(d.goc, p.group_of_cta.data(), p.group_of_cta.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-  ED_TRY_CUDA(cudaMemcpyAsync(d.order, p.order.data(), p.order.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-  ED_TRY_CUDA(cudaMemsetAsync(d.bar, 0, 2 * p.groups.size() * sizeof(unsigned), s));
+// The batch's plan for max_ctas CTAs, uploaded to `mem`; sets the plan's fields of a and the grid.
+ed_status upload_plan(const BatchRun& R, int sched, int max_ctas, void* mem, BArgs& a, int* grid, cudaStream_t s) {
+  const Plan p = make_plan(R.work, R.dims, kScheds[sched], max_ctas);
+  double* part = (double*)mem;
+  BGroup* groups = (BGroup*)(part + 2 * (size_t)max_ctas);
+  int* goc = (int*)(groups + max_ctas);
+  int* order = goc + max_ctas;
+  unsigned* bar = (unsigned*)(order + R.n);
+  ED_TRY_CUDA(cudaMemcpyAsync(groups, p.groups.data(), p.groups.size() * sizeof(BGroup), cudaMemcpyHostToDevice, s));
+  ED_TRY_CUDA(cudaMemcpyAsync(goc, p.group_of_cta.data(), p.group_of_cta.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+  ED_TRY_CUDA(cudaMemcpyAsync(order, p.order.data(), p.order.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+  ED_TRY_CUDA(cudaMemsetAsync(bar, 0, 2 * (size_t)max_ctas * sizeof(unsigned), s));
+  // (the plan's host arrays may go: copies from pageable memory are staged when the call returns,
+  // and the caller synchronises the stream before the block is freed)
+  a.order = order;
+  a.groups = groups;
+  a.group_of_cta = goc;
+  a.part_a = part;
+  a.part_b = part + max_ctas;
+  a.bar_count = bar;
+  a.bar_gen = bar + max_ctas;
+  *grid = p.grid;
   return ED_OK;
 }
 
-// One cooperative launch of the whole batch, captured in a CUDA graph and replayed once.
-// p: the plan of the (first) Lanczos launch; p2: the plan of a mixed solve's Ritz and
-// refinement launches (their kernels may allow fewer CTAs per SM; all state between the
-// launches is per instance, so each launch can pack the instances its own way).
-ed_status run_plan(BatchRun& R, const Plan& p, const Plan* p2, const ed_opts* o, int check,
-                   cudaStream_t s, float* ms_out) {
+// The whole batch: Algorithm 1 in one cooperative launch and, for a mixed solve, the Ritz vectors
+// and the refinement in one each, over a plan for their kernels' residency (all state between the
+// launches is per instance).
+ed_status run_batch(BatchRun& R, int sched, const ed_opts* o, int check, cudaStream_t s, float* ms_out) {
   const void* kernel = o->dtype == ED_F64_NATIVE ? (const void*)batched_lanczos_kernel<double>
                                                  : (const void*)batched_lanczos_kernel<float>;
-  PlanDev d, d2;
-  ed_status st = upload_plan(p, d, s);
-  if (st != ED_OK) return st;
-  if (R.mixed && (st = upload_plan(*p2, d2, s)) != ED_OK) return st;
   ED_TRY_CUDA(cudaMemsetAsync(R.d_misc, 0, sizeof(int), s));
-  BArgs a;
+  BArgs a = {};
   a.inst = R.d_inst;
   a.st = R.d_state;
   const size_t stride = (size_t)o->max_steps + 2;
   a.alpha = R.d_scal;
   a.beta = R.d_scal + stride * R.n;
   a.E0 = R.d_scal + 2 * stride * R.n;
-  a.order = d.order;
-  a.groups = d.groups;
-  a.group_of_cta = d.goc;
-  a.part_a = d.part;
-  a.part_b = d.part + p.grid;
-  a.bar_count = d.bar;
-  a.bar_gen = d.bar + p.groups.size();
   a.error = R.d_misc;
   a.max_steps = o->max_steps;
   a.check = check;
@@ -997,71 +991,36 @@ ed_status run_plan(BatchRun& R, const Plan& p, const Plan* p2, const ed_opts* o,
   a.E02 = R.d_scal2 ? R.d_scal2 + 2 * stride2 * R.n : nullptr;
   a.refine_steps = R.refine_steps;
   a.refine_tol = R.refine_tol;
-  a.refine = 0;
   a.store = R.mixed ? 1 : 0;
-  BArgs ar = a;  // mixed solves: the Ritz launch and the FP64 refinement over plan p2
-  if (R.mixed) {
-    ar.order = d2.order;
-    ar.groups = d2.groups;
-    ar.group_of_cta = d2.goc;
-    ar.part_a = d2.part;
-    ar.part_b = d2.part + p2->grid;
-    ar.bar_count = d2.bar;
-    ar.bar_gen = d2.bar + p2->groups.size();
-  }
-  ar.store = 0;
-  BArgs a2 = ar;
-  a2.refine = 1;
+  const auto t0 = std::chrono::steady_clock::now();
+  int grid = 0;
+  ed_status r = upload_plan(R, sched, R.max_ctas, R.d_plan, a, &grid, s);
+  if (r != ED_OK) return r;
   void* args[] = {&a};
-  void* argsr[] = {&ar};
-  void* args2[] = {&a2};
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  ED_TRY_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  const size_t dsm = bsmem_bytes(o->max_steps), dsm2 = bsmem_bytes(R.refine_steps);
-  cudaError_t le = cudaLaunchCooperativeKernel(kernel, p.grid, kBThreads, args, dsm, s);
-  if (le == cudaSuccess && R.mixed)
-    le = cudaLaunchCooperativeKernel((const void*)batched_ritz_kernel, p2->grid, kBThreads, argsr,
-                                     ritz_bytes(o->max_steps), s);
-  if (le == cudaSuccess && R.mixed)
-    le = cudaLaunchCooperativeKernel((const void*)batched_lanczos_kernel<double>, p2->grid, kBThreads,
-                                     args2, dsm2, s);
-  cudaError_t ce = cudaStreamEndCapture(s, &graph);
-  if (le != cudaSuccess || ce != cudaSuccess) {
-    if (graph) cudaGraphDestroy(graph);
-    set_error("batched Lanczos: capture of the cooperative launch failed: %s",
-              cudaGetErrorString(le != cudaSuccess ? le : ce));
-    return ED_ERR_CUDA;
-  }
-  cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
-  cudaGraphDestroy(graph);
-  if (ie != cudaSuccess) {
-    set_error("batched Lanczos: graph instantiate failed: %s", cudaGetErrorString(ie));
-    return ED_ERR_CUDA;
-  }
-  cudaEvent_t e0, e1;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
-  cudaEventRecord(e0, s);
-  cudaError_t ge = cudaGraphLaunch(exec, s);
-  cudaEventRecord(e1, s);
-  cudaError_t se = cudaStreamSynchronize(s);
-  float ms = 0.f;
-  cudaEventElapsedTime(&ms, e0, e1);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  cudaGraphExecDestroy(exec);
-  if (ge != cudaSuccess || se != cudaSuccess) {
-    set_error("batched Lanczos: %s", cudaGetErrorString(ge != cudaSuccess ? ge : se));
-    return ED_ERR_CUDA;
+  ED_TRY_CUDA(cudaLaunchCooperativeKernel(kernel, grid, kBThreads, args, bsmem_bytes(o->max_steps), s));
+  if (R.mixed) {
+    BArgs b = a;
+    b.store = 0;
+    if ((r = upload_plan(R, sched, R.max_ctas2, R.d_plan2, b, &grid, s)) != ED_OK) return r;
+    void* args2[] = {&b};
+    ED_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)batched_ritz_kernel, grid, kBThreads, args2,
+                                            ritz_bytes(o->max_steps), s));
+    b.refine = 1;  // (a launch copies its arguments)
+    ED_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)batched_lanczos_kernel<double>, grid, kBThreads, args2,
+                                            bsmem_bytes(R.refine_steps), s));
+    R.hs2.resize(R.n);
+    ED_TRY_CUDA(cudaMemcpyAsync(R.hs2.data(), R.d_state2, R.n * sizeof(BState), cudaMemcpyDeviceToHost, s));
   }
   int err = 0;
-  ED_TRY_CUDA(cudaMemcpy(&err, R.d_misc, sizeof(int), cudaMemcpyDeviceToHost));
+  R.hs.resize(R.n);
+  ED_TRY_CUDA(cudaMemcpyAsync(R.hs.data(), R.d_state, R.n * sizeof(BState), cudaMemcpyDeviceToHost, s));
+  ED_TRY_CUDA(cudaMemcpyAsync(&err, R.d_misc, sizeof(int), cudaMemcpyDeviceToHost, s));
+  ED_TRY_CUDA(cudaStreamSynchronize(s));
   if (err) {
     set_error("batched Lanczos: a group barrier timed out");
     return ED_ERR_TIMEOUT;
   }
-  if (ms_out) *ms_out = ms;
+  if (ms_out) *ms_out = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();
   return ED_OK;
 }
 
@@ -1152,21 +1111,79 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
     ED_CHECK_ARG(!b->has_tau(), "%s: basis %d has complex amplitudes", fn, i);
     ED_CHECK_ARG(b->dim < (1LL << 31), "%s: instance %d too large", fn, i);
     R.dims[i] = (int)b->dim;
-    R.work[i] = (long long)b->dim * (b->up.maxhops + b->dn.maxhops + 4);
+    // (the element-by-element H.v takes about 1.4 times as long as the row-ordered one)
+    R.work[i] = (long long)b->dim * (b->up.maxhops + b->dn.maxhops + 4) * (blayout_rows(b) ? 5 : 7);
     ED_CHECK_ARG(b->up.dim * (int64_t)blayout_ld(b) < (1LL << 31), "%s: instance %d too large", fn, i);
     total += blayout_elems(b);
   }
   const size_t esize = o->dtype == ED_F64_NATIVE ? 8 : 4;
-  const size_t stride = (size_t)o->max_steps + 2;
-  ED_TRY_CUDA(cudaMalloc((void**)&R.vec, 2 * total * esize));
+  const size_t stride = (size_t)o->max_steps + 2, stride2 = (size_t)refine_steps + 2;
+  R.stream = s;
+  // a cooperative launch needs every CTA resident: grids of (resident CTAs per SM) x SMs
+  int per_sm = 0, per_sm2 = 0;
+  if (o->dtype == ED_F64_NATIVE)
+    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_lanczos_kernel<double>,
+                                                              kBThreads, bsmem_bytes(o->max_steps)));
+  else
+    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_lanczos_kernel<float>,
+                                                              kBThreads, bsmem_bytes(o->max_steps)));
+  if (mixed) {  // the Ritz and refinement launches share a limit
+    int pm = 0, pd = 0;
+    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pm, batched_ritz_kernel, kBThreads,
+                                                              ritz_bytes(o->max_steps)));
+    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pd, batched_lanczos_kernel<double>,
+                                                              kBThreads, bsmem_bytes(refine_steps)));
+    per_sm2 = std::min(pm, pd);
+  }
+  ED_CHECK_ARG(per_sm >= 1 && (!mixed || per_sm2 >= 1), "%s: the batched kernels do not fit an SM", fn);
+  R.max_ctas = sm_count() * std::min(per_sm, o->dtype == ED_F64_NATIVE
+                                                 ? bctas_per_sm<double>() : bctas_per_sm<float>());
+  R.max_ctas2 = sm_count() * std::min(std::max(per_sm2, 1), kBCtasPerSm);
+  // ---- one block for the work vectors, states, scalars and plans
+  {
+    size_t at = 0;
+    auto place = [&](size_t bytes) {
+      const size_t o0 = at;
+      at += (bytes + 255) / 256 * 256;
+      return o0;
+    };
+    const size_t o_vec = place(2 * total * esize), o_inst = place(n * sizeof(BInst)), o_st = place(n * sizeof(BState)),
+                 o_misc = place(sizeof(int)), o_plan = place(plan_bytes(R.max_ctas, n)),
+                 o_plan2 = place(mixed ? plan_bytes(R.max_ctas2, n) : 0),
+                 o_dvec = place(mixed ? 2 * total * sizeof(double) : 0), o_st2 = place(mixed ? n * sizeof(BState) : 0),
+                 o_zero = at, o_scal = place(3 * stride * n * sizeof(double)),
+                 o_scal2 = place(mixed ? 3 * stride2 * n * sizeof(double) : 0),
+                 o_rw = place(mixed ? 4 * stride * n * sizeof(double) : 0);
+    cudaMemPool_t pool = psi_pool();
+    const cudaError_t e = pool ? cudaMallocFromPoolAsync(&R.mem, at, pool, s) : cudaMallocAsync(&R.mem, at, s);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      R.mem = nullptr;
+      set_error("%s: %zu bytes of device memory are not available", fn, at);
+      return e == cudaErrorMemoryAllocation ? ED_ERR_OOM : ED_ERR_CUDA;
+    }
+    char* m = (char*)R.mem;
+    R.vec = m + o_vec;
+    R.d_inst = (BInst*)(m + o_inst);
+    R.d_state = (BState*)(m + o_st);
+    R.d_misc = (int*)(m + o_misc);
+    R.d_plan = m + o_plan;
+    R.d_plan2 = m + o_plan2;
+    R.d_scal = (double*)(m + o_scal);
+    if (mixed) {
+      R.dvec = m + o_dvec;
+      R.d_state2 = (BState*)(m + o_st2);
+      R.d_scal2 = (double*)(m + o_scal2);
+      R.d_rwork = (double*)(m + o_rw);
+    }
+    ED_TRY_CUDA(cudaMemsetAsync(m + o_zero, 0, at - o_zero, s));
+  }
   if (mixed) {
     R.mixed = true;
     R.refine_steps = refine_steps;
     R.refine_tol = refine_tol;
-    const size_t stride2 = (size_t)refine_steps + 2;
     const size_t vbytes = total * (size_t)o->max_steps * sizeof(float);
     cudaMemPool_t pool = vstore_pool();
-    R.stream = s;
     const cudaError_t ve = pool ? cudaMallocFromPoolAsync(&R.vstore, vbytes, pool, s)
                                 : cudaMalloc(&R.vstore, vbytes);
     if (ve != cudaSuccess) {
@@ -1176,12 +1193,6 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
       return ED_ERR_OOM;
     }
     R.pooled = pool != nullptr;
-    ED_TRY_CUDA(cudaMalloc(&R.dvec, 2 * total * sizeof(double)));
-    ED_TRY_CUDA(cudaMalloc((void**)&R.d_rwork, 4 * stride * n * sizeof(double)));
-    ED_TRY_CUDA(cudaMalloc((void**)&R.d_state2, n * sizeof(BState)));
-    ED_TRY_CUDA(cudaMalloc((void**)&R.d_scal2, 3 * stride2 * n * sizeof(double)));
-    ED_TRY_CUDA(cudaMemsetAsync(R.d_scal2, 0, 3 * stride2 * n * sizeof(double), s));
-    ED_TRY_CUDA(cudaMemsetAsync(R.d_rwork, 0, 4 * stride * n * sizeof(double), s));
   }
   size_t off = 0;
   for (int i = 0; i < n; ++i) {
@@ -1213,33 +1224,7 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
     I.t = params[i].t;
     I.U = params[i].U;
   }
-  ED_TRY_CUDA(cudaMalloc((void**)&R.d_inst, n * sizeof(BInst)));
-  ED_TRY_CUDA(cudaMalloc((void**)&R.d_state, n * sizeof(BState)));
-  ED_TRY_CUDA(cudaMalloc((void**)&R.d_scal, 3 * stride * n * sizeof(double)));
-  ED_TRY_CUDA(cudaMalloc((void**)&R.d_misc, sizeof(int)));
   ED_TRY_CUDA(cudaMemcpyAsync(R.d_inst, R.hinst.data(), n * sizeof(BInst), cudaMemcpyHostToDevice, s));
-  ED_TRY_CUDA(cudaMemsetAsync(R.d_scal, 0, 3 * stride * n * sizeof(double), s));
-
-  // a cooperative launch needs every CTA resident: grids of (resident CTAs per SM) x SMs
-  int per_sm = 0, per_sm2 = 0;
-  if (o->dtype == ED_F64_NATIVE)
-    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_lanczos_kernel<double>,
-                                                              kBThreads, bsmem_bytes(o->max_steps)));
-  else
-    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_lanczos_kernel<float>,
-                                                              kBThreads, bsmem_bytes(o->max_steps)));
-  if (mixed) {  // the Ritz and refinement launches share a plan
-    int pm = 0, pd = 0;
-    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pm, batched_ritz_kernel, kBThreads,
-                                                              ritz_bytes(o->max_steps)));
-    ED_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pd, batched_lanczos_kernel<double>,
-                                                              kBThreads, bsmem_bytes(refine_steps)));
-    per_sm2 = std::min(pm, pd);
-  }
-  ED_CHECK_ARG(per_sm >= 1 && (!mixed || per_sm2 >= 1), "%s: the batched kernels do not fit an SM", fn);
-  const int max_ctas = sm_count() * std::min(per_sm, o->dtype == ED_F64_NATIVE
-                                                         ? bctas_per_sm<double>() : bctas_per_sm<float>());
-  const int max_ctas2 = sm_count() * std::min(std::max(per_sm2, 1), kBCtasPerSm);
   const int check = 4;  // E0(j) every 4 steps (and at the stop step)
   int sched = o->schedule;
   if (sched < 0) {
@@ -1247,7 +1232,7 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
     // schedules pack the same H.v work in both forms), keep the best
     std::string key;
     for (int i = 0; i < n; ++i) key += std::to_string(R.work[i]) + ",";
-    key += std::to_string(max_ctas) + "/" + std::to_string((int)o->dtype);
+    key += std::to_string(R.max_ctas) + "/" + std::to_string((int)o->dtype);
     {
       std::lock_guard<std::mutex> lk(g_tune_mu);
       auto it = g_tune_cache.find(key);
@@ -1262,9 +1247,8 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
       R.mixed = false;
       float best = 1e30f;
       for (int k = 0; k < kNumScheds; ++k) {
-        const Plan p = make_plan(R.work, R.dims, kScheds[k], max_ctas);
         float ms = 0.f;
-        ed_status r = run_plan(R, p, nullptr, &ot, check, s, &ms);
+        ed_status r = run_batch(R, k, &ot, check, s, &ms);
         if (r != ED_OK) return r;
         if (ms < best) best = ms, sched = k;
       }
@@ -1273,23 +1257,14 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
       g_tune_cache[key] = sched;
     }
   }
-  const Plan p = make_plan(R.work, R.dims, kScheds[sched], max_ctas);
-  const Plan p2 = mixed ? make_plan(R.work, R.dims, kScheds[sched], max_ctas2) : Plan();
-  float ms = 0.f;
-  ed_status r = run_plan(R, p, mixed ? &p2 : nullptr, o, check, s, &ms);
+  ed_status r = run_batch(R, sched, o, check, s, nullptr);
   if (r != ED_OK) return r;
-  std::vector<BState> hs(n), hs2(mixed ? n : 0);
-  ED_TRY_CUDA(cudaMemcpy(hs.data(), R.d_state, n * sizeof(BState), cudaMemcpyDeviceToHost));
-  const size_t stride_out = mixed ? (size_t)refine_steps + 2 : stride;
+  const std::vector<BState>&hs = R.hs, &hs2 = R.hs2;
+  const size_t stride_out = mixed ? stride2 : stride;
   std::vector<double> hE(stride_out * n);
-  if (mixed) {
-    ED_TRY_CUDA(cudaMemcpy(hs2.data(), R.d_state2, n * sizeof(BState), cudaMemcpyDeviceToHost));
-    ED_TRY_CUDA(cudaMemcpy(hE.data(), R.d_scal2 + 2 * stride_out * n, stride_out * n * sizeof(double),
-                           cudaMemcpyDeviceToHost));
-  } else {
-    ED_TRY_CUDA(cudaMemcpy(hE.data(), R.d_scal + 2 * stride * n, stride * n * sizeof(double),
-                           cudaMemcpyDeviceToHost));
-  }
+  ED_TRY_CUDA(cudaMemcpyAsync(hE.data(), mixed ? R.d_scal2 + 2 * stride2 * n : R.d_scal + 2 * stride * n,
+                              stride_out * n * sizeof(double), cudaMemcpyDeviceToHost, s));
+  ED_TRY_CUDA(cudaStreamSynchronize(s));
   bool all_conv = true;
   for (int i = 0; i < n; ++i) {
     const BState& F = mixed ? hs2[i] : hs[i];

@@ -42,7 +42,6 @@ hv2s_kernel(Hv2sArgs a, const E* __restrict__ x, E* __restrict__ y,
   __shared__ double red[33];
   if (S->status != 0) return;
   const int ld = a.ld;
-  const int MH = a.maxhops_up > 0 ? a.maxhops_up : 1;
   constexpr int G = hv2_group<E, 1>();
   E* xs = reinterpret_cast<E*>(smem);
   int64_t* upoff = reinterpret_cast<int64_t*>(smem + ((size_t)a.nslots * sizeof(E) + 15) / 16 * 16);

@@ -132,6 +132,8 @@ void lz_cache_free(const ed_basis* b);
 // A basis was built (+1) or destroyed (-1): with the last one the ground-state pool (memory of
 // kept Lanczos vectors, ed_lanczos.cu) is given back.
 void psi_pool_basis(int delta);
+// That pool on the current device (NULL: not available); at most 16 GB stay in it while idle.
+cudaMemPool_t psi_pool();
 // Free the fused H.v down tables cached on a basis (called by ed_basis_destroy).
 void hv2_tables_free(const ed_basis* b);
 

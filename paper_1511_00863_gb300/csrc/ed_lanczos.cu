@@ -1148,7 +1148,7 @@ extern "C" ed_status ed_lanczos_solve(const ed_basis* b, const ed_params* p, con
 
 // ------------------------------------------------------------------ ground-state vector
 namespace ed {
-// Memory of the vectors a ground-state call keeps: a pool per device, so that the next call
+// Memory of the vectors a ground-state call keeps and of a batch's work: a pool per device, so that the next call
 // does not map the same gigabytes again (0.75 ms per GB). It holds at most kPsiKeep bytes while
 // idle and gives them back when the last basis is destroyed.
 constexpr uint64_t kPsiKeep = 16ull << 30;
@@ -1156,7 +1156,7 @@ static std::mutex g_psi_mu;
 static cudaMemPool_t g_psi_pool[64] = {};
 static int64_t g_psi_bases = 0;
 
-static cudaMemPool_t psi_pool() {
+cudaMemPool_t psi_pool() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
   std::lock_guard<std::mutex> lk(g_psi_mu);

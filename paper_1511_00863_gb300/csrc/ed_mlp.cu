@@ -29,7 +29,6 @@
 namespace ed {
 
 constexpr int kH = 64;         // hidden units
-constexpr int kMaxIn = 2 * kMaxSites + 1;
 constexpr int kTile = 64;      // samples per tile in the training kernel
 constexpr int kMThreads = 256;
 
