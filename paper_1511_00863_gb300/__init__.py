@@ -113,10 +113,20 @@ def _check(status: int) -> int:
     return status
 
 
+_raw_stream = None  # () -> the current CUDA stream's handle
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return c_void_p(torch.cuda.current_stream().cuda_stream)
+        global _raw_stream
+        if _raw_stream is None:
+            import torch
+            torch.cuda.current_stream()  # (initialises CUDA)
+            get, dev = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+            # the handle without building a Stream object, where this torch has the call
+            _raw_stream = ((lambda: get(dev())) if get and dev
+                           else (lambda: torch.cuda.current_stream().cuda_stream))
+        return c_void_p(_raw_stream())
     if isinstance(stream, int):
         return c_void_p(stream)
     return c_void_p(stream.cuda_stream)
@@ -137,6 +147,21 @@ def _ptr(t, dtype_code=None, numel=None):
     if numel is not None and t.numel() != numel:
         raise ValueError(f"expected {numel} elements, got {t.numel()}")
     return c_void_p(t.data_ptr())
+
+
+_TORCH_CODES: dict = {}  # torch dtype -> code, filled on first use
+_TENSOR: type = type(None)  # torch.Tensor from then on
+
+
+def _torch_code(dtype):
+    """dtype_code of a torch dtype by one lookup (None: not one)."""
+    if not _TORCH_CODES:
+        import torch
+        global _TENSOR
+        _TENSOR = torch.Tensor
+        _TORCH_CODES.update({torch.float64: ED_F64, torch.float32: ED_F32, torch.complex64: ED_C32,
+                             torch.complex128: ED_C64})
+    return _TORCH_CODES.get(dtype)
 
 
 def dtype_code(dtype) -> int:
@@ -263,11 +288,20 @@ def ed_basis_destroy(basis) -> None:
 
 # ------------------------------------------------------------------------ H.v
 def ed_hv(basis, t: float, U: float, x, y, stream=None) -> None:
-    code = dtype_code(x.dtype)
-    dim = ed_basis_dims(basis)[2]
-    p = ed_params(t, U)
-    _check(_lib.ed_hv(basis, byref(p), code, _ptr(x, code, dim), _ptr(y, code, dim),
-                      _stream(stream)))
+    # the shortest call of the library: checks as _ptr's, without its lookups
+    code = _torch_code(x.dtype)
+    if code is None:
+        code = dtype_code(x.dtype)
+    dim = c_int64()
+    s = _lib.ed_basis_dims(basis, None, None, byref(dim))
+    if s < 0:
+        _check(s)
+    if not (type(x) is type(y) is _TENSOR and x.is_cuda and y.is_cuda and x.dtype == y.dtype
+            and x.is_contiguous() and y.is_contiguous() and x.numel() == y.numel() == dim.value):
+        _ptr(x, code, dim.value), _ptr(y, code, dim.value)  # raises, or a subclass of Tensor
+    s = _lib.ed_hv(basis, byref(ed_params(t, U)), code, x.data_ptr(), y.data_ptr(), _stream(stream))
+    if s < 0:
+        _check(s)
 
 
 def ed_start_vector(dim: int, seed: int, out, stream=None) -> None:

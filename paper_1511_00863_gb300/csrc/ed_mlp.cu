@@ -60,6 +60,26 @@ __device__ __forceinline__ float tanh_sfu(float x) {
   return y;
 }
 
+// Two FP32 additions / multiply-adds in one instruction (PTX f32x2, sm_100 and later); each half is
+// rounded as by fadd / fmaf.
+__device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 x, x, y;\n\t"
+      "mov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
+      "fma.rn.f32x2 x, x, y, z;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
+
 // ------------------------------------------------------------------ inference
 // 5th-generation tensor cores: a CTA of 4 warps evaluates tiles of 128 basis states, one
 // state per thread (TMEM lane). The features of the tile (bits as 0/1, bf16(U/8), zero
@@ -69,7 +89,10 @@ __device__ __forceinline__ float tanh_sfu(float x) {
 // and commits to an mbarrier; every thread then reads its row of the accumulator with
 // tcgen05.ld and applies
 // bias (CUDA cores) and tanh (special-function unit); the 64 -> 2 output layer stays on the
-// CUDA cores.
+// CUDA cores. 128 tanh per state on the special-function unit (16 per cycle and SM) are 0.31 ms for
+// 11.8 M states; the other instructions have to fit beside them: features come from a table of
+// bytes (16 bytes of operand per load), additions and the output layer go two at a time, states are
+// carried from tile to tile without a division.
 // Waits on the mbarrier are bounded (1 s of the global timer); on expiry the kernel sets
 // *err, frees its TMEM and returns.
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -87,7 +110,7 @@ constexpr int kTcCtasPerSm = 5;
 
 struct TcLayout {
   int K1;
-  uint32_t a1, a2, b1, b2, par, mbar, tslot, total;
+  uint32_t a1, a2, b1, b2, par, lut, mbar, tslot, total;
 };
 
 __host__ __device__ inline TcLayout tc_layout(int nin) {
@@ -99,7 +122,8 @@ __host__ __device__ inline TcLayout tc_layout(int nin) {
   t.b1 = up(t.a2 + (uint32_t)kTcRows * kH * 2, 1024);
   t.b2 = up(t.b1 + (uint32_t)kH * t.K1 * 2, 1024);
   t.par = up(t.b2 + (uint32_t)kH * kH * 2, 1024);
-  t.mbar = up(t.par + (uint32_t)(4 * kH + 2) * 4, 16);
+  t.lut = up(t.par + (uint32_t)(4 * kH + 2) * 4, 16);
+  t.mbar = t.lut + 256 * 16;
   t.tslot = t.mbar + 8;
   t.total = up(t.tslot + 8, 1024);
   return t;
@@ -122,6 +146,7 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
   float* sb2 = sb1 + kH;
   float* sW3 = sb2 + kH;
   float* sb3 = sW3 + 2 * kH;
+  uint4* lut = reinterpret_cast<uint4*>(tsm + ly.lut);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(tsm + ly.tslot);
   const uint32_t mbar = smem_addr(tsm + ly.mbar);
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -144,6 +169,11 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
     sW3[2 * i + 1] = bf16r(params[d.oW3 + 2 * i + 1]);
   }
   if (tid < 2) sb3[tid] = bf16r(params[d.ob3 + tid]);
+  // the bf16 features (0 or 1) of every byte
+  for (int i = tid; i < 256; i += blockDim.x) {
+    auto pair = [&](int k) { return ((i >> k) & 1 ? 0x3F80u : 0u) | ((i >> (k + 1)) & 1 ? 0x3F800000u : 0u); };
+    lut[i] = make_uint4(pair(0), pair(2), pair(4), pair(6));
+  }
   if (tid == 0) mbar_init(mbar, 1);
   if (warp == 0) tc_alloc(smem_addr(tslot), kTcCols);
   fence_smem_to_async();
@@ -152,7 +182,7 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
   tc_fence_after_sync();
   const uint32_t tmem = *tslot;
   const uint32_t lanes = (uint32_t)(warp * 32) << 16;  // this warp's TMEM lane quarter
-  const float u8 = bf16r(U * 0.125f);
+  const uint32_t u8bits = pack_bf16(U * 0.125f, 0.f);  // bf16(U/8) in the low half
   const uint32_t idesc = tc_idesc_bf16_f32(kTcRows, kH);
   const uint32_t a1s = smem_addr(A1), a2s = smem_addr(A2), b1s = smem_addr(B1), b2s = smem_addr(B2);
   const uint32_t sbo1 = (uint32_t)(K1 >> 3) << 7, sbo2 = (uint32_t)(kH >> 3) << 7;
@@ -160,23 +190,35 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
   uint32_t phase = 0;
   bool ok = true;
   const int64_t ntiles = (dim + kTcRows - 1) / kTcRows;
-  for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+  // this thread's state (up rank, down rank), carried from one tile of the CTA to the next
+  const int64_t step = (int64_t)gridDim.x * kTcRows, su = step / dim_dn, sd = step - su * dim_dn;
+  int64_t u = ((int64_t)blockIdx.x * kTcRows + tid) / dim_dn;
+  int64_t dd = (int64_t)blockIdx.x * kTcRows + tid - u * dim_dn;
+  for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, u += su, dd += sd) {
+    if (dd >= dim_dn) {
+      dd -= dim_dn;
+      ++u;
+    }
     const int64_t e = tile * kTcRows + tid;
     const bool valid = e < dim;
     uint32_t ub = 0, db = 0;
     if (valid) {
-      const int64_t u = e / dim_dn;
       ub = upb[u];
-      db = dnb[e - u * dim_dn];
+      db = dnb[dd];
     }
-    auto feat = [&](int f) -> float {
-      if (f < L) return (float)((ub >> f) & 1u);
-      if (f < 2 * L) return (float)((db >> (f - L)) & 1u);
-      return f == 2 * L ? u8 : 0.f;
-    };
+    // the bits of both species in feature order, eight features (16 bytes) per table entry; the U
+    // feature (2 L) comes after them, zeros to K1
+    const unsigned long long bits = (unsigned long long)ub | ((unsigned long long)db << L);
     for (int j = 0; j < K1; j += 8) {
-      const uint4 w = make_uint4(pack_bf16(feat(j), feat(j + 1)), pack_bf16(feat(j + 2), feat(j + 3)),
-                                 pack_bf16(feat(j + 4), feat(j + 5)), pack_bf16(feat(j + 6), feat(j + 7)));
+      uint4 w = lut[j < 64 ? (bits >> j) & 0xFFu : 0u];
+      if (j == (2 * L & ~7)) {
+        const uint32_t v = u8bits << (16 * (2 * L & 1));
+        const int q = (2 * L & 7) >> 1;
+        if (q == 0) w.x |= v;
+        else if (q == 1) w.y |= v;
+        else if (q == 2) w.z |= v;
+        else w.w |= v;
+      }
       *reinterpret_cast<uint4*>(A1 + cm_offset(tid, j, K1)) = w;
     }
     // ---- layer 1 on the tensor cores
@@ -202,8 +244,10 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
       uint32_t w[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        w[q] = pack_bf16(tanh_sfu(h[j + 2 * q] + sb1[j + 2 * q]),
-                         tanh_sfu(h[j + 2 * q + 1] + sb1[j + 2 * q + 1]));
+      {
+        const float2 t = add2(make_float2(h[j + 2 * q], h[j + 2 * q + 1]), ld2(sb1 + j + 2 * q));
+        w[q] = pack_bf16(tanh_sfu(t.x), tanh_sfu(t.y));
+      }
       *reinterpret_cast<uint4*>(A2 + cm_offset(tid, j, kH)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
     // ---- layer 2 on the tensor cores
@@ -224,16 +268,18 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
     tc_ld32(tmem + lanes, h);
     tc_ld32(tmem + lanes + 32, h + 32);
     // ---- output layer on the CUDA cores
-    float a = sb3[0], z = sb3[1];
+    float2 az = ld2(sb3);
 #pragma unroll
-    for (int n = 0; n < kH; ++n) {
-      const float t = tanh_sfu(h[n] + sb2[n]);
-      a = fmaf(t, sW3[2 * n], a);
-      z = fmaf(t, sW3[2 * n + 1], z);
+    for (int n = 0; n < kH; n += 2) {
+      const float2 x = add2(make_float2(h[n], h[n + 1]), ld2(sb2 + n));
+      const float t0 = tanh_sfu(x.x), t1 = tanh_sfu(x.y);
+      const float4 w = *reinterpret_cast<const float4*>(sW3 + 2 * n);
+      az = fma2(make_float2(t0, t0), make_float2(w.x, w.y), az);
+      az = fma2(make_float2(t1, t1), make_float2(w.z, w.w), az);
     }
     if (valid) {
-      const float v = expf(a);
-      out[e] = (T)(z >= 0.f ? v : -v);
+      const float v = expf(az.x);
+      out[e] = (T)(az.y >= 0.f ? v : -v);
     }
     tc_fence_before_sync();  // this tile's TMEM reads before the next tile's MMAs
   }
