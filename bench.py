@@ -38,18 +38,10 @@ FALLBACK_HBM_GBS = 6800.0
 # the kernel's sources are unchanged since that capture.
 KERNEL_SOURCES = ["paper_1511_00863_gb300/csrc/ed_hv2_kernel.cuh", "paper_1511_00863_gb300/csrc/ed_fixed.cuh",
                   "paper_1511_00863_gb300/csrc/ed_internal.cuh", "paper_1511_00863_gb300/csrc/ed_tables.h"]
-TRAFFIC_SOURCES_SHA256 = "d5cddba73f3a3d16aa105a94ec04438c502f7512267e7f10f94116b3c2604841"
+TRAFFIC_SOURCES_SHA256 = "201131d14b9ac948eada79ffce9f0db932fa6b7328fd4a912b449cb07e688f31"
 MEASURED_TRAFFIC = {
-    ("torus4x4_5_5", "f64", 8): {"bytes": 474670848 + 136560640,
+    ("torus4x4_5_5", "f64", 8): {"bytes": 479295232 + 133789696,
                                  "profile": "profiles/hv2_kernel_torus4x4_5_5_int64.md"},
-    ("torus4x4_5_5", "f64", 9): {"bytes": 458221568 + 135683072,
-                                 "profile": "profiles/hv2_kernel_torus4x4_5_5_int64.md"},
-    ("torus4x4_5_5", "f32", 1): {"bytes": 179300352 + 51745280,
-                                 "profile": "profiles/hv2_kernel_torus4x4_5_5_f32.md"},
-    ("ring16_8_8", "f32", 2): {"bytes": 2449393920 + 634859520,
-                               "profile": "profiles/hv2_kernel_ring16_8_8_f32.md"},
-    ("ring16_8_8", "f64", 10): {"bytes": 6075339520 + 1332783104,
-                                "profile": "profiles/hv2_kernel_ring16_8_8_f32.md"},
 }
 
 
