@@ -298,7 +298,6 @@ static ed_status hv2_build_split(const ed_basis* b, int mode, int ld, cudaStream
   p->smem = split_smem(*t, b, mode == kHv2Fx ? 8 : 4);
   p->ld = ld;
   p->grid = (int)b->up.dim;
-  p->ticket = b->up.dim * (int64_t)ld >= kTicketMin;
   p->nslots = split_slots(*t);
   for (int i = 0; i < 3; ++i) p->cst[i] = t->cstart[i];
   const int64_t n = b->dn.dim;
@@ -321,7 +320,7 @@ static ed_status hv2_build_split(const ed_basis* b, int mode, int ld, cudaStream
   if (e == cudaSuccess) e = cudaMemcpyAsync(p->colpos, t->pos.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
 #define HV2S_ATTR(K, E, V_, T, MB) \
-  if (e == cudaSuccess && p->kind == K) e = one_wave(hv2s_kernel<E, V_, T, MB>, T, p);
+  if (e == cudaSuccess && p->kind == K) e = allow_max_smem(hv2s_kernel<E, V_, T, MB>);
   HV2S_KINDS(HV2S_ATTR)
 #undef HV2S_ATTR
   if (e != cudaSuccess) {
@@ -488,7 +487,6 @@ ed_status hv2_launch(const Hv2Plan* p, const ed_basis* b, double t, double U, co
     c.dim_up = b->up.dim;
     c.ld = p->ld;
     c.maxhops_up = b->up.maxhops;
-    c.ticket = p->ticket;
     c.nslots = p->nslots;
     c.cstart0 = p->cst[0];
     c.cstart1 = p->cst[1];

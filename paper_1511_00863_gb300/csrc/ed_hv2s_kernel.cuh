@@ -28,7 +28,7 @@ struct Hv2sArgs {
   const int32_t* __restrict__ hop_up;    // basis table [maxhops_up][dim_up]
   const int32_t* __restrict__ order;     // up-row visit order (NULL = rank order)
   int64_t dim_up;
-  int ld, maxhops_up, nslots, ticket;    // nslots: longest slice + G
+  int ld, maxhops_up, nslots;            // nslots: longest slice + G
   int cstart0, cstart1, cstart2;         // slices [cstart0, cstart1), [cstart1, cstart2)
   float t, U;                            // FP32 variant
 };
@@ -60,10 +60,12 @@ hv2s_kernel(Hv2sArgs a, const E* __restrict__ x, E* __restrict__ y,
   }
   DotAcc<float> dotf;
   A192 dota;
-  // one resident wave of CTAs, each takes rows blockIdx.x, blockIdx.x + gridDim.x, ...
-  for (int g = blockIdx.x; g < (int)a.dim_up; g += gridDim.x) {
+  // One CTA per row: its reduction is 1% of its 100-180 us, and as the hardware starts CTAs in order
+  // the rows in flight stay neighbours, whose rows L2 then holds. One resident wave over every
+  // grid-th row (hv2_kernel's form) took 24.3 instead of 20.6 ms on the 18-site 9/9 basis in FP32 and
+  // 64.0 instead of 55.7 ms in int64; with the rows handed out by a counter 22.4 and 59.1 ms.
+  const int g = blockIdx.x;
   const int64_t u = a.order ? (int64_t)a.order[g] : g;
-  __syncthreads();
   if (threadIdx.x < 32)
     hv2_up_list(a.hop_up, a.maxhops_up, a.dim_up, u, ld, upoff, &npos_s, &nneg_s);
   __syncthreads();
@@ -151,13 +153,11 @@ hv2s_kernel(Hv2sArgs a, const E* __restrict__ x, E* __restrict__ y,
       stcs_pack(reinterpret_cast<Pack<E, V>*>(yp), W);
     }
   }
-  }
   if constexpr (sizeof(E) == 4) {
     const double v = block_sum(dotf.get(), red);
     if (threadIdx.x == 0) reinterpret_cast<double*>(partial)[blockIdx.x] = v;
-    if (a.ticket) hv_finish(S, reinterpret_cast<const double*>(partial), gridDim.x, red);
   } else {
-    fx_hv_end(S, cur, dota.w0, dota.w1, dota.w2, reinterpret_cast<long long*>(partial), a.ticket);
+    fx_hv_end(S, cur, dota.w0, dota.w1, dota.w2, reinterpret_cast<long long*>(partial), 0);
   }
 }
 
