@@ -19,13 +19,14 @@
 // The grid is one resident wave; a CTA takes every grid-th row group (in the order that keeps
 // neighbours in L2).
 // Measured against the row-staged kernels with one padded list length per basis (ed_hv.cu,
-// ed_hvc.cu), which stay for rows too long for this one: FP32, 14-site ring 7/7: 178 -> 103 us;
-// FP64, 4x4 5/5: 1664 -> 1107 us; complex FP64 on the 4x4 checkerboard-type lattice (73 hops per
-// state, 4 classes): 18.9 -> 6.6 ms; FP64, 12-site ring 3/3: 8.8 -> 6 us.
+// ed_hvc.cu), which stay for rows too long or too short for this one (rows_usable): FP32, 14-site
+// ring 7/7: 178 -> 103 us; FP64, 4x4 5/5: 1664 -> 1107 us; complex FP64 on the 4x4 checkerboard-type
+// lattice (73 hops per state, 4 classes): 18.9 -> 6.6 ms.
 #include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "ed_internal.cuh"
@@ -484,11 +485,33 @@ static ed_status rows_launch(const ed_basis* b, const RowsArgs& a, const E* x, E
   return ED_OK;
 }
 
-// Whether this kernel takes the basis: rows of at least 96 columns (shorter ones leave most of a
-// CTA idle: the element-parallel kernel) whose two copies fit in shared memory.
+// Whether this kernel takes the basis. Its rows fit in shared memory twice, and they are long enough
+// to occupy a CTA: a row of 120 columns is four warps' work in the down part and one in the up part
+// of 12, while the row-staged kernel (ed_hv.cu, ed_hvc.cu) keeps eight small CTAs of two rows on an SM.
+// The lines, with both kernels' times of one ed_hv call (row-staged / this kernel, us) on either side:
+//  * FP32: 12,870 rows x 120 columns 23 / 50, 6,435 x 455 37 / 45, 1,001 x 2,002 31 / 35; but 8,008 x
+//    560 54 / 46, 12,870 x 1,820 265 / 181. Rows of a multiple of 4 columns (16-byte loads) from 500 on,
+//    others from 1,200 on where rows come in pairs (launch_hv_rows) or from 5,000 on. With few rows
+//    (four CTAs per SM or fewer) the down part's length counts: 120 x 252 5.0 / 4.5, 462 x 330 8.8 / 5.6.
+//  * FP64: 18,564 x 153 120 / 122, 3,003 x 105 18 / 21; 1,716 x 286 28 / 22. In the Lanczos-fused form
+//    495 x 220 loses 14%, 715 x 286 gains 12%.
+//  * complex FP32: 6,435 x 455 50 / 65, 924 x 495 14.5 / 16, 38,760 x 190 127 / 232; 1,287 x 286 11.3 /
+//    10.4, 12,870 x 560 126 / 116. Few rows: 455 x 105 5.2 / 4.4.
+//  * complex FP64: 6,435 x 105 116 / 136, 8,568 x 153 183 / 186; 462 x 165 20 / 15.5; with amplitude
+//    classes (fewer multiply-adds, the bound) 12,870 x 120 already 1,090 / 855.
 template <typename E>
 bool rows_usable(const ed_basis* b) {
-  return b->rows.C > 0 && b->dn.dim >= 96 && rows_smem<E, 1>(b) + 4096 <= (size_t)smem_optin_max();
+  const int64_t nd = b->dn.dim, nu = b->up.dim, sms = sm_count();
+  if (b->rows.C == 0 || nd < 96 || rows_smem<E, 1>(b) + 4096 > (size_t)smem_optin_max()) return false;
+  if constexpr (std::is_same<E, float>::value)
+    return nd % 4 == 0 ? nd >= 500 || (nd >= 240 && nu <= 4 * sms)
+                       : nd >= 5000 || (nd >= 1200 && nu >= 8 * sms) || (nd >= 240 && nu <= 4 * sms);
+  else if constexpr (std::is_same<E, double>::value)
+    return nd >= 240;
+  else if constexpr (std::is_same<E, float2>::value)
+    return nu <= 2 * sms || nd >= 1000 || (nd >= 280 && (nd % 2 == 0 || nu <= 4 * sms));
+  else
+    return nd >= 160 || nu <= 2 * sms || b->rows.C > 1;
 }
 
 template <typename E>
