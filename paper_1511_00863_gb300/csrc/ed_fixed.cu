@@ -264,7 +264,7 @@ fx_hv_global_kernel(FxHvArgs a, const long long* __restrict__ x, long long* __re
 // Whole CTA: b_{j+1} and f_{j+1}'s scale from the n partial records of ||Q||^2, then the
 // coefficients of the next H.v.
 __device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long long* pb, int nb,
-                                               const FxPlanArgs& p, double* vscale) {
+                                               const FxPlanArgs& p, const LzStore& store) {
   I192 sum;
   long long mx;
   fx_sum_partials(pb, nb, sum, mx);
@@ -276,7 +276,8 @@ __device__ __forceinline__ void fx_finish_step(LzScalars* S, int cur, const long
   if (finish_step(S, j, beta)) {
     S->scale[1 - cur] = sw / beta;
     S->fx_max[1 - cur] = mx;
-    if (vscale) vscale[j] = sw / beta;
+    if (store.vscale) store.vscale[j] = sw / beta;
+    if (store.vmax) store.vmax[j] = mx;
     fx_plan_step(S, 1 - cur, p);
   }
 }
@@ -340,12 +341,12 @@ fx_update_kernel(LzScalars* S, int cur, const long long* __restrict__ xc, long l
     }
   }
   fx_block_reduce(a192_get(q2), mx, pb + 4 * blockIdx.x);
-  if (finish && last_cta(&S->tick_upd)) fx_finish_step(S, cur, pb, gridDim.x, plan, kKeep ? store.vscale : nullptr);
+  if (finish && last_cta(&S->tick_upd)) fx_finish_step(S, cur, pb, gridDim.x, plan, store);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
 fx_finish_kernel(LzScalars* S, int cur, const long long* __restrict__ pb, int nb, FxPlanArgs plan) {
-  if (S->status == 0) fx_finish_step(S, cur, pb, nb, plan, nullptr);
+  if (S->status == 0) fx_finish_step(S, cur, pb, nb, plan, LzStore{nullptr, nullptr, nullptr});
 }
 
 // ------------------------------------------------------------------ ground-state vector

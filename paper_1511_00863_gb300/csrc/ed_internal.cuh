@@ -197,10 +197,12 @@ ed_status hvc_prepare(const ed_basis* b, ed_dtype dtype);
 inline bool is_complex(ed_dtype d) { return d == ED_C32 || d == ED_C64; }
 
 // Where a run keeps its Lanczos vectors (device tables; slots NULL: nowhere): slot k receives
-// the raw vector of f_{k+1} from the update pass, vscale[k] its scale. A NULL slot is skipped.
+// the raw vector of f_{k+1} from the update pass, vscale[k] its scale and (fixed point, where not
+// NULL) vmax[k] its largest |X|. A NULL slot is skipped.
 struct LzStore {
   void* const* slots;
   double* vscale;
+  long long* vmax;
 };
 
 // Row-ordered H.v (ed_rows.cu): tables built with the basis (t_bond: host amplitudes or NULL);

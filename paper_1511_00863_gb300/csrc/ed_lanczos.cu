@@ -398,12 +398,13 @@ struct ed_lanczos {
   FxRun fxr{};
   Hv2Plan* plan = nullptr;  // fused H.v on the padded layout (ed_hv2.cu), if it fits
   Reorth* ro = nullptr;     // stored Lanczos vectors when opts.reorth != 0 (ed_reorth.cu)
-  LzStore store{nullptr, nullptr};  // where the update pass keeps the vectors
+  LzStore store{nullptr, nullptr, nullptr};  // where the update pass keeps the vectors
   cudaGraphExec_t graph[4] = {};  // without / with the convergence test, + 2: vectors kept in `slots`
-  // ground-state vectors only: slot table and scales of the kept vectors, y of T_m with the
-  // inverse iteration's work, ranks by column
+  // ground-state vectors only: slot table, scales and maxima of the kept vectors, y of T_m with
+  // the inverse iteration's work, ranks by column
   void** slots = nullptr;
   double* vscale = nullptr;
+  long long* vmax = nullptr;
   double* ywork = nullptr;
   int32_t* rank = nullptr;
   // solves only (lz_iterate): the checks' stream, fork and join events of the capture, one event
@@ -584,7 +585,7 @@ extern "C" void ed_lanczos_destroy(ed_lanczos* st) {
     if (g) cudaGraphExecDestroy(g);
   for (cudaEvent_t e : st->ev_batch)
     if (e) cudaEventDestroy(e);
-  for (void* q : {(void*)st->slots, (void*)st->vscale, (void*)st->ywork, (void*)st->rank})
+  for (void* q : {(void*)st->slots, (void*)st->vscale, (void*)st->vmax, (void*)st->ywork, (void*)st->rank})
     if (q) cudaFree(q);
   if (st->ev_fork) cudaEventDestroy(st->ev_fork);
   if (st->ev_join) cudaEventDestroy(st->ev_join);
@@ -1214,7 +1215,8 @@ struct KeptVectors {
   ~KeptVectors() {
     for (void* q : blocks) cudaFreeAsync(q, st->stream);
   }
-  // Slots 0 .. n - 1; what does not fit leaves the run without kept vectors (complete false).
+  void* slot(int k) const { return (char*)blocks[k / per_block] + (size_t)(k % per_block) * vbytes; }
+  // Slots 0 .. n - 1; from the first that does not fit on (complete false) the run keeps no more.
   ed_status grow(int n) {
     while (complete && ready < n) {
       const size_t bytes = (size_t)per_block * vbytes;
@@ -1238,20 +1240,44 @@ struct KeptVectors {
 
 }  // namespace
 
-// psi on a started state: Algorithm 1 with its vectors kept where memory allows (then one pass
-// over them sums psi; the run itself is most of the time), else a second run of the same steps
-// that adds y_j f_j step by step. Both sums are the same integers.
+// The run of st, whose scalars are in st->host, from f_k on again: buffers and scalars from the kept
+// vectors of f_{k-1} and f_k (k >= 2), the tridiagonal up to a_{k-1}, b_k from the first time.
+static ed_status lz_resume(ed_lanczos* st, int k, size_t vbytes, void* const* slot) {
+  cudaStream_t s = st->stream;
+  LzScalars& h = *st->host;  // (pinned, and the stream has passed its last copy)
+  h.j = k - 1;
+  h.status = h.conv_j = h.row_next = 0;
+  h.tick_chk = h.tick_hv = h.tick_upd = 0;
+  memset(h.fx_dot, 0, sizeof(h.fx_dot));
+  h.tscale = 0.0;
+  for (int i = 1; i < k; ++i) h.tscale = std::max(h.tscale, std::fabs(h.alpha[i]) + h.beta[i]);
+  ED_TRY_CUDA(cudaMemcpyAsync(st->S, &h, sizeof(h), cudaMemcpyHostToDevice, s));
+  st->cur = 0;
+  for (int i = 0; i < 2; ++i) {  // buffer 0: f_k, buffer 1: f_{k-1}
+    ED_TRY_CUDA(cudaMemcpyAsync(st->B[i], slot[i], vbytes, cudaMemcpyDeviceToDevice, s));
+    ED_TRY_CUDA(cudaMemcpyAsync(&st->S->scale[i], st->vscale + k - 1 - i, sizeof(double), cudaMemcpyDeviceToDevice, s));
+    ED_TRY_CUDA(cudaMemcpyAsync(&st->S->fx_max[i], st->vmax + k - 1 - i, sizeof(long long), cudaMemcpyDeviceToDevice, s));
+  }
+  return ED_OK;
+}
+
+// psi on a started state: Algorithm 1 with its vectors kept where memory allows; one pass over
+// them sums psi (the run itself is most of the time). Where memory ends before the run, the steps
+// behind the last kept vector are made again from it, adding y_j f_j step by step, all of them when
+// nothing fits. All sums are the same integers. Half-filled 16-site ring (1.3 GB a vector, 72 of
+// them in the 96 GB): 622 ms; with all steps made again 909 ms, with nothing kept 839 ms.
 static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p, const ed_opts* o,
                            const void* f1, long long* P, double* E0, int32_t* steps) {
   cudaStream_t s = st->stream;
   if (!st->ywork) {
     if (cudaMalloc((void**)&st->slots, (ED_MAX_STEPS + 2) * sizeof(void*)) != cudaSuccess ||
         cudaMalloc((void**)&st->vscale, (ED_MAX_STEPS + 2) * sizeof(double)) != cudaSuccess ||
+        cudaMalloc((void**)&st->vmax, (ED_MAX_STEPS + 2) * sizeof(long long)) != cudaSuccess ||
         cudaMalloc((void**)&st->ywork, 3 * (ED_MAX_STEPS + 4) * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
-      for (void* q : {(void*)st->slots, (void*)st->vscale})
+      for (void* q : {(void*)st->slots, (void*)st->vscale, (void*)st->vmax})
         if (q) cudaFree(q);
-      st->slots = nullptr, st->vscale = nullptr;
+      st->slots = nullptr, st->vscale = nullptr, st->vmax = nullptr;
       set_error("ed_lanczos_ground_state: out of device memory");
       return ED_ERR_OOM;
     }
@@ -1261,12 +1287,13 @@ static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p
   if (r != ED_OK) return r;
   if ((r = fx_prepare(b)) != ED_OK) return r;
   int m = 0, status = 0;
+  double lam = NAN;
   double* y = st->ywork;
-  bool summed = false;
+  int have = 0;  // psi holds the terms of f_1 .. f_have
   {
     struct Unset {  // later solves on the state keep no vectors
       ed_lanczos* st;
-      ~Unset() { st->store = LzStore{nullptr, nullptr}; }
+      ~Unset() { st->store = LzStore{nullptr, nullptr, nullptr}; }
     } unset{st};
     KeptVectors kept(st);
     const bool own = !st->ro;  // a reorthogonalising run keeps its vectors by itself
@@ -1276,7 +1303,8 @@ static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p
       if (kept.complete) {
         ED_TRY_CUDA(cudaMemcpyAsync(kept.blocks[0], st->B[0], kept.vbytes, cudaMemcpyDeviceToDevice, s));
         ED_TRY_CUDA(cudaMemcpyAsync(st->vscale, &st->S->scale[0], sizeof(double), cudaMemcpyDeviceToDevice, s));
-        st->store = LzStore{st->slots, st->vscale};
+        ED_TRY_CUDA(cudaMemcpyAsync(st->vmax, &st->S->fx_max[0], sizeof(long long), cudaMemcpyDeviceToDevice, s));
+        st->store = LzStore{st->slots, st->vscale, st->vmax};
       }
     }
     r = lz_iterate(st, p, o, false, &m, &status,
@@ -1288,21 +1316,31 @@ static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p
     }
     lz_ritz_kernel<<<1, 32, 5 * (size_t)(m + 2) * sizeof(double), s>>>(st->S, m, st->host->E0[m], y);
     ED_TRY_CUDA(cudaGetLastError());
-    summed = !own || kept.complete;
-    if (summed &&
-        (r = fx_psi_sum(b, y, m, own ? st->store : ro_slots(st->ro), st->ld, st->rank, P, (long long*)st->pb, s)) != ED_OK)
+    lam = st->host->E0[m];
+    have = own ? std::min(kept.ready, m) : m;
+    if (have < std::min(m, 2)) have = 0;  // (a run goes on from two vectors)
+    if (have > 0 &&
+        (r = fx_psi_sum(b, y, have, own ? st->store : ro_slots(st->ro), st->ld, st->rank, P, (long long*)st->pb, s)) != ED_OK)
       return r;
+    if (have > 0 && have < m) {
+      void* const last[2] = {kept.slot(have - 1), kept.slot(have - 2)};
+      if ((r = lz_resume(st, have, kept.vbytes, last)) != ED_OK) return r;
+    }
   }
-  const double lam = st->host->E0[m];
+  const bool summed = have == m;
   if (!summed) {
-    if ((r = lz_reset(st, o, f1)) != ED_OK) return r;
-    ED_TRY_CUDA(cudaMemsetAsync(P, 0, (size_t)b->dim * sizeof(long long), s));
+    auto add = [&](int j) {  // the term of f_j, the running vector
+      return fx_psi_accum(b, st->S, st->cur, y, j, (const long long*)st->B[st->cur], st->ld, hv2_colpos(st->plan), P, s);
+    };
+    if (have == 0) {
+      if ((r = lz_reset(st, o, f1)) != ED_OK) return r;
+      ED_TRY_CUDA(cudaMemsetAsync(P, 0, (size_t)b->dim * sizeof(long long), s));
+      if ((r = add(++have)) != ED_OK) return r;
+    }
     if ((r = lz_plan(st, p)) != ED_OK) return r;
-    for (int j = 1; j <= m; ++j) {
-      if ((r = fx_psi_accum(b, st->S, st->cur, y, j, (const long long*)st->B[st->cur], st->ld,
-                            hv2_colpos(st->plan), P, s)) != ED_OK)
-        return r;
-      if (j < m && (r = lz_launch_step(st, p, s)) != ED_OK) return r;
+    while (have < m) {
+      if ((r = lz_launch_step(st, p, s)) != ED_OK) return r;
+      if ((r = add(++have)) != ED_OK) return r;
     }
   }
   if ((r = fx_psi_finish(b, P, summed, (long long*)st->pb, s)) != ED_OK) return r;

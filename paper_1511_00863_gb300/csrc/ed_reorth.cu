@@ -445,7 +445,7 @@ ed_status ro_create(int mode, ed_dtype dtype, int64_t n, int max_steps, int64_t 
   return ED_OK;
 }
 
-LzStore ro_slots(const Reorth* r) { return LzStore{r->slot, r->vscale}; }
+LzStore ro_slots(const Reorth* r) { return LzStore{r->slot, r->vscale, nullptr}; }
 
 template <typename T>
 static void ro_store_t(const Reorth* r, const LzScalars* S, int buf, const void* src, cudaStream_t s) {
