@@ -343,8 +343,11 @@ __device__ __forceinline__ void mm_forward(float (&acc)[4][4], const float* A, c
   }
 }
 
-// acc[q][r] += sum_s A[s][4 ty + q] B[s][4 tx + r] over the tile's samples in order.
-__device__ __forceinline__ void mm_outer(float (&acc)[4][4], const float* A, const float* B, int ty, int tx) {
+// sum[q][r] += sum_s A[s][4 ty + q] B[s][4 tx + r] over the tile's samples in order. The tile's sum is
+// formed by itself: carried on through all tiles of a CTA, a chain of additions grows with the batch
+// (55,000 of them at 2^24 samples instead of 64 and one per tile).
+__device__ __forceinline__ void mm_outer(float (&sum)[4][4], const float* A, const float* B, int ty, int tx) {
+  float acc[4][4] = {};
 #pragma unroll 4
   for (int t = 0; t < kTile; ++t) {
     const float4 a = ld4(A + t * kLdT + 4 * ty), b = ld4(B + t * kLdT + 4 * tx);
@@ -353,6 +356,10 @@ __device__ __forceinline__ void mm_outer(float (&acc)[4][4], const float* A, con
 #pragma unroll
       for (int r = 0; r < 4; ++r) acc[q][r] = fmaf(get4(a, q), get4(b, r), acc[q][r]);
   }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) sum[q][r] += acc[q][r];
 }
 
 __global__ void __launch_bounds__(kMThreads, 2)
@@ -531,8 +538,11 @@ mlp_grad_kernel(const float* __restrict__ params, int L, float U, const uint32_t
     // ---- weight gradients
     mm_outer(gW2, H1B, H2, ty, tx);
     if (4 * ty < n4) mm_outer(gW1, X, H1, ty, tx);
-    if (d.nin > kH && tid < kH)
-      for (int t = 0; t < kTile; ++t) gW1last = fmaf(X[t * kLdT + kH], H1[t * kLdT + tid], gW1last);
+    if (d.nin > kH && tid < kH) {
+      float acc = 0.f;
+      for (int t = 0; t < kTile; ++t) acc = fmaf(X[t * kLdT + kH], H1[t * kLdT + tid], acc);
+      gW1last += acc;
+    }
     if (tid >= 2 * kH) {  // b1, b2
       const float* G = tid < 3 * kH ? H1 + (tid - 2 * kH) : H2 + (tid - 3 * kH);
       float acc = 0.f;
