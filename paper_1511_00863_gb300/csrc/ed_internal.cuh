@@ -332,8 +332,14 @@ template <> struct DotAcc<float> {
     const float s = hi + p;
     const float bb = s - hi;
     const float err = (hi - (s - bb)) + (p - bb);
-    hi = s;
-    lo += err + e;
+    const float l = lo + (err + e);
+    // renormalised (FastTwoSum): a low part that grows rounds off more at every product, and a CTA of
+    // the H.v gives a thread 20-1,700 of them. Equal products, relative error: 720 of them 6e-11 ->
+    // 6e-13, 1,740 3e-10 -> 1e-12 (72, one row group of the half-filled 16-site ring, 6e-13 -> 6e-14).
+    // Three additions: FP32 H.v of that ring 0.6% slower, complex FP32 1-2%. (Pairs per row group,
+    // summed in FP64 or as three FP32 terms, cost 7% and 2-3%.)
+    hi = s + l;
+    lo = l - (hi - s);
   }
   __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
 };
