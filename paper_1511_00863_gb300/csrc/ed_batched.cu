@@ -861,33 +861,6 @@ using namespace ed;
 
 namespace {
 
-// The FP32 vector store of batched mixed solves (Sum dim x max_steps x 4 bytes, gigabytes for
-// a large batch) comes from a per-device memory pool of the library whose release threshold
-// keeps the memory reserved after a solve frees it: a repeated solve does not map the store
-// again (mapping 12 GB took about 9 ms per call). Process-local; nothing outlasts the process.
-cudaMemPool_t vstore_pool() {
-  static std::mutex mu;
-  static std::map<int, cudaMemPool_t> pools;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-  std::lock_guard<std::mutex> lk(mu);
-  auto it = pools.find(dev);
-  if (it != pools.end()) return it->second;
-  cudaMemPoolProps props = {};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = dev;
-  cudaMemPool_t pool = nullptr;
-  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  uint64_t keep = UINT64_MAX;
-  cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-  pools[dev] = pool;
-  return pool;
-}
-
 // Layout of an instance's vectors: the row-ordered H.v where the basis has its tables (one hop
 // class) and a block of rows and its up-hop lists fit the staging area, with rows padded to 4
 // elements; else dense rows. Rows shorter than 96 columns leave most warps of the down part idle.
@@ -1184,8 +1157,7 @@ static ed_status solve_batched(int32_t n, const ed_basis* const* bases, const ed
     R.refine_tol = refine_tol;
     const size_t vbytes = total * (size_t)o->max_steps * sizeof(float);
     cudaMemPool_t pool = vstore_pool();
-    const cudaError_t ve = pool ? cudaMallocFromPoolAsync(&R.vstore, vbytes, pool, s)
-                                : cudaMalloc(&R.vstore, vbytes);
+    const cudaError_t ve = pool ? cudaMallocFromPoolAsync(&R.vstore, vbytes, pool, s) : cudaMalloc(&R.vstore, vbytes);
     if (ve != cudaSuccess) {
       cudaGetLastError();
       R.vstore = nullptr;

@@ -134,6 +134,11 @@ void lz_cache_free(const ed_basis* b);
 void psi_pool_basis(int delta);
 // That pool on the current device (NULL: not available); at most 16 GB stay in it while idle.
 cudaMemPool_t psi_pool();
+// The pool of the batched mixed solves' vector stores (keeps what it has while idle).
+cudaMemPool_t vstore_pool();
+// Bytes both pools hold idle on the current device. They are as good as free: the driver takes them
+// back from a pool when an allocation of the process would fail otherwise.
+uint64_t pools_idle();
 // Free the fused H.v down tables cached on a basis (called by ed_basis_destroy).
 void hv2_tables_free(const ed_basis* b);
 

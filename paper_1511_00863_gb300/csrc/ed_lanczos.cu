@@ -1149,19 +1149,20 @@ extern "C" ed_status ed_lanczos_solve(const ed_basis* b, const ed_params* p, con
 
 // ------------------------------------------------------------------ ground-state vector
 namespace ed {
-// Memory of the vectors a ground-state call keeps and of a batch's work: a pool per device, so that the next call
-// does not map the same gigabytes again (0.75 ms per GB). It holds at most kPsiKeep bytes while
-// idle and gives them back when the last basis is destroyed.
+// Two memory pools per device, so that the next call does not map the same gigabytes again (0.75 ms
+// per GB). psi: the vectors a ground-state call keeps and a batch's work; it holds at most kPsiKeep
+// bytes while idle and gives them back when the last basis is destroyed. vstore: the FP32 vector
+// stores of batched mixed solves (12 GB for 256 instances), kept in the process.
 constexpr uint64_t kPsiKeep = 16ull << 30;
 static std::mutex g_psi_mu;
-static cudaMemPool_t g_psi_pool[64] = {};
+static cudaMemPool_t g_psi_pool[64] = {}, g_vstore_pool[64] = {};
 static int64_t g_psi_bases = 0;
 
-cudaMemPool_t psi_pool() {
+static cudaMemPool_t lib_pool(cudaMemPool_t (&pools)[64], uint64_t keep) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
   std::lock_guard<std::mutex> lk(g_psi_mu);
-  if (g_psi_pool[dev]) return g_psi_pool[dev];
+  if (pools[dev]) return pools[dev];
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
@@ -1171,9 +1172,24 @@ cudaMemPool_t psi_pool() {
     cudaGetLastError();
     return nullptr;
   }
-  uint64_t keep = kPsiKeep;
   cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-  return g_psi_pool[dev] = pool;
+  return pools[dev] = pool;
+}
+cudaMemPool_t psi_pool() { return lib_pool(g_psi_pool, kPsiKeep); }
+cudaMemPool_t vstore_pool() { return lib_pool(g_vstore_pool, UINT64_MAX); }
+
+uint64_t pools_idle() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::lock_guard<std::mutex> lk(g_psi_mu);
+  uint64_t idle = 0;
+  for (cudaMemPool_t p : {g_psi_pool[dev], g_vstore_pool[dev]}) {
+    uint64_t reserved = 0, used = 0;
+    if (p && cudaMemPoolGetAttribute(p, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+        cudaMemPoolGetAttribute(p, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+      idle += reserved - used;
+  }
+  return idle;
 }
 
 void psi_pool_basis(int delta) {
@@ -1392,13 +1408,14 @@ extern "C" ed_status ed_lanczos_solve_mixed(const ed_basis* b, const ed_params* 
   ed_opts o32 = *o;
   o32.reorth = 3;
   {
-    // the FP32 phase keeps at most as many vectors as fit in half the free device memory
+    // the FP32 phase keeps at most as many vectors as fit in half the free device memory (and
+    // of what the library's pools hold idle)
     // and in 96 GB; a shorter FP32 phase leaves more of the convergence to the refinement
     // steps
     size_t free_b = 0, total_b = 0;
     ED_TRY_CUDA(cudaMemGetInfo(&free_b, &total_b));
     const double vbytes = (double)b->up.dim * (double)((b->dn.dim + 31) / 32 * 32) * 4.0;
-    const double budget = std::min((double)free_b / 2.0, 96e9);
+    const double budget = std::min(((double)free_b + (double)pools_idle()) / 2.0, 96e9);
     const int cap = (int)std::min(budget / vbytes - 1.0, (double)ED_MAX_STEPS);
     ED_CHECK_ARG(cap >= 2, "ed_lanczos_solve_mixed: device memory for FP32 vectors too small");
     if (o32.max_steps > cap) o32.max_steps = cap;
