@@ -1084,9 +1084,11 @@ static ed_status solve_on(ed_lanczos* st, const ed_basis* b, const ed_params* p,
 
 // Run fn(st) on the basis's cached state for opts o (allocated on first use), or on a
 // private state when another thread holds the cache; the work is ordered after the work
-// already queued on the caller's stream.
+// already queued on the caller's stream. A state made by this call whose work vectors take more than
+// keep_bytes is not kept.
 template <typename Fn>
-static ed_status with_state(const ed_basis* b, const ed_opts* o, cudaStream_t user, Fn fn) {
+static ed_status with_state(const ed_basis* b, const ed_opts* o, cudaStream_t user, Fn fn,
+                            double keep_bytes = INFINITY) {
   SolveCache* C = nullptr;
   {
     std::lock_guard<std::mutex> lk(g_cache_mu);
@@ -1120,6 +1122,11 @@ static ed_status with_state(const ed_basis* b, const ed_opts* o, cudaStream_t us
         st = e.st;
     if (!st) {
       if ((r = lz_alloc(b, o, s, &st)) != ED_OK) return r;
+      if (2.0 * (double)st->n * (double)st->esize > keep_bytes) {
+        r = fn(st);
+        ed_lanczos_destroy(st);
+        return r;
+      }
       C->entries.push_back({(int)o->dtype, o->schedule, o->reorth, slots, st});
     }
     return fn(st);
@@ -1256,6 +1263,10 @@ struct KeptVectors {
 
 }  // namespace
 
+// A ground-state call keeps its work vectors on the basis up to this size: larger ones leave the device
+// as free as the call found it, and making them again is 1% of the call (2 GB: 3 of 330 ms).
+constexpr double kGroundKeep = 1e9;
+
 // The run of st, whose scalars are in st->host, from f_k on again: buffers and scalars from the kept
 // vectors of f_{k-1} and f_k (k >= 2), the tridiagonal up to a_{k-1}, b_k from the first time.
 static ed_status lz_resume(ed_lanczos* st, int k, size_t vbytes, void* const* slot) {
@@ -1383,7 +1394,7 @@ extern "C" ed_status ed_lanczos_ground_state(const ed_basis* b, const ed_params*
   ED_CHECK_ARG(aligned16(psi), "ed_lanczos_ground_state: psi must be 16-byte aligned");
   return with_state(b, o, (cudaStream_t)stream, [&](ed_lanczos* st) {
     return ground_on(st, b, p, o, f1, (long long*)psi, E0, steps);
-  });
+  }, kGroundKeep);
 }
 
 extern "C" ed_status ed_lanczos_solve_mixed(const ed_basis* b, const ed_params* p,

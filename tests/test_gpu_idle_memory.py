@@ -1,5 +1,6 @@
 """Memory that the library's pools hold idle (vectors of earlier ground-state calls, stores of batched
-solves) counts as free: later calls get it, and nothing fails or is cut short for it."""
+solves) counts as free: later calls get it, nothing fails or is cut short for it, and a large
+ground-state call leaves no work vectors behind."""
 import pytest
 
 import ed_inputs
@@ -82,3 +83,21 @@ def test_batched_solve_gets_idle_memory(idle):
     finally:
         del hog
         ed.ed_basis_destroy(b)
+
+
+def test_large_ground_state_leaves_no_work_vectors():
+    import torch
+    import paper_1511_00863_gb300 as ed
+    b = ed.ed_build_basis(16, ed_inputs.ring_bonds(16), 8, 7)  # two vectors of 1.2 GB
+    try:
+        psi = torch.empty(ed.ed_basis_dims(b)[2], dtype=torch.float64, device="cuda")
+        hog = _hog(int(2.5 * psi.numel() * 8) + (256 << 20))  # no room for kept vectors: none idle afterwards
+        try:
+            before = _free()
+            ed.ed_lanczos_ground_state(b, 1.0, 4.0, ed.make_opts(max_steps=4, tol=0.0, seed=4), psi)
+            assert before - _free() <= 256 << 20
+        finally:
+            del hog
+    finally:
+        ed.ed_basis_destroy(b)
+        torch.cuda.empty_cache()
