@@ -162,17 +162,21 @@ static ed_status build_species(SpeciesTables& sp, int n_sites, int n, const int2
 // table): breadth-first search from a low-degree vertex of a far end (two sweeps), each
 // vertex's unvisited neighbours taken by increasing degree (ties by index), every
 // connected component in turn, the result reversed. Deterministic.
-static ed_status rcm_order(const SpeciesTables& sp, cudaStream_t s, std::vector<int32_t>& order) {
+// `beside` is called once the table is on the host: what it enqueues runs beside the search.
+template <typename Beside>
+static ed_status rcm_order(const SpeciesTables& sp, cudaStream_t s, std::vector<int32_t>& order, Beside beside) {
   const int64_t n = sp.dim;
   const int mh = sp.maxhops;
   order.resize(n);
   if (mh == 0 || n < 3) {
     for (int64_t i = 0; i < n; ++i) order[i] = (int32_t)i;
-    return ED_OK;
+    return beside();
   }
   std::vector<int32_t> tab((size_t)mh * n);
   ED_TRY_CUDA(cudaMemcpyAsync(tab.data(), sp.hop, tab.size() * 4, cudaMemcpyDeviceToHost, s));
   ED_TRY_CUDA(cudaStreamSynchronize(s));
+  const ed_status r = beside();
+  if (r != ED_OK) return r;
   std::vector<int32_t> deg(n, 0);
   auto nb = [&](int64_t v, int k) { return (int64_t)((uint32_t)tab[(size_t)k * n + v] & kTargetMask); };
   for (int64_t v = 0; v < n; ++v)
@@ -307,16 +311,20 @@ extern "C" ed_status ed_build_basis(const ed_lattice* L, int32_t n_up, int32_t n
     std::swap(B->up, B->dn);
     B->swapped = true;
   }
+  RowsPlan rows;
+  rows_plan(L->n_sites, n_up, n_dn, L->t_bond, L->n_bonds, rows);
+  auto row_tables = [&] { return rows_build(B, rows, s); };
+  std::vector<int32_t> order;
   if (B->up.dim <= kMaxOrderedRows && B->up.maxhops > 0) {
-    std::vector<int32_t> order;
-    if ((st = rcm_order(B->up, s, order)) != ED_OK) return fail(st);
+    if ((st = rcm_order(B->up, s, order, row_tables)) != ED_OK) return fail(st);
     if (cudaMalloc((void**)&B->up_order, order.size() * 4) != cudaSuccess ||
         cudaMemcpyAsync(B->up_order, order.data(), order.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) {
       set_error("ed_build_basis: row order upload failed");
       return fail(ED_ERR_CUDA);
     }
+  } else if ((st = row_tables()) != ED_OK) {
+    return fail(st);
   }
-  if ((st = rows_build(B, L->t_bond, s)) != ED_OK) return fail(st);
   if (cudaStreamSynchronize(s) != cudaSuccess) {
     set_error("ed_build_basis: %s", cudaGetErrorString(cudaGetLastError()));
     return fail(ED_ERR_CUDA);

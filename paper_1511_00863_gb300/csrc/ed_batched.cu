@@ -866,7 +866,7 @@ namespace {
 // elements; else dense rows. Rows shorter than 96 columns leave most warps of the down part idle.
 bool blayout_rows(const ed_basis* b) {
   const int64_t ld = (b->dn.dim + 3) / 4 * 4;
-  return b->rows.C == 1 && b->rows.ucnt == nullptr && b->dn.dim >= 96 && b->up.maxhops * 2 <= kBLists &&
+  return b->rows.C == 1 && b->rows.ucnt == nullptr && b->up.maxhops * 2 <= kBLists &&
          (2 * ld + 1) * 8 + 4 * kBLists <= kBRowFloats * 4;
 }
 int blayout_ld(const ed_basis* b) { return blayout_rows(b) ? (int)((b->dn.dim + 3) / 4 * 4) : (int)b->dn.dim; }

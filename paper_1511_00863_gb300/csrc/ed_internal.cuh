@@ -6,6 +6,7 @@
 
 #include <cstdarg>
 #include <cstdio>
+#include <vector>
 
 #include "ed.h"
 #include "ed_tables.h"  // hop-entry layout (kTargetMask, kSignBit)
@@ -52,6 +53,7 @@ struct SpeciesTables {
 // Tables of the row-ordered H.v (ed_rows.cu), built with the basis where its rows are short
 // enough; C = 0: none.
 constexpr int kMaxClasses = 16;
+constexpr int kMinRowCols = 96;  // shorter rows leave most of a CTA idle everywhere
 struct HvRows {
   int C = 0;                 // hop classes: distinct amplitudes up to sign
   int nchunks = 0;           // groups of 32 down columns
@@ -210,10 +212,18 @@ struct LzStore {
   long long* vmax;
 };
 
-// Row-ordered H.v (ed_rows.cu): tables built with the basis (t_bond: host amplitudes or NULL);
+// Row-ordered H.v (ed_rows.cu): tables built with the basis (rows_plan: classes of the host amplitudes
+// t_bond, or NULL; rows_build enqueues the rest);
 // E = float, double, float2 or double2 (complex). Preferred to launch_hv / launch_hvc where
 // rows_usable.
-ed_status rows_build(ed_basis* b, const double* t_bond, cudaStream_t s);
+struct RowsPlan {
+  int C = 0;                 // hop classes, 0: no tables
+  std::vector<double2> amp;  // [C]
+  std::vector<uint8_t> cls;  // amplitude number -> class | flip << 7 (empty: no amplitudes)
+  std::vector<char> host;    // the copy's source
+};
+void rows_plan(int n_sites, int n_up, int n_dn, const double* t_bond, int n_bonds, RowsPlan& p);
+ed_status rows_build(ed_basis* b, RowsPlan& p, cudaStream_t s);
 void rows_free(ed_basis* b);
 template <typename E>
 bool rows_usable(const ed_basis* b);

@@ -34,61 +34,151 @@
 namespace ed {
 
 // ------------------------------------------------------------------ tables
-// counts[s * C + c] = hops of state s in class c (cls: class | flip << 7 of an amplitude number;
-// NULL: class 0).
-__global__ void rows_count_kernel(const int32_t* __restrict__ hop, const int32_t* __restrict__ hopa,
-                                  const uint8_t* __restrict__ cls, int64_t dim, int maxhops, int C,
-                                  uint8_t* __restrict__ counts) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < dim; s += (int64_t)gridDim.x * blockDim.x) {
-    for (int c = 0; c < C; ++c) {
-      int n = 0;
-      for (int k = 0; k < maxhops; ++k) {
-        const uint32_t e = (uint32_t)hop[(int64_t)k * dim + s];
-        if ((int64_t)(e & kTargetMask) >= dim) break;
-        n += !cls || (cls[hopa[(int64_t)k * dim + s]] & 0x7F) == c;
-      }
-      counts[s * C + c] = (uint8_t)n;
+// f(class, entry with the amplitude's flip in its sign) for the hops of state s in table order (cls:
+// class | flip << 7 of an amplitude number; NULL: class 0), four loaded before the first is taken: one
+// state's list is a chain of dependent loads otherwise, 1 us a hop.
+template <typename F>
+__device__ __forceinline__ void for_hops(const int32_t* __restrict__ hop, const int32_t* __restrict__ hopa,
+                                         const uint8_t* __restrict__ cls, int64_t dim, int maxhops, int64_t s, F f) {
+  for (int k = 0; k < maxhops; k += 4) {
+    uint32_t e[4], m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) e[i] = k + i < maxhops ? (uint32_t)hop[(int64_t)(k + i) * dim + s] : (uint32_t)dim;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      m[i] = cls && (int64_t)(e[i] & kTargetMask) < dim ? cls[hopa[(int64_t)(k + i) * dim + s]] : 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if ((int64_t)(e[i] & kTargetMask) >= dim) return;
+      f((int)(m[i] & 0x7F), e[i] ^ (m[i] >> 7 << 31));
     }
+  }
+}
+
+constexpr int kRowsThreads = 128;
+
+// counts[s * C + c] = hops of state s in class c.
+__global__ void __launch_bounds__(kRowsThreads)
+rows_count_kernel(const int32_t* __restrict__ hop, const int32_t* __restrict__ hopa, const uint8_t* __restrict__ cls,
+                  int64_t dim, int maxhops, int C, uint8_t* __restrict__ counts) {
+  __shared__ uint8_t n[kMaxClasses][kRowsThreads];
+  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < dim; s += (int64_t)gridDim.x * blockDim.x) {
+    for (int c = 0; c < C; ++c) n[c][threadIdx.x] = 0;
+    for_hops(hop, hopa, cls, dim, maxhops, s, [&](int c, uint32_t) { ++n[c][threadIdx.x]; });
+    for (int c = 0; c < C; ++c) counts[s * C + c] = n[c][threadIdx.x];
   }
 }
 
 // Down table: per chunk of 32 columns and class the hops of perm's columns, kc[chunk * C + c] rows
 // of 32 entries (target, sign in bit 15; the zero column dim pads short lists).
-__global__ void rows_down_kernel(const int32_t* __restrict__ hop, const int32_t* __restrict__ hopa,
-                                 const uint8_t* __restrict__ cls, int64_t dim, int maxhops, int C,
-                                 const int32_t* __restrict__ perm, const int32_t* __restrict__ base,
-                                 const uint8_t* __restrict__ kc, int nchunks, uint16_t* __restrict__ tab) {
+__global__ void __launch_bounds__(kRowsThreads)
+rows_down_kernel(const int32_t* __restrict__ hop, const int32_t* __restrict__ hopa, const uint8_t* __restrict__ cls,
+                 int64_t dim, int maxhops, int C, const int32_t* __restrict__ perm, const int32_t* __restrict__ base,
+                 const uint8_t* __restrict__ kc, int nchunks, uint16_t* __restrict__ tab) {
+  __shared__ uint16_t at[kMaxClasses][kRowsThreads];  // the class's next row
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 32 * nchunks; i += gridDim.x * blockDim.x) {
     const int ch = i >> 5, d = perm[i];
     uint16_t* t = tab + base[ch] + (i & 31);
-    for (int c = 0; c < C; ++c) {
-      int n = 0;
-      for (int k = 0; k < maxhops && d >= 0; ++k) {
-        const uint32_t e = (uint32_t)hop[(int64_t)k * dim + d];
-        if ((int64_t)(e & kTargetMask) >= dim) break;
-        const uint8_t m = cls ? cls[hopa[(int64_t)k * dim + d]] : 0;
-        if ((m & 0x7F) != c) continue;
-        t[32 * n++] = (uint16_t)((e & kTargetMask) | (((e >> 31) ^ (m >> 7)) << 15));
-      }
-      for (; n < kc[ch * C + c]; ++n) t[32 * n] = (uint16_t)dim;
-      t += 32 * kc[ch * C + c];
+    for (int c = 0, row = 0; c < C; row += kc[ch * C + c], ++c) at[c][threadIdx.x] = (uint16_t)row;
+    if (d >= 0)
+      for_hops(hop, hopa, cls, dim, maxhops, d, [&](int c, uint32_t e) {
+        t[32 * at[c][threadIdx.x]++] = (uint16_t)((e & kTargetMask) | (e >> 31 << 15));
+      });
+    for (int c = 0, end = 0; c < C; ++c) {
+      end += kc[ch * C + c];
+      for (int row = at[c][threadIdx.x]; row < end; ++row) t[32 * row] = (uint16_t)dim;
     }
   }
 }
 
-// Up table with per-bond amplitudes: the hops of a row class by class, sign flips applied.
-__global__ void rows_up_kernel(const int32_t* __restrict__ hop, const int32_t* __restrict__ hopa,
-                               const uint8_t* __restrict__ cls, int64_t dim, int maxhops, int C,
-                               int32_t* __restrict__ out) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < dim; s += (int64_t)gridDim.x * blockDim.x) {
-    int n = 0;
-    for (int c = 0; c < C; ++c)
-      for (int k = 0; k < maxhops; ++k) {
-        const uint32_t e = (uint32_t)hop[(int64_t)k * dim + s];
-        if ((int64_t)(e & kTargetMask) >= dim) break;
-        const uint8_t m = cls[hopa[(int64_t)k * dim + s]];
-        if ((m & 0x7F) == c) out[(int64_t)n++ * dim + s] = (int32_t)(e ^ ((uint32_t)(m >> 7) << 31));
+// Exclusive sum of v over the CTA's threads (kSortThreads of them; sm: 32 words).
+constexpr int kSortThreads = 1024;
+__device__ __forceinline__ int block_scan(int v, int* sm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int in = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int w = __shfl_up_sync(0xffffffffu, in, o);
+    if (lane >= o) in += w;
+  }
+  if (lane == 31) sm[warp] = in;
+  __syncthreads();
+  int pre = lane < warp ? sm[lane] : 0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) pre += __shfl_xor_sync(0xffffffffu, pre, o);
+  __syncthreads();
+  return pre + in - v;
+}
+
+// Columns by their hop counts, descending, class 0 first, ties by rank (perm, -1 pads), then a
+// chunk's rows per class (kc) and start in the table (base). One CTA: a stable counting sort per class,
+// the last class first; a warp takes a run of columns, 32 at a time, ranked by __match_any_sync.
+__global__ void __launch_bounds__(kSortThreads)
+rows_sort_kernel(const uint8_t* __restrict__ counts, int nd, int C, int nchunks, int32_t* __restrict__ perm,
+                 int32_t* __restrict__ tmp, uint8_t* __restrict__ kc, int32_t* __restrict__ base) {
+  __shared__ int place[256][32];  // [255 - count][warp]: columns, then where the next one goes
+  __shared__ int sm[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int run = (nd + 32 * 32 - 1) / (32 * 32) * 32, i0 = warp * run, i1 = min(nd, i0 + run);
+  int* flat = &place[0][0];
+  for (int c = C - 1; c >= 0; --c) {
+    const int32_t* src = c & 1 ? perm : tmp;  // the last sort (class 0) writes perm
+    int32_t* dst = c & 1 ? tmp : perm;
+    for (int i = threadIdx.x; i < 256 * 32; i += kSortThreads) flat[i] = 0;
+    __syncthreads();
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int i = i0; i < i1; i += 32) {
+        const int q = i + lane;
+        const int d = q < i1 ? (c == C - 1 ? q : src[q]) : 0;
+        const int key = q < i1 ? 255 - counts[(int64_t)d * C + c] : 256;
+        const unsigned same = __match_any_sync(0xffffffffu, key);
+        int* p = key < 256 ? &place[key][warp] : nullptr;
+        if (pass && p) dst[*p + __popc(same & ((1u << lane) - 1u))] = d;
+        __syncwarp();
+        if (p && lane == __ffs(same) - 1) *p += __popc(same);
+        __syncwarp();
       }
+      __syncthreads();
+      if (pass) continue;
+      int v[8], sum = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) sum += v[k] = flat[8 * threadIdx.x + k];
+      int at = block_scan(sum, sm);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        flat[8 * threadIdx.x + k] = at;
+        at += v[k];
+      }
+      __syncthreads();
+    }
+  }
+  for (int i = nd + threadIdx.x; i < 32 * nchunks; i += kSortThreads) perm[i] = -1;
+  __syncthreads();
+  for (int ch = warp; ch < nchunks; ch += 32) {
+    const int d = perm[32 * ch + lane];
+    int rows = 0;
+    for (int c = 0; c < C; ++c) {
+      const unsigned n = __reduce_max_sync(0xffffffffu, d >= 0 ? (unsigned)counts[(int64_t)d * C + c] : 0u);
+      if (lane == 0) kc[ch * C + c] = (uint8_t)n;
+      rows += (int)n;
+    }
+    if (lane == 0) base[ch] = 32 * rows;
+  }
+  __syncthreads();
+  const int t = threadIdx.x, n = t < nchunks ? base[t] : 0;  // (nchunks <= 1,024: rows below 32,767 columns)
+  const int at = block_scan(n, sm);
+  if (t < nchunks) base[t] = at;
+}
+
+// Up table with per-bond amplitudes: the hops of a row class by class, sign flips applied.
+__global__ void __launch_bounds__(kRowsThreads)
+rows_up_kernel(const int32_t* __restrict__ hop, const int32_t* __restrict__ hopa, const uint8_t* __restrict__ cls,
+               int64_t dim, int maxhops, int C, const uint8_t* __restrict__ counts, int32_t* __restrict__ out) {
+  __shared__ uint16_t at[kMaxClasses][kRowsThreads];
+  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < dim; s += (int64_t)gridDim.x * blockDim.x) {
+    for (int c = 0, n = 0; c < C; n += counts[s * C + c], ++c) at[c][threadIdx.x] = (uint16_t)n;
+    for_hops(hop, hopa, cls, dim, maxhops, s,
+             [&](int c, uint32_t e) { out[(int64_t)at[c][threadIdx.x]++ * dim + s] = (int32_t)e; });
   }
 }
 
@@ -97,112 +187,84 @@ void rows_free(ed_basis* b) {
   b->rows = HvRows();
 }
 
-ed_status rows_build(ed_basis* b, const double* t_bond, cudaStream_t s) {
-  const int64_t nd = b->dn.dim, nu = b->up.dim;
-  if (nu < kMinRowsStaged || nd >= 0x7FFF || b->dn.maxhops > 255 || b->up.maxhops > 255) return ED_OK;
-  // ---- classes: distinct amplitudes up to sign (amplitude number 2 q: tau_q, 2 q + 1: its
-  // conjugate, the gather amplitudes over -t)
-  std::vector<double2> amp;
-  std::vector<uint8_t> cls;
+// Classes: distinct amplitudes up to sign (amplitude number 2 q: tau_q, 2 q + 1: its conjugate, the
+// gather amplitudes over -t). p.C = 0: no tables for this basis.
+void rows_plan(int n_sites, int n_up, int n_dn, const double* t_bond, int n_bonds, RowsPlan& p) {
   if (t_bond) {
-    cls.resize(2 * (size_t)b->n_bonds);
-    for (size_t i = 0; i < cls.size(); ++i) {
+    p.cls.resize(2 * (size_t)n_bonds);
+    for (size_t i = 0; i < p.cls.size(); ++i) {
       const double re = t_bond[2 * (i / 2)], im = (i & 1) ? -t_bond[2 * (i / 2) + 1] : t_bond[2 * (i / 2) + 1];
       size_t c = 0;
-      while (c < amp.size() && !(amp[c].x == re && amp[c].y == im) && !(amp[c].x == -re && amp[c].y == -im)) ++c;
-      if (c == amp.size()) amp.push_back(make_double2(re, im));
-      cls[i] = (uint8_t)(c | (amp[c].x == re && amp[c].y == im ? 0 : 0x80));
-      if (amp.size() > kMaxClasses) return ED_OK;  // too many to pay: the plain kernels
+      while (c < p.amp.size() && !(p.amp[c].x == re && p.amp[c].y == im) && !(p.amp[c].x == -re && p.amp[c].y == -im))
+        ++c;
+      if (c == p.amp.size()) p.amp.push_back(make_double2(re, im));
+      p.cls[i] = (uint8_t)(c | (p.amp[c].x == re && p.amp[c].y == im ? 0 : 0x80));
+      if (p.amp.size() > kMaxClasses) return;  // too many to pay: the plain kernels
     }
-  }
-  if (amp.empty()) amp.push_back(make_double2(1.0, 0.0));
-  const int C = (int)amp.size();
-  const int nch = (int)((nd + 31) / 32);
-  // ---- hop counts per class, then columns sorted by them
-  uint8_t* d_cls = nullptr;
-  uint8_t* d_cnt = nullptr;
-  std::vector<uint8_t> cnt((size_t)nd * C), ucnt(t_bond ? (size_t)nu * C : 0);
-  struct Release {
-    uint8_t *&a, *&b;
-    ~Release() {
-      if (a) cudaFree(a);
-      if (b) cudaFree(b);
-    }
-  } release{d_cls, d_cnt};
-  if (!cls.empty()) {
-    ED_TRY_CUDA(cudaMalloc((void**)&d_cls, cls.size()));
-    ED_TRY_CUDA(cudaMemcpyAsync(d_cls, cls.data(), cls.size(), cudaMemcpyHostToDevice, s));
-  }
-  ED_TRY_CUDA(cudaMalloc((void**)&d_cnt, cnt.size() + ucnt.size()));
-  auto grid = [](int64_t n) { return (unsigned)std::min<int64_t>((n + 127) / 128, 1024); };
-  rows_count_kernel<<<grid(nd), 128, 0, s>>>(b->dn.hop, b->dn.hopa, d_cls, nd, b->dn.maxhops, C, d_cnt);
-  if (t_bond)
-    rows_count_kernel<<<grid(nu), 128, 0, s>>>(b->up.hop, b->up.hopa, d_cls, nu, b->up.maxhops, C, d_cnt + cnt.size());
-  ED_TRY_CUDA(cudaGetLastError());
-  ED_TRY_CUDA(cudaMemcpyAsync(cnt.data(), d_cnt, cnt.size(), cudaMemcpyDeviceToHost, s));
-  if (t_bond)
-    ED_TRY_CUDA(cudaMemcpyAsync(ucnt.data(), d_cnt + cnt.size(), ucnt.size(), cudaMemcpyDeviceToHost, s));
-  ED_TRY_CUDA(cudaStreamSynchronize(s));
-  if (t_bond) {
     // per element: 2 additions per hop and 4 multiply-adds per class and species, against 4
     // multiply-adds per hop of the plain kernels: taken while the classes cost no more than the
-    // additions save (4 classes for 73 hops on the checkerboard-type lattice)
-    const double hops = std::accumulate(cnt.begin(), cnt.end(), 0.0) / (double)nd +
-                        std::accumulate(ucnt.begin(), ucnt.end(), 0.0) / (double)nu;
-    if (8.0 * C > 2.0 * hops) return ED_OK;
+    // additions save (4 classes for 73 hops on the checkerboard-type lattice). A bond's ends are
+    // occupied differently, so it hops, in 2 n (L - n) / (L (L - 1)) of a species' states.
+    const double L = n_sites, pairs = L > 1 ? L * (L - 1) : 1;
+    const double hops = 2.0 * n_bonds * (n_up * (L - n_up) + n_dn * (L - n_dn)) / pairs;
+    if (8.0 * (double)p.amp.size() > 2.0 * hops && !p.amp.empty()) return;
   }
-  std::vector<int32_t> perm(32 * (size_t)nch, -1), base(nch);
-  if (C == 1) {
-    std::vector<int32_t> start(257, 0);
-    for (uint8_t n : cnt) ++start[256 - n];
-    for (int n = 1; n <= 256; ++n) start[n] += start[n - 1];
-    for (int64_t d = 0; d < nd; ++d) perm[start[255 - cnt[d]]++] = (int32_t)d;
-  } else {
-    std::iota(perm.begin(), perm.begin() + nd, 0);
-    std::stable_sort(perm.begin(), perm.begin() + nd, [&](int32_t x, int32_t y) {
-      return memcmp(&cnt[(size_t)x * C], &cnt[(size_t)y * C], C) > 0;
-    });
-  }
-  std::vector<uint8_t> kc((size_t)nch * C, 0);
-  int32_t total = 0;
-  for (int ch = 0; ch < nch; ++ch) {
-    base[ch] = total;
-    for (int l = 0; l < 32; ++l)
-      for (int c = 0; c < C && perm[32 * ch + l] >= 0; ++c)
-        kc[(size_t)ch * C + c] = std::max(kc[(size_t)ch * C + c], cnt[(size_t)perm[32 * ch + l] * C + c]);
-    for (int c = 0; c < C; ++c) total += 32 * kc[(size_t)ch * C + c];
-  }
-  // ---- one allocation for everything
+  if (p.amp.empty()) p.amp.push_back(make_double2(1.0, 0.0));
+  p.C = (int)p.amp.size();
+}
+
+// Enqueue the tables: five launches and a copy at most, no wait (p and t_bond's classes stay until s
+// has passed them). Sorted on the host, with the counts' way there and back, they made ed_build_basis
+// 4-8% longer, 20% with amplitudes; so they are made beside the host's work on the row order.
+ed_status rows_build(ed_basis* b, RowsPlan& p, cudaStream_t s) {
+  const int64_t nd = b->dn.dim, nu = b->up.dim;
+  if (p.C == 0 || nu < kMinRowsStaged || nd < kMinRowCols || nd >= 0x7FFF || b->dn.maxhops > 255 || b->up.maxhops > 255)
+    return ED_OK;
+  const int C = p.C, nch = (int)((nd + 31) / 32);
+  const bool amps = !p.cls.empty();
+  // one allocation: amplitudes and classes (from the host), the counts and the sort's second buffer,
+  // the tables. A chunk has a row per hop of a class at most, a bond one hop.
   HvRows& r = b->rows;
   auto up16 = [](size_t n) { return (n + 15) / 16 * 16; };
-  const size_t o_amp = 0, o_perm = up16(o_amp + C * sizeof(double2)), o_base = up16(o_perm + perm.size() * 4),
-               o_kc = up16(o_base + base.size() * 4), o_tab = up16(o_kc + kc.size()),
-               o_ucnt = up16(o_tab + (size_t)total * 2), o_up = up16(o_ucnt + ucnt.size()),
-               bytes = o_up + (t_bond ? (size_t)b->up.maxhops * nu * 4 : 0);
-  ED_TRY_CUDA(cudaMalloc(&r.mem, bytes + 16));
+  const size_t rows = (size_t)nch * (amps ? std::min(C * b->dn.maxhops, b->n_bonds) : b->dn.maxhops);
+  const size_t o_cls = up16(C * sizeof(double2)), o_cnt = up16(o_cls + p.cls.size()), o_ucnt = up16(o_cnt + nd * C),
+               o_tmp = up16(o_ucnt + (amps ? nu * C : 0)), o_perm = up16(o_tmp + nd * 4),
+               o_base = up16(o_perm + 32 * (size_t)nch * 4), o_kc = up16(o_base + nch * 4),
+               o_tab = up16(o_kc + (size_t)nch * C), o_up = up16(o_tab + rows * 64),
+               bytes = o_up + (amps ? (size_t)b->up.maxhops * nu * 4 : 0);
+  const cudaError_t e = cudaMalloc(&r.mem, bytes + 16);
+  if (e == cudaErrorMemoryAllocation) {  // the basis goes without (the row-staged kernels serve it)
+    cudaGetLastError();
+    r.mem = nullptr;
+    return ED_OK;
+  }
+  ED_TRY_CUDA(e);
   char* m = (char*)r.mem;
-  r.amp = (double2*)(m + o_amp);
+  uint8_t* cls = amps ? (uint8_t*)(m + o_cls) : nullptr;
+  uint8_t* cnt = (uint8_t*)(m + o_cnt);
+  r.amp = (double2*)m;
+  r.ucnt = amps ? (uint8_t*)(m + o_ucnt) : nullptr;
   r.perm = (int32_t*)(m + o_perm);
   r.base = (int32_t*)(m + o_base);
   r.kc = (uint8_t*)(m + o_kc);
   r.tab = (uint16_t*)(m + o_tab);
-  r.ucnt = t_bond ? (uint8_t*)(m + o_ucnt) : nullptr;
-  r.up = t_bond ? (int32_t*)(m + o_up) : b->up.hop;
+  r.up = amps ? (int32_t*)(m + o_up) : b->up.hop;
   r.nchunks = nch;
-  // (the host arrays outlive the copies: the stream is synchronised before they go)
-  ED_TRY_CUDA(cudaMemcpyAsync(r.amp, amp.data(), C * sizeof(double2), cudaMemcpyHostToDevice, s));
-  ED_TRY_CUDA(cudaMemcpyAsync(r.perm, perm.data(), perm.size() * 4, cudaMemcpyHostToDevice, s));
-  ED_TRY_CUDA(cudaMemcpyAsync(r.base, base.data(), base.size() * 4, cudaMemcpyHostToDevice, s));
-  ED_TRY_CUDA(cudaMemcpyAsync(r.kc, kc.data(), kc.size(), cudaMemcpyHostToDevice, s));
-  rows_down_kernel<<<grid(32 * (int64_t)nch), 128, 0, s>>>(b->dn.hop, b->dn.hopa, d_cls, nd, b->dn.maxhops, C,
-                                                           r.perm, r.base, r.kc, nch, r.tab);
-  if (t_bond) {
-    ED_TRY_CUDA(cudaMemcpyAsync(r.ucnt, ucnt.data(), ucnt.size(), cudaMemcpyHostToDevice, s));
-    rows_up_kernel<<<grid(nu), 128, 0, s>>>(b->up.hop, b->up.hopa, d_cls, nu, b->up.maxhops, C, r.up);
+  p.host.resize(o_cnt);
+  memcpy(p.host.data(), p.amp.data(), C * sizeof(double2));
+  if (amps) memcpy(&p.host[o_cls], p.cls.data(), p.cls.size());
+  ED_TRY_CUDA(cudaMemcpyAsync(m, p.host.data(), o_cnt, cudaMemcpyHostToDevice, s));
+  auto grid = [](int64_t n) { return (unsigned)std::min<int64_t>((n + kRowsThreads - 1) / kRowsThreads, 1024); };
+  rows_count_kernel<<<grid(nd), kRowsThreads, 0, s>>>(b->dn.hop, b->dn.hopa, cls, nd, b->dn.maxhops, C, cnt);
+  rows_sort_kernel<<<1, kSortThreads, 0, s>>>(cnt, (int)nd, C, nch, r.perm, (int32_t*)(m + o_tmp), r.kc, r.base);
+  rows_down_kernel<<<grid(32 * (int64_t)nch), kRowsThreads, 0, s>>>(b->dn.hop, b->dn.hopa, cls, nd, b->dn.maxhops, C,
+                                                                    r.perm, r.base, r.kc, nch, r.tab);
+  if (amps) {
+    rows_count_kernel<<<grid(nu), kRowsThreads, 0, s>>>(b->up.hop, b->up.hopa, cls, nu, b->up.maxhops, C, r.ucnt);
+    rows_up_kernel<<<grid(nu), kRowsThreads, 0, s>>>(b->up.hop, b->up.hopa, cls, nu, b->up.maxhops, C, r.ucnt, r.up);
   }
   ED_TRY_CUDA(cudaGetLastError());
-  ED_TRY_CUDA(cudaStreamSynchronize(s));
-  r.C = C;  // usable from here on
+  r.C = C;
   return ED_OK;
 }
 
@@ -502,7 +564,7 @@ static ed_status rows_launch(const ed_basis* b, const RowsArgs& a, const E* x, E
 template <typename E>
 bool rows_usable(const ed_basis* b) {
   const int64_t nd = b->dn.dim, nu = b->up.dim, sms = sm_count();
-  if (b->rows.C == 0 || nd < 96 || rows_smem<E, 1>(b) + 4096 > (size_t)smem_optin_max()) return false;
+  if (b->rows.C == 0 || rows_smem<E, 1>(b) + 4096 > (size_t)smem_optin_max()) return false;
   if constexpr (std::is_same<E, float>::value)
     return nd % 4 == 0 ? nd >= 500 || (nd >= 240 && nu <= 4 * sms)
                        : nd >= 5000 || (nd >= 1200 && nu >= 8 * sms) || (nd >= 240 && nu <= 4 * sms);
