@@ -26,7 +26,8 @@ struct Hv2Plan {
   uchar2* kpn = nullptr;      // per chunk of 32 V columns: positive, negative table rows
   uint8_t* slot_lo = nullptr;  // per column: slot within its group of G
   uint32_t* dn_pad = nullptr;  // down bits by column
-  int32_t* colpos = nullptr;  // column of each down rank
+  int32_t* colpos = nullptr;  // column of each down rank [dim_dn], then the down rank of each column
+  int32_t* rank = nullptr;    // [ld], -1 for a pad (colpos + dim_dn)
   int cst[3] = {0, 0, 0};     // split-row plans: slice starts
   int nslots = 0;             // split-row plans: shared-memory slots (longest slice + G)
   uint16_t* xtab = nullptr;   // split-row plans: cross-slice rows
@@ -156,15 +157,23 @@ static ed_status compute_down_tables(const ed_basis* b, int ld, const KindInfo& 
                            ld, ki.V, ki.G, cplx, out);
 }
 
+// The host copy of a plan's colpos and rank.
+static std::vector<int32_t> plan_columns(const std::vector<int32_t>& pos, int64_t n, int ld) {
+  std::vector<int32_t> h((size_t)n + ld, -1);
+  for (int64_t i = 0; i < n; ++i) h[n + (h[i] = pos[i])] = (int32_t)i;
+  return h;
+}
+
 static ed_status upload_down_tables(const DownTables& t, int64_t n, cudaStream_t s, Hv2Plan* p) {
   const int ld = t.ld;
   const size_t tbytes = t.cplx ? t.tab32.size() * 4 : t.tab.size() * 2;
+  const std::vector<int32_t> cols = plan_columns(t.pos, n, ld);
   const void* tdata = t.cplx ? (const void*)t.tab32.data() : (const void*)t.tab.data();
   if (cudaMalloc(&p->dtab, tbytes) != cudaSuccess ||
       cudaMalloc((void**)&p->kpn, t.kpn.size()) != cudaSuccess ||
       cudaMalloc((void**)&p->slot_lo, (size_t)ld) != cudaSuccess ||
       cudaMalloc((void**)&p->dn_pad, (size_t)ld * 4) != cudaSuccess ||
-      cudaMalloc((void**)&p->colpos, (size_t)(n > 0 ? n : 1) * 4) != cudaSuccess) {
+      cudaMalloc((void**)&p->colpos, cols.size() * 4) != cudaSuccess) {
     set_error("H.v tables: out of device memory");
     return ED_ERR_OOM;
   }
@@ -172,7 +181,8 @@ static ed_status upload_down_tables(const DownTables& t, int64_t n, cudaStream_t
   ED_TRY_CUDA(cudaMemcpyAsync(p->kpn, t.kpn.data(), t.kpn.size(), cudaMemcpyHostToDevice, s));
   ED_TRY_CUDA(cudaMemcpyAsync(p->slot_lo, t.lo.data(), t.lo.size(), cudaMemcpyHostToDevice, s));
   ED_TRY_CUDA(cudaMemcpyAsync(p->dn_pad, t.pad.data(), t.pad.size() * 4, cudaMemcpyHostToDevice, s));
-  ED_TRY_CUDA(cudaMemcpyAsync(p->colpos, t.pos.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s));
+  ED_TRY_CUDA(cudaMemcpyAsync(p->colpos, cols.data(), cols.size() * 4, cudaMemcpyHostToDevice, s));
+  p->rank = p->colpos + n;
   ED_TRY_CUDA(cudaStreamSynchronize(s));
   return ED_OK;
 }
@@ -301,12 +311,13 @@ static ed_status hv2_build_split(const ed_basis* b, int mode, int ld, cudaStream
   p->nslots = split_slots(*t);
   for (int i = 0; i < 3; ++i) p->cst[i] = t->cstart[i];
   const int64_t n = b->dn.dim;
+  const std::vector<int32_t> cols = plan_columns(t->pos, n, ld);
   if (cudaMalloc(&p->dtab, t->tab.size() * 2) != cudaSuccess ||
       cudaMalloc((void**)&p->xtab, t->xtab.size() * 2) != cudaSuccess ||
       cudaMalloc((void**)&p->kpn, t->kpn.size()) != cudaSuccess ||
       cudaMalloc((void**)&p->slot_lo, (size_t)ld) != cudaSuccess ||
       cudaMalloc((void**)&p->dn_pad, (size_t)ld * 4) != cudaSuccess ||
-      cudaMalloc((void**)&p->colpos, (size_t)(n > 0 ? n : 1) * 4) != cudaSuccess) {
+      cudaMalloc((void**)&p->colpos, cols.size() * 4) != cudaSuccess) {
     cudaGetLastError();
     hv2_free(p);
     set_error("H.v split tables: out of device memory");
@@ -317,7 +328,8 @@ static ed_status hv2_build_split(const ed_basis* b, int mode, int ld, cudaStream
   if (e == cudaSuccess) e = cudaMemcpyAsync(p->kpn, t->kpn.data(), t->kpn.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(p->slot_lo, t->lo.data(), (size_t)ld, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(p->dn_pad, t->pad.data(), (size_t)ld * 4, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p->colpos, t->pos.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(p->colpos, cols.data(), cols.size() * 4, cudaMemcpyHostToDevice, s);
+  p->rank = p->colpos + n;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
 #define HV2S_ATTR(K, E, V_, T, MB) \
   if (e == cudaSuccess && p->kind == K) e = allow_max_smem(hv2s_kernel<E, V_, T, MB>);
@@ -398,6 +410,7 @@ ed_status hv2_build(const ed_basis* b, int mode, int ld, int schedule, cudaStrea
 }
 
 const int32_t* hv2_colpos(const Hv2Plan* p) { return p ? p->colpos : nullptr; }
+const int32_t* hv2_rank(const Hv2Plan* p) { return p ? p->rank : nullptr; }
 
 int hv2_grid(const Hv2Plan* p) { return p ? p->grid : 0; }
 bool hv2_ticket(const Hv2Plan* p) { return p && p->ticket; }

@@ -318,6 +318,8 @@ bool hv2_ticket(const Hv2Plan* p);
 int hv2_split_ld(const ed_basis* b, int mode, int schedule, cudaStream_t s);
 // Column of each down rank in the plan's row layout (device, dim_dn entries).
 const int32_t* hv2_colpos(const Hv2Plan* p);
+// ... and the down rank of each column (-1: a pad) of the plan's [ld] columns.
+const int32_t* hv2_rank(const Hv2Plan* p);
 int hv2_kind(const Hv2Plan* p);
 // Time every fused H.v variant that fits on x (f_j) and y (f_{j-1} / w) with scalars S
 // (zeroed: a neutral step) and return the fastest variant id (0 if none fits).

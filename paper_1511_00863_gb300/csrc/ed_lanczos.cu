@@ -186,14 +186,10 @@ fx_copy_in_kernel(const double* __restrict__ f, RowRuns L, int vb, int E, long l
   fx_block_reduce(a192_get(acc), mx, part + 4 * blockIdx.x);
 }
 
-// rank[p] = the down rank at column p, -1 for a pad.
-__global__ void rank_kernel(const int32_t* __restrict__ colpos, int64_t cols, int64_t ld,
-                            int32_t* __restrict__ rank, int pads) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (pads ? ld : cols);
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (pads) rank[i] = -1;
-    else rank[colpos ? colpos[i] : i] = (int32_t)i;
-  }
+// The rank table of rank order: column p is rank p, -1 for a pad.
+__global__ void rank_kernel(int64_t cols, int64_t ld, int32_t* __restrict__ rank) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ld; i += (int64_t)gridDim.x * blockDim.x)
+    rank[i] = i < cols ? (int32_t)i : -1;
 }
 
 __global__ void init_scalars_kernel(LzScalars* S, const double* __restrict__ partial,
@@ -401,7 +397,7 @@ struct ed_lanczos {
   LzStore store{nullptr, nullptr, nullptr};  // where the update pass keeps the vectors
   cudaGraphExec_t graph[4] = {};  // without / with the convergence test, + 2: vectors kept in `slots`
   // ground-state vectors only: slot table, scales and maxima of the kept vectors, y of T_m with
-  // the inverse iteration's work, ranks by column
+  // the inverse iteration's work, ranks by column without a plan
   void** slots = nullptr;
   double* vscale = nullptr;
   long long* vmax = nullptr;
@@ -607,19 +603,18 @@ extern "C" void ed_lanczos_destroy(ed_lanczos* st) {
 // variant would cost more than their solves.
 constexpr int64_t kAutotuneMinDim = (int64_t)1 << 22;
 
-// The state's table of ranks by column (built on first use).
-static ed_status lz_rank(ed_lanczos* st) {
-  if (st->rank) return ED_OK;
+// The state's table of ranks by column: its plan's, or of rank order (built on first use).
+static ed_status lz_rank(ed_lanczos* st, const int32_t** out) {
+  if ((*out = hv2_rank(st->plan)) != nullptr || (*out = st->rank) != nullptr) return ED_OK;
   if (cudaMalloc((void**)&st->rank, (size_t)st->ld * sizeof(int32_t)) != cudaSuccess) {
     cudaGetLastError();
     st->rank = nullptr;
     set_error("Lanczos column ranks: out of device memory");
     return ED_ERR_OOM;
   }
-  const int g = red_grid(st->ld);
-  rank_kernel<<<g, kRedThreads, 0, st->stream>>>(hv2_colpos(st->plan), st->basis->dn.dim, st->ld, st->rank, 1);
-  rank_kernel<<<g, kRedThreads, 0, st->stream>>>(hv2_colpos(st->plan), st->basis->dn.dim, st->ld, st->rank, 0);
+  rank_kernel<<<red_grid(st->ld), kRedThreads, 0, st->stream>>>(st->basis->dn.dim, st->ld, st->rank);
   ED_TRY_CUDA(cudaGetLastError());
+  *out = st->rank;
   return ED_OK;
 }
 
@@ -698,15 +693,11 @@ static ed_status lz_alloc(const ed_basis* b, const ed_opts* o, cudaStream_t s, e
     ed_status pr = hv2_build(b, mode, (int)st->ld, sched, s, &st->plan);
     if (pr != ED_OK) return fail(pr);
   }
-  // pads hold 0 from here on: every pass writes 0 there or leaves them
-  for (int i = 0; i < 2; ++i)
-    if (cudaMemsetAsync(st->B[i], 0, st->n * st->esize, s) != cudaSuccess) {
-      set_error("Lanczos work vectors: clearing failed");
-      return fail(ED_ERR_CUDA);
-    }
-  if (st->plan) {
-    const ed_status rr = lz_rank(st);
-    if (rr != ED_OK) return fail(rr);
+  // pads hold 0: lz_reset writes buffer 0 with its pads and clears buffer 1 in floating point; in
+  // fixed point that stays cleared from here on (every pass writes 0 into pads or leaves them)
+  if (st->fx && cudaMemsetAsync(st->B[1], 0, st->n * st->esize, s) != cudaSuccess) {
+    set_error("Lanczos work vectors: clearing failed");
+    return fail(ED_ERR_CUDA);
   }
   *out = st;
   return ED_OK;
@@ -746,7 +737,7 @@ static ed_status lz_reset(ed_lanczos* st, const ed_opts* o, const void* f1) {
   ED_CHECK_ARG((int64_t)g <= st->npb, "internal: partial buffer too small");
   st->cur = 0;
   // rank order (general kernels) without a plan
-  const RowRuns L = row_runs(b->up.dim, b->dn.dim, st->ld, cx, st->plan ? st->rank : nullptr);
+  const RowRuns L = row_runs(b->up.dim, b->dn.dim, st->ld, cx, hv2_rank(st->plan));
   if (st->fx) {
     long long* part = (long long*)st->pb;
     if (f1 == nullptr) {
@@ -1309,7 +1300,8 @@ static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p
       return ED_ERR_OOM;
     }
   }
-  ed_status r = lz_rank(st);
+  const int32_t* rank = nullptr;
+  ed_status r = lz_rank(st, &rank);
   if (r == ED_OK) r = lz_reset(st, o, f1);
   if (r != ED_OK) return r;
   if ((r = fx_prepare(b)) != ED_OK) return r;
@@ -1347,7 +1339,7 @@ static ed_status ground_on(ed_lanczos* st, const ed_basis* b, const ed_params* p
     have = own ? std::min(kept.ready, m) : m;
     if (have < std::min(m, 2)) have = 0;  // (a run goes on from two vectors)
     if (have > 0 &&
-        (r = fx_psi_sum(b, y, have, own ? st->store : ro_slots(st->ro), st->ld, st->rank, P, (long long*)st->pb, s)) != ED_OK)
+        (r = fx_psi_sum(b, y, have, own ? st->store : ro_slots(st->ro), st->ld, rank, P, (long long*)st->pb, s)) != ED_OK)
       return r;
     if (have > 0 && have < m) {
       void* const last[2] = {kept.slot(have - 1), kept.slot(have - 2)};
