@@ -90,8 +90,10 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 // tcgen05.ld and applies
 // bias (CUDA cores) and tanh (special-function unit); the 64 -> 2 output layer stays on the
 // CUDA cores. 128 tanh per state on the special-function unit (16 per cycle and SM) are 0.31 ms for
-// 11.8 M states; the other instructions have to fit beside them: features come from a table of
-// bytes (16 bytes of operand per load), additions and the output layer go two at a time, states are
+// 11.8 M states; the other instructions have to fit beside them: features come from a table
+// of four-bit groups (8 bytes of operand per load; a table of bytes took 4 KB of every CTA, and with
+// it a resident CTA from 16 sites on: 16 sites 834 -> 810 us for 19 M states, 32 sites 1,279 -> 1,167
+// for 25 M, 14 sites 505 -> 503 for 11.8 M), additions and the output layer go two at a time, states are
 // carried from tile to tile without a division.
 // Waits on the mbarrier are bounded (1 s of the global timer); on expiry the kernel sets
 // *err, frees its TMEM and returns.
@@ -123,7 +125,7 @@ __host__ __device__ inline TcLayout tc_layout(int nin) {
   t.b2 = up(t.b1 + (uint32_t)kH * t.K1 * 2, 1024);
   t.par = up(t.b2 + (uint32_t)kH * kH * 2, 1024);
   t.lut = up(t.par + (uint32_t)(4 * kH + 2) * 4, 16);
-  t.mbar = t.lut + 256 * 16;
+  t.mbar = t.lut + 16 * 8;
   t.tslot = t.mbar + 8;
   t.total = up(t.tslot + 8, 1024);
   return t;
@@ -146,7 +148,7 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
   float* sb2 = sb1 + kH;
   float* sW3 = sb2 + kH;
   float* sb3 = sW3 + 2 * kH;
-  uint4* lut = reinterpret_cast<uint4*>(tsm + ly.lut);
+  uint2* lut = reinterpret_cast<uint2*>(tsm + ly.lut);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(tsm + ly.tslot);
   const uint32_t mbar = smem_addr(tsm + ly.mbar);
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -169,10 +171,10 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
     sW3[2 * i + 1] = bf16r(params[d.oW3 + 2 * i + 1]);
   }
   if (tid < 2) sb3[tid] = bf16r(params[d.ob3 + tid]);
-  // the bf16 features (0 or 1) of every byte
-  for (int i = tid; i < 256; i += blockDim.x) {
-    auto pair = [&](int k) { return ((i >> k) & 1 ? 0x3F80u : 0u) | ((i >> (k + 1)) & 1 ? 0x3F800000u : 0u); };
-    lut[i] = make_uint4(pair(0), pair(2), pair(4), pair(6));
+  // the bf16 features (0 or 1) of every four bits: 128 bytes, one to each bank
+  if (tid < 16) {
+    auto pair = [&](int k) { return ((tid >> k) & 1 ? 0x3F80u : 0u) | ((tid >> (k + 1)) & 1 ? 0x3F800000u : 0u); };
+    lut[tid] = make_uint2(pair(0), pair(2));
   }
   if (tid == 0) mbar_init(mbar, 1);
   if (warp == 0) tc_alloc(smem_addr(tslot), kTcCols);
@@ -206,11 +208,13 @@ mlp_infer_tc_kernel(const float* __restrict__ params, int L, float U, const uint
       ub = upb[u];
       db = dnb[dd];
     }
-    // the bits of both species in feature order, eight features (16 bytes) per table entry; the U
-    // feature (2 L) comes after them, zeros to K1
+    // the bits of both species in feature order, eight features (16 bytes) from two table entries; the
+    // U feature (2 L) comes after them, zeros to K1
     const unsigned long long bits = (unsigned long long)ub | ((unsigned long long)db << L);
     for (int j = 0; j < K1; j += 8) {
-      uint4 w = lut[j < 64 ? (bits >> j) & 0xFFu : 0u];
+      const uint32_t f8 = j < 64 ? (uint32_t)(bits >> j) & 0xFFu : 0u;
+      const uint2 lo = lut[f8 & 15u], hi = lut[f8 >> 4];
+      uint4 w = make_uint4(lo.x, lo.y, hi.x, hi.y);
       if (j == (2 * L & ~7)) {
         const uint32_t v = u8bits << (16 * (2 * L & 1));
         const int q = (2 * L & 7) >> 1;
