@@ -216,7 +216,7 @@ static int global_grid(const ed_basis* b) {
 template <typename T, bool kLz>
 static ed_status launch_any(const ed_basis* b, const HvArgs& a, const T* x, T* y,
                             cudaStream_t s, const LzHvArgs& lz, int* grid_out) {
-  if (rows_usable<T>(b)) return launch_hv_rows<T>(b, a.t, a.U, x, y, a.ld, s, kLz ? &lz : nullptr, grid_out);
+  if (rows_usable<T>(b, kLz)) return launch_hv_rows<T>(b, a.t, a.U, x, y, a.ld, s, kLz ? &lz : nullptr, grid_out);
   const size_t lim = (size_t)max_smem_optin();
   const bool rows = b->up.dim >= kMinRowsStaged;
   if (rows && staged_smem<T, 2>(b) <= lim) return launch_staged<T, 2, kLz>(a, b, x, y, s, lz, grid_out);
@@ -246,7 +246,7 @@ static ed_status set_smem_attr(const ed_basis* b) {
 
 template <typename T>
 static ed_status prepare_t(const ed_basis* b) {
-  if (rows_usable<T>(b)) return ED_OK;  // (that launch looks after itself)
+  if (rows_usable<T>(b, true)) return ED_OK;  // (that launch looks after itself)
   const size_t lim = (size_t)max_smem_optin();
   if (staged_smem<T, 2>(b) <= lim && b->up.dim >= 2) return set_smem_attr<T, 2>(b);
   if (staged_smem<T, 1>(b) <= lim) return set_smem_attr<T, 1>(b);

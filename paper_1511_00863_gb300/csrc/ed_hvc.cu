@@ -324,7 +324,7 @@ static int hvc_global_grid(const ed_basis* b) {
 
 template <typename T>
 static ed_status hvc_prepare_t(const ed_basis* b) {
-  if (rows_usable<typename CVec<T>::type>(b)) return ED_OK;  // (that launch looks after itself)
+  if (rows_usable<typename CVec<T>::type>(b, true)) return ED_OK;  // (that launch looks after itself)
   const int R = hvc_rows<T>(b);
   if (R == 2) {
     ED_TRY_CUDA(allow_max_smem(hvc_staged_kernel<T, 2, true>));
@@ -344,7 +344,7 @@ template <typename T>
 ed_status launch_hvc(const ed_basis* b, double t, double U, const void* x, void* y, int64_t ld,
                      cudaStream_t s, const LzHvArgs* lz, int* grid_out) {
   typedef typename CVec<T>::type V;
-  if (rows_usable<V>(b)) return launch_hv_rows<V>(b, t, U, (const V*)x, (V*)y, ld, s, lz, grid_out);
+  if (rows_usable<V>(b, lz != nullptr)) return launch_hv_rows<V>(b, t, U, (const V*)x, (V*)y, ld, s, lz, grid_out);
   const HvcArgs a = hvc_args(b, t, U, ld);
   const LzHvArgs none{nullptr, 0, nullptr};
   const int R = hvc_rows<T>(b);

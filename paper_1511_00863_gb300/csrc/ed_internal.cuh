@@ -215,7 +215,7 @@ struct LzStore {
 // Row-ordered H.v (ed_rows.cu): tables built with the basis (rows_plan: classes of the host amplitudes
 // t_bond, or NULL; rows_build enqueues the rest);
 // E = float, double, float2 or double2 (complex). Preferred to launch_hv / launch_hvc where
-// rows_usable.
+// rows_usable (lz: the Lanczos-fused form).
 struct RowsPlan {
   int C = 0;                 // hop classes, 0: no tables
   std::vector<double2> amp;  // [C]
@@ -226,7 +226,7 @@ void rows_plan(int n_sites, int n_up, int n_dn, const double* t_bond, int n_bond
 ed_status rows_build(ed_basis* b, RowsPlan& p, cudaStream_t s);
 void rows_free(ed_basis* b);
 template <typename E>
-bool rows_usable(const ed_basis* b);
+bool rows_usable(const ed_basis* b, bool lz);
 template <typename E>
 ed_status launch_hv_rows(const ed_basis* b, double t, double U, const E* x, E* y, int64_t ld,
                          cudaStream_t s, const LzHvArgs* lz, int* grid_out);
