@@ -59,8 +59,8 @@ typedef enum {
  *                 eigensolve in FP64. Dot products and norms: each thread accumulates its
  *                 products as a compensated FP32 pair (exact product by FMA, error-free
  *                 sums: the Dot2 scheme of Ogita, Rump & Oishi 2005, about twice FP32
- *                 precision), converted to FP64 once per thread and summed in FP64 across
- *                 threads and CTAs.
+ *                 precision, the pair renormalised after every product), converted to FP64
+ *                 once per thread and summed in FP64 across threads and CTAs.
  *  ED_F64_NATIVE  FP64 vectors and FP64 arithmetic throughout (the plain method).
  *  ED_C32         complex vectors (interleaved re, im) of FP32 pairs, complex FP32 H.v
  *                 arithmetic; a_j, b_j (real for Hermitian H), dot products and the
@@ -129,7 +129,7 @@ typedef struct {
  *             see ed_lanczos_schedule); -1 = for bases of at least 2^22 states, the fastest
  *             variant for this basis and dtype, found by timing every variant that fits on
  *             the first run's buffers and remembered by the basis; smaller bases take the
- *             default variant. ED_F64_NATIVE always uses the general kernels.
+ *             default variant. ED_F64_NATIVE and ED_C64 have no fused variants.
  *             Batched solves: see ed_lanczos_solve_batched. */
 typedef struct {
   int32_t max_steps;
@@ -284,10 +284,13 @@ ed_status ed_lanczos_solve_mixed(const ed_basis* basis, const ed_params* params,
                                  double* E0_fp32, int32_t* steps64, double* residual);
 
 /* ed_lanczos_solve_batched - Algorithm 1 for n independent instances (basis i with
- * params[i], a HOST array of n) in one persistent cooperative kernel launch. opts apply to every instance (dtype ED_F32: FP32 vectors and H.v, dot
+ * params[i], a HOST array of n) in one persistent cooperative kernel launch. Its device memory
+ * (two vectors per instance and scalars) comes from the library's pool (see
+ * ed_lanczos_ground_state). opts apply to every instance (dtype ED_F32: FP32 vectors and H.v, dot
  * products as for ED_F32 (compensated FP32 per thread, FP64 across threads); or
  * ED_F64_NATIVE: FP64 vectors and H.v; FP64 a_j, b_j and tridiagonal solve either way;
- * start vector of opts->seed for every instance; reorth 0). The convergence test of opts is evaluated every 4 steps.
+ * start vector of opts->seed for every instance; reorth 0). The convergence test of opts is
+ * evaluated every 4 steps.
  * opts->schedule picks how instances are packed onto groups of CTAs (0..6; 5 sizes groups
  * in proportion to each instance's work per step, 6 to that work times log2 of its
  * dimension, an estimate of its step count); -1 lets the library time every schedule on
@@ -302,7 +305,7 @@ ed_status ed_lanczos_solve_batched(int32_t n, const ed_basis* const* bases,
                                    int32_t* schedule_used);
 
 /* ed_lanczos_solve_batched_mixed - E0 of n independent instances to FP64 accuracy with most
- * steps in FP32, in one persistent cooperative kernel launch (the batched form of
+ * steps in FP32, in three persistent cooperative kernel launches (the batched form of
  * ed_lanczos_solve_mixed). Per instance: Algorithm 1 (Sec. 2.2) in FP32 as in
  * ed_lanczos_solve_batched (opts: dtype ED_F32, max_steps, tol checked every 4 steps, seed,
  * schedule), keeping its Lanczos vectors on the device (Sum_i dim_i x max_steps x 4 bytes,
@@ -324,11 +327,18 @@ ed_status ed_lanczos_solve_batched_mixed(int32_t n, const ed_basis* const* bases
 
 /* ed_lanczos_ground_state - the ground-state vector: Algorithm 1 to convergence (ED_F64
  * only), the eigenvector y of T_m for its lowest eigenvalue (inverse iteration on the
- * device), then the same Lanczos vectors regenerated from f1 and summed, psi = sum_j y_j
- * f_j, exactly in int64 fixed point. psi: DEVICE array of dim FP64, normalised, with the
- * sign fixed so that its largest-magnitude entry (lowest index on ties) is positive. E0 and
- * steps as ed_lanczos_solve. The paper computes E0 only (Sec. 2.2); the vector is the
- * training data of the learned start vector. */
+ * device), and psi = sum_j y_j f_j over the Lanczos vectors, exactly in int64 fixed point.
+ * psi: DEVICE array of dim FP64, normalised, with the sign fixed so that its
+ * largest-magnitude entry (lowest index on ties) is positive. E0 and steps as
+ * ed_lanczos_solve. The paper computes E0 only (Sec. 2.2); the vector is the training data
+ * of the learned start vector.
+ * The run keeps its vectors (8 bytes per element and step) while they fit in half the free
+ * device memory and in 96 GB; the vectors behind the last kept one are made a second time by
+ * the same steps. psi does not depend on how many were kept. The memory comes from a pool of
+ * the library, taken as the run goes on: up to 16 GB of it stay reserved while idle, serve
+ * later calls (batched solves too) and any allocation of the process that needs them, and are
+ * given back with the last basis. Work vectors of up to 1 GB stay with the basis as in
+ * ed_lanczos_solve, larger ones are freed. */
 ed_status ed_lanczos_ground_state(const ed_basis* basis, const ed_params* params,
                                   const ed_opts* opts, const void* f1, void* stream, double* psi,
                                   double* E0, int32_t* steps);

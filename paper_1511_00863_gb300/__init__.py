@@ -429,7 +429,7 @@ def ed_lanczos_solve_batched(bases, ts, Us, opts: ed_opts, stream=None,
 def ed_lanczos_solve_batched_mixed(bases, ts, Us, opts: ed_opts, refine_steps: int = 32,
                                    refine_tol: float = 1e-12, stream=None,
                                    raise_not_converged: bool = True) -> dict:
-    """All instances in one persistent launch: FP32 Lanczos (opts), Ritz vector, FP64
+    """All instances in three persistent launches: FP32 Lanczos (opts), Ritz vectors, FP64
     refinement (see include/ed.h)."""
     n = len(bases)
     arr = (c_void_p * n)(*[b.value if isinstance(b, c_void_p) else b for b in bases])

@@ -198,12 +198,6 @@ __device__ __forceinline__ long long start_int(uint64_t seed, uint64_t i) {
   return (long long)(z >> 11) - (1LL << 52);
 }
 
-// Coefficient c = m * 2^e with m an int64 mantissa, |m| < 2^62 for the largest of a set.
-struct FxCoef {
-  long long m;
-  int e;
-};
-
 // ------------------------------------------------------------------ reductions
 // Block reduction of a 192-bit sum and a max; thread 0 writes out[0..3] =
 // (lo bits 0..63, lo bits 64..127, hi, max).

@@ -382,8 +382,8 @@ __device__ __forceinline__ double block_sum(double v, double* sm) {
 
 // True in the CTA that is the last of its launch to get here (for all its threads); it sees
 // what thread 0 of every other CTA wrote before. The update pass ends in that CTA instead of a
-// launch of its own (the fence and the ticket take 2-4 us, so passes whose CTAs are many or
-// short-lived, the H.v, leave their records to the next pass).
+// launch of its own, the fused H.v on long vectors too (kTicketMin). The fence and the ticket take
+// 2-4 us, so passes with many short-lived CTAs leave their records to the next pass.
 __device__ __forceinline__ bool last_cta(unsigned* ticket) {
   __shared__ int last_s;
   if (threadIdx.x == 0) {

@@ -31,7 +31,7 @@ namespace ed {
 
 // ------------------------------------------------------------------ start vector
 // Element i of the start vector is h_i 2^-52 / ||.||, h_i = (top 53 bits of the (i+1)-th
-// SplitMix64 output) - 2^52 (split_mix, ed_fixed.cuh). Everything per element is integer
+// SplitMix64 output) - 2^52 (start_int, ed_fixed.cuh). Everything per element is integer
 // arithmetic: GB300's FP64 rate made the conversion, the product and the rounding of an element
 // 15-17 ps and its share of the norm 7 ps (2.8 ms of a 166 M element FP32 start).
 
@@ -914,7 +914,7 @@ extern "C" ed_status ed_lanczos_energy(ed_lanczos* st, double* E0, int32_t* step
 
 // ------------------------------------------------------------------ solve
 // ed_lanczos_solve keeps, per basis, one allocated state per (dtype, schedule) and its
-// instantiated two-step graph, so repeated solves skip allocation and capture; a solve that
+// instantiated graph of two to eight steps (lz_graph), so repeated solves skip allocation and capture; a solve that
 // finds the cache busy (another thread) uses a private state instead.
 struct SolveCache {
   std::mutex mu;
