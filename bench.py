@@ -38,9 +38,9 @@ FALLBACK_HBM_GBS = 6800.0
 # the kernel's sources are unchanged since that capture.
 KERNEL_SOURCES = ["paper_1511_00863_gb300/csrc/ed_hv2_kernel.cuh", "paper_1511_00863_gb300/csrc/ed_fixed.cuh",
                   "paper_1511_00863_gb300/csrc/ed_internal.cuh", "paper_1511_00863_gb300/csrc/ed_tables.h"]
-TRAFFIC_SOURCES_SHA256 = "201131d14b9ac948eada79ffce9f0db932fa6b7328fd4a912b449cb07e688f31"
+TRAFFIC_SOURCES_SHA256 = "29060772e34034b306e297f1f04d8b83506a4d72fcf9ed021d5f343f8a27c8cd"
 MEASURED_TRAFFIC = {
-    ("torus4x4_5_5", "f64", 8): {"bytes": 479295232 + 133789696,
+    ("torus4x4_5_5", "f64", 8): {"bytes": 479839744 + 133579264,
                                  "profile": "profiles/hv2_kernel_torus4x4_5_5_int64.md"},
 }
 
@@ -516,7 +516,7 @@ def _hv_roofline(dim, du, dd, tabs, esize, hv_ms, workload, dtype, variant, t_bo
             "kernel": (f"hv2s_kernel variant {variant} (fused Lanczos H.v, rows staged as two slices)"
                        if variant >= 30 else
                        f"hv2_kernel variant {variant} (fused Lanczos H.v)" if variant > 0 else
-                       "general H.v kernels (rows too few for the fused kernel)"),
+                       "row-ordered or general H.v kernels (no fused variant)"),
             "bytes_per_launch": hv_bytes, "launch_ms": hv_ms,
             "peak_source": f"{peak_kind} HBM copy bandwidth"}
 

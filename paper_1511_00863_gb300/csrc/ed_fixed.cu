@@ -392,10 +392,11 @@ __device__ __forceinline__ void fx_psi_records(long long bv, long long bi, const
 }
 
 // P = sum_k round(y_{k+1} s_k 2^60 X_k) over the m stored vectors, two columns per thread, and
-// the records of P. HBM bound: every vector is read once, coalesced, four of them in flight;
-// the element goes to its rank (scattered within its row) once. Against regenerating the
-// vectors (a second run of the m H.v and update passes and a read-modify-write of P per step)
-// the half-filled 14-site ring's 78 vectors of 94 MB take about 1.4 ms instead of 26.
+// the records of P. Every vector is read once, coalesced, four of them in flight; the element goes
+// to its rank (scattered within its row) once. Bound by the ALU (66%: a 128-bit product and a
+// rounding shift per element and vector) before HBM (3.5 TB/s): 24 vectors of 95 MB take 0.66 ms.
+// Against regenerating the vectors (a second run of the m H.v and update passes and a
+// read-modify-write of P per step) the half-filled 14-site ring's 78 take 2.1 ms instead of 26.
 __global__ void __launch_bounds__(kFxThreads)
 fx_psi_sum_kernel(const double* __restrict__ y, int m, LzStore store, int64_t rows, int64_t cols,
                   int64_t ld, const int32_t* __restrict__ rank, long long* __restrict__ P,
