@@ -223,10 +223,18 @@ ed_status rows_build(ed_basis* b, RowsPlan& p, cudaStream_t s) {
   const int C = p.C, nch = (int)((nd + 31) / 32);
   const bool amps = !p.cls.empty();
   // one allocation: amplitudes and classes (from the host), the counts and the sort's second buffer,
-  // the tables. A chunk has a row per hop of a class at most, a bond one hop.
+  // the tables. A chunk has as many rows of a class as one of its columns has hops in it: one per bond
+  // at most, or two where the two directions of a bond are of different classes (complex amplitudes:
+  // columns that hop one way and columns that hop the other can share a chunk).
   HvRows& r = b->rows;
   auto up16 = [](size_t n) { return (n + 15) / 16 * 16; };
-  const size_t rows = (size_t)nch * (amps ? std::min(C * b->dn.maxhops, b->n_bonds) : b->dn.maxhops);
+  int chunk_rows = b->dn.maxhops;
+  if (amps) {
+    int n = 0;
+    for (size_t q = 0; q < p.cls.size(); q += 2) n += (p.cls[q] & 0x7F) == (p.cls[q + 1] & 0x7F) ? 1 : 2;
+    chunk_rows = std::min(C * b->dn.maxhops, n);
+  }
+  const size_t rows = (size_t)nch * chunk_rows;
   const size_t o_cls = up16(C * sizeof(double2)), o_cnt = up16(o_cls + p.cls.size()), o_ucnt = up16(o_cnt + nd * C),
                o_tmp = up16(o_ucnt + (amps ? nu * C : 0)), o_perm = up16(o_tmp + nd * 4),
                o_base = up16(o_perm + 32 * (size_t)nch * 4), o_kc = up16(o_base + nch * 4),
