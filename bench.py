@@ -432,7 +432,7 @@ def batched_study(ed, rel=1e-8):
                     for b, t, U in zip(bases, ts, Us)]
         _mixed()
         mix, t_m = _timed(_mixed)
-        # the batch in FP32 with its FP64 refinement (three cooperative launches in one graph)
+        # the batch in FP32 with its FP64 refinement (three cooperative launches)
         bm_opts = ed.make_opts(max_steps=200, tol=1e-9, seed=4, dtype="f32", schedule=-1)
         def _bmixed():
             return ed.ed_lanczos_solve_batched_mixed(bases, ts, Us, bm_opts, refine_steps=64,
