@@ -292,7 +292,8 @@ ed_status ro_count(const Reorth* r, cudaStream_t s, int* count);
 ed_status ro_ritz_vector(const Reorth* r, const double* y, int m, int64_t dim, int64_t cols,
                          int64_t ld, const int32_t* colpos, double* psi, cudaStream_t s);
 
-// Vectors from this length on let the fused H.v's last CTA finish a_j (a fence and a ticket per
+// Vectors from this length on, of two row groups and more per CTA (hv2_build), let the fused H.v's last
+// CTA finish a_j (a fence and a ticket per
 // CTA and the last one's sum, 6-8 us in all); below, every CTA of the update pass sums the H.v's
 // records first (2-9 us, growing with the waiting memory traffic): H.v + update 440 against 453
 // us on the 4x4 lattice (19 M), 18.5 against 19.5 us on the 12-site ring (48,400). Kernels with
