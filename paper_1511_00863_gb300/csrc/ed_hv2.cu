@@ -295,7 +295,8 @@ static cudaError_t one_wave(K kernel, int threads, Hv2Plan* p) {
   cudaError_t e = allow_max_smem(kernel);
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, p->smem);
-  if (e == cudaSuccess && per_sm >= 1) p->grid = std::min(p->grid, per_sm * sm_count());
+  if (e == cudaSuccess && per_sm >= 1 && !(per_sm == 1 && p->grid < 2 * sm_count()))
+    p->grid = std::min(p->grid, per_sm * sm_count());
   return e;
 }
 
