@@ -333,6 +333,13 @@ ed_status hv2_launch(const Hv2Plan* p, const ed_basis* b, double t, double U, co
 // launch_hvc, the fixed-point kernels, the fused plans): the size of the partial-sum buffer.
 int64_t hv_max_grid(const ed_basis* b);
 
+// +-1 from a sign in bit 31 (a select between two constants lets the compiler form both the sum and the
+// difference, two FP64 instructions)
+__device__ __forceinline__ float sign_one(uint32_t e, float) { return __uint_as_float(0x3F800000u | (e & kSignBit)); }
+__device__ __forceinline__ double sign_one(uint32_t e, double) {
+  return __hiloint2double((int)(0x3FF00000u | (e & kSignBit)), 0);
+}
+
 // ---------------------------------------------------------------- reductions
 // Dot-product accumulator: FP64 for FP64 data; for FP32 data an exact product (FMA
 // error term) fed into a compensated FP32 pair, converted to FP64 once per thread.

@@ -299,11 +299,6 @@ template <> struct RowElem<double> { typedef double T; static constexpr int kWid
 template <> struct RowElem<float2> { typedef float T; static constexpr int kWide = 2; };
 template <> struct RowElem<double2> { typedef double T; static constexpr int kWide = 1; };
 
-// +-1 from a sign in bit 31
-__device__ __forceinline__ float sign_one(uint32_t e, float) { return __uint_as_float(0x3F800000u | (e & kSignBit)); }
-__device__ __forceinline__ double sign_one(uint32_t e, double) {
-  return __hiloint2double((int)(0x3FF00000u | (e & kSignBit)), 0);
-}
 template <typename T> __device__ __forceinline__ void row_mad(T& a, T c, T x) { a = fma(c, x, a); }
 __device__ __forceinline__ void row_mad(float2& a, float c, float2 x) { a.x = fma(c, x.x, a.x), a.y = fma(c, x.y, a.y); }
 __device__ __forceinline__ void row_mad(double2& a, double c, double2 x) { a.x = fma(c, x.x, a.x), a.y = fma(c, x.y, a.y); }
@@ -563,11 +558,12 @@ static ed_status rows_launch(const ed_basis* b, const RowsArgs& a, const E* x, E
 //    560 54 / 46, 12,870 x 1,820 265 / 181. Rows of a multiple of 4 columns (16-byte loads) from 500 on,
 //    others from 1,200 on where rows come in pairs (launch_hv_rows) or from 5,000 on. With few rows
 //    (four CTAs per SM or fewer) the down part's length counts: 120 x 252 5.0 / 4.5, 462 x 330 8.8 / 5.6.
-//  * FP64: 18,564 x 153 120 / 122, 3,003 x 105 18 / 21, 495 x 220 7.4 / 8.9; 1,716 x 286 28 / 22. With few
+//  * FP64: 12,870 x 120 65 / 92, 3,003 x 105 17 / 23, 18,564 x 153 120 / 122, 495 x 220 7.4 / 8.9; 1,716 x 286 28 / 22. With few
 //    rows 252 x 210 6.2 / 6.0, 220 x 220 5.6 / 5.6 (its sums round less), in the Lanczos-fused form 2-4% less.
 //  * complex FP32: 6,435 x 455 50 / 65, 924 x 495 14.5 / 16, 38,760 x 190 127 / 232; 1,287 x 286 11.3 /
 //    10.4, 12,870 x 560 126 / 116. Few rows: 455 x 105 5.2 / 4.4.
-//  * complex FP64: 6,435 x 105 116 / 136, 8,568 x 153 183 / 186; 462 x 165 20 / 15.5; with amplitude
+//  * complex FP64: 3,003 x 105 34 / 66, 12,870 x 120 142 / 275 (8,568 x 153 183 / 186 and 462 x 165 20 / 15.5 while
+//    the row-staged kernel multiplied at every hop); with amplitude
 //    classes (fewer multiply-adds, the bound) 12,870 x 120 already 1,090 / 855.
 template <typename E>
 bool rows_usable(const ed_basis* b, bool lz) {
