@@ -469,6 +469,9 @@ mlp_grad_kernel(const float* __restrict__ params, int L, float U, const uint32_t
       if (k < n) {
         float a = sb3[0], z = sb3[1];
         const float* h = H2 + tid * kLdT;
+        // (unrolled whole, its 192 loads took the registers of the running gradients to local memory: 780
+        // bytes of spills; 16,384 samples 68.6 -> 65.7 us, 2^20 1,474 -> 1,356)
+#pragma unroll 16
         for (int o = 0; o < kH; ++o) {
           a = fmaf(h[o], W3[2 * o], a);
           z = fmaf(h[o], W3[2 * o + 1], z);
