@@ -11,9 +11,11 @@
 //     coalesced along d (consecutive threads own consecutive d);
 //   * the diagonal   y[u,d] += U popc(up[u] & dn[d]) x[u,d]   uses the integer popcount.
 // Rounding: the hops of a species are added with their signs alone, each sum is multiplied once, and the
-// diagonal, often the largest term, comes last: the arithmetic of the row-ordered kernel (ed_rows.cu), bit
-// for bit, whichever of the two a basis takes. (The diagonal first and t with every hop rounded up to
-// half as much again, 2.2e-16 of the result instead of 1.4e-16 in FP64.)
+// diagonal, often the largest term, comes last: the arithmetic of the row-ordered kernel (ed_rows.cu),
+// whichever of the two a basis takes. (The diagonal first and t with every hop rounded up to three times
+// as much: 4.9e-16 of the result instead of 1.4e-16 in FP64, 12,870 x 120 states.)
+#include <cmath>
+
 #include "ed_internal.cuh"
 
 namespace ed {
@@ -28,6 +30,7 @@ struct HvArgs {
   int64_t dim_up, dim_dn, ld;
   int maxhops_up, maxhops_dn;
   double t, U;
+  float Uh, Ul;  // U = Uh + Ul to 48 bits
 };
 
 // acc += coef(entry_k) v_k over a state's hops in table order (the
@@ -67,7 +70,7 @@ __global__ void __launch_bounds__(kHvThreads)
 hv_staged_kernel(HvArgs a, const T* __restrict__ x, T* __restrict__ y, LzHvArgs lz) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[33];
-  __shared__ T diag[kMaxSites + 1];  // U n
+  __shared__ T diag[sizeof(T) == 8 ? kMaxSites + 1 : 1];
   T sc = T(1), bsp = T(0);
   if (kLz) {
     if (lz.S->status != 0) return;
@@ -81,7 +84,15 @@ hv_staged_kernel(HvArgs a, const T* __restrict__ x, T* __restrict__ y, LzHvArgs 
   int32_t* ut = reinterpret_cast<int32_t*>(xs + (size_t)(dn + 1) * R);
   const int64_t u0 = (int64_t)blockIdx.x * R;
   const T tt = (T)a.t;
-  if (threadIdx.x <= kMaxSites) diag[threadIdx.x] = (T)(a.U * (double)threadIdx.x);
+  // U n: FP64 from a table, made by the last warps, which short rows leave without elements to stage. FP32
+  // as n Uh + n Ul, which rounds as U n does: 33 FP64 products and conversions per CTA, or a table from the
+  // host, are seen in a call on 14 columns (7.1 us; 7.7, 7.8).
+  const int dg = (int)threadIdx.x - (kHvThreads - 1 - kMaxSites);
+  if (sizeof(T) == 8 && dg >= 0) diag[dg] = (T)(a.U * (double)dg);
+  auto un = [&](int n) -> T {
+    if constexpr (sizeof(T) == 8) return diag[n];
+    else return fmaf((float)n, a.Uh, (float)n * a.Ul);
+  };
 
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -120,7 +131,7 @@ hv_staged_kernel(HvArgs a, const T* __restrict__ x, T* __restrict__ y, LzHvArgs 
         hv_add_hops(up, ut + r * a.maxhops_up, 1, a.maxhops_up, a.dim_up, [](uint32_t e) { return sign_one(e, T()); },
                     [&](int64_t tg) { return x[tg * a.ld + d]; });
         const T hop = fma(-tt, up, -tt * acc[r]);
-        acc[r] = fma(diag[__popc(ub[r] & db)], xs[d * R + r], hop);
+        acc[r] = fma(un(__popc(ub[r] & db)), xs[d * R + r], hop);
         if (kLz) {
           const T f = sc * xs[d * R + r];
           const T w = sc * acc[r] - bsp * y[u * a.ld + d];
@@ -191,6 +202,8 @@ static HvArgs make_args(const ed_basis* b, double t, double U, int64_t ld) {
   a.maxhops_dn = b->dn.maxhops;
   a.t = t;
   a.U = U;
+  a.Uh = (float)U;
+  a.Ul = std::isfinite(a.Uh) ? (float)(U - (double)a.Uh) : 0.f;
   return a;
 }
 

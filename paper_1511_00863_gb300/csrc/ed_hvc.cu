@@ -16,7 +16,7 @@
 // the Lanczos epilogue (kLz): w = s_cur H B_cur - b_j s_prev B_prev over B_prev, and per-CTA
 // partial sums of Re(w . conj f_j) (the real dot product of the interleaved vectors), so
 // the real Lanczos driver runs unchanged on 2 dim scalars. Without per-bond amplitudes the staged kernel
-// adds the hops with their signs and multiplies once, as the row-ordered kernel does (bit for bit).
+// adds the hops with their signs and multiplies once, as the row-ordered kernel does.
 #include "ed_internal.cuh"
 
 namespace ed {
@@ -162,7 +162,8 @@ hvc_staged_kernel(HvcArgs a, const typename CVec<T>::type* __restrict__ x,
     sc = (T)lz.S->scale[lz.cur];
     bsp = (T)(lz.S->beta[j] * lz.S->scale[1 - lz.cur]);
   }
-  if (threadIdx.x <= kMaxSites) diag[threadIdx.x] = (T)(a.U * (double)threadIdx.x);
+  const int dg = (int)threadIdx.x - (kHvcThreads - 1 - kMaxSites);
+  if (dg >= 0) diag[dg] = (T)(a.U * (double)dg);
   const int dn = (int)a.dim_dn;
   const int MH = a.maxhops_up > 0 ? a.maxhops_up : 1;
   V* xs = reinterpret_cast<V*>(smem);                 // [(dn + 1) * R], zero slot at dn

@@ -558,13 +558,13 @@ static ed_status rows_launch(const ed_basis* b, const RowsArgs& a, const E* x, E
 //    560 54 / 46, 12,870 x 1,820 265 / 181. Rows of a multiple of 4 columns (16-byte loads) from 500 on,
 //    others from 1,200 on where rows come in pairs (launch_hv_rows) or from 5,000 on. With few rows
 //    (four CTAs per SM or fewer) the down part's length counts: 120 x 252 5.0 / 4.5, 462 x 330 8.8 / 5.6.
-//  * FP64: 12,870 x 120 65 / 92, 3,003 x 105 17 / 23, 18,564 x 153 120 / 122, 495 x 220 7.4 / 8.9; 1,716 x 286 28 / 22. With few
-//    rows 252 x 210 6.2 / 6.0, 220 x 220 5.6 / 5.6 (its sums round less), in the Lanczos-fused form 2-4% less.
+//  * FP64: 12,870 x 120 65 / 92, 3,003 x 105 17 / 23, 18,564 x 153 120 / 122, 495 x 220 7.4 / 8.9;
+//    1,716 x 286 28 / 22. With few rows 330 x 165 6.1 / 5.5, 165 x 165 5.3 / 4.9, 153 x 153 3.9 / 4.3, 462 x 165 6.5 / 7.4; in the
+//    Lanczos-fused form the row-staged kernel takes 2-4% less.
 //  * complex FP32: 6,435 x 455 50 / 65, 924 x 495 14.5 / 16, 38,760 x 190 127 / 232; 1,287 x 286 11.3 /
-//    10.4, 12,870 x 560 126 / 116. Few rows: 455 x 105 5.2 / 4.4.
-//  * complex FP64: 3,003 x 105 34 / 66, 12,870 x 120 142 / 275 (8,568 x 153 183 / 186 and 462 x 165 20 / 15.5 while
-//    the row-staged kernel multiplied at every hop); with amplitude
-//    classes (fewer multiply-adds, the bound) 12,870 x 120 already 1,090 / 855.
+//    10.4, 12,870 x 560 126 / 116. Few rows: 330 x 165 5.1 / 4.4, 455 x 105 4.6 / 4.3, 462 x 165 5.5 / 6.2.
+//  * complex FP64: 3,003 x 105 34 / 66, 12,870 x 120 142 / 275 (8,568 x 153 183 / 186 and 462 x 165
+//    20 / 15.5 while the row-staged kernel multiplied at every hop); with amplitude classes (fewer multiply-adds, the bound) 12,870 x 120 already 1,090 / 855.
 template <typename E>
 bool rows_usable(const ed_basis* b, bool lz) {
   const int64_t nd = b->dn.dim, nu = b->up.dim, sms = sm_count();
@@ -573,9 +573,9 @@ bool rows_usable(const ed_basis* b, bool lz) {
     return nd % 4 == 0 ? nd >= 500 || (nd >= 240 && nu <= 4 * sms)
                        : nd >= 5000 || (nd >= 1200 && nu >= 8 * sms) || (nd >= 240 && nu <= 4 * sms);
   else if constexpr (std::is_same<E, double>::value)
-    return nd >= 240 || (nd >= 200 && nu <= 2 * sms && !lz);
+    return nd >= 240 || (nd >= 160 && nu <= 3 * sms && !lz);
   else if constexpr (std::is_same<E, float2>::value)
-    return nu <= 2 * sms || nd >= 1000 || (nd >= 280 && (nd % 2 == 0 || nu <= 4 * sms));
+    return nu <= 3 * sms || nd >= 1000 || (nd >= 280 && (nd % 2 == 0 || nu <= 4 * sms));
   else
     return nd >= 160 || nu <= 2 * sms || b->rows.C > 1;
 }
